@@ -63,11 +63,11 @@ typedef enum {
  * block of rows, a row of V or X, a column of C or Z) is aligned to an
  * exponent at or above its largest and held as a 104-bit integer (four
  * 26-bit limbs; the ten most significant limb products are kept) or, in Gram
- * products with 16 or more columns on one side, as a 105-bit integer of
- * fifteen balanced 7-bit digits whose products are summed on the tensor cores
- * (FP16 integer digits, exact FP32 sums; the 120 most significant digit pairs
- * are kept; a column's alignment exponent sits up to two binades above its
- * largest, so that it rarely has to grow).  Each product then carries an
+ * products with more than 8 columns on one side, as a 110-bit integer of
+ * fourteen 8-bit digits whose products are summed on the tensor cores (FP16
+ * integer digits, exact FP32 sums; the digit pairs of weight 2^-112 of the
+ * largest and above are kept; a column's alignment exponent sits up to two
+ * binades above its largest, so that it rarely has to grow).  Each product then carries an
  * error below 2^-101 max|x| max|y| (integer limbs) or 2^-96 max|x| max|y|
  * (tensor-core digits), the sums of the kept products are exact, and every
  * result is rounded once.  Exact sums are

@@ -9,9 +9,7 @@
 // plain digits D_s in [0, 127], each the FP16 subnormal +-D_s 2^-24 whose bit
 // pattern is the digit with the value's sign, so products of two digits are
 // exact and FP32 sums of fewer than 2^24 units of 2^-48 are exact.  The Gram
-// kernel (umma_gram.cu) uses balanced digits (below), FP16 integers of at
-// most 64 in magnitude (128 for the top digit), whose products are smaller
-// and let its accumulators run longer between drains.
+// kernel (umma_gram.cu) has balanced 8-bit digits of its own.
 #pragma once
 
 #include <cuda.h>
@@ -181,131 +179,65 @@ __device__ __forceinline__ void tmem_ld3(unsigned a0, unsigned a1, unsigned a2, 
   }
 }
 
-// Six groups: three of the accumulators and three of the running sums.
-template <int NY>
-__device__ __forceinline__ void tmem_ld3x2(unsigned a0, unsigned a1, unsigned a2, unsigned b0, unsigned b1,
-                                           unsigned b2, unsigned (&v)[3][NY], unsigned (&w)[3][NY]) {
-  if constexpr (NY == 4) {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%24];\n"
-        "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%4,%5,%6,%7}, [%25];\n"
-        "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%8,%9,%10,%11}, [%26];\n"
-        "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%12,%13,%14,%15}, [%27];\n"
-        "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%16,%17,%18,%19}, [%28];\n"
-        "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%20,%21,%22,%23}, [%29];\n"
-        "tcgen05.wait::ld.sync.aligned;\n"
-        : "=r"(v[0][0]), "=r"(v[0][1]), "=r"(v[0][2]), "=r"(v[0][3]), "=r"(v[1][0]), "=r"(v[1][1]), "=r"(v[1][2]),
-          "=r"(v[1][3]), "=r"(v[2][0]), "=r"(v[2][1]), "=r"(v[2][2]), "=r"(v[2][3]), "=r"(w[0][0]), "=r"(w[0][1]),
-          "=r"(w[0][2]), "=r"(w[0][3]), "=r"(w[1][0]), "=r"(w[1][1]), "=r"(w[1][2]), "=r"(w[1][3]), "=r"(w[2][0]),
-          "=r"(w[2][1]), "=r"(w[2][2]), "=r"(w[2][3])
-        : "r"(a0), "r"(a1), "r"(a2), "r"(b0), "r"(b1), "r"(b2)
-        : "memory");
-  } else {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x2.b32 {%0,%1}, [%12];\n"
-        "tcgen05.ld.sync.aligned.32x32b.x2.b32 {%2,%3}, [%13];\n"
-        "tcgen05.ld.sync.aligned.32x32b.x2.b32 {%4,%5}, [%14];\n"
-        "tcgen05.ld.sync.aligned.32x32b.x2.b32 {%6,%7}, [%15];\n"
-        "tcgen05.ld.sync.aligned.32x32b.x2.b32 {%8,%9}, [%16];\n"
-        "tcgen05.ld.sync.aligned.32x32b.x2.b32 {%10,%11}, [%17];\n"
-        "tcgen05.wait::ld.sync.aligned;\n"
-        : "=r"(v[0][0]), "=r"(v[0][1]), "=r"(v[1][0]), "=r"(v[1][1]), "=r"(v[2][0]), "=r"(v[2][1]), "=r"(w[0][0]),
-          "=r"(w[0][1]), "=r"(w[1][0]), "=r"(w[1][1]), "=r"(w[2][0]), "=r"(w[2][1])
-        : "r"(a0), "r"(a1), "r"(a2), "r"(b0), "r"(b1), "r"(b2)
-        : "memory");
-  }
-}
-// The same loads without the wait; tmem_wait_ld_regs completes them (it names
-// the destination registers so that no use can move above the wait).
-template <int NY>
-__device__ __forceinline__ void tmem_ld3x2_nowait(unsigned a0, unsigned a1, unsigned a2, unsigned b0, unsigned b1,
-                                                  unsigned b2, unsigned (&v)[3][NY], unsigned (&w)[3][NY]) {
-  if constexpr (NY == 4) {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%24];\n"
-        "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%4,%5,%6,%7}, [%25];\n"
-        "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%8,%9,%10,%11}, [%26];\n"
-        "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%12,%13,%14,%15}, [%27];\n"
-        "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%16,%17,%18,%19}, [%28];\n"
-        "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%20,%21,%22,%23}, [%29];\n"
-        : "=r"(v[0][0]), "=r"(v[0][1]), "=r"(v[0][2]), "=r"(v[0][3]), "=r"(v[1][0]), "=r"(v[1][1]), "=r"(v[1][2]),
-          "=r"(v[1][3]), "=r"(v[2][0]), "=r"(v[2][1]), "=r"(v[2][2]), "=r"(v[2][3]), "=r"(w[0][0]), "=r"(w[0][1]),
-          "=r"(w[0][2]), "=r"(w[0][3]), "=r"(w[1][0]), "=r"(w[1][1]), "=r"(w[1][2]), "=r"(w[1][3]), "=r"(w[2][0]),
-          "=r"(w[2][1]), "=r"(w[2][2]), "=r"(w[2][3])
-        : "r"(a0), "r"(a1), "r"(a2), "r"(b0), "r"(b1), "r"(b2)
-        : "memory");
-  } else {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x2.b32 {%0,%1}, [%12];\n"
-        "tcgen05.ld.sync.aligned.32x32b.x2.b32 {%2,%3}, [%13];\n"
-        "tcgen05.ld.sync.aligned.32x32b.x2.b32 {%4,%5}, [%14];\n"
-        "tcgen05.ld.sync.aligned.32x32b.x2.b32 {%6,%7}, [%15];\n"
-        "tcgen05.ld.sync.aligned.32x32b.x2.b32 {%8,%9}, [%16];\n"
-        "tcgen05.ld.sync.aligned.32x32b.x2.b32 {%10,%11}, [%17];\n"
-        : "=r"(v[0][0]), "=r"(v[0][1]), "=r"(v[1][0]), "=r"(v[1][1]), "=r"(v[2][0]), "=r"(v[2][1]), "=r"(w[0][0]),
-          "=r"(w[0][1]), "=r"(w[1][0]), "=r"(w[1][1]), "=r"(w[2][0]), "=r"(w[2][1])
-        : "r"(a0), "r"(a1), "r"(a2), "r"(b0), "r"(b1), "r"(b2)
-        : "memory");
-  }
-}
-template <int NY>
-__device__ __forceinline__ void tmem_wait_ld_regs(unsigned (&v)[3][NY], unsigned (&w)[3][NY]) {
-  if constexpr (NY == 4) {
-    asm volatile("tcgen05.wait::ld.sync.aligned;"
-                 : "+r"(v[0][0]), "+r"(v[0][1]), "+r"(v[0][2]), "+r"(v[0][3]), "+r"(v[1][0]), "+r"(v[1][1]),
-                   "+r"(v[1][2]), "+r"(v[1][3]), "+r"(v[2][0]), "+r"(v[2][1]), "+r"(v[2][2]), "+r"(v[2][3]),
-                   "+r"(w[0][0]), "+r"(w[0][1]), "+r"(w[0][2]), "+r"(w[0][3]), "+r"(w[1][0]), "+r"(w[1][1]),
-                   "+r"(w[1][2]), "+r"(w[1][3]), "+r"(w[2][0]), "+r"(w[2][1]), "+r"(w[2][2]), "+r"(w[2][3])
-                 :
-                 : "memory");
-  } else {
-    asm volatile("tcgen05.wait::ld.sync.aligned;"
-                 : "+r"(v[0][0]), "+r"(v[0][1]), "+r"(v[1][0]), "+r"(v[1][1]), "+r"(v[2][0]), "+r"(v[2][1]),
-                   "+r"(w[0][0]), "+r"(w[0][1]), "+r"(w[1][0]), "+r"(w[1][1]), "+r"(w[2][0]), "+r"(w[2][1])
-                 :
-                 : "memory");
-  }
-}
-template <int NY>
-__device__ __forceinline__ void tmem_st3(unsigned a0, unsigned a1, unsigned a2, const unsigned (&v)[3][NY]) {
-  if constexpr (NY == 4) {
-    asm volatile(
-        "tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%3,%4,%5,%6};\n"
-        "tcgen05.st.sync.aligned.32x32b.x4.b32 [%1], {%7,%8,%9,%10};\n"
-        "tcgen05.st.sync.aligned.32x32b.x4.b32 [%2], {%11,%12,%13,%14};\n" ::"r"(a0),
-        "r"(a1), "r"(a2), "r"(v[0][0]), "r"(v[0][1]), "r"(v[0][2]), "r"(v[0][3]), "r"(v[1][0]), "r"(v[1][1]),
-        "r"(v[1][2]), "r"(v[1][3]), "r"(v[2][0]), "r"(v[2][1]), "r"(v[2][2]), "r"(v[2][3])
-        : "memory");
-  } else {
-    asm volatile(
-        "tcgen05.st.sync.aligned.32x32b.x2.b32 [%0], {%3,%4};\n"
-        "tcgen05.st.sync.aligned.32x32b.x2.b32 [%1], {%5,%6};\n"
-        "tcgen05.st.sync.aligned.32x32b.x2.b32 [%2], {%7,%8};\n" ::"r"(a0),
-        "r"(a1), "r"(a2), "r"(v[0][0]), "r"(v[0][1]), "r"(v[1][0]), "r"(v[1][1]), "r"(v[2][0]), "r"(v[2][1])
-        : "memory");
-  }
-}
-// Zeros into three column blocks of NY columns (one zero register for all).
-template <int NY>
-__device__ __forceinline__ void tmem_zero3(unsigned a0, unsigned a1, unsigned a2) {
-  const unsigned z = 0u;
-  if constexpr (NY == 4) {
-    asm volatile(
-        "tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%3,%3,%3,%3};\n"
-        "tcgen05.st.sync.aligned.32x32b.x4.b32 [%1], {%3,%3,%3,%3};\n"
-        "tcgen05.st.sync.aligned.32x32b.x4.b32 [%2], {%3,%3,%3,%3};\n" ::"r"(a0),
-        "r"(a1), "r"(a2), "r"(z)
-        : "memory");
-  } else {
-    asm volatile(
-        "tcgen05.st.sync.aligned.32x32b.x2.b32 [%0], {%3,%3};\n"
-        "tcgen05.st.sync.aligned.32x32b.x2.b32 [%1], {%3,%3};\n"
-        "tcgen05.st.sync.aligned.32x32b.x2.b32 [%2], {%3,%3};\n" ::"r"(a0),
-        "r"(a1), "r"(a2), "r"(z)
-        : "memory");
-  }
-}
 __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+
+// N consecutive TMEM columns of this warp's 32 lanes (N = 8 or 16).
+template <int N>
+__device__ __forceinline__ void tmem_ldn(unsigned a, unsigned (&v)[N]) {
+  if constexpr (N == 16) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]), "=r"(v[8]),
+          "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
+        : "r"(a)
+        : "memory");
+  } else {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
+                 : "r"(a)
+                 : "memory");
+  }
+}
+// Completes the loads into v (named, so that no use can move above the wait).
+template <int N>
+__device__ __forceinline__ void tmem_waitn(unsigned (&v)[N]) {
+  if constexpr (N == 16) {
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+r"(v[0]), "+r"(v[1]), "+r"(v[2]), "+r"(v[3]), "+r"(v[4]), "+r"(v[5]), "+r"(v[6]), "+r"(v[7]),
+                   "+r"(v[8]), "+r"(v[9]), "+r"(v[10]), "+r"(v[11]), "+r"(v[12]), "+r"(v[13]), "+r"(v[14]), "+r"(v[15])
+                 :
+                 : "memory");
+  } else {
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+r"(v[0]), "+r"(v[1]), "+r"(v[2]), "+r"(v[3]), "+r"(v[4]), "+r"(v[5]), "+r"(v[6]), "+r"(v[7])
+                 :
+                 : "memory");
+  }
+}
+template <int N>
+__device__ __forceinline__ void tmem_stn(unsigned a, const unsigned (&v)[N]) {
+  if constexpr (N == 16) {
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};" ::"r"(a),
+        "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]), "r"(v[8]), "r"(v[9]),
+        "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]), "r"(v[15])
+        : "memory");
+  } else {
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"r"(a), "r"(v[0]), "r"(v[1]),
+                 "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7])
+                 : "memory");
+  }
+}
+template <int N>
+__device__ __forceinline__ void tmem_zeron(unsigned a) {
+  const unsigned z = 0u;
+  if constexpr (N == 16)
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1};" ::"r"(a),
+                 "r"(z)
+                 : "memory");
+  else
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%1,%1,%1,%1,%1,%1,%1};" ::"r"(a), "r"(z) : "memory");
+}
 
 __device__ __forceinline__ void mbar_arrive_expect_tx(unsigned bar, unsigned bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
@@ -406,47 +338,6 @@ __device__ __forceinline__ unsigned pair_word(const PairLanes& p, unsigned signs
   asm("lop3.b32 %0, %1, %2, %3, 0xEA;" : "=r"(w) : "r"(zs), "n"(0x007f007fu), "r"(signs));
   return w;
 }
-// The 15 digit words of two consecutive rows (low half: row r, high half:
-// row r + 1) into their slabs, slab s at dst + s * stride.
-template <int S>
-__device__ __forceinline__ void store_digits(unsigned char* dst, unsigned stride, const PairLanes& p,
-                                             unsigned signs) {
-  if constexpr (S < NS) {
-    *reinterpret_cast<unsigned*>(dst + S * stride) = pair_word<S>(p, signs);
-    store_digits<S + 1>(dst, stride, p, signs);
-  }
-}
-
-// Balanced digits.  With B = sum_s 64 * 2^(98 - 7s) (64 in every digit
-// place), X' = X + B has 7-bit fields f_s in [0, 127] for s >= 1 and a top
-// field f_0 = X' >> 98 in [0, 192] (X < 2^105), and
-//   X = sum_s (f_s - 64) 2^(98 - 7s),   D_s = f_s - 64,
-// so D_s is in [-64, 63] for s >= 1 and in [-64, 128] for s = 0: products
-// of two digits are at most 2^12 (2^13 with D_0, 2^14 for D_0^2) instead of
-// 127^2 for unsigned 7-bit digits.  On the tensor cores a digit is the FP16
-// integer sign(x) D_s: the field is placed in the significand of the FP16
-// 1024 (bit pattern 0x6400 | f, the value 1024 + f), and one f16x2 FMA
-// forms sign * (1024 + f) - sign * 1088 = sign (f - 64) exactly (integers
-// below 2048 are exact in FP16).
-constexpr unsigned kBias0 = 0x08102040u, kBias1 = 0x40810204u, kBias2 = 0x04081020u, kBias3 = 0x102u;
-__device__ __forceinline__ void add_bias(unsigned (&w)[4]) {
-  asm("add.cc.u32 %0, %0, %4;\n\t"
-      "addc.cc.u32 %1, %1, %5;\n\t"
-      "addc.cc.u32 %2, %2, %6;\n\t"
-      "addc.u32 %3, %3, %7;"
-      : "+r"(w[0]), "+r"(w[1]), "+r"(w[2]), "+r"(w[3])
-      : "n"(kBias0), "n"(kBias1), "n"(kBias2), "n"(kBias3));
-}
-// add_bias for X with its low word zero (a value within 20 binades of A):
-// the low word becomes the bias's own and carries nothing.
-__device__ __forceinline__ void add_bias_near(unsigned (&w)[4]) {
-  w[0] = kBias0;
-  asm("add.cc.u32 %0, %0, %3;\n\t"
-      "addc.cc.u32 %1, %1, %4;\n\t"
-      "addc.u32 %2, %2, %5;"
-      : "+r"(w[1]), "+r"(w[2]), "+r"(w[3])
-      : "n"(kBias1), "n"(kBias2), "n"(kBias3));
-}
 // The FP16 exponent field of 1024 in both halves, as a register (so that
 // the digit's mask and this constant fit one three-input logic operation).
 __device__ __forceinline__ unsigned exp1024x2() {
@@ -459,49 +350,5 @@ __device__ __forceinline__ unsigned hfma2(unsigned a, unsigned b, unsigned c) {
   asm("fma.rn.f16x2 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(c));
   return d;
 }
-// Signs of a pair (bit 15: value a, bit 31: value b) -> the f16x2 factors
-// (+-1, +-1) and addends (-+1088, -+1088) of the digit FMA.
-struct PairSign {
-  unsigned mul, add, e1024;
-};
-__device__ __forceinline__ PairSign pair_sign(unsigned signs, unsigned e1024) {
-  return PairSign{0x3C003C00u | signs, 0xE440E440u ^ signs, e1024};
-}
-// Balanced digit word of slab S for the pair (lanes of X'): low half value a,
-// high half value b, both FP16 integers sign * D_S.
-template <int S>
-__device__ __forceinline__ unsigned bal_word(const PairLanes& p, PairSign sg) {
-  constexpr int q = 98 - 7 * S, k = q >> 4, o = q & 15;
-  constexpr unsigned m = S == 0 ? 0x00ff00ffu : 0x007f007fu;  // the top field has 8 bits
-  constexpr bool low = o <= (S == 0 ? 8 : 9);
-  constexpr int sh = low ? o : o - 8;
-  const unsigned z = low ? p.Z[k] : p.Z8[k];
-  // the shift as a high-half multiplication (the FMA pipe), then one
-  // three-input logic operation (z & m) | e1024 (the ALU)
-  unsigned zs = z, f;
-  if constexpr (sh > 0) asm("mul.hi.u32 %0, %1, %2;" : "=r"(zs) : "r"(z), "n"(1u << (32 - sh)));
-  asm("lop3.b32 %0, %1, %2, %3, 0xEA;" : "=r"(f) : "r"(zs), "n"(m), "r"(sg.e1024));
-  return hfma2(f, sg.mul, sg.add);
-}
-template <int S>
-__device__ __forceinline__ void store_bal_digits(unsigned char* dst, unsigned stride, const PairLanes& p,
-                                                 PairSign sg) {
-  if constexpr (S < NS) {
-    *reinterpret_cast<unsigned*>(dst + S * stride) = bal_word<S>(p, sg);
-    store_bal_digits<S + 1>(dst, stride, p, sg);
-  }
-}
-// The same for a pair whose X have their low 32 bits zero (add_bias_near):
-// the fields of slabs 11..14 (bits 0..27) are then the bias's, so those
-// digits are zero.
-template <int S>
-__device__ __forceinline__ void store_bal_digits_near(unsigned char* dst, unsigned stride, const PairLanes& p,
-                                                      PairSign sg) {
-  if constexpr (S < NS) {
-    *reinterpret_cast<unsigned*>(dst + S * stride) = S >= 11 ? 0u : bal_word<S>(p, sg);
-    store_bal_digits_near<S + 1>(dst, stride, p, sg);
-  }
-}
-
 }  // namespace umma
 }  // namespace eo

@@ -6,12 +6,15 @@
 // run on the tensor cores:
 //
 //  * each value x of a column is aligned to the column's alignment exponent
-//    A and held as X = floor(|x| 2^(1127 - A)) < 2^105, written with 15
-//    balanced digits, X = sum_s D_s 2^(98 - 7s), D_s in [-64, 63] (D_0 in
-//    [-64, 128]; umma.cuh: the fields of X + sum_s 64 2^(98 - 7s), less 64);
-//  * a digit is the FP16 integer sign(x) D_s, so every product of two digits
-//    is an integer of at most 2^12 (2^14 for the two top digits) and FP32
-//    sums of such products are exact while they stay within 2^24;
+//    A and held as X = floor(|x| 2^(1132 - A)) < 2^110, written with 14
+//    balanced base-256 digits, X = sum_s D_s 2^(104 - 8s), D_s in [-128, 127]
+//    (D_0 in [0, 65]; the fields of X + sum_s 128 2^(104 - 8s), less 128);
+//  * a digit is the FP16 integer sign(x) D_s, so a product of two digits is
+//    an integer of at most 2^14 and FP32 sums of up to 1024 such products are
+//    exact;
+//  * a value within 25 binades of A has digits 10..13 zero (its X has a zero
+//    low word); panels whose values all are such ("near", nearly always)
+//    store and multiply only ten digit slabs;
 //  * a column's alignment exponent starts at the first panel's largest
 //    exponent plus EO_GRAM_HEADROOM binades and grows (to the new largest
 //    exponent plus the headroom) only when a value's exponent exceeds it:
@@ -23,40 +26,68 @@
 //    the Y slabs t = 0 .. T-1 (N = T x kyp) and writes at TMEM column offset
 //    J q kyp, so the product of slabs s = Jq + j and t lands in column block
 //    c = Jq + t of lane block j: column block c of lane block j collects the
-//    digit diagonal d = c + j, and the 120 digit pairs with d <= 14 take
-//    15 / J + 1 MMAs per 16 rows;
-//  * every R rows (R such that no accumulator can exceed 2^24 in magnitude:
-//    the largest per-row sum of digit-pair bounds that a column block
-//    collects, group_bound below) the accumulators are read back
-//    (tcgen05.ld), converted to integers, added to 32-bit running sums per
-//    (lane, column) and set back to zero; a group of three column blocks
-//    whose per-row bound is smaller is drained only every 2nd, 4th or 8th
-//    time.  The running sums are folded into a 128-bit total W in the units
-//    of the integer engine (value = W 2^(Ax + Ay - 2148)) every 8192 rows,
-//    before an alignment exponent grows, and at the end.  The row-chunk
-//    partials go through the same exact, order-free reduction
+//    digit diagonal d = c + j; pairs with d > 14 are dropped;
+//  * a symmetric 16-column product needs one MMA per 16 rows (q = 0): with
+//    U(i, j) the sum of its column blocks c <= 7 and V(i, j) that of c >= 8
+//    (s <= 7, t >= 8), the pairs with s >= 8 are those of V transposed, and
+//    G(i, j) = U(i, j) + V(i, j) + V(j, i);
+//  * before an accumulator can exceed 2^24 in magnitude (group_pairs below)
+//    the accumulators are read back (tcgen05.ld), converted to integers,
+//    added to 32-bit running sums per (lane, column) kept in TMEM and set
+//    back to zero.  The running sums are folded into a 128-bit total W in the
+//    units of the integer engine (value = W 2^(Ax + Ay - 2148)) every
+//    kFoldDrains drains, before an alignment exponent grows, and at the end.
+//    The row-chunk partials go through the same exact, order-free reduction
 //    (fx_gram_reduce).
 //
-// Error per product x y: the dropped digit pairs (d >= 15) weigh less than
-// 14.2 * 2^103 units^2 (units of 2^(Ax - 1127), 2^(Ay - 1127)), and a value
-// more than 52 binades below A is truncated by less than one unit; with
-// max|x| >= 2^(104 - h) units for a headroom h, the error is below
-// 22.2 * 2^(2h - 105) max|x| max|y| (h = 2: 2^-96.5).  Pipeline per CTA (one
-// per SM): TMA loads
-// of the FP64 panels (128-byte swizzle, two panels ahead), conversion of
-// panel p into one of two digit buffers while the tensor cores run panel
-// p-1, one warp issuing the MMAs and committing them to an mbarrier per
-// buffer.  Every wait is bounded; a wait that runs out marks the partials
-// non-finite, so the result is NaN.  Inputs that TMA cannot address (a base
-// address not 16-byte aligned or an odd leading dimension) are copied by the
-// converter threads themselves with cp.async (the DIRECT variant).
+// Error per product x y: the dropped digit pairs (d >= 15, twelve of weight
+// 2^88 and fewer of smaller weights, each product at most 2^14) sum to less
+// than 2^105.7 units^2 (units of 2^(Ax - 1132), 2^(Ay - 1132)), and a value
+// more than 57 binades below A is truncated by less than one unit, 2^110 for
+// a product; with max|x| >= 2^(109 - h) units for a headroom h the error is
+// below 2^(2h - 107) max|x| max|y| (h = 2: 2^-103), under the 2^-96 that
+// include/eo.h states.
+//
+// Pipeline per CTA (one per SM, 16 warps of 128 registers): the values of a
+// panel of P rows arrive by TMA (two panels ahead, 16-row boxes with 128-byte
+// swizzle).  A converter thread owns eight consecutive rows of one column of
+// every panel, so that its column's alignment exponent stays in a register and
+// its digits of a slab are one 16-byte shared-memory store (one row of a core
+// matrix: eight lanes fill one, no bank conflicts).  Per panel it cuts its
+// values as if they were near, takes the next panel's values from the staging
+// buffer and looks whether they are (one unsigned range test), and, once every
+// warp has stored the previous panel, stores its digits into the buffer that
+// the MMAs of two panels ago have released, drains its share of the
+// accumulators when due, and arrives; the sixteenth warp then issues the
+// panel's MMAs and the copies of the panel after the next.  A panel that was
+// seen to hold a value above its column's exponent, a zero, or a value below
+// the near window sends every warp through a slower branch with barriers:
+// exponents grow, zeros are masked, and with a value below the window the
+// panel is stored and multiplied in parts with all 14 slabs.  Every wait is
+// bounded; a wait that runs out marks the partials non-finite, so the result
+// is NaN.  Operands that TMA cannot address (a base not 16-byte aligned, an
+// odd leading dimension, FP32) are copied by the converter threads with
+// cp.async into the same places.
+//
+// What bounds it: issue and latency of the digit conversion (ALU pipe 48 % of
+// active cycles, issue 51 %, tensor pipe 29 %, shared-memory data pipe 56 % of
+// its wavefronts), not DRAM (30 %).  8-bit digits cost two ALU operations per
+// pair of values and two digits (a byte permutation, or a masked merge, and an
+// f16x2 FMA on the other pipe each) where 7-bit digits took three, and ten
+// stored slabs instead of fifteen.  Measured, 4e6 rows against the 7-bit form
+// (15 slabs, items of two rows, 19 converter warps): V^T Y 64 x 16 1.41 -> 1.04
+// ms (2.5 TB/s), X^T X 16 columns 0.395 -> 0.283, 64 columns (strips) 4.6 ->
+// 3.06.  Tried and slower: loads straight into registers (each 128-bit load
+// costs 20 wavefronts of the shared data pipe: 1.30 ms), one bulk copy per
+// column (80 a panel: 2.41 ms), four warps that only drain (each drain takes
+// one of them 3,600 cycles, which the MMAs wait for: 1.08 ms), a barrier per
+// panel over all warps (1.20 ms).
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
 #include <algorithm>
 #include <cstdlib>
 #include <mutex>
-#include <type_traits>
 
 #include "common.cuh"
 #include "fx.cuh"
@@ -68,55 +99,81 @@ namespace {
 using namespace fx;
 using namespace umma;
 
-// 19 converter warps and the MMA warp: five warps per SM sub-partition, so
-// that each may hold 96 registers (a sixth warp on one of them caps every
-// thread at 80, and the kernel spills).
-#ifndef EO_GRAM_CONV_WARPS
-#define EO_GRAM_CONV_WARPS 19
-#endif
-constexpr int kConvWarps = EO_GRAM_CONV_WARPS;  // staging and conversion (16 to 19)
-constexpr int kDrainWarps = 16;  // the first 16 also drain TMEM: 4 per lane quarter
-constexpr int kConvThreads = 32 * kConvWarps;
-constexpr int kThreads = kConvThreads + 32;  // plus one MMA-issuing warp
-static_assert(kConvWarps >= kDrainWarps, "every drain warp converts");
-constexpr int kLanes = 128;   // MMA M = TMEM lanes
-constexpr int kMaxItems = 3;  // items (two rows of one column) per thread and panel
+constexpr int kConvWarps = 15;              // convert
+constexpr int kWarps = kConvWarps + 1;      // all drain TMEM (4 per lane quarter); the last issues MMAs and copies
+constexpr int kThreads = 32 * kWarps;
+constexpr int kIssuer = 32 * kConvWarps;    // the thread that issues the MMAs
+constexpr int kLanes = 128;                   // MMA M = TMEM lanes
+constexpr int kNear = 10, kAll = 14;          // digit slabs of a near panel, of any panel
+constexpr int kDiag = 14;                     // last digit diagonal kept
 constexpr int kOffsetDigits = 2148;
-constexpr int kFoldRows = 8192;  // rows between folds of the 32-bit running sums
+// Running sums grow by at most 2^24 per drain: exact in 32 bits for 127.
+constexpr int kFoldDrains = 96;
+constexpr int kPairRows = 1024;  // digit products of magnitude <= 2^14 that an FP32 accumulator holds exactly
 constexpr size_t kSmemCap = 225 * 1024;
 // Binades of headroom above a column's largest exponent when its alignment
 // exponent is set (see the error bound above).
 #ifndef EO_GRAM_HEADROOM
 #define EO_GRAM_HEADROOM 2
 #endif
+constexpr int kNearBits = 25;  // values within this many binades of A have a zero low word
 
-struct UPlan {
-  int kxp, kyp, J, nq;  // X tile width (J = 128 / kxp lane blocks), Y tile width, MMAs per k-step
-  int ntx, nty;         // tiles over X and Y columns
-  int shared;           // X and Y are one matrix held once (symmetric, kx <= 16)
-  int P;                // rows per panel (multiple of 16)
-  int drain_panels;     // panels accumulated in TMEM between drains
-  int fold_drains;      // drains between folds of the running sums
-  int drain_log;        // 3 bits per group g of column blocks 3g..3g+2: log2 of the drains it may skip + 1
-  int nslots;           // staged columns per CTA
-  unsigned dig_bytes;   // one digit buffer (A part, then B part unless shared)
-  unsigned a_bytes;     // A part of a digit buffer
-  unsigned stage_bytes; // one staging buffer: P / 16 TMA boxes of X (16 rows x kxp), then of Y
+// Digit pairs per row that a column block of any lane block collects at most,
+// with ns digits per value: pairs (s, t) = (J q + j, c - J q), all < ns.
+constexpr int group_pairs(int J, int ns, int nq) {
+  int worst = 0;
+  for (int c = 0; c <= kDiag; ++c)
+    for (int j = 0; j < J; ++j) {
+      int b = 0;
+      for (int q = 0; q < nq; ++q)
+        if (J * q + j < ns && c - J * q >= 0 && c - J * q < ns) ++b;
+      worst = b > worst ? b : worst;
+    }
+  return worst;
+}
+
+// Geometry of one tile: KXP X columns by KYP Y columns; SHARED: Y = X (one
+// operand held, 16 columns).  A warp converts 16 columns by 16 rows.
+template <int KXP_, int KYP_, bool SHARED_>
+struct Geo {
+  static constexpr int KXP = KXP_, KYP = KYP_;
+  static constexpr bool SHARED = SHARED_;
+  static constexpr int COLS = KXP + (SHARED ? 0 : KYP);             // columns held
+  static constexpr int NCG = (COLS + 15) / 16;                      // groups of 16 columns
+  static constexpr int J = kLanes / KXP;                            // X slabs per MMA
+  static constexpr int NQN = SHARED ? 1 : (kNear + J - 1) / J;      // MMAs per 16 rows, near panels
+  static constexpr int NQA = SHARED ? 1 : (kAll + J - 1) / J;       // any panel
+  static constexpr int SAN = SHARED ? kNear : NQN * J;              // X slabs held (the last ones zero), near
+  static constexpr int SAA = SHARED ? kAll : NQA * J;               // any
+  // A K chunk (8 rows) of an operand holds its slabs' columns, 16 bytes each, slab after slab.
+  static constexpr unsigned LAN = 16u * SAN * KXP, LBN = SHARED ? 0u : 16u * kNear * KYP;
+  static constexpr unsigned LAA = 16u * SAA * KXP, LBA = SHARED ? 0u : 16u * kAll * KYP;
+  static constexpr unsigned up1024(unsigned b) { return (b + 1023u) & ~1023u; }
+  static constexpr size_t bytes(int p) {  // two digit buffers, two staging buffers, two exponents a column
+    return up1024(2u * (LAN + LBN) * (p / 8)) + 2 * (size_t)up1024(8u * COLS * p) + 2 * sizeof(int) * COLS;
+  }
+  // rows per panel that fit the warps and shared memory
+  static constexpr int rows() {
+    int p = 16;
+    while (NCG * (p + 16) / 16 <= kConvWarps && bytes(p + 16) <= kSmemCap) p += 16;
+    return p;
+  }
 };
-
-// ------------------------------------------------------------ kernel
-// Warps 0..kConvWarps-1 stage, scan and convert (named barrier 1), the
-// first 16 of them also drain TMEM; warp kConvWarps issues the MMAs: per
-// panel p it waits for ready[p & 1] (one arrival per converter thread: the
-// digits of p are in buffer p & 1 and TMEM is drained if due), issues the
-// MMAs and commits them to full[p & 1], which the converters wait on before
-// they reuse the buffer (panel p + 2) or read TMEM.
-// DIRECT: the operands cannot be read by TMA (a leading dimension that is
-// not a whole number of 16-byte units, or a base that is not 16-byte
-// aligned): every converter thread then copies its own items of panel p + 2
-// into private shared-memory slots with 8-byte cp.async (zeros beyond the
-// matrix) and reads them back at panel p; the rest is the same.
-constexpr unsigned kDirectStageBytes = 2u * kMaxItems * kConvThreads * 16u;
+template <int KXP_, int KYP_, bool SHARED_>
+struct Plan : Geo<KXP_, KYP_, SHARED_> {
+  using B = Geo<KXP_, KYP_, SHARED_>;
+  static constexpr int P = B::rows();
+  static constexpr unsigned b_off = B::LAN * (P / 8), dig_bytes = (B::LAN + B::LBN) * (P / 8);
+  static constexpr unsigned stage_off = B::up1024(2 * dig_bytes), copy_bytes = 8u * B::COLS * P, stage_bytes = B::up1024(copy_bytes);
+  // A panel with all slabs is multiplied in NF steps of at most FK K steps (16 rows)
+  static constexpr int FK = (int)(dig_bytes / (2 * (B::LAA + B::LBA))), NF = (P / 16 + FK - 1) / FK;
+  static constexpr unsigned b_off_all = B::LAA * (2 * FK);
+  static constexpr int pairs_near = group_pairs(B::J, kNear, B::NQN), pairs_all = group_pairs(B::J, kAll, B::NQA);
+  static constexpr size_t smem = B::bytes(P) + 1024;
+  static_assert(FK >= 1 && P * pairs_near <= kPairRows && 16 * FK * pairs_all <= kPairRows, "a step fits the accumulators");
+  static_assert(2 * (size_t)dig_bytes >= (SHARED_ ? 2u : 1u) * (size_t)kLanes * KYP_ * 16, "final sums fit the digit buffers");
+  static_assert(dig_bytes % 16 == 0 && B::LAA / 16 < (1u << 14), "descriptor strides");
+};
 
 // An FP32 value widened to FP64 exactly in integer arithmetic (the FP64
 // conversion unit is slow on this GPU); zeros, subnormals, infinities and
@@ -128,89 +185,225 @@ __device__ __forceinline__ double widen(float f) {
   return __hiloint2double((int)((b & 0x80000000u) | ((e + 896u) << 20) | ((b & 0x7fffffu) >> 3)), (int)(b << 29));
 }
 
-// PAD: the tile has padded columns (beyond kx or ky, e.g. kx = 40 in a
-// 64-column plan): their digits are zeroed once and never converted.
-// T: the element type of X and Y; FP32 (the EO_F32 mode) only with DIRECT
-// loads, every value widened to FP64 exactly as it is read.  KXPC, PC: the
-// plan's X tile width and panel rows when known at compile time (the hot
-// plans: slab strides become immediate store offsets), 0 = from the plan.
-template <int KYP, bool DIRECT, bool PAD, typename T = double, int KXPC = 0, int PC = 0>
+// Bias of the balanced digits: 128 in each of the digit places 1..13 (bits
+// 0..103); the top digit is not negative and takes none.
+constexpr unsigned kB = 0x80808080u, kBTop = 0x80u;
+
+// Words 1..3 of X + bias for a value within kNearBits binades of A (X's word 0
+// is zero): the significand times 2^bo, bo = t - 32 with X = m 2^t, t = 57 - A
+// + e, so bo is in [0, 25].  bo has the sign bit (above the exponent field)
+// added as 2^11; shifts take their amount modulo 32.  cA = 25 - A.
+// ZERO: a value that is zero gives X = 0 (else the implicit bit would stand).
+template <bool ZERO>
+__device__ __forceinline__ void near_words(double x, int cA, unsigned& w1, unsigned& w2, unsigned& w3) {
+  const unsigned hi = hi32(x), lo = lo32(x);
+  const unsigned bo = (hi >> 20) + (unsigned)cA;
+  unsigned mh = (hi & 0xfffffu) | 0x100000u;
+  if (ZERO) mh = ((hi & 0x7fffffffu) | lo) ? mh : 0u;
+  w1 = __funnelshift_l(0u, lo, bo);
+  w2 = __funnelshift_l(lo, mh, bo);
+  w3 = __funnelshift_l(mh, 0u, bo);
+  asm("add.cc.u32 %0, %0, %3;\n\t"
+      "addc.cc.u32 %1, %1, %3;\n\t"
+      "addc.u32 %2, %2, %4;"
+      : "+r"(w1), "+r"(w2), "+r"(w3)
+      : "n"(kB), "n"(kBTop));
+}
+
+// X + bias of any value (A >= its exponent), four words.
+__device__ __forceinline__ void any_words(double x, int A, unsigned (&w)[4]) {
+  xwords(x, A - 5, w);  // floor(|x| 2^(1127 - (A - 5)))
+  asm("add.cc.u32 %0, %0, %4;\n\t"
+      "addc.cc.u32 %1, %1, %4;\n\t"
+      "addc.cc.u32 %2, %2, %4;\n\t"
+      "addc.u32 %3, %3, %5;"
+      : "+r"(w[0]), "+r"(w[1]), "+r"(w[2]), "+r"(w[3])
+      : "n"(kB), "n"(kBTop));
+}
+
+// f16x2 factors (+-1, +-1) of a pair's digit FMA sign (1024 + f) + addend,
+// with the addends -sign 1152 (f - 128) and, for the top digit, -sign 1024.
+struct Sign2 {
+  unsigned mul, add;
+};
+__device__ __forceinline__ unsigned hmul2(unsigned a, unsigned b) {
+  unsigned d;
+  asm("mul.rn.f16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
+  return d;
+}
+__device__ __forceinline__ Sign2 sign2(double a, double b) {
+  Sign2 s;
+  asm("lop3.b32 %0, %1, %2, %3, 0xEA;"
+      : "=r"(s.mul)
+      : "r"(__byte_perm(hi32(a), hi32(b), 0x7632)), "n"(0x80008000u), "r"(0x3C003C00u));
+  s.add = hmul2(s.mul, 0xE480E480u);
+  return s;
+}
+__device__ __forceinline__ Sign2 top(Sign2 s) { return Sign2{s.mul, hmul2(s.mul, 0xE400E400u)}; }
+// Both digits of a byte-interleaved lane word z = [lo a, hi a, lo b, hi b].
+__device__ __forceinline__ unsigned digit_lo(unsigned z, unsigned e1024, Sign2 s) {
+  unsigned f;
+  asm("lop3.b32 %0, %1, %2, %3, 0xEA;" : "=r"(f) : "r"(z), "n"(0x00ff00ffu), "r"(e1024));  // (z & m) | 1024
+  return hfma2(f, s.mul, s.add);
+}
+__device__ __forceinline__ unsigned digit_hi(unsigned z, unsigned e1024, Sign2 s) {
+  return hfma2(__byte_perm(z, e1024, 0x7371), s.mul, s.add);  // [z1, 0x64, z3, 0x64]
+}
+
+__device__ __forceinline__ void st_digits(unsigned addr, unsigned a, unsigned b, unsigned c, unsigned d) {
+  asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
+}
+
+// The ten near slabs of eight values (pairs m = rows 2m, 2m + 1) whose lane
+// words are z, slab s at dst + s * stride.
+__device__ __forceinline__ void store_near(unsigned dst, unsigned stride, const unsigned (&z)[4][5],
+                                           const Sign2 (&sg)[4], unsigned e1024) {
+#pragma unroll
+  for (int i = 0; i < 5; ++i) {  // digits 2i (high bytes) and 2i + 1 (low bytes)
+    const Sign2 s0 = i ? sg[0] : top(sg[0]), s1 = i ? sg[1] : top(sg[1]);
+    const Sign2 s2 = i ? sg[2] : top(sg[2]), s3 = i ? sg[3] : top(sg[3]);
+    st_digits(dst + (unsigned)(2 * i) * stride, digit_hi(z[0][i], e1024, s0), digit_hi(z[1][i], e1024, s1),
+              digit_hi(z[2][i], e1024, s2), digit_hi(z[3][i], e1024, s3));
+    st_digits(dst + (unsigned)(2 * i + 1) * stride, digit_lo(z[0][i], e1024, sg[0]), digit_lo(z[1][i], e1024, sg[1]),
+              digit_lo(z[2][i], e1024, sg[2]), digit_lo(z[3][i], e1024, sg[3]));
+  }
+}
+
+// Barrier 0 over the CTA, true if any thread passes true.
+__device__ __forceinline__ bool bar_any(bool v) { return __syncthreads_or(v ? 1 : 0) != 0; }
+
+// Lane words of the eight values' near digits and their signs.
+template <bool ZERO>
+__device__ __forceinline__ void near_lanes(const double (&v)[8], int A, unsigned (&z)[4][5], Sign2 (&sg)[4]) {
+#pragma unroll
+  for (int m = 0; m < 4; ++m) {
+    unsigned a1, a2, a3, b1, b2, b3;
+    const double a = v[2 * m], b = v[2 * m + 1];
+    near_words<ZERO>(a, 25 - A, a1, a2, a3);
+    near_words<ZERO>(b, 25 - A, b1, b2, b3);
+    sg[m] = sign2(a, b);
+    z[m][0] = __byte_perm(a3, b3, 0x5410);
+    z[m][1] = __byte_perm(a2, b2, 0x7632);
+    z[m][2] = __byte_perm(a2, b2, 0x5410);
+    z[m][3] = __byte_perm(a1, b1, 0x7632);
+    z[m][4] = __byte_perm(a1, b1, 0x5410);
+  }
+}
+
+__device__ __forceinline__ double2 ld_shared2(unsigned addr) {
+  double2 d;
+  asm volatile("ld.shared.v2.f64 {%0, %1}, [%2];" : "=d"(d.x), "=d"(d.y) : "r"(addr));
+  return d;
+}
+
+// Accumulators -> running sums (256 columns on) for the column blocks q, q + 4,
+// .. of this warp's lanes (the four warps of a lane quarter share them out);
+// accumulators back to zero.
+template <int KYP>
+__device__ __forceinline__ void drain(unsigned ta, int q) {
+#pragma unroll 1
+  for (int c = q; c <= kDiag; c += 4) {
+    unsigned a[KYP], s[KYP];
+    const unsigned t = ta + (unsigned)(c * KYP);
+    tmem_ldn<KYP>(t, a);
+    tmem_ldn<KYP>(t + 256u, s);
+    tmem_waitn<KYP>(a);
+    tmem_waitn<KYP>(s);
+#pragma unroll
+    for (int y = 0; y < KYP; ++y) s[y] += (unsigned)__float2int_rn(__uint_as_float(a[y]));
+    tmem_stn<KYP>(t + 256u, s);
+    tmem_zeron<KYP>(t);
+  }
+  tmem_wait_st();
+}
+
+// Running sums of this thread's TMEM lane (NY columns of every column block,
+// from address ts) -> the totals (units 2^(Ax + Ay - 2148)).
+// With h = sum_d S_d 2^(8 (14 - d)) the value is h 2^(Ax + Ay - 2168); h = H 2^24
+// + l (H: diagonals 0..11) and the total takes floor(h 2^-20) = H 2^4 + floor(l
+// 2^-20).  Rare, and out of line: its 128-bit sums would cost the panel loop
+// registers.  jl: the lane's digit phase (column block c holds diagonal c + jl).
+template <class G>
+__device__ __noinline__ void fold(unsigned ts, int jl, i128* tot) {
+  constexpr int KYP = G::KYP, NY = KYP / 4;
+#pragma unroll 1
+  for (int part = 0; part < (G::SHARED ? 2 : 1); ++part) {  // SHARED: U from blocks c < J, V from the others
+    i128 h[NY];
+    long long l[NY];
+#pragma unroll
+    for (int y = 0; y < NY; ++y) {
+      h[y] = 0;
+      l[y] = 0;
+    }
+    // Horner over the diagonals d = c + jl; a block outside the part adds zero
+#pragma unroll 1
+    for (int c0 = 0; c0 <= kDiag; c0 += 3) {
+      unsigned s[3][NY];
+      tmem_ld3<NY>(ts + c0 * KYP, ts + (c0 + 1) * KYP, ts + (c0 + 2) * KYP, s);
+#pragma unroll
+      for (int u = 0; u < 3; ++u) {
+        const int c = c0 + u, d = c + jl;
+        const bool in = !G::SHARED || (c < G::J) == (part == 0);
+#pragma unroll
+        for (int y = 0; y < NY; ++y) {
+          const int x = in ? (int)s[u][y] : 0;
+          if (d <= 11) h[y] = (h[y] << 8) + (i128)x;
+          else if (d <= kDiag) l[y] = l[y] * 256 + x;
+        }
+      }
+    }
+#pragma unroll
+    for (int y = 0; y < NY; ++y) tot[part * NY + y] += (h[y] << 4) + (i128)(l[y] >> 20);
+  }
+}
+
+// ------------------------------------------------------------ kernel
+template <class G, typename T, bool TMA>
 __global__ void __launch_bounds__(kThreads, 1)
     umma_gram_partial_kernel(int64_t n, int kx, const T* __restrict__ X, int64_t ldx, int ky,
-                             const T* __restrict__ Y, int64_t ldy, UPlan pl, int64_t rows_per_chunk,
+                             const T* __restrict__ Y, int64_t ldy, int64_t rows_per_chunk,
                              const __grid_constant__ CUtensorMap tmx, const __grid_constant__ CUtensorMap tmy,
                              FxPart* __restrict__ parts, const int* gate) {
-  static_assert(sizeof(T) == 8 || DIRECT, "FP32 operands are copied by the converter threads");
-  // The compile-time plans: (KXPC, PC) = (64, 32) with separate X and Y
-  // (V^T Y, 64 + 16 columns) and (16, 128) with X = Y (symmetric, 16
-  // columns); TMA loads, no padded columns.  Their items are numbered A
-  // items first (kNA of them), then B items (kNB), so that whether an item
-  // exists and which operand it belongs to is known per item slot at compile
-  // time or is uniform over a warp.
-  constexpr bool kHot = KXPC > 0;
-  constexpr bool kHotShared = KXPC == 16;
-  constexpr int kNA = kHot ? KXPC * PC / 2 : 0, kNB = kHot && !kHotShared ? KYP * PC / 2 : 0;
-  static_assert(!kHot || ((KXPC == 64 && PC == 32) || (KXPC == 16 && PC == 128)), "compile-time plans");
-  static_assert(!kHot || (!DIRECT && !PAD && KYP == 16), "compile-time plans load by TMA");
-  static_assert(!kHot || (kNA + kNB <= kMaxItems * kConvThreads && kNA % 32 == 0 && kNB % 32 == 0),
-                "compile-time plans: whole warps of items");
+  static_assert(sizeof(T) == 8 || !TMA, "FP32 operands are copied by the converter threads");
   if (gate && *gate == 0) return;
-  // Y columns of one converter thread in a drain (four warps share a TMEM
-  // lane quarter), handled NH times NY at a time
-  constexpr int NYT = KYP * 4 / kDrainWarps;
-  constexpr int NY = NYT < 4 ? NYT : 4;
-  constexpr int NH = NYT / NY;
-  const int kxp = KXPC ? KXPC : pl.kxp, P = PC ? PC : pl.P;
-  const int nslots = KXPC ? (pl.shared ? KXPC : KXPC + KYP) : pl.nslots;
-  const int tx = blockIdx.x / pl.nty, ty = blockIdx.x % pl.nty;
-  const int x0 = tx * kxp, y0 = ty * KYP;  // first X / Y column of the tile
-  const unsigned SBO = (unsigned)P * 16;   // bytes per 8-row group of a slab (P / 8 core matrices)
+  constexpr int KXP = G::KXP, KYP = G::KYP, J = G::J, P = G::P;
+  constexpr bool SHARED = G::SHARED;
+  // Y columns of one draining thread (four warps share a TMEM lane quarter)
+  constexpr int NY = KYP / 4;
+  constexpr int kParts = SHARED ? 2 : 1;  // totals per output of a lane: U (and V)
+  const int y0 = blockIdx.x * KYP;        // first Y column of the tile
 
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   // 1024-byte aligned base (the 128-byte swizzle of the TMA boxes is anchored there)
-  unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
-  unsigned char* stage = smem;                                 // 2 staging buffers (TMA boxes; DIRECT: slots)
-  const size_t stage_region = DIRECT ? max(2 * (size_t)pl.stage_bytes, (size_t)kDirectStageBytes)
-                                     : 2 * (size_t)pl.stage_bytes;
-  unsigned char* dig = stage + stage_region;                   // 2 digit buffers
-  int* Erun = reinterpret_cast<int*>(dig + 2 * (size_t)pl.dig_bytes);
-  int* pmax = Erun + 2 * nslots;  // three panels' column maxima (Erun: running exponents, two buffers)
-  __shared__ __align__(8) unsigned long long full_bar[2], ready_bar[2], stage_bar[2];
+  unsigned char* dig = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);  // 2 digit buffers
+  unsigned char* stage = dig + G::stage_off;             // 2 staging buffers
+  int* Erun = reinterpret_cast<int*>(stage + 2 * (size_t)G::stage_bytes);  // running exponents (0: none yet)
+  int* Enew = Erun + G::COLS;                                              // the same with the current panel
+  __shared__ __align__(8) unsigned long long full_bar[2], stage_bar[2], ready_bar[2];
   __shared__ unsigned tmem_base;
   __shared__ int flag, bad;
-  // far[b]: the last panel in digit buffer b with an item off the near path
-  // (its digit slabs 11..14 may be nonzero); written by the converters before
-  // they mark the panel ready, read by the MMA warp after that
-  __shared__ int far[2];
+  // spec[p & 1] = p: panel p holds a value that is not near; written before the arrivals for panel p - 1
+  __shared__ int spec[2];
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
   // ---- set-up: TMEM (accumulators in columns 0..255, running sums in 256..511),
-  // barriers, zero slabs, exponents
+  // barriers, zero digits (padded columns and slabs stay zero), exponents
   if (warp == 0) tmem_alloc(smem_u32(&tmem_base), 512);
   if (tid == 0) {
     for (int b = 0; b < 2; ++b) {
       mbar_init(smem_u32(&full_bar[b]), 1);
-      mbar_init(smem_u32(&ready_bar[b]), kConvThreads);
       mbar_init(smem_u32(&stage_bar[b]), 1);
+      mbar_init(smem_u32(&ready_bar[b]), kConvWarps);
+      spec[b] = -1;
     }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     flag = 0;
     bad = 0;
-    far[0] = far[1] = -1;
   }
-  for (int c = tid; c < 5 * nslots; c += kThreads) Erun[c] = 0;  // Erun and pmax
-  {  // slab 15 of every operand stays zero
-    const unsigned za = (unsigned)kxp / 8u * SBO, zb = (unsigned)KYP / 8u * SBO;  // bytes of one slab
-    for (int b = 0; b < 2; ++b) {
-      unsigned* pa = reinterpret_cast<unsigned*>(dig + (size_t)b * pl.dig_bytes + 15u * za);
-      for (unsigned e = tid; e < za / 4; e += kThreads) pa[e] = 0u;
-      if (!pl.shared) {
-        unsigned* pb = reinterpret_cast<unsigned*>(dig + (size_t)b * pl.dig_bytes + pl.a_bytes + 15u * zb);
-        for (unsigned e = tid; e < zb / 4; e += kThreads) pb[e] = 0u;
-      }
-    }
-  }
+  for (int c = tid; c < 2 * G::COLS; c += kThreads) Erun[c] = 0;  // Erun and Enew
+  for (unsigned e = tid; e < 2 * G::dig_bytes / 16; e += kThreads)
+    reinterpret_cast<uint4*>(dig)[e] = make_uint4(0u, 0u, 0u, 0u);
   fence_proxy_async();
   tc_fence_before();
   __syncthreads();
@@ -221,511 +414,383 @@ __global__ void __launch_bounds__(kThreads, 1)
   const int64_t r1 = min(n, r0 + rows_per_chunk);
   const int npan = r0 < r1 ? (int)((r1 - r0 + P - 1) / P) : 0;
   const unsigned dig_s = smem_u32(dig);
-  const unsigned fb0 = smem_u32(&full_bar[0]), rb0 = smem_u32(&ready_bar[0]), sb0 = smem_u32(&stage_bar[0]);
-  // TMA loads of panel p into staging buffer p & 1: P / 16 boxes of 16 rows per operand
-  const unsigned xbox = (unsigned)kxp * 128u, ybox = (unsigned)KYP * 128u;
-  auto load_panel = [&](int p) {
-    const unsigned bar = sb0 + 8u * (unsigned)(p & 1);
-    const unsigned dst = smem_u32(stage) + (unsigned)(p & 1) * pl.stage_bytes;
-    const int xr = (int)(r0 + (int64_t)p * P);
-    mbar_arrive_expect_tx(bar, pl.stage_bytes);
-    for (int h = 0; h < P / 16; ++h) {
-      tma_load_2d(dst + (unsigned)h * xbox, &tmx, xr + 16 * h, x0, bar);
-      if (!pl.shared) tma_load_2d(dst + (unsigned)(P / 16) * xbox + (unsigned)h * ybox, &tmy, xr + 16 * h, y0, bar);
-    }
+  const unsigned fb0 = smem_u32(&full_bar[0]);
+
+  // ---- this thread's item: eight consecutive rows of one column of every panel
+  const int cg = warp % G::NCG, kc = (warp / G::NCG) * 2 + (lane >> 4);  // column group, K chunk
+  const int slot = cg * 16 + (lane & 15);      // column held
+  const bool isb = !SHARED && cg * 16 >= KXP;  // of the Y operand (uniform over the warp)
+  const int lc = slot - (isb ? KXP : 0);
+  const bool mine = warp < kConvWarps && kc < P / 8 && slot < G::COLS;  // the thread has an item
+  const bool valid = mine && (isb ? y0 + lc < ky : lc < kx);
+  const unsigned dst_near = dig_s + (isb ? G::b_off + (unsigned)kc * G::LBN : (unsigned)kc * G::LAN) + (unsigned)lc * 16u;
+  const unsigned e1024 = exp1024x2();
+
+  // ---- staging: panel p's values in staging buffer p & 1, P / 16 boxes of
+  // 16 rows (128 bytes, 128-byte swizzle) of X's columns, then of Y's.  TMA:
+  // the last warp copies a whole panel (rows past the matrix read as zero, the
+  // rows of the next chunk are masked).  Else (a base not 16-byte aligned, an
+  // odd leading dimension, FP32) every converter thread copies its own item
+  // into its own place, element by element.
+  constexpr unsigned xbox = KXP * 128u, ybox = KYP * 128u;
+  const unsigned stage_s = smem_u32(stage), sb0 = smem_u32(&stage_bar[0]);
+  const T* src = valid ? (isb ? Y + (size_t)(y0 + lc) * ldy : X + (size_t)lc * ldx) + r0 + 8 * kc : nullptr;
+  const unsigned item = (isb ? (P / 16) * xbox : 0u) + (unsigned)(kc >> 1) * (isb ? ybox : xbox) + (unsigned)lc * 128u;
+  // 16-byte unit u (rows 2u, 2u + 1) of the item
+  auto unit = [&](int p, int u) {
+    return (unsigned)(p & 1) * G::stage_bytes + item + (((unsigned)(4 * (kc & 1) + u) ^ (unsigned)(lc & 7)) << 4);
   };
-  if (!DIRECT && tid == 0) {
-    for (int p = 0; p < 2 && p < npan; ++p) load_panel(p);
-  }
-
-  // the partial sums of this thread's lane: lane block jl (digit phase), X column xl
-  const int Lq = (warp & 3) * 32, L = Lq + lane;
-  const int jl = L >> (31 - __clz(kxp)), xl = L & (kxp - 1);
-  const int yq = (warp >> 2) * NYT;  // first of this thread's NYT Y columns (drain warps)
-  const bool drainer = warp < kDrainWarps;
-  i128 W[NYT];
-#pragma unroll
-  for (int y = 0; y < NYT; ++y) W[y] = 0;
-
-  if (warp == kConvWarps) {
-    // ---------------- MMA issuer
-    if (lane == 0) {
-      int p = 0;
-      for (; p < npan; ++p) {
-        const int db = p & 1;
-        if (!mbar_wait(rb0 + 8u * db, (unsigned)(p >> 1) & 1u, &bad)) break;
-        tc_fence_after();
-        const unsigned abase = dig_s + (unsigned)db * pl.dig_bytes;
-        const unsigned bbase = pl.shared ? abase : abase + pl.a_bytes;
-        // every item of the panel on the near path: digit slabs 11..14 of
-        // both operands are zero, and the MMAs that would only multiply them
-        // are left out (exactly the same sums)
-        const int ns = *reinterpret_cast<volatile int*>(&far[db]) == p ? NS : 11;
-        for (int ks = 0; ks < P / 16; ++ks) {
-          for (int q = 0; q < pl.nq; ++q) {
-            if (pl.J * q >= ns) break;  // all of this MMA's X slabs are zero
-            const int nt = min(NS - pl.J * q, ns);
-            const int Tp = KYP == 16 ? nt : (nt + 1) & ~1;  // N a multiple of 16
-            const unsigned long long ad =
-                sdesc(abase + (unsigned)(pl.J * q * kxp / 8) * SBO + (unsigned)ks * 256u, 128u, SBO);
-            const unsigned long long bd = sdesc(bbase + (unsigned)ks * 256u, 128u, SBO);
-            mma_f16(taddr + (unsigned)(KYP * pl.J * q), ad, bd, idesc_f16(kLanes, KYP * Tp),
-                    1u);  // the accumulators start at zero and drains zero them
-          }
-        }
-        mma_commit(fb0 + 8u * db);
-      }
-      // the last committed MMAs finish before TMEM and shared memory are released
-      if (p > 0) mbar_wait_final(fb0 + 8u * ((p - 1) & 1), (unsigned)((p - 1) >> 1) & 1u, &bad);
-    }
-    __syncwarp();
-  } else {
-    // ---------------- converters: staging, exponents, digits, drains
-    const unsigned tacc = taddr + ((unsigned)Lq << 16) + (unsigned)yq;
-    const unsigned tsum = tacc + 256u;
-    if (drainer) {
-      unsigned z[3][NY];
-#pragma unroll
-      for (int u = 0; u < 3; ++u)
-#pragma unroll
-        for (int y = 0; y < NY; ++y) z[u][y] = 0u;
-#pragma unroll
-      for (int hh = 0; hh < NH; ++hh)
-#pragma unroll
-        for (int c0 = 0; c0 < NS; c0 += 3) {
-          const unsigned ts = tsum + 4u * hh, ta = tacc + 4u * hh;
-          tmem_st3<NY>(ts + c0 * KYP, ts + (c0 + 1) * KYP, ts + (c0 + 2) * KYP, z);
-          tmem_st3<NY>(ta + c0 * KYP, ta + (c0 + 1) * KYP, ta + (c0 + 2) * KYP, z);
-        }
-      tmem_wait_st();
-    }
-
-    // TMEM accumulators -> TMEM running sums (column block c of lane block
-    // jl: diagonal c + jl) for the groups of three column blocks G0 .. 4 (the
-    // groups due at a drain are always such a suffix: a group's period is a
-    // power of two no shorter than that of any later group); a drained
-    // group's accumulators are set back to zero.  The loads of the next group
-    // are in flight while a group is added.
-    unsigned tacc_h = tacc, tsum_h = tsum;  // the NY columns being drained
-    auto load = [&](int c0, unsigned (&v)[3][NY], unsigned (&sm)[3][NY]) {
-      tmem_ld3x2_nowait<NY>(tacc_h + c0 * KYP, tacc_h + (c0 + 1) * KYP, tacc_h + (c0 + 2) * KYP, tsum_h + c0 * KYP,
-                            tsum_h + (c0 + 1) * KYP, tsum_h + (c0 + 2) * KYP, v, sm);
-    };
-    auto add_store = [&](int c0, unsigned (&v)[3][NY], unsigned (&sm)[3][NY]) {
-      // (column blocks with c + jl > 14 collect no kept diagonal: the fold skips them)
-#pragma unroll
-      for (int u = 0; u < 3; ++u)
-#pragma unroll
-        for (int y = 0; y < NY; ++y) sm[u][y] += (unsigned)__float2int_rn(__uint_as_float(v[u][y]));
-      tmem_st3<NY>(tsum_h + c0 * KYP, tsum_h + (c0 + 1) * KYP, tsum_h + (c0 + 2) * KYP, sm);
-      tmem_zero3<NY>(tacc_h + c0 * KYP, tacc_h + (c0 + 1) * KYP, tacc_h + (c0 + 2) * KYP);
-    };
-    auto drain_from = [&](auto g0) {
-      constexpr int G0 = decltype(g0)::value;
-      unsigned va[3][NY], sa[3][NY], vb[3][NY], sb[3][NY];
-      load(3 * G0, va, sa);
-      tmem_wait_ld_regs<NY>(va, sa);
-      if constexpr (G0 + 1 <= 4) load(3 * (G0 + 1), vb, sb);
-      add_store(3 * G0, va, sa);
-      if constexpr (G0 + 1 <= 4) {
-        tmem_wait_ld_regs<NY>(vb, sb);
-        if constexpr (G0 + 2 <= 4) load(3 * (G0 + 2), va, sa);
-        add_store(3 * (G0 + 1), vb, sb);
-      }
-      if constexpr (G0 + 2 <= 4) {
-        tmem_wait_ld_regs<NY>(va, sa);
-        if constexpr (G0 + 3 <= 4) load(3 * (G0 + 3), vb, sb);
-        add_store(3 * (G0 + 2), va, sa);
-      }
-      if constexpr (G0 + 3 <= 4) {
-        tmem_wait_ld_regs<NY>(vb, sb);
-        if constexpr (G0 + 4 <= 4) load(3 * (G0 + 4), va, sa);
-        add_store(3 * (G0 + 3), vb, sb);
-      }
-      if constexpr (G0 + 4 <= 4) {
-        tmem_wait_ld_regs<NY>(va, sa);
-        add_store(3 * (G0 + 4), va, sa);
-      }
-      tmem_wait_st();
-    };
-    auto drain = [&](int g0) {
-#pragma unroll
-      for (int hh = 0; hh < NH; ++hh) {
-        tacc_h = tacc + 4u * hh;
-        tsum_h = tsum + 4u * hh;
-        switch (g0) {
-          case 0: drain_from(std::integral_constant<int, 0>{}); break;
-          case 1: drain_from(std::integral_constant<int, 1>{}); break;
-          case 2: drain_from(std::integral_constant<int, 2>{}); break;
-          case 3: drain_from(std::integral_constant<int, 3>{}); break;
-          case 4: drain_from(std::integral_constant<int, 4>{}); break;
-          default: break;  // no group due
+  auto fetch = [&](int p) {
+    if constexpr (TMA) {
+      if (tid == kIssuer) {
+        const unsigned bar = sb0 + 8u * (unsigned)(p & 1), dst = stage_s + (unsigned)(p & 1) * G::stage_bytes;
+        const int xr = (int)(r0 + (int64_t)p * P);
+        fence_proxy_async();
+        mbar_arrive_expect_tx(bar, G::copy_bytes);
+        for (int h = 0; h < P / 16; ++h) {
+          tma_load_2d(dst + (unsigned)h * xbox, &tmx, xr + 16 * h, 0, bar);
+          if (!SHARED) tma_load_2d(dst + (P / 16) * xbox + (unsigned)h * ybox, &tmy, xr + 16 * h, y0, bar);
         }
       }
-    };
-    auto fold = [&]() {  // running sums -> W (units 2^(Ax + Ay - 2148)), sums back to zero
+    } else {
+      // a copy of no bytes (a row past the chunk: the place is zero-filled)
+      // names the partials array as its source, an address that is always valid
+      const T* z = reinterpret_cast<const T*>(parts);
+      const int64_t pr = (int64_t)p * P, left = r1 - (r0 + pr + 8 * kc);
+      if (valid) {
 #pragma unroll
-      for (int hh = 0; hh < NH; ++hh) {
-        const unsigned ts = tsum + 4u * hh;
-        i128 h[NY];
-#pragma unroll
-        for (int y = 0; y < NY; ++y) h[y] = 0;
-#pragma unroll
-        for (int c0 = 0; c0 < NS; c0 += 3) {
-          unsigned sm[3][NY];
-          tmem_ld3<NY>(ts + c0 * KYP, ts + (c0 + 1) * KYP, ts + (c0 + 2) * KYP, sm);
-#pragma unroll
-          for (int u = 0; u < 3; ++u)
-#pragma unroll
-            for (int y = 0; y < NY; ++y)
-              if (c0 + u + jl <= 14) h[y] = (h[y] << 7) + (i128)(int)sm[u][y];
-#pragma unroll
-          for (int u = 0; u < 3; ++u)
-#pragma unroll
-            for (int y = 0; y < NY; ++y) sm[u][y] = 0u;
-          tmem_st3<NY>(ts + c0 * KYP, ts + (c0 + 1) * KYP, ts + (c0 + 2) * KYP, sm);
-        }
-        tmem_wait_st();
-#pragma unroll
-        for (int y = 0; y < NY; ++y) W[hh * NY + y] += h[y] >> 8;
-      }
-    };
-
-    // This thread's items (two rows of one column) of every panel: i = tid +
-    // k * kConvThreads.  Within a warp, lanes l, l ^ 8, l ^ 16, l ^ 24 share a column,
-    // the eight columns of a quarter warp read distinct 16-byte chunks of the
-    // swizzled boxes, and the 32 digit words a warp stores per slab fill 128
-    // contiguous bytes.  it_s: column << 16 | staging offset / 16; it_d:
-    // digit offset | B operand << 31.
-    // Item i of a panel goes to thread slot i % kConvThreads, slot k = i /
-    // kConvThreads; thread tid holds slot titem, rotated so that the slots
-    // past the last whole round of items (the third item of some threads)
-    // fall to the converter warps that do not drain TMEM.  In the hot plans
-    // the kNA items of the A operand come first and the kNB items of the B
-    // operand after them (item_valid, item_b below).
-    const int titem = (tid + 32 * (kConvWarps - kDrainWarps)) % kConvThreads;
-    const int half = P >> 1, ncg = nslots >> 3;
-    const int nitems = nslots * half;
-    unsigned it_s[kMaxItems], it_d[kMaxItems];
-#pragma unroll
-    for (int k = 0; k < kMaxItems; ++k) {
-      int c, rh, cl, rl;
-      if constexpr (kHot) {
-        // an empty slot (past the kNA + kNB items) takes item 0's column, so
-        // that every column index stays below nslots
-        const int i0 = titem + k * kConvThreads;
-        const bool live = i0 < kNA + kNB;
-        const bool kb = live && i0 >= kNA;
-        const int i = kb ? i0 - kNA : (live ? i0 : 0);
-        const int g = kb ? KYP / 8 : KXPC / 8;  // column groups of the operand
-        cl = i & 7;
-        rl = (i >> 3) & 3;
-        c = ((i >> 5) % g) * 8 + cl + (kb ? KXPC : 0);
-        rh = (i >> 5) / g;
-      } else {
-        const int i = titem + k * kConvThreads;
-        cl = i & 7;
-        rl = (i >> 3) & 3;
-        c = ((i >> 5) % ncg) * 8 + cl;
-        rh = (i >> 5) / ncg;
-      }
-      const int r = (rh * 4 + rl) * 2;
-      const bool isb = !pl.shared && c >= kxp;
-      const int lc = isb ? c - kxp : c;
-      const unsigned so = (isb ? (unsigned)(P / 16) * xbox : 0u) + (unsigned)(r >> 4) * (isb ? ybox : xbox) +
-                          (unsigned)lc * 128u + ((((unsigned)(r & 15) >> 1) ^ (unsigned)(lc & 7)) << 4);
-      it_s[k] = ((unsigned)c << 16) | (so >> 4);
-      it_d[k] = ((isb ? pl.a_bytes : 0u) + (unsigned)(lc >> 3) * SBO + (unsigned)rh * 128u +
-                 (unsigned)(lc & 7) * 16u + (unsigned)rl * 4u) |
-                ((unsigned)isb << 31);
-      if constexpr (PAD) {  // bit 30: a padded column, whose digits stay zero
-        if (titem + k * kConvThreads < nitems && !(isb ? y0 + lc < ky : x0 + lc < kx)) it_d[k] |= 1u << 30;
-      }
-    }
-    // item k exists for this thread; it belongs to the B operand
-    auto item_valid = [&](int k) -> bool {
-      if constexpr (kHot) {
-        if (k * kConvThreads >= kNA + kNB) return false;
-        if ((k + 1) * kConvThreads <= kNA + kNB) return true;
-        return titem + k * kConvThreads < kNA + kNB;
-      } else {
-        return titem + k * kConvThreads < nitems;
-      }
-    };
-    auto item_b = [&](int k) -> bool {
-      if constexpr (kHot) {
-        if (kNB == 0 || (k + 1) * kConvThreads <= kNA) return false;
-        if (k * kConvThreads >= kNA) return true;
-        return titem + k * kConvThreads >= kNA;
-      } else {
-        return (it_d[k] >> 31) != 0u;
-      }
-    };
-    const unsigned stride_a = (unsigned)kxp / 8u * SBO, stride_b = (unsigned)KYP / 8u * SBO;
-    if constexpr (PAD) {  // the digit words of padded columns: zero once, in both buffers
-#pragma unroll
-      for (int k = 0; k < kMaxItems; ++k) {
-        if (it_d[k] & 0x40000000u) {
-          for (int b = 0; b < 2; ++b) {
-            unsigned char* d = dig + (size_t)b * pl.dig_bytes + (it_d[k] & 0x3fffffffu);
-            const unsigned strd = (it_d[k] >> 31) ? stride_b : stride_a;
-            for (int sl = 0; sl < NS; ++sl) *reinterpret_cast<unsigned*>(d + sl * strd) = 0u;
-          }
-        }
-      }
-    }
-
-    // DIRECT: each item's column (null: zeros) and row offset in the panel
-    const T* gcol[kMaxItems];
-    int irow[kMaxItems];
-    const unsigned slot0 = smem_u32(stage) + (unsigned)tid * 16u;
-    // a copy of no bytes (a row past the chunk: the slot is zero-filled) names
-    // the partials array as its source, an address that is always valid
-    const T* zsrc = reinterpret_cast<const T*>(parts);
-    auto prefetch = [&](int pp) {  // this thread's items of panel pp into slot buffer pp & 1
-      const int64_t base = r0 + (int64_t)pp * P;
-#pragma unroll
-      for (int k = 0; k < kMaxItems; ++k) {
-        if (!gcol[k]) continue;
-        const int64_t row = base + irow[k];
-        const unsigned d = slot0 + (unsigned)(((pp & 1) * kMaxItems + k) * kConvThreads) * 16u;
-        if constexpr (sizeof(T) == 8) {
-          cp_async8z(d, row < r1 ? gcol[k] + row : zsrc, row < r1 ? 8u : 0u);
-          cp_async8z(d + 8u, row + 1 < r1 ? gcol[k] + row + 1 : zsrc, row + 1 < r1 ? 8u : 0u);
-        } else {
-          cp_async4z(d, row < r1 ? gcol[k] + row : zsrc, row < r1 ? 4u : 0u);
-          cp_async4z(d + 4u, row + 1 < r1 ? gcol[k] + row + 1 : zsrc, row + 1 < r1 ? 4u : 0u);
+        for (int m = 0; m < 8; ++m) {
+          const unsigned d = stage_s + unit(p, m >> 1) + (unsigned)(m & 1) * 8u;
+          if constexpr (sizeof(T) == 8) cp_async8z(d, m < left ? src + pr + m : z, m < left ? 8u : 0u);
+          else cp_async4z(d, m < left ? src + pr + m : z, m < left ? 4u : 0u);
         }
       }
       cp_async_commit_group();
-    };
-    if constexpr (DIRECT) {
-#pragma unroll
-      for (int k = 0; k < kMaxItems; ++k) {
-        const int i = titem + k * kConvThreads;
-        const int cl = i & 7, rl = (i >> 3) & 3, rest = i >> 5;
-        const int c = (rest % ncg) * 8 + cl, rh = rest / ncg;
-        const bool isb = !pl.shared && c >= kxp;
-        const int lc = isb ? c - kxp : c, gc = isb ? y0 + lc : x0 + lc;
-        const bool ok = i < nitems && gc < (isb ? ky : kx);
-        gcol[k] = ok ? (isb ? Y + (size_t)gc * ldy : X + (size_t)gc * ldx) : nullptr;
-        irow[k] = (rh * 4 + rl) * 2;
-      }
-      prefetch(0);
-      prefetch(1);
     }
-
-    // One barrier per panel.  The values of panel p are in registers and
-    // the maxima of its columns complete in pmax[p % 3] when panel p begins
-    // (both done during panel p-1): a converter aligns and converts p, drains
-    // TMEM if due, marks p ready for the MMA warp, then reads and scans panel
-    // p+1 while those MMAs run; the barrier that ends the panel completes
-    // that scan.  The running exponents through panel q sit in Erun[q & 1],
-    // the maxima of panel q in pmax[q % 3]; a buffer is rewritten only after
-    // the barrier that follows its last read.
-    auto stage_values = [&](int q, double2 (&v)[kMaxItems]) {  // this thread's items of panel q
-      if constexpr (DIRECT) {
-        asm volatile("cp.async.wait_group 1;" ::: "memory");  // panel q's copies (q + 1's may be in flight)
+  };
+  // Panel p's values (zeros past the chunk).  The units of an item differ in
+  // bits 4 and 5 of their address only (the swizzle's), as an exclusive or.
+  double v[8];
+  const unsigned item_s = stage_s + (mine ? unit(0, 0) : 0u);
+  auto load = [&](int p) {
+    if constexpr (TMA) mbar_wait(sb0 + 8u * (unsigned)(p & 1), (unsigned)(p >> 1) & 1u, &bad);
+    else asm volatile("cp.async.wait_group 1;" ::: "memory");  // p + 1's may be in flight
+    const unsigned at = item_s + (unsigned)(p & 1) * G::stage_bytes;
 #pragma unroll
-        for (int k = 0; k < kMaxItems; ++k) {
-          const unsigned char* slot = stage + ((size_t)((q & 1) * kMaxItems + k) * kConvThreads + tid) * 16u;
-          if constexpr (sizeof(T) == 8) {
-            v[k] = gcol[k] ? *reinterpret_cast<const double2*>(slot) : make_double2(0.0, 0.0);
-          } else {
-            const float2 f = gcol[k] ? *reinterpret_cast<const float2*>(slot) : make_float2(0.0f, 0.0f);
-            v[k] = make_double2(widen(f.x), widen(f.y));
+    for (int m = 0; m < 4; ++m) {
+      const double2 d = ld_shared2(at ^ ((unsigned)m << 4));
+      if constexpr (sizeof(T) == 8) {
+        v[2 * m] = d.x;
+        v[2 * m + 1] = d.y;
+      } else {
+        v[2 * m] = widen(__int_as_float(__double2loint(d.x)));
+        v[2 * m + 1] = widen(__int_as_float(__double2loint(d.y)));
+      }
+    }
+    if (TMA && p + 1 == npan) {  // (the copies zero-fill rows past the chunk, but not the tensor map)
+      const int64_t left = r1 - (r0 + (int64_t)p * P + 8 * kc);
+#pragma unroll
+      for (int m = 0; m < 8; ++m)
+        if (m >= left) v[m] = 0.0;
+    }
+  };
+  // The column's window: a value is near when (2 |hi word| - wlo) < wrange, unsigned.
+  int te = 0;  // running exponent of this thread's column (0: none)
+  unsigned wlo = 0, wrange = valid ? 0u : 0xffffffffu;
+  auto set_window = [&]() {
+    const int A = max(te, 1), f = max(A - kNearBits, 1);
+    wlo = (unsigned)f << 21;
+    wrange = ((unsigned)(A + 1) << 21) - wlo;
+  };
+  auto outside = [&]() {
+    unsigned k = 0;
+#pragma unroll
+    for (int m = 0; m < 8; ++m) k = max(k, 2u * hi32(v[m]) - wlo);
+    return k >= wrange;
+  };
+  if (npan > 0) {
+    fetch(0);
+    if (!TMA || npan > 1) fetch(1);
+  }
+
+  // ---- drains: this thread's TMEM lane: lane block jl (digit phase), X column xl
+  const int Lq = (warp & 3) * 32, L = Lq + lane;
+  const int jl = L / KXP, xl = L % KXP;
+  const int yq = (warp >> 2) * NY;  // first of this thread's NY Y columns
+  const unsigned tq = taddr + ((unsigned)Lq << 16);             // the lane quarter's columns
+  const unsigned tsum = tq + (unsigned)yq + 256u;               // the running sums of its columns
+  // the exact totals; touched once per fold, so they are kept out of registers
+  i128 totals[kParts * NY];
+  i128* tot = totals;
+  asm volatile("" : "+l"(tot)::"memory");
+  for (int y = 0; y < kParts * NY; ++y) tot[y] = 0;
+
+  // the running sums and, first, the accumulators at zero (this warp's share of the column blocks)
+  auto zero_blocks = [&](unsigned t) {
+#pragma unroll 1
+    for (int c = warp >> 2; c <= kDiag; c += 4) tmem_zeron<KYP>(t + (unsigned)(c * KYP));
+    tmem_wait_st();
+  };
+  zero_blocks(tq);
+  zero_blocks(tq + 256u);
+  tc_fence_before();
+
+  // ---- steps: one digit buffer filled and multiplied (a near panel, or half
+  // of a panel with all slabs).  Step `step` uses buffer step & 1.
+  int step = 0;          // steps converted so far
+  int pend = 0;          // K steps (16 rows) of the last converted step, not issued yet (0: none)
+  bool pend_all = false; // ... with all slabs
+  int used = 0;          // row-pairs (of kPairRows) the accumulators hold, the pending step included
+  int drains = 0;        // since the last fold
+  auto issue = [&]() {   // the pending step's MMAs (after a barrier that follows its stores)
+    if (pend > 0 && tid == kIssuer) {
+      tc_fence_after();
+      const int b = (step - 1) & 1;
+      const unsigned ab = dig_s + (unsigned)b * G::dig_bytes;
+      if (!pend_all) {
+        for (int ks = 0; ks < pend; ++ks) {
+          const unsigned long long bd = SHARED ? sdesc(ab + (unsigned)ks * 2u * G::LAN, G::LAN, 128u)
+                                               : sdesc(ab + G::b_off + (unsigned)ks * 2u * G::LBN, G::LBN, 128u);
+#pragma unroll
+          for (int q = 0; q < G::NQN; ++q) {
+            constexpr int even = KYP == 8 ? 1 : 0;  // N is a multiple of 16
+            const int nt = (min(kNear, kDiag + 1 - J * q) + even) & ~even;
+            mma_f16(taddr + (unsigned)(KYP * J * q),
+                    sdesc(ab + (unsigned)(J * q * KXP) * 16u + (unsigned)ks * 2u * G::LAN, G::LAN, 128u), bd,
+                    idesc_f16(kLanes, KYP * nt), 1u);  // the accumulators start at zero and drains zero them
           }
         }
-        prefetch(q + 2);  // into the slots just read (zeros past the chunk)
       } else {
-        mbar_wait(sb0 + 8u * (unsigned)(q & 1), (unsigned)(q >> 1) & 1u, &bad);  // panel q staged
-        const unsigned char* st = stage + (size_t)(q & 1) * pl.stage_bytes;
-#pragma unroll
-        for (int k = 0; k < kMaxItems; ++k)
-          v[k] = item_valid(k) ? *reinterpret_cast<const double2*>(st + ((it_s[k] & 0xffffu) << 4))
-                               : make_double2(0.0, 0.0);
+        for (int ks = 0; ks < pend; ++ks) {
+          const unsigned long long bd = SHARED ? sdesc(ab + (unsigned)ks * 2u * G::LAA, G::LAA, 128u)
+                                               : sdesc(ab + G::b_off_all + (unsigned)ks * 2u * G::LBA, G::LBA, 128u);
+#pragma unroll 1
+          for (int q = 0; q < G::NQA; ++q) {
+            constexpr int even = KYP == 8 ? 1 : 0;
+            const int nt = (min(kAll, kDiag + 1 - J * q) + even) & ~even;
+            mma_f16(taddr + (unsigned)(KYP * J * q),
+                    sdesc(ab + (unsigned)(J * q * KXP) * 16u + (unsigned)ks * 2u * G::LAA, G::LAA, 128u), bd,
+                    idesc_f16(kLanes, KYP * nt), 1u);
+          }
+        }
       }
-    };
-    // largest exponent of each column of a panel into pmq (the exponent
-    // field of the larger |x| bit pattern; bit 0 set when any bit is, so
-    // that subnormals count) where it exceeds the column's running
-    // exponent, one shared-memory atomic per such item (cheaper than
-    // reducing the four items of a column in a warp by shuffles first);
-    // true if one of this thread's columns exceeds te[k], its nonzero
-    // running exponent
-    auto scan = [&](const double2 (&v)[kMaxItems], int* pmq, const int (&te)[kMaxItems]) -> bool {
-      bool g = false;
+      mma_commit(fb0 + 8u * b);
+    }
+    pend = 0;
+  };
+  // wait for the MMAs of step s (committed to its buffer's barrier)
+  auto wait_step = [&](int s) { mbar_wait(fb0 + 8u * (unsigned)(s & 1), (unsigned)(s >> 1) & 1u, &bad); };
+  // Empties the accumulators (after the MMAs of the steps before s) and, when
+  // due or asked for, folds the running sums.
+  auto empty = [&](int s, bool full) {
+    ++drains;
+    full |= drains >= kFoldDrains;
+    wait_step(s - 1);
+    tc_fence_after();
+    drain<KYP>(tq, warp >> 2);
+    if (full) {  // all of the lane quarter's blocks are drained
+      asm volatile("bar.sync %0, 128;" ::"r"(1 + (warp & 3)) : "memory");
+      fold<G>(tsum, jl, tot);
+      asm volatile("bar.sync %0, 128;" ::"r"(1 + (warp & 3)) : "memory");
+      zero_blocks(tq + 256u);
+    }
+    tc_fence_before();
+    if (full) drains = 0;
+    used = 0;
+  };
+  // the step just converted (cost row-pairs) becomes the pending one; the
+  // accumulators are emptied first when they could not hold it
+  auto finish_step = [&](int ks, bool all, int cost) {
+    fence_proxy_async();
+    if (used + cost > kPairRows) empty(step, false);
+    used += cost;
+    pend = ks;
+    pend_all = all;
+    ++step;
+  };
+
+  int dirty = 0;  // bit b: buffer b was last used with all slabs (its zero slabs and columns are to be zeroed again)
+
+  // the near digits of this thread's item into step `step`'s buffer
+  auto put = [&](const unsigned (&z)[4][5], const Sign2 (&sg)[4]) {
+    const unsigned at = dst_near + (unsigned)(step & 1) * G::dig_bytes;
+    if (mine) {
+      if (step >= 2) wait_step(step - 2);  // the buffer's last MMAs are done
+      if (valid) {
+        if (isb) store_near(at, 16u * KYP, z, sg, e1024);
+        else store_near(at, 16u * KXP, z, sg, e1024);
+      }
+      if ((dirty >> (step & 1)) & 1) {  // zero slabs, and the padded columns
+        const unsigned st = 16u * (unsigned)(isb ? KYP : KXP);
+        const int s1 = isb || SHARED ? kNear : G::SAN;
+        for (int s = valid ? kNear : 0; s < s1; ++s) st_digits(at + (unsigned)s * st, 0u, 0u, 0u, 0u);
+      }
+    }
+    dirty &= ~(1 << (step & 1));
+  };
+  // One panel: convert panel p (its values are in v), take panel p + 1's values
+  // and look whether they are near, then, once every warp has stored panel p - 1
+  // (ready), store the digits and arrive.  The last warp issues panel p - 1's
+  // MMAs and the copies of panel p + 1's successor at that point instead.
+  const bool conv = warp < kConvWarps;
+  const unsigned rb0 = smem_u32(&ready_bar[0]);
+  if (npan > 0) {
+    if (conv) load(0);
+    if (tid == 0) spec[0] = 0;  // no exponents yet
+  }
+  __syncthreads();
+  if (TMA && npan > 2) fetch(2);  // (TMA: panel 0's values are in registers)
+#pragma unroll 1
+  for (int p = 0; p < npan; ++p) {
+    unsigned z[4][5];
+    Sign2 sg[4];
+    bool off = false;
+    if (conv) {
+      near_lanes<false>(v, max(te, 1), z, sg);
+      if constexpr (!TMA) fetch(p + 2);
+      if (p + 1 < npan) {
+        load(p + 1);
+        off = outside();
+      }
+    }
+    if (p > 0) {
+      if (!mbar_wait(rb0 + 8u * (unsigned)((p - 1) & 1), (unsigned)((p - 1) >> 1) & 1u, &bad)) break;
+      if (!conv) {
+        // every warp has taken panel p's values: its staging buffer is free
+        if (TMA && p + 2 < npan) fetch(p + 2);
+        issue();  // panel p - 1's
+      }
+    }
+    int ks = P / 16, cost = P * G::pairs_near;
+    bool all = false;
+    if (*reinterpret_cast<volatile int*>(&spec[p & 1]) == p) {
+      // Panel p holds a value that is not near: every warp comes here.
+      __syncthreads();
+      double u[8];
+      unsigned m = 0;  // largest magnitude
+      const int64_t pr = (int64_t)p * P;
 #pragma unroll
-      for (int k = 0; k < kMaxItems; ++k) {
-        if (!item_valid(k)) continue;  // an empty slot
-        // the larger magnitude's bit pattern; its exponent exceeds te[k]
-        // exactly when the pattern reaches (te[k] + 1) << 20.  A panel's
-        // maxima are only ever used as max(running exponent, panel
-        // maximum), so an item within its column's running exponent changes
-        // nothing (with steady exponents, nearly all items).  Subnormals
-        // (exponent field 0) never raise a column: its alignment exponent is
-        // at least 1 anyway.  Items past the panel's end hold zeros.
-        const unsigned m = max(hi32(v[k].x) & 0x7fffffffu, hi32(v[k].y) & 0x7fffffffu);
-        if (m >= ((unsigned)te[k] + 1u) << 20) {
+      for (int i = 0; i < 8; ++i) {
+        u[i] = (valid && r0 + pr + 8 * kc + i < r1) ? (sizeof(T) == 8 ? (double)src[pr + i] : widen((float)src[pr + i])) : 0.0;
+        m = max(m, abs_hi(u[i]));
+      }
+      // exponents (subnormals never raise a column: its alignment exponent is at least 1)
+      const bool up = valid && m >= ((unsigned)te + 1u) << 20;
+      if (bar_any(up)) {
+        if (up) {
           const int e = (int)(m >> 20);
           if (e == 2047) flag = 1;
-          atomicMax(&pmq[it_s[k] >> 16], e + EO_GRAM_HEADROOM);
-          g |= te[k] != 0;
+          // (finite exponents stay below 2047, so that an Inf or NaN always raises)
+          atomicMax(&Enew[slot], e == 2047 ? e : min(e + EO_GRAM_HEADROOM, 2046));
         }
-      }
-      return g;
-    };
-
-    double2 v[kMaxItems];
-    bool grew = false;  // a column of the current panel exceeds its running exponent
-    if (npan > 0) {
-      stage_values(0, v);
-      const int none[kMaxItems] = {};
-      (void)scan(v, pmax, none);  // nothing has accumulated yet
-    }
-    bar_conv<kConvThreads>();
-    if (!DIRECT && tid == 0 && 2 < npan) {  // staging buffer 0 is read: panel 2
-      fence_proxy_async();
-      load_panel(2);
-    }
-
-    int undrained = 0, drains = 0, ev = 0, pc = 0;  // ev: drains since the last full one
-    for (int p = 0; p < npan; ++p) {
-      const int db = p & 1;
-      const int pn = pc == 2 ? 0 : pc + 1, pz = pn == 2 ? 0 : pn + 1;  // (p + 1) % 3, (p + 2) % 3
-      const int* eprev = Erun + (db ^ 1) * nslots;  // through panel p-1
-      const int* pcur = pmax + pc * nslots;         // panel p
-      if (tid < nslots) {
-        Erun[db * nslots + tid] = max(eprev[tid], pcur[tid]);  // through panel p
-        pmax[pz * nslots + tid] = 0;                           // panel p-1's, read for the last time in p-1
-      }
-      int A[kMaxItems], te[kMaxItems];  // te: running exponent through panel p of the item's column
-#pragma unroll
-      for (int k = 0; k < kMaxItems; ++k) {
-        const int c = (int)(it_s[k] >> 16);
-        te[k] = max(eprev[c], pcur[c]);
-        A[k] = max(te[k], 1);
-      }
-
-      // the digit buffer db is free once the MMAs of panel p-2 are done
-      if (p >= 2) mbar_wait(fb0 + 8u * db, (unsigned)((p - 2) >> 1) & 1u, &bad);
-      // digits of panel p
-      unsigned char* dbuf = dig + (size_t)db * pl.dig_bytes;
-      const unsigned e1024 = exp1024x2();
-      bool off_near = false;  // an item of this warp took the general path
-#pragma unroll
-      for (int k = 0; k < kMaxItems; ++k) {
-        const bool valid = item_valid(k) && (!PAD || !(it_d[k] & 0x40000000u));
-        // every value of the warp's items normal and within 20 binades of its
-        // alignment exponent (nearly always): the words without selects
-        const bool near =
-            __all_sync(0xffffffffu, !valid || min(abs_hi(v[k].x), abs_hi(v[k].y)) >= near_floor(A[k]));
-        off_near |= !near;
+        __syncthreads();
+        if (used > 0) {
+          empty(step, true);
+          // totals onto the new grid: divide by 2^(growth of both columns' exponents)
+          const int ysb = SHARED ? 0 : KXP;
+          for (int y = 0; y < NY; ++y) {
+            const int cy = ysb + yq + y;
+            const int dx = Erun[xl] ? Enew[xl] - Erun[xl] : 0;
+            const int dy = Erun[cy] ? Enew[cy] - Erun[cy] : 0;
+            for (int q = 0; q < kParts; ++q) tot[q * NY + y] = w_shift(tot[q * NY + y], dx + dy);
+          }
+        }
+        __syncthreads();
+        if (tid < G::COLS) Erun[tid] = Enew[tid];
         if (valid) {
-          unsigned wa[4], wb[4];
-          const unsigned signs = ((hi32(v[k].x) >> 31) << 15) | (hi32(v[k].y) & 0x80000000u);
-          // operand A or B (warp-uniform; known at compile time in the hot
-          // plans): two copies of the stores, so that with a compile-time
-          // plan the slab stride is an immediate offset
-          unsigned char* dst = dbuf + (it_d[k] & (PAD ? 0x3fffffffu : 0x7fffffffu));
-          if (near) {
-            xwords_near(v[k].x, 52 - A[k], wa);
-            xwords_near(v[k].y, 52 - A[k], wb);
-            add_bias_near(wa);
-            add_bias_near(wb);
-            if (item_b(k))
-              store_bal_digits_near<0>(dst, stride_b, pair_lanes(wa, wb), pair_sign(signs, e1024));
-            else
-              store_bal_digits_near<0>(dst, stride_a, pair_lanes(wa, wb), pair_sign(signs, e1024));
-          } else {
-            xwords(v[k].x, A[k], wa);
-            xwords(v[k].y, A[k], wb);
-            add_bias(wa);
-            add_bias(wb);
-            if (item_b(k))
-              store_bal_digits<0>(dst, stride_b, pair_lanes(wa, wb), pair_sign(signs, e1024));
-            else
-              store_bal_digits<0>(dst, stride_a, pair_lanes(wa, wb), pair_sign(signs, e1024));
+          te = Enew[slot];
+          set_window();
+        }
+        __syncthreads();
+      }
+      // a nonzero value (normal or not) below the window
+      const int A = max(te, 1);
+      bool below = false;
+      const unsigned floor = (unsigned)max(A - kNearBits, 1) << 20;
+#pragma unroll
+      for (int i = 0; i < 8; ++i) below |= valid && (abs_hi(u[i]) | lo32(u[i])) != 0u && abs_hi(u[i]) < floor;
+      all = bar_any(below);
+      if (!all) {
+        unsigned y[4][5];
+        Sign2 sy[4];
+        near_lanes<true>(u, A, y, sy);
+        put(y, sy);
+      } else {
+        Sign2 sy[4];
+#pragma unroll 1
+        for (int h = 0; h < G::NF; ++h) {
+          if (h) {  // the previous step's digits are stored: its MMAs
+            finish_step(G::FK, true, 16 * G::FK * G::pairs_all);
+            __syncthreads();
+            issue();
           }
-        }
-      }
-      if (off_near && lane == 0) far[db] = p;
-      fence_proxy_async();
-
-      // this thread's accumulators (its own TMEM lanes and columns) are drained
-      // before it marks panel p ready
-      if ((grew || undrained >= pl.drain_panels) && undrained > 0) {
-        // a full drain before a fold or a growth; otherwise the groups whose
-        // period ends here
-        const bool full = grew || drains + 1 == pl.fold_drains;
-        int g0 = 0;  // first group due
-        if (!full) {
-          g0 = 5;
+          const unsigned db = (unsigned)(step & 1) * G::dig_bytes;
+          if (step >= 2) wait_step(step - 2);
+          const int k = kc - h * 2 * G::FK;  // K chunk within the step
+          if (mine && k >= 0 && k < 2 * G::FK) {
+            const unsigned dst =
+                dig_s + db + (isb ? G::b_off_all + (unsigned)k * G::LBA : (unsigned)k * G::LAA) + (unsigned)lc * 16u;
+            const unsigned st = 16u * (unsigned)(isb ? KYP : KXP);
+            unsigned y[4][7];
 #pragma unroll
-          for (int g = 4; g >= 0; --g) {
-            const int per = 1 << ((pl.drain_log >> (3 * g)) & 7);
-            if (g0 == g + 1 && ((ev + 1) & (per - 1)) == 0) g0 = g;
+            for (int i = 0; i < 4; ++i) {
+              unsigned a[4], b[4];
+              any_words(u[2 * i], A, a);
+              any_words(u[2 * i + 1], A, b);
+              sy[i] = sign2(u[2 * i], u[2 * i + 1]);
+              y[i][0] = __byte_perm(a[3], b[3], 0x5410);
+#pragma unroll
+              for (int j = 0; j < 3; ++j) {
+                y[i][1 + 2 * j] = __byte_perm(a[2 - j], b[2 - j], 0x7632);
+                y[i][2 + 2 * j] = __byte_perm(a[2 - j], b[2 - j], 0x5410);
+              }
+            }
+#pragma unroll
+            for (int i = 0; i < 7; ++i) {
+              const Sign2 s0 = i ? sy[0] : top(sy[0]), s1 = i ? sy[1] : top(sy[1]);
+              const Sign2 s2 = i ? sy[2] : top(sy[2]), s3 = i ? sy[3] : top(sy[3]);
+              st_digits(dst + (unsigned)(2 * i) * st, digit_hi(y[0][i], e1024, s0), digit_hi(y[1][i], e1024, s1),
+                        digit_hi(y[2][i], e1024, s2), digit_hi(y[3][i], e1024, s3));
+              st_digits(dst + (unsigned)(2 * i + 1) * st, digit_lo(y[0][i], e1024, sy[0]), digit_lo(y[1][i], e1024, sy[1]),
+                        digit_lo(y[2][i], e1024, sy[2]), digit_lo(y[3][i], e1024, sy[3]));
+            }
+            if (!isb)
+              for (int s = kAll; s < G::SAA; ++s) st_digits(dst + (unsigned)s * st, 0u, 0u, 0u, 0u);
           }
+          dirty |= 1 << (step & 1);
         }
-        if (drainer) {
-          // all MMAs so far (the last commit is panel p-1's) are done before TMEM is read
-          mbar_wait(fb0 + 8u * ((p - 1) & 1), (unsigned)((p - 1) >> 1) & 1u, &bad);
-          tc_fence_after();
-          drain(g0);
-          if (full) fold();
-        }
-        ++drains;
-        ++ev;
-        if (full) {
-          drains = 0;
-          ev = 0;
-        }
-        if (grew && drainer) {  // totals onto the new grid: divide by 2^(growth of both columns' exponents)
-          const int ysb = pl.shared ? 0 : kxp;
-#pragma unroll
-          for (int y = 0; y < NYT; ++y) {
-            const int cx = xl, cy = ysb + yq + y;
-            const int dx = eprev[cx] ? max(eprev[cx], pcur[cx]) - eprev[cx] : 0;
-            const int dy = eprev[cy] ? max(eprev[cy], pcur[cy]) - eprev[cy] : 0;
-            W[y] = w_shift(W[y], dx + dy);
-          }
-        }
-        tc_fence_before();
-        undrained = 0;
+        ks = P / 16 - (G::NF - 1) * G::FK;
+        cost = 16 * ks * G::pairs_all;
       }
-      mbar_arrive(rb0 + 8u * db);  // digits of p ready (and TMEM drained if it was due)
-      ++undrained;
-
-      // panel p+1: values and column maxima (growth against the exponents through p)
-      bool gl = false;
-      double2 vn[kMaxItems];
+      // panel p + 1's values again (they are still staged; nothing but the
+      // loop's state is kept across this branch) and their look, as the
+      // exponents may have grown
+      if (conv && p + 1 < npan) {
+        load(p + 1);
+        off = outside();
+      } else {
 #pragma unroll
-      for (int k = 0; k < kMaxItems; ++k) vn[k] = make_double2(0.0, 0.0);
-      if (p + 1 < npan) {
-        stage_values(p + 1, vn);
-        gl = scan(vn, pmax + pn * nslots, te);
+        for (int i = 0; i < 8; ++i) v[i] = 0.0;
       }
-      grew = bar_conv_or<kConvThreads>(gl);
-      if (!DIRECT && tid == 0 && p + 3 < npan) {  // staging buffer (p + 1) & 1 is read: panel p + 3
-        fence_proxy_async();
-        load_panel(p + 3);
-      }
-#pragma unroll
-      for (int k = 0; k < kMaxItems; ++k) v[k] = vn[k];
-      pc = pn;
+    } else {
+      put(z, sg);
     }
-
-    if constexpr (DIRECT) asm volatile("cp.async.wait_all;" ::: "memory");  // the last (empty) copies
-    // last drain and fold
-    if (npan > 0 && drainer) {
-      mbar_wait(fb0 + 8u * ((npan - 1) & 1), (unsigned)((npan - 1) >> 1) & 1u, &bad);
-      tc_fence_after();
-      drain(0);
-      fold();
-      tc_fence_before();
+    finish_step(ks, all, cost);
+    if (conv) {
+      if (off) *reinterpret_cast<volatile int*>(&spec[(p + 1) & 1]) = p + 1;
+      __syncwarp();
+      if (lane == 0) mbar_arrive(rb0 + 8u * (unsigned)(p & 1));
     }
   }
 
+  if constexpr (!TMA) asm volatile("cp.async.wait_all;" ::: "memory");  // the last (empty) copies
+  // the last step's MMAs, drain and fold
+  __syncthreads();
+  issue();
+  if (step > 0) {
+    if (warp == 0) mbar_wait_final(fb0 + 8u * (unsigned)((step - 1) & 1), (unsigned)((step - 1) >> 1) & 1u, &bad);
+    empty(step, true);
+  }
   __syncthreads();
   if (warp == 0) {
     tc_fence_after();
@@ -733,25 +798,22 @@ __global__ void __launch_bounds__(kThreads, 1)
   }
 
   // sum the lane blocks (digit phase j) of every output and write the partials
-  i128* red = reinterpret_cast<i128*>(dig);  // 128 lanes x KYP entries (the MMAs are done)
-  if (warp < kDrainWarps) {
-#pragma unroll
-    for (int y = 0; y < NYT; ++y) red[L * KYP + yq + y] = W[y];
-  }
+  i128* red = reinterpret_cast<i128*>(dig);  // kParts x 128 lanes x KYP entries (the MMAs are done)
+  for (int q = 0; q < kParts; ++q)
+    for (int y = 0; y < NY; ++y) red[(q * kLanes + L) * KYP + yq + y] = tot[q * NY + y];
   __syncthreads();
-  const int J = pl.J;
-  const int* Efin = Erun + ((npan - 1) & 1) * nslots;  // running exponents through the last panel
-  for (int e = tid; e < kxp * KYP; e += kThreads) {
-    const int xo = e / KYP, yo = e % KYP;
-    const int i = x0 + xo, j = y0 + yo;
+  for (int e = tid; e < KXP * KYP; e += kThreads) {
+    const int i = e / KYP, yo = e % KYP, j = y0 + yo;
     if (i >= kx || j >= ky) continue;
     i128 w = 0;
-    for (int b = 0; b < J; ++b) w += red[(b * kxp + xo) * KYP + yo];
-    const int cy = pl.shared ? yo : kxp + yo;
+    for (int b = 0; b < J; ++b) {
+      w += red[(b * KXP + i) * KYP + yo];
+      if constexpr (SHARED) w += red[(kLanes + b * KXP + i) * KYP + yo] + red[(kLanes + b * KXP + yo) * KYP + i];
+    }
     FxPart o;
     o.wl = (long long)(unsigned long long)(u128)w;
     o.wh = (long long)(w >> 64);
-    o.s = max(Efin[xo], 1) + max(Efin[cy], 1) - kOffsetDigits;
+    o.s = max(Erun[i], 1) + max(Erun[(SHARED ? 0 : KXP) + yo], 1) - kOffsetDigits;
     o.flag = flag | bad;
     o.pad = 0;
     parts[(size_t)blockIdx.y * ((size_t)kx * ky) + (size_t)j * kx + i] = o;
@@ -759,90 +821,28 @@ __global__ void __launch_bounds__(kThreads, 1)
 }
 
 // ------------------------------------------------------------ host side
-int pow2_at_least(int v) {
-  int p = 1;
-  while (p < v) p <<= 1;
-  return p;
-}
-
-// Largest |digit| of slab s: balanced digits are in [-64, 63] except the top
-// one, in [-64, 128].
-constexpr long long digit_bound(int s) { return s == 0 ? 128 : 64; }
-
-// Largest per-row sum of |D_s D_t| that a column block c in [c0, c1] of any
-// lane block j collects: the pairs (s, t) = (J q + j, c - J q) with J q <= c
-// and J q + j <= 14.
-long long group_bound(int c0, int c1, int J) {
-  long long worst = 0;
-  for (int c = c0; c <= c1; ++c)
-    for (int j = 0; j < J; ++j) {
-      long long b = 0;
-      for (int q = 0; J * q <= c && J * q + j <= 14; ++q) b += digit_bound(J * q + j) * digit_bound(c - J * q);
-      worst = std::max(worst, b);
-    }
-  return worst;
-}
+// Tile and launch geometry of one product: X tile width kxp >= kx (16, 32 or
+// 64), Y tile width kyp, row chunks.
+struct UPlan {
+  int kxp, kyp, nty;
+  bool shared;
+};
 
 UPlan make_plan(int kx, int ky, bool sym) {
   UPlan p{};
-  if (sym && kx <= 16) {
-    p.shared = 1;
-    p.kxp = 16;
-    p.kyp = 16;
-  } else {
-    p.kxp = std::min(128, std::max(16, pow2_at_least(kx)));
-    p.kyp = ky <= 8 ? 8 : 16;
-  }
-  p.J = kLanes / p.kxp;
-  p.nq = 14 / p.J + 1;
-  p.ntx = (kx + p.kxp - 1) / p.kxp;
+  p.shared = sym && kx <= 16;
+  p.kxp = kx <= 16 ? 16 : (kx <= 32 ? 32 : 64);
+  p.kyp = p.shared || ky > 8 ? 16 : 8;
   p.nty = p.shared ? 1 : (ky + p.kyp - 1) / p.kyp;
-  p.nslots = p.shared ? p.kxp : p.kxp + p.kyp;
-  // rows an accumulator may absorb: the largest sum of digit-pair bounds
-  // that one column block collects per row (below 2^24 in total)
-  const long long row_bound = group_bound(0, 14, p.J);
-  const int rows_cap = (int)((1ll << 24) / row_bound);
-  int best = 16;
-  for (int P = 16; P <= 128; P *= 2) {
-    if (P > rows_cap || (size_t)p.nslots * P / 2 > (size_t)kMaxItems * kConvThreads) break;
-    const size_t dig = (size_t)32 * P * (p.shared ? p.kxp : p.kxp + p.kyp);
-    const size_t stg = (size_t)p.nslots * P * 8;
-    const size_t red = (size_t)kLanes * p.kyp * 16;
-    if (std::max(2 * dig, red) + 2 * stg + 20 * (size_t)p.nslots + 1024 > kSmemCap) break;
-    best = P;
-  }
-  p.P = best;
-  p.drain_panels = std::max(1, rows_cap / p.P);
-  // a drain adds at most drain rows x row_bound to a 32-bit running sum
-  const long long per_drain = (long long)p.drain_panels * p.P * row_bound;
-  p.fold_drains = (int)std::max(1ll, std::min<long long>(kFoldRows / (p.drain_panels * p.P),
-                                                          ((1ll << 31) - 1) / per_drain));
-  // Column block c of a lane block collects at most c / J + 1 digit pairs
-  // per row, so a group of three blocks stays exact for 2^24 / (its largest
-  // per-row bound) rows: it is drained every 2^g-th drain (g <= 3).
-  p.drain_log = 0;
-  for (int g = 0; g < 5; ++g) {
-    const long long dmax = (1ll << 24) / (group_bound(3 * g, std::min(3 * g + 2, 14), p.J) * p.drain_panels * p.P);
-    int lg = 0;
-    while (lg < 3 && (2ll << lg) <= dmax) ++lg;
-    p.drain_log |= lg << (3 * g);
-  }
-  p.a_bytes = (unsigned)(32 * p.P * p.kxp);
-  p.dig_bytes = (unsigned)(32 * p.P * (p.shared ? p.kxp : p.kxp + p.kyp));
-  p.stage_bytes = (unsigned)(p.nslots * p.P * 8);
   return p;
 }
 
-size_t plan_smem(const UPlan& p) {
-  const size_t red = (size_t)kLanes * p.kyp * 16;
-  return std::max(2 * (size_t)p.dig_bytes, red) + 2 * (size_t)p.stage_bytes + 5 * sizeof(int) * p.nslots + 1024;
-}
+constexpr int kMinRows = 64;  // rows of the smallest row chunk
 
 int num_chunks(int64_t n, const UPlan& p) {
-  const int tiles = p.ntx * p.nty;
-  const int64_t by_rows = (n + p.P - 1) / p.P;
-  const int64_t want = std::max<int64_t>(1, (152 + tiles - 1) / tiles);  // one CTA per SM
-  const int64_t need = (n + (1ll << 22) - 1) >> 22;                     // <= 2^22 rows per chunk
+  const int64_t by_rows = (n + kMinRows - 1) / kMinRows;
+  const int64_t want = std::max<int64_t>(1, (152 + p.nty - 1) / p.nty);  // one CTA per SM
+  const int64_t need = (n + (1ll << 22) - 1) >> 22;                       // <= 2^22 rows per chunk
   return (int)std::max<int64_t>(1, std::min(by_rows, std::max(want, need)));
 }
 
@@ -852,7 +852,7 @@ int capped_chunks(int64_t n, const UPlan& p, int ctas) {
   const int c = num_chunks(n, p);
   if (ctas <= 0) return c;
   const int64_t need = (n + (1ll << 22) - 1) >> 22;
-  const int64_t cap = std::max<int64_t>(1, ctas / (p.ntx * p.nty));
+  const int64_t cap = std::max<int64_t>(1, ctas / p.nty);
   return (int)std::max<int64_t>(std::max<int64_t>(1, need), std::min<int64_t>(c, cap));
 }
 
@@ -882,21 +882,37 @@ bool make_map(CUtensorMap* m, const double* A, int64_t n, int k, int64_t ld, int
              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-size_t plan_smem_direct(const UPlan& p) {
-  return plan_smem(p) - 2 * (size_t)p.stage_bytes + std::max<size_t>(2 * (size_t)p.stage_bytes, kDirectStageBytes);
+struct Maps {
+  CUtensorMap x, y;
+};
+
+template <class G, typename T, bool TMA>
+cudaError_t launch_kernel(const UPlan& plan, int chunks, int64_t n, int kx, const T* X, int64_t ldx, int ky,
+                          const T* Y, int64_t ldy, int64_t rpc, const Maps& maps, FxPart* parts, const int* gate,
+                          cudaStream_t st) {
+  cudaError_t e = set_dyn_smem(umma_gram_partial_kernel<G, T, TMA>, G::smem);
+  if (e != cudaSuccess) return e;
+  umma_gram_partial_kernel<G, T, TMA>
+      <<<dim3(plan.nty, chunks), kThreads, G::smem, st>>>(n, kx, X, ldx, ky, Y, ldy, rpc, maps.x, maps.y, parts, gate);
+  return cudaGetLastError();
 }
 
-template <int KYP, bool DIRECT, bool PAD, typename T = double, int KXPC = 0, int PC = 0>
-cudaError_t launch_kernel(const UPlan& plan, int chunks, int64_t n, int kx, const T* X, int64_t ldx, int ky,
-                          const T* Y, int64_t ldy, int64_t rpc, const CUtensorMap& tmx, const CUtensorMap& tmy,
-                          FxPart* parts, const int* gate, cudaStream_t st) {
-  const size_t smem = DIRECT ? plan_smem_direct(plan) : plan_smem(plan);
-  cudaError_t e = set_dyn_smem(umma_gram_partial_kernel<KYP, DIRECT, PAD, T, KXPC, PC>, smem);
-  if (e != cudaSuccess) return e;
-  dim3 grid(plan.ntx * plan.nty, chunks);
-  umma_gram_partial_kernel<KYP, DIRECT, PAD, T, KXPC, PC>
-      <<<grid, kThreads, smem, st>>>(n, kx, X, ldx, ky, Y, ldy, plan, rpc, tmx, tmy, parts, gate);
-  return cudaGetLastError();
+template <typename T, bool TMA>
+cudaError_t launch_plan(const UPlan& plan, int chunks, int64_t n, int kx, const T* X, int64_t ldx, int ky,
+                        const T* Y, int64_t ldy, int64_t rpc, const Maps& maps, FxPart* parts, const int* gate,
+                        cudaStream_t st) {
+#define EO_UMMA_LAUNCH(A, B, S) \
+  return launch_kernel<Plan<A, B, S>, T, TMA>(plan, chunks, n, kx, X, ldx, ky, Y, ldy, rpc, maps, parts, gate, st)
+  if (plan.shared) EO_UMMA_LAUNCH(16, 16, true);
+  if (plan.kyp == 16) {
+    if (plan.kxp == 16) EO_UMMA_LAUNCH(16, 16, false);
+    if (plan.kxp == 32) EO_UMMA_LAUNCH(32, 16, false);
+    EO_UMMA_LAUNCH(64, 16, false);
+  }
+  if (plan.kxp == 16) EO_UMMA_LAUNCH(16, 8, false);
+  if (plan.kxp == 32) EO_UMMA_LAUNCH(32, 8, false);
+  EO_UMMA_LAUNCH(64, 8, false);
+#undef EO_UMMA_LAUNCH
 }
 
 // One thread waits for a phase of an mbarrier that nothing completes, bounded
@@ -923,181 +939,110 @@ cudaError_t umma_gram_take_wait_record(unsigned* out) { return take_wait_record(
 
 namespace {
 
-// How one product reaches its operands: by TMA (tensor maps) or by the
-// converter threads' own copies (direct); neither: the integer limbs.
-struct Route {
-  UPlan plan;
-  bool tma_ok, direct;
-  CUtensorMap tmx, tmy;
-};
-void route(Route& r, int64_t n, int kx, const double* X, int64_t ldx, int ky, const double* Y, int64_t ldy,
-           bool sym) {
-  r.plan = make_plan(kx, ky, sym);
-  r.tmx = CUtensorMap{};
-  r.tmy = CUtensorMap{};
-  // TMA addresses 16-byte aligned bases and leading dimensions of whole 16-byte units
-  r.tma_ok = (uintptr_t)X % 16 == 0 && (uintptr_t)Y % 16 == 0 && ldx % 2 == 0 && ldy % 2 == 0 && n < (1ll << 31) &&
-             make_map(&r.tmx, X, n, kx, ldx, r.plan.kxp) && make_map(&r.tmy, Y, n, ky, ldy, r.plan.kyp);
-  // EO_DD_GRAM_LOADS=direct uses the copies for TMA-addressable operands too.
-  const char* lm = getenv("EO_DD_GRAM_LOADS");
-  const bool force_direct = lm && lm[0] == 'd';
-  r.direct = (!r.tma_ok || force_direct) && (uintptr_t)X % 8 == 0 && (uintptr_t)Y % 8 == 0 &&
-             plan_smem_direct(r.plan) <= kSmemCap;
-}
-
 // A symmetric product with more than 16 columns runs as column strips of 16:
 // strip c0 .. c1 - 1 is X[:, 0:c1]^T X[:, c0:c1] (the first one the symmetric
 // 16-column product), of which the reduction keeps the entries on and above
 // the diagonal of G and mirrors them (so G is exactly symmetric).  Each
-// value is converted once per strip that reads it, where the one-tile plans
-// of X^T Y over all columns convert it once per 16-column Y tile and once
-// more as the Y operand.
-bool use_strips(int64_t n, int kx, const double* X, int64_t ldx, bool sym) {
-  if (!sym || kx <= 16) return false;
-  for (int c0 = 0; c0 < kx; c0 += 16) {
-    const int c1 = std::min(kx, c0 + 16);
-    Route r;
-    route(r, n, c1, X, ldx, c1 - c0, X + (size_t)c0 * ldx, ldx, c0 == 0);
-    if (!r.tma_ok && !r.direct) return false;
-  }
-  return true;
-}
-
-cudaError_t launch_one(const Route& r, int64_t n, int kx, const double* X, int64_t ldx, int ky, const double* Y,
-                       int64_t ldy, void* scratch, double* G_hi, double* G_lo, int ldg, const int* gate,
-                       cudaStream_t st, int ctas, bool sym, int jo) {
-  const UPlan& plan = r.plan;
-  const bool direct = r.direct;
-  const CUtensorMap& tmx = r.tmx;
-  const CUtensorMap& tmy = r.tmy;
+// value is converted once per strip that reads it, where one-tile plans of
+// X^T Y over all columns convert it once per 16-column Y tile and once more
+// as the Y operand.
+template <typename T>
+cudaError_t launch_one(int64_t n, int kx, const T* X, int64_t ldx, int ky, const T* Y, int64_t ldy, void* scratch,
+                       double* G_hi, double* G_lo, int ldg, const int* gate, cudaStream_t st, int ctas, bool sym,
+                       int jo, bool shared) {
+  const UPlan plan = make_plan(kx, ky, shared);
   const int chunks = capped_chunks(n, plan, ctas);
+  // whole K steps per chunk: at most 15 rows of imbalance, and every chunk's
+  // first row keeps its column's alignment
   int64_t rpc = (n + chunks - 1) / chunks;
-  rpc = std::max<int64_t>(plan.P, (rpc + plan.P - 1) / plan.P * plan.P);
+  rpc = std::max<int64_t>(16, (rpc + 15) / 16 * 16);
   FxPart* parts = static_cast<FxPart*>(scratch);
-  const bool pad = plan.ntx * plan.kxp > kx || (!plan.shared && plan.nty * plan.kyp > ky);
+  alignas(64) Maps maps{};
   cudaError_t e;
-#define EO_UMMA_LAUNCH(K, D, PD) \
-  launch_kernel<K, D, PD>(plan, chunks, n, kx, X, ldx, ky, Y, ldy, rpc, tmx, tmy, parts, gate, st)
-  // the two plans of the projection step: V^T Y (64 + 16 columns, 32-row
-  // panels) and a symmetric 16-column Gram (128-row panels)
-  const bool hot_vty = !direct && !pad && plan.kyp == 16 && !plan.shared && plan.kxp == 64 && plan.P == 32;
-  const bool hot_sym = !direct && !pad && plan.kyp == 16 && plan.shared && plan.kxp == 16 && plan.P == 128;
-  if (hot_vty)
-    e = launch_kernel<16, false, false, double, 64, 32>(plan, chunks, n, kx, X, ldx, ky, Y, ldy, rpc, tmx, tmy, parts,
-                                                        gate, st);
-  else if (hot_sym)
-    e = launch_kernel<16, false, false, double, 16, 128>(plan, chunks, n, kx, X, ldx, ky, Y, ldy, rpc, tmx, tmy,
-                                                         parts, gate, st);
-  else if (plan.kyp == 16)
-    e = direct ? (pad ? EO_UMMA_LAUNCH(16, true, true) : EO_UMMA_LAUNCH(16, true, false))
-               : (pad ? EO_UMMA_LAUNCH(16, false, true) : EO_UMMA_LAUNCH(16, false, false));
-  else
-    e = direct ? (pad ? EO_UMMA_LAUNCH(8, true, true) : EO_UMMA_LAUNCH(8, true, false))
-               : (pad ? EO_UMMA_LAUNCH(8, false, true) : EO_UMMA_LAUNCH(8, false, false));
-#undef EO_UMMA_LAUNCH
+  bool tma = false;
+  if constexpr (sizeof(T) == 8) {
+    // TMA addresses 16-byte aligned bases and leading dimensions of whole
+    // 16-byte units, rows below 2^31 (a box may start past the last row)
+    const char* lm = getenv("EO_DD_GRAM_LOADS");  // "direct": the threads' own copies for such operands too
+    tma = (uintptr_t)X % 16 == 0 && (uintptr_t)Y % 16 == 0 && ldx % 2 == 0 && ldy % 2 == 0 && n < (1ll << 31) - 1024 &&
+          !(lm && lm[0] == 'd') && make_map(&maps.x, X, n, kx, ldx, plan.kxp) &&
+          make_map(&maps.y, Y, n, ky, ldy, plan.kyp);
+    e = tma ? launch_plan<T, true>(plan, chunks, n, kx, X, ldx, ky, Y, ldy, rpc, maps, parts, gate, st)
+            : launch_plan<T, false>(plan, chunks, n, kx, X, ldx, ky, Y, ldy, rpc, maps, parts, gate, st);
+  } else {
+    e = launch_plan<T, false>(plan, chunks, n, kx, X, ldx, ky, Y, ldy, rpc, maps, parts, gate, st);
+  }
   if (e != cudaSuccess) return e;
   return launch_fx_reduce(kx, ky, sym, chunks, parts, G_hi, G_lo, ldg, gate, st, jo);
+}
+
+template <typename T>
+cudaError_t launch_gram_t(int64_t n, int kx, const T* X, int64_t ldx, int ky, const T* Y, int64_t ldy, bool sym,
+                          void* scratch, double* G_hi, double* G_lo, int ldg, const int* gate, cudaStream_t st,
+                          int ctas) {
+  if (!sym) return launch_one(n, kx, X, ldx, ky, Y, ldy, scratch, G_hi, G_lo, ldg, gate, st, ctas, false, 0, false);
+  for (int c0 = 0; c0 < kx; c0 += 16) {
+    const int c1 = std::min(kx, c0 + 16);
+    cudaError_t e = launch_one(n, c1, X, ldx, c1 - c0, X + (size_t)c0 * ldx, ldx, scratch, G_hi, G_lo, ldg, gate, st,
+                               ctas, true, c0, c0 == 0);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 }  // namespace
 
 size_t umma_gram_scratch_bytes(int64_t n, int kx, int ky, bool sym) {
-  if (sym) ky = kx;
-  size_t b = (size_t)num_chunks(n, make_plan(kx, ky, sym)) * (size_t)kx * ky * sizeof(FxPart);
-  if (sym && kx > 16) {  // the column strips (one after another: the largest)
-    for (int c0 = 0; c0 < kx; c0 += 16) {
-      const int c1 = std::min(kx, c0 + 16);
-      b = std::max(b, (size_t)num_chunks(n, make_plan(c1, c1 - c0, c0 == 0)) * (size_t)c1 * (c1 - c0) *
-                          sizeof(FxPart));
-    }
+  if (!sym) return (size_t)num_chunks(n, make_plan(kx, ky, false)) * (size_t)kx * ky * sizeof(FxPart);
+  size_t b = 0;  // the column strips (one after another: the largest)
+  for (int c0 = 0; c0 < kx; c0 += 16) {
+    const int c1 = std::min(kx, c0 + 16);
+    b = std::max(b, (size_t)num_chunks(n, make_plan(c1, c1 - c0, c0 == 0)) * (size_t)c1 * (c1 - c0) * sizeof(FxPart));
   }
   return b;
 }
 
 int umma_gram_ctas(int64_t n, int kx, int ky, bool sym, int ctas) {
-  if (sym) ky = kx;
-  const UPlan plan = make_plan(kx, ky, sym);
-  int c = plan.ntx * plan.nty * capped_chunks(n, plan, ctas);
-  if (sym && kx > 16) {
-    for (int c0 = 0; c0 < kx; c0 += 16) {
-      const int c1 = std::min(kx, c0 + 16);
-      const UPlan ps = make_plan(c1, c1 - c0, c0 == 0);
-      c = std::max(c, ps.ntx * ps.nty * capped_chunks(n, ps, ctas));
-    }
+  if (!sym) {
+    const UPlan plan = make_plan(kx, ky, false);
+    return plan.nty * capped_chunks(n, plan, ctas);
+  }
+  int c = 0;
+  for (int c0 = 0; c0 < kx; c0 += 16) {
+    const int c1 = std::min(kx, c0 + 16);
+    const UPlan ps = make_plan(c1, c1 - c0, c0 == 0);
+    c = std::max(c, ps.nty * capped_chunks(n, ps, ctas));
   }
   return c;
 }
 
 int umma_gram_launches(int64_t n, int kx, const double* X, int64_t ldx, int ky, const double* Y, int64_t ldy,
                        bool sym) {
+  (void)n;
+  (void)X;
+  (void)ldx;
   (void)ky;
   (void)Y;
   (void)ldy;
-  return use_strips(n, kx, X, ldx, sym) ? 2 * ((kx + 15) / 16) : 2;
+  return sym ? 2 * ((kx + 15) / 16) : 2;
 }
 
 cudaError_t launch_umma_gram(int64_t n, int kx, const double* X, int64_t ldx, int ky, const double* Y, int64_t ldy,
                              bool sym, void* scratch, double* G_hi, double* G_lo, int ldg, const int* gate,
                              cudaStream_t st, int ctas) {
-  if (sym) {
-    Y = X;
-    ldy = ldx;
-    ky = kx;
-  }
-  if (use_strips(n, kx, X, ldx, sym)) {
-    for (int c0 = 0; c0 < kx; c0 += 16) {
-      const int c1 = std::min(kx, c0 + 16);
-      const double* Xs = X + (size_t)c0 * ldx;
-      Route r;
-      route(r, n, c1, X, ldx, c1 - c0, Xs, ldx, c0 == 0);
-      cudaError_t e =
-          launch_one(r, n, c1, X, ldx, c1 - c0, Xs, ldx, scratch, G_hi, G_lo, ldg, gate, st, ctas, true, c0);
-      if (e != cudaSuccess) return e;
-    }
-    return cudaSuccess;
-  }
-  Route r;
-  route(r, n, kx, X, ldx, ky, Y, ldy, sym);
-  // without TMA: the converters copy their own items (when the slots fit), else the integer limbs
-  if (!r.tma_ok && !r.direct)
-    return launch_fx_gram(n, kx, X, ldx, ky, Y, ldy, sym, scratch, G_hi, G_lo, ldg, gate, st, ctas);
-  return launch_one(r, n, kx, X, ldx, ky, Y, ldy, scratch, G_hi, G_lo, ldg, gate, st, ctas, sym, 0);
+  return launch_gram_t<double>(n, kx, X, ldx, ky, Y, ldy, sym, scratch, G_hi, G_lo, ldg, gate, st, ctas);
 }
 
 bool umma_gram_f32_supported(const float* X, const float* Y, int kx, int ky, bool sym) {
-  if (sym) {
-    Y = X;
-    ky = kx;
-  }
-  return (uintptr_t)X % 4 == 0 && (uintptr_t)Y % 4 == 0 && plan_smem_direct(make_plan(kx, ky, sym)) <= kSmemCap;
+  (void)kx;
+  (void)ky;
+  return (uintptr_t)X % 4 == 0 && (sym || (uintptr_t)Y % 4 == 0);
 }
 
 cudaError_t launch_umma_gram_f32(int64_t n, int kx, const float* X, int64_t ldx, int ky, const float* Y,
                                  int64_t ldy, bool sym, void* scratch, double* G_hi, double* G_lo, int ldg,
                                  const int* gate, cudaStream_t st) {
-  if (sym) {
-    Y = X;
-    ldy = ldx;
-    ky = kx;
-  }
-  const UPlan plan = make_plan(kx, ky, sym);
-  alignas(64) CUtensorMap tm{};  // unused: FP32 operands are copied by the converter threads
-  const int chunks = capped_chunks(n, plan, 0);
-  int64_t rpc = (n + chunks - 1) / chunks;
-  rpc = std::max<int64_t>(plan.P, (rpc + plan.P - 1) / plan.P * plan.P);
-  FxPart* parts = static_cast<FxPart*>(scratch);
-  const bool pad = plan.ntx * plan.kxp > kx || (!plan.shared && plan.nty * plan.kyp > ky);
-  cudaError_t e;
-  if (plan.kyp == 16)
-    e = pad ? launch_kernel<16, true, true, float>(plan, chunks, n, kx, X, ldx, ky, Y, ldy, rpc, tm, tm, parts, gate, st)
-            : launch_kernel<16, true, false, float>(plan, chunks, n, kx, X, ldx, ky, Y, ldy, rpc, tm, tm, parts, gate,
-                                                    st);
-  else
-    e = pad ? launch_kernel<8, true, true, float>(plan, chunks, n, kx, X, ldx, ky, Y, ldy, rpc, tm, tm, parts, gate, st)
-            : launch_kernel<8, true, false, float>(plan, chunks, n, kx, X, ldx, ky, Y, ldy, rpc, tm, tm, parts, gate,
-                                                   st);
-  if (e != cudaSuccess) return e;
-  return launch_fx_reduce(kx, ky, sym, chunks, parts, G_hi, G_lo, ldg, gate, st);
+  return launch_gram_t<float>(n, kx, X, ldx, ky, Y, ldy, sym, scratch, G_hi, G_lo, ldg, gate, st, 0);
 }
 
 }  // namespace eo
