@@ -15,16 +15,23 @@
 //                D = diag(M)^{-1/2} and Z = D U Lambda^{+1/2}, columns in
 //                ascending eigenvalue order, each eigenvector's largest
 //                entry positive (the SVQB of Stathopoulos and Wu, 2002).
-// In EO_DD the arithmetic is DD throughout (divisions, reciprocals and
-// square roots by Newton-Raphson); otherwise it is FP64.
+// In EO_DD and EO_DD_EFT the arithmetic is floating point with a 128-bit
+// significand on the integer pipe (wide.cuh: more accurate than double-double
+// and, on this GPU, several times faster), double-double in the pivoted
+// Cholesky; otherwise it is FP64.
 #include <algorithm>
+#include <type_traits>
 
 #include "common.cuh"
+#include "wide.cuh"
 
 namespace eo {
 namespace {
 
+using namespace fx;
+
 constexpr int kThreads = 256;
+constexpr int kJacThreads = 512;
 // Jacobi rotates a pair while |a_pq| > eps sqrt(|a_pp a_qq|).  The rotations
 // of a sweep leave off-diagonal entries at the rounding level of the
 // arithmetic (2^-106 in DD, 2^-53 in FP64), so eps sits a few bits above it:
@@ -91,8 +98,6 @@ struct Ar<MODE_DD> {
   }
 };
 
-__device__ __forceinline__ double dabs(double x) { return x < 0 ? -x : x; }
-
 __global__ void status_init_kernel(DevStatus* s, int k) {
   for (int i = threadIdx.x; i < 64; i += blockDim.x) s->gate[i] = i == 0;
   if (threadIdx.x == 0) {
@@ -108,31 +113,198 @@ __device__ void finish_gates(const SmallGates& g, int run_update, int want_next)
   if (g.next) *g.next = want_next;
 }
 
+// ------------------------------------------------- the two arithmetics
+
+// Vectors of numbers in shared memory, and the operations on them.
+struct F64 {
+  typedef double T;
+  static constexpr size_t kBytes = 8;
+  struct Vec {
+    double* p;
+    __device__ __forceinline__ T get(int i) const { return p[i]; }
+    __device__ __forceinline__ void set(int i, T v) const { p[i] = v; }
+  };
+  // n vectors of the given lengths, one after another
+  static __device__ __forceinline__ Vec vec(void* base, size_t total, size_t off) {
+    (void)total;
+    return Vec{static_cast<double*>(base) + off};
+  }
+  static __device__ __forceinline__ T zero() { return 0.0; }
+  static __device__ __forceinline__ T one() { return 1.0; }
+  static __device__ __forceinline__ T neg(T a) { return -a; }
+  static __device__ __forceinline__ T from(double hi, double lo) {
+    (void)lo;
+    return hi;
+  }
+  static __device__ __forceinline__ void to(T a, double& hi, double& lo) {
+    hi = a;
+    lo = 0.0;
+  }
+  static __device__ __forceinline__ T sub(T a, T b) { return __dsub_rn(a, b); }
+  static __device__ __forceinline__ T mul(T a, T b) { return __dmul_rn(a, b); }
+  static __device__ __forceinline__ T fma(T a, T b, T c) { return __fma_rn(a, b, c); }
+  static __device__ __forceinline__ T dot2(T a, T x, T b, T y) { return __dadd_rn(__dmul_rn(a, x), __dmul_rn(b, y)); }
+  static __device__ __forceinline__ T recip(T a) { return __drcp_rn(a); }
+  static __device__ __forceinline__ T sqrt(T a) { return __dsqrt_rn(a); }
+  static __device__ __forceinline__ T rsqrt(T a) { return __ddiv_rn(1.0, __dsqrt_rn(a)); }
+  static __device__ __forceinline__ bool is_zero(T a) { return a == 0.0; }
+  static __device__ __forceinline__ bool is_neg(T a) { return a < 0.0; }
+  static __device__ __forceinline__ bool less(T a, T b) { return a < b; }
+  static __device__ __forceinline__ T shfl_xor(T a, int m) { return __shfl_xor_sync(0xffffffffu, a, m); }
+  // a pivot that the elimination can divide by (ref: the matrix's own diagonal entry)
+  static __device__ __forceinline__ bool pivot_ok(T d, int ref) {
+    (void)ref;
+    return d > 0.0;
+  }
+  static __device__ __forceinline__ int scale_of(T a) {
+    (void)a;
+    return 0;
+  }
+  // The rotation that zeroes apq: whether |apq| > eps sqrt(|app aqq|), c and s.
+  static __device__ __forceinline__ bool rotation(T app, T aqq, T apq, T& c, T& sn) {
+    constexpr double eps = kJacobiEpsFP64;
+    const double scale = ::sqrt(fabs(app) * fabs(aqq));
+    if (!(fabs(apq) > eps * scale && apq != 0.0)) return false;
+    const double th = __dsub_rn(aqq, app) / (2.0 * apq);
+    const double t = fabs(th) > 1e150 ? 0.5 / th : copysign(1.0 / (fabs(th) + ::sqrt(::fma(th, th, 1.0))), th);
+    c = __ddiv_rn(1.0, __dsqrt_rn(__dadd_rn(1.0, __dmul_rn(t, t))));
+    sn = __dmul_rn(c, t);
+    return true;
+  }
+};
+
+struct Wide {
+  typedef wide T;
+  static constexpr size_t kBytes = 20;  // significand, exponent and sign in arrays of their own
+  struct Vec {
+    u128* m;
+    int* es;  // 2 e + s
+    __device__ __forceinline__ T get(int i) const {
+      const int x = es[i];
+      return wide{m[i], x >> 1, x & 1};
+    }
+    __device__ __forceinline__ void set(int i, T v) const {
+      m[i] = v.m;
+      es[i] = 2 * v.e + v.s;
+    }
+  };
+  static __device__ __forceinline__ Vec vec(void* base, size_t total, size_t off) {
+    u128* m = static_cast<u128*>(base);
+    return Vec{m + off, reinterpret_cast<int*>(m + total) + off};
+  }
+  static __device__ __forceinline__ T zero() { return wide_zero(); }
+  static __device__ __forceinline__ T one() { return wide_one(); }
+  static __device__ __forceinline__ T neg(T a) { return wide_neg(a); }
+  static __device__ __forceinline__ T from(double hi, double lo) { return wide_from(hi, lo); }
+  static __device__ __forceinline__ void to(T a, double& hi, double& lo) { wide_to_dd(a, hi, lo); }
+  static __device__ __forceinline__ T sub(T a, T b) { return wide_sub(a, b); }
+  static __device__ __forceinline__ T mul(T a, T b) { return wide_mul(a, b); }
+  static __device__ __forceinline__ T fma(T a, T b, T c) { return wide_fma(a, b, c); }
+  static __device__ __forceinline__ T dot2(T a, T x, T b, T y) { return wide_dot2(a, x, b, y); }
+  static __device__ __forceinline__ T recip(T a) { return wide_recip(a); }
+  static __device__ __forceinline__ T sqrt(T a) { return wide_sqrt(a); }
+  static __device__ __forceinline__ T rsqrt(T a) { return wide_rsqrt(a); }
+  static __device__ __forceinline__ bool is_zero(T a) { return wide_is_zero(a); }
+  static __device__ __forceinline__ bool is_neg(T a) { return a.s != 0 && !wide_is_zero(a); }
+  static __device__ __forceinline__ bool less(T a, T b) {  // a < b
+    const bool na = is_neg(a), nb = is_neg(b);
+    return na != nb ? na : (na ? wide_abs_gt(a, b) : wide_abs_gt(b, a));
+  }
+  static __device__ __forceinline__ T shfl_xor(T a, int m) {
+    unsigned long long h = (unsigned long long)(a.m >> 64), l = (unsigned long long)a.m;
+    h = __shfl_xor_sync(0xffffffffu, h, m);
+    l = __shfl_xor_sync(0xffffffffu, l, m);
+    const int x = __shfl_xor_sync(0xffffffffu, 2 * a.e + a.s, m);
+    return wide{((u128)h << 64) | l, x >> 1, x & 1};
+  }
+  // The Gram matrix is given to 2^-106: a pivot 118 binades below its diagonal
+  // entry is what rounding left of an exact zero.
+  static __device__ __forceinline__ bool pivot_ok(T d, int ref) { return !wide_is_zero(d) && d.s == 0 && d.e > ref - 118; }
+  static __device__ __forceinline__ int scale_of(T a) { return a.e; }
+  // The rotation that zeroes apq, whether |apq| > 2^-100 sqrt(|app aqq|): the
+  // tangent t from FP32 (24 bits: the remainder of apq is left to later
+  // sweeps), then c = (1 + t^2)^(-1/2) and s = t c to 2^-119, so that the
+  // rotation is orthogonal to that precision.
+  static __device__ __forceinline__ bool rotation(T app, T aqq, T apq, T& c, T& sn) {
+    static_assert(kJacobiEpsDD == 0x1p-100, "the test below");
+    if (wide_is_zero(apq)) return false;
+    const float fpq = wide_top(apq);
+    const int D = 2 * apq.e - app.e - aqq.e + 200;  // log2 of apq^2 2^200 / (app aqq), up to the significands
+    if (D < -2 || (D <= 2 && !(ldexpf(fpq * fpq, D) > wide_top(app) * wide_top(aqq)))) return false;
+    const wide d = wide_sub(aqq, app);
+    const int x = d.e - apq.e - 1;  // th = d / (2 apq) = +-(top d / top apq) 2^x
+    float t;
+    int te = 0;  // |t| 2^te
+    if (wide_is_zero(d) || x < -40) {
+      t = 1.0f;
+    } else if (x > 40) {
+      t = fpq / wide_top(d);  // 1 / (2 th)
+      te = -x - 1;
+    } else {
+      const float th = ldexpf(wide_top(d) / fpq, x);
+      t = 1.0f / (th + sqrtf(fmaf(th, th, 1.0f)));
+    }
+    const float g = te < -20 ? 1.0f : fmaf(ldexpf(t, te), ldexpf(t, te), 1.0f);  // 1 + t^2
+    const unsigned bits = __float_as_uint(t);                                       // t in (2^-43, 2)
+    const unsigned mt = (bits & 0x7fffffu) | 0x800000u;
+    te += (int)(bits >> 23) - 127;
+    const wide tw{(u128)mt << 104, te, wide_is_zero(d) ? 0 : d.s ^ apq.s};
+    // 1 + t^2 = G 2^-126: t^2 = mt^2 2^(2 te - 46) (te <= 0, or t = 1 up to its rounding)
+    const unsigned long long q = (unsigned long long)mt * mt;
+    const int sh = 80 + 2 * te;
+    const u128 t2 = sh >= 0 ? (u128)q << sh : shr128((u128)q, -sh);
+    c = wide_norm(rsqrt_fixed(((u128)1 << 126) + t2, g), 0, 0);
+    sn = wide_mul(tw, c);
+    return true;
+  }
+};
+
+// Packed upper triangle.
+__device__ __forceinline__ int tri(int i, int j) { return j * (j + 1) / 2 + i; }  // i <= j
+__device__ __forceinline__ int sym(int i, int j) { return i <= j ? tri(i, j) : tri(j, i); }
+__device__ __forceinline__ void untri(int t, int& i, int& j) {  // the entry with tri(i, j) = t
+  j = (int)((sqrtf(8.0f * (float)t + 1.0f) - 1.0f) * 0.5f);
+  if ((j + 1) * (j + 2) / 2 <= t) ++j;
+  if (j * (j + 1) / 2 > t) --j;
+  i = t - j * (j + 1) / 2;
+}
+
+// M's upper triangle into A; false (everywhere) if it has a NaN or Inf.  Ends with a barrier.
+template <class N>
+__device__ __forceinline__ bool load_upper(int k, const double* Mh, const double* Ml, int ldm, bool use_lo,
+                                           typename N::Vec A, int threads) {
+  bool ok = true;
+  for (int t = threadIdx.x; t < k * (k + 1) / 2; t += threads) {
+    int i, j;
+    untri(t, i, j);
+    const double h = Mh[(size_t)j * ldm + i], l = Ml && use_lo ? Ml[(size_t)j * ldm + i] : 0.0;
+    const bool fin = isfinite(h) && isfinite(l);
+    ok = ok && fin;
+    A.set(t, fin ? N::from(h, l) : N::zero());
+  }
+  return __syncthreads_and(ok ? 1 : 0) != 0;
+}
+
 // ------------------------------------------------------------ Cholesky
 
-template <int MODE>
+template <class N>
 __device__ __forceinline__ void chol_small_body(int k, const double* Mh, const double* Ml, int ldm, SmallWs* ws,
                                                 double* Rh_u, double* Rl_u, int ldr, DevStatus* st, SmallGates g,
                                                 int pass, int passes, double thr, int* info_user) {
-  using A_ = Ar<MODE>;
+  typedef typename N::T T;
   if (*g.run == 0) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  dd* A = reinterpret_cast<dd*>(smem_raw);  // A(i,j) = A[j*k+i]; R overwrites the upper triangle
-  dd* Z = A + k * k;
-  dd* Tb = Z + k * k;  // W = L^{-1}
-  __shared__ int flag;
+  const int nt = k * (k + 1) / 2;
+  // upper triangles: A(i, j), i <= j (becomes R); S, the products of a step;
+  // W = L^{-1}, W(l, c) (c <= l) at tri(c, l)
+  const typename N::Vec A = N::vec(smem_raw, 3 * (size_t)nt, 0), S = N::vec(smem_raw, 3 * (size_t)nt, nt),
+                        W = N::vec(smem_raw, 3 * (size_t)nt, 2 * (size_t)nt);
+  __shared__ int flag, ref[KMAX];
+  __shared__ double dhi[KMAX];
+  __shared__ T piv_inv;
   const int tid = threadIdx.x;
   if (tid == 0) flag = 0;
-  __syncthreads();
-  for (int t = tid; t < k * k; t += kThreads) {
-    const int i = t % k, j = t / k;
-    const int a = min(i, j), b = max(i, j);
-    dd v = dd{Mh[(size_t)b * ldm + a], Ml ? Ml[(size_t)b * ldm + a] : 0.0};
-    if (MODE != MODE_DD) v.lo = 0.0;
-    if (!dd_finite(v)) atomicExch(&flag, -1);
-    A[t] = v;
-  }
-  __syncthreads();
+  if (!load_upper<N>(k, Mh, Ml, ldm, true, A, kThreads) && tid == 0) flag = -1;
   // Square-root-free (L D L^T) elimination on the upper triangle: at step j
   // the pivot d_j = A(j,j) and the row A(j, j+1..) are those of the
   // standard algorithm before scaling, the Schur complement takes
@@ -140,44 +312,44 @@ __device__ __forceinline__ void chol_small_body(int k, const double* Mh, const d
   // takes W(l,:) -= L(l,j) W(j,:).  The products do not depend on the pivot,
   // so they run while one thread forms 1/d_j: the dependent chain of a step
   // is one reciprocal and one multiply-subtract.  Afterwards
-  // R = D^{1/2} L^T and Z = R^{-1} = L^{-T} D^{-1/2} (W: Tb, W(l,c) = Tb[c k + l];
-  // the products: Z, as scratch).
-  __shared__ dd piv_inv;
-  for (int t = tid; t < k * k; t += kThreads) Tb[t] = dd{(t % k) == (t / k) ? 1.0 : 0.0, 0.0};
+  // R = D^{1/2} L^T and Z = R^{-1} = L^{-T} D^{-1/2}.
+  for (int t = tid; t < nt; t += kThreads) {
+    int i, j;
+    untri(t, i, j);
+    W.set(t, i == j ? N::one() : N::zero());
+    if (i == j) ref[j] = N::scale_of(A.get(t));
+  }
   __syncthreads();
   if (flag == 0) {
     for (int j = 0; j < k; ++j) {
       const int m = k - j - 1, np = m * (m + 1) / 2, nq = m * (j + 1);
       if (tid == kThreads - 1) {
-        const dd d = A[j * k + j];
-        if (!(d.hi > 0.0)) flag = j + 1;
-        else piv_inv = A_::recip(d);
+        const T d = A.get(tri(j, j));
+        if (!N::pivot_ok(d, ref[j])) flag = j + 1;
+        else piv_inv = N::recip(d);
       }
       for (int t = tid; t < np + nq; t += kThreads) {
-        if (t < np) {  // (a, b) = j + 1 + (u, v), u <= v, t = v (v + 1) / 2 + u
-          int v = (int)((sqrtf(8.0f * (float)t + 1.0f) - 1.0f) * 0.5f);
-          if ((v + 1) * (v + 2) / 2 <= t) ++v;
-          if (v * (v + 1) / 2 > t) --v;
-          const int a = j + 1 + t - v * (v + 1) / 2, b = j + 1 + v;
-          Z[t] = A_::mul(A[a * k + j], A[b * k + j]);
+        if (t < np) {  // (a, b) = j + 1 + (u, v), u <= v
+          int u, v;
+          untri(t, u, v);
+          S.set(t, N::mul(A.get(tri(j, j + 1 + u)), A.get(tri(j, j + 1 + v))));
         } else {  // W row l = j + 1 + q % m, column c = q / m <= j
           const int q = t - np, l = j + 1 + q % m, c = q / m;
-          Z[t] = A_::mul(A[l * k + j], Tb[c * k + j]);
+          S.set(t, N::mul(A.get(tri(j, l)), W.get(tri(c, j))));
         }
       }
       __syncthreads();
       if (flag) break;
-      const dd w = piv_inv;
+      const T w = piv_inv;
       for (int t = tid; t < np + nq; t += kThreads) {
         if (t < np) {
-          int v = (int)((sqrtf(8.0f * (float)t + 1.0f) - 1.0f) * 0.5f);
-          if ((v + 1) * (v + 2) / 2 <= t) ++v;
-          if (v * (v + 1) / 2 > t) --v;
-          const int a = j + 1 + t - v * (v + 1) / 2, b = j + 1 + v;
-          A[b * k + a] = A_::sub(A[b * k + a], A_::mul(Z[t], w));
+          int u, v;
+          untri(t, u, v);
+          const int e = tri(j + 1 + u, j + 1 + v);
+          A.set(e, N::sub(A.get(e), N::mul(S.get(t), w)));
         } else {
-          const int q = t - np, l = j + 1 + q % m, c = q / m;
-          Tb[c * k + l] = A_::sub(Tb[c * k + l], A_::mul(Z[t], w));
+          const int q = t - np, e = tri(q / m, j + 1 + q % m);
+          W.set(e, N::sub(W.get(e), N::mul(S.get(t), w)));
         }
       }
       __syncthreads();
@@ -191,57 +363,59 @@ __device__ __forceinline__ void chol_small_body(int k, const double* Mh, const d
     }
     return;
   }
-  // s_j = sqrt(d_j) and 1 / s_j (kept in the diagonal of Z for the moment)
+  // s_j = sqrt(d_j) and 1 / s_j (in S(j) for the moment)
   for (int j = tid; j < k; j += kThreads) {
-    const dd r = A_::sqrt(A[j * k + j]);
-    A[j * k + j] = r;
-    Z[j * k + j] = A_::recip(r);
+    const T r = N::sqrt(A.get(tri(j, j)));
+    A.set(tri(j, j), r);
+    S.set(j, N::recip(r));
+    double lo;
+    N::to(r, dhi[j], lo);
   }
   __syncthreads();
-  // R(j, l) = A(j, l) / s_j (l > j); Z(i, j) = W(j, i) / s_j (i < j)
+  // R(i, j) = A(i, j) / s_i; Z(i, j) = W(j, i) / s_j (i <= j), straight to memory
   for (int t = tid; t < k * k; t += kThreads) {
     const int i = t % k, j = t / k;
-    if (i < j) {
-      A[j * k + i] = A_::mul(A[j * k + i], Z[i * k + i]);
-      Z[t] = A_::mul(Tb[i * k + j], Z[j * k + j]);
-    } else if (i > j) {
-      Z[t] = dd{0.0, 0.0};
-    }
-  }
-  __syncthreads();
-  for (int t = tid; t < k * k; t += kThreads) {
-    const int i = t % k, j = t / k;
-    ws->Zh[j * KMAX + i] = Z[t].hi;
-    ws->Zl[j * KMAX + i] = Z[t].lo;
-  }
-  __syncthreads();
-  // T <- R T (upper triangular product); T = R on the first pass.
-  for (int t = tid; t < k * k; t += kThreads) {
-    const int i = t % k, j = t / k;
-    dd v = dd{0.0, 0.0};
+    double h = 0.0, l = 0.0;
     if (i <= j) {
-      if (pass == 0) {
-        v = A[j * k + i];
-      } else {
-        for (int l = i; l <= j; ++l)
-          v = A_::fma(A[l * k + i], dd{ws->Th[j * KMAX + l], ws->Tl[j * KMAX + l]}, v);
-      }
+      if (i < j) A.set(tri(i, j), N::mul(A.get(tri(i, j)), S.get(i)));
+      N::to(i < j ? N::mul(W.get(tri(i, j)), S.get(j)) : S.get(j), h, l);
     }
-    Z[t] = v;  // Z's copy is already in global memory
+    ws->Zh[j * KMAX + i] = h;
+    ws->Zl[j * KMAX + i] = l;
+  }
+  __syncthreads();
+  // T <- R T (upper triangular product; the old T into W); T = R on the first pass.
+  if (pass != 0) {
+    for (int t = tid; t < nt; t += kThreads) {
+      int i, j;
+      untri(t, i, j);
+      W.set(t, N::from(ws->Th[j * KMAX + i], ws->Tl[j * KMAX + i]));
+    }
   }
   __syncthreads();
   for (int t = tid; t < k * k; t += kThreads) {
     const int i = t % k, j = t / k;
-    ws->Th[j * KMAX + i] = Z[t].hi;
-    ws->Tl[j * KMAX + i] = Z[t].lo;
-    if (Rh_u) Rh_u[(size_t)j * ldr + i] = Z[t].hi;
-    if (Rl_u) Rl_u[(size_t)j * ldr + i] = Z[t].lo;
+    double h = 0.0, l = 0.0;
+    if (i <= j) {
+      T v;
+      if (pass == 0) {
+        v = A.get(tri(i, j));
+      } else {
+        v = N::zero();
+        for (int q = i; q <= j; ++q) v = N::fma(A.get(tri(i, q)), W.get(tri(q, j)), v);
+      }
+      N::to(v, h, l);
+    }
+    ws->Th[j * KMAX + i] = h;
+    ws->Tl[j * KMAX + i] = l;
+    if (Rh_u) Rh_u[(size_t)j * ldr + i] = h;
+    if (Rl_u) Rl_u[(size_t)j * ldr + i] = l;
   }
   if (tid == 0) {
     double dmax = 0.0, dmin = 1e308;
     for (int i = 0; i < k; ++i) {
-      dmax = fmax(dmax, A[i * k + i].hi);
-      dmin = fmin(dmin, A[i * k + i].hi);
+      dmax = fmax(dmax, dhi[i]);
+      dmin = fmin(dmin, dhi[i]);
     }
     int next = 0;
     if (pass == 0) next = passes == 2 ? 1 : (passes == 0 ? (dmax > thr * dmin) : 0);
@@ -425,38 +599,29 @@ __global__ void __launch_bounds__(kThreads)
 
 // --------------------------------------------------------------- SVQB
 
-template <int MODE>
+template <class N>
 __device__ __forceinline__ void svqb_small_body(int k, const double* Mh, const double* Ml, int ldm, SmallWs* ws,
                                                 double* Zh_u, double* Zl_u, int ldz, double tol, DevStatus* st,
-                                                SmallGates g, int pass, int passes, double thr, double eps,
-                                                int* rank_user, bool rotated) {
-  using A_ = Ar<MODE>;
+                                                SmallGates g, int pass, int passes, double thr, int* rank_user,
+                                                bool rotated) {
+  typedef typename N::T T;
   if (*g.run == 0) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  dd* A = reinterpret_cast<dd*>(smem_raw);  // k*k (upper triangle read during the sweeps)
-  dd* A2 = A + k * k;                        // k*k: the next A
-  dd* U = A2 + k * k;                        // k*k
-  dd* cs = U + k * k;                        // 2 * (k/2 + 1): c, s per pair
-  dd* dv = cs + 2 * (k / 2 + 1);             // k: D = diag(M)^{-1/2} (rotated form)
-  int* pr = reinterpret_cast<int*>(dv + k);  // 2 * (k/2 + 1): p, q per pair
-  int* perm = pr + 2 * (k / 2 + 1);          // k: eigenpair of column j (rotated form)
-  __shared__ int flag, rot_count;
-  const int tid = threadIdx.x;
+  const int nt = k * (k + 1) / 2;
   const int kk = k + (k & 1);  // even number of players; index k is a dummy
   const int npairs = kk / 2;
-  if (tid == 0) flag = 0;
-  __syncthreads();
-  for (int t = tid; t < k * k; t += kThreads) {
-    const int i = t % k, j = t / k;
-    const int a = min(i, j), b = max(i, j);
-    dd v = dd{Mh[(size_t)b * ldm + a], Ml ? Ml[(size_t)b * ldm + a] : 0.0};
-    if (MODE != MODE_DD) v.lo = 0.0;
-    if (!dd_finite(v)) atomicExch(&flag, -1);
-    A[t] = v;
-    U[t] = dd{i == j ? 1.0 : 0.0, 0.0};
-  }
-  __syncthreads();
-  if (flag != 0) {
+  // A and the next A (upper triangles), U (columns), c and s per pair, D = diag(M)^{-1/2} (rotated form)
+  const size_t total = 2 * (size_t)nt + (size_t)k * k + 2 * (size_t)npairs + k;
+  typename N::Vec A = N::vec(smem_raw, total, 0), A2 = N::vec(smem_raw, total, nt);
+  const typename N::Vec U = N::vec(smem_raw, total, 2 * (size_t)nt),
+                        cs = N::vec(smem_raw, total, 2 * (size_t)nt + (size_t)k * k),
+                        dv = N::vec(smem_raw, total, 2 * (size_t)nt + (size_t)k * k + 2 * (size_t)npairs);
+  __shared__ int pr[KMAX + 2];   // p, q per pair
+  __shared__ int perm[KMAX];     // eigenpair of column j (rotated form)
+  __shared__ int rotates[KMAX / 2 + 1];
+  __shared__ int rot_count, next_unit;
+  const int tid = threadIdx.x, lane = tid & 31;
+  if (!load_upper<N>(k, Mh, Ml, ldm, true, A, kJacThreads)) {
     if (tid == 0) {
       st->rank = -1;
       finish_gates(g, 0, 0);
@@ -464,97 +629,104 @@ __device__ __forceinline__ void svqb_small_body(int k, const double* Mh, const d
     }
     return;
   }
+  for (int t = tid; t < k * k; t += kJacThreads) U.set(t, t % k == t / k ? N::one() : N::zero());
   if (rotated) {  // the Jacobi runs on D M D (unit diagonal; a zero diagonal gives d_i = 0)
-    for (int i = tid; i < k; i += kThreads) {
-      const dd m = A[i * k + i];
-      dv[i] = m.hi > 0.0 ? A_::div(dd{1.0, 0.0}, A_::sqrt(m)) : dd{0.0, 0.0};
+    for (int i = tid; i < k; i += kJacThreads) {
+      const T m = A.get(tri(i, i));
+      dv.set(i, !N::is_zero(m) && !N::is_neg(m) ? N::rsqrt(m) : N::zero());
       perm[i] = i;
     }
     __syncthreads();
-    for (int t = tid; t < k * k; t += kThreads) A[t] = A_::mul(A_::mul(dv[t % k], A[t]), dv[t / k]);
-    __syncthreads();
+    for (int t = tid; t < nt; t += kJacThreads) {
+      int i, j;
+      untri(t, i, j);
+      A.set(t, N::mul(N::mul(dv.get(i), A.get(t)), dv.get(j)));
+    }
   }
+  __syncthreads();
   // Sweeps of the parallel (round-robin) ordering.  Per step: (1) each pair's
-  // rotation: the angle in FP64 from the hi parts (t = tan(phi)), then
-  // c = 1 / sqrt(1 + t^2) and s = t c in the mode's arithmetic, so that the
-  // rotation is orthogonal to that precision while it zeroes a_pq only to
-  // FP64 accuracy (the remainder is left in A and removed by later sweeps);
-  // (2) A' = J^T A J by 2x2 blocks of pairs on the upper triangle, into the
-  // second buffer, and U <- U J in place.
-  auto upper = [&](const dd* B, int r, int c) { return B[max(r, c) * k + min(r, c)]; };
+  // rotation (N::rotation: the angle in a short format, c and s orthogonal to
+  // full precision; the remainder of a_pq is removed by later sweeps); (2) A' =
+  // J^T A J by 2x2 blocks of pairs on the upper triangle, into the second
+  // buffer, and U <- U J in place.  The warps take units of (2) from a counter:
+  // first 16 blocks a unit (a pair of lanes per block: each multiplies a row by
+  // J_Q, then, after an exchange, a column by J_P^T), then 64 entries of U.
+  const int nblk = npairs * (npairs + 1) / 2, ablk = (nblk + 15) / 16, uent = 2 * npairs * k, nunits = ablk + (uent + 63) / 64;
   for (int sweep = 0; sweep < 40; ++sweep) {
     if (tid == 0) rot_count = 0;
     __syncthreads();
     for (int step = 0; step < kk - 1; ++step) {
       // round-robin pairing: player 0 fixed, the others rotate by `step`
-      for (int p = tid; p < npairs; p += kThreads) {
+      if (tid < npairs) {
         auto player = [&](int pos) { return pos == 0 ? 0 : 1 + (pos - 1 + step) % (kk - 1); };
-        int a = player(p), b = player(kk - 1 - p);
-        int lo = min(a, b), hi = max(a, b);
-        dd c = dd{1.0, 0.0}, sn = dd{0.0, 0.0};
-        if (hi < k) {
-          const dd apq = A[hi * k + lo];
-          const dd app = A[lo * k + lo], aqq = A[hi * k + hi];
-          const double scale = sqrt(dabs(app.hi) * dabs(aqq.hi));
-          if (dabs(apq.hi) > eps * scale && apq.hi != 0.0) {
-            const double th = A_::sub(aqq, app).hi / (2.0 * apq.hi);
-            const double t = dabs(th) > 1e150 ? 0.5 / th : copysign(1.0 / (dabs(th) + sqrt(fma(th, th, 1.0))), th);
-            c = A_::rsqrt(A_::add(dd{1.0, 0.0}, A_::mul(dd{t, 0.0}, dd{t, 0.0})));
-            sn = A_::mul(c, dd{t, 0.0});
-            atomicAdd(&rot_count, 1);
+        const int a = player(tid), b = player(kk - 1 - tid);
+        const int lo = min(a, b), hi = max(a, b);
+        T c = N::one(), sn = N::zero();
+        const bool rot = hi < k && N::rotation(A.get(tri(lo, lo)), A.get(tri(hi, hi)), A.get(tri(lo, hi)), c, sn);
+        if (rot) atomicAdd(&rot_count, 1);
+        rotates[tid] = rot;
+        cs.set(2 * tid, c);
+        cs.set(2 * tid + 1, sn);
+        pr[2 * tid] = lo;
+        pr[2 * tid + 1] = hi;
+      }
+      if (tid == kJacThreads - 1) next_unit = 0;
+      __syncthreads();
+      for (;;) {
+        int unit = 0;
+        if (lane == 0) unit = atomicAdd(&next_unit, 1);
+        unit = __shfl_sync(0xffffffffu, unit, 0);
+        if (unit >= nunits) break;
+        if (unit < ablk) {
+          // A2 = J^T A J, block (P, Q) of rows {lo_P, hi_P} and columns {lo_Q, hi_Q}, P <= Q
+          const int b = unit * 16 + (lane >> 1), r = lane & 1;
+          const bool act = b < nblk;
+          int P, Q;
+          untri(act ? b : 0, P, Q);
+          const int r0 = pr[2 * P], r1 = pr[2 * P + 1], c0 = pr[2 * Q], c1 = pr[2 * Q + 1];
+          const bool v1 = r1 < k, w1 = c1 < k;  // r0, c0 < k always (the dummy index is the larger)
+          const int row = r ? r1 : r0;
+          const bool have = !r || v1;
+          T t0 = have ? A.get(sym(row, c0)) : N::zero();
+          T t1 = have && w1 ? A.get(sym(row, c1)) : N::zero();
+          if (rotates[Q]) {  // row r of B J_Q
+            const T c = cs.get(2 * Q), sn = cs.get(2 * Q + 1);
+            const T x = N::dot2(t0, c, t1, N::neg(sn));
+            t1 = N::dot2(t0, sn, t1, c);
+            t0 = x;
+          }
+          const T other = N::shfl_xor(r ? t0 : t1, 1);
+          T y0 = r ? other : t0, y1 = r ? t1 : other;  // column r
+          if (rotates[P]) {  // J_P^T (B J_Q)
+            const T c = cs.get(2 * P), sn = cs.get(2 * P + 1);
+            const T x = N::dot2(c, y0, N::neg(sn), y1);
+            y1 = N::dot2(sn, y0, c, y1);
+            y0 = x;
+          }
+          if (act && (!r || w1)) {
+            const int col = r ? c1 : c0;
+            A2.set(sym(r0, col), y0);
+            if (v1 && (P != Q || r)) A2.set(sym(r1, col), y1);  // (P = Q: (r1, c0) is the mirror of (r0, c1))
+          }
+        } else {
+          // U <- U J, columns lo_Q, hi_Q of row m: a pair of lanes per row and pair
+          for (int h = 0; h < 2; ++h) {
+            const int t = (unit - ablk) * 64 + h * 32 + lane;
+            const int q = (t >> 1) / k, m = (t >> 1) % k, r = t & 1;
+            const bool act = t < uent && rotates[q] != 0;
+            T v = N::zero();
+            if (act) {
+              const T c = cs.get(2 * q), sn = cs.get(2 * q + 1);
+              const T x = U.get(pr[2 * q] * k + m), y = U.get(pr[2 * q + 1] * k + m);
+              v = r ? N::dot2(sn, x, c, y) : N::dot2(c, x, N::neg(sn), y);
+            }
+            __syncwarp();  // both lanes have read the entries that they replace
+            if (act) U.set(pr[2 * q + r] * k + m, v);
           }
         }
-        cs[2 * p] = c;
-        cs[2 * p + 1] = sn;
-        pr[2 * p] = lo;
-        pr[2 * p + 1] = hi;
       }
       __syncthreads();
-      // A2 = J^T A J, block (P, Q) of rows {lo_P, hi_P} and columns {lo_Q, hi_Q}, P <= Q
-      for (int t = tid; t < npairs * (npairs + 1) / 2; t += kThreads) {
-        int Q = (int)((sqrtf(8.0f * t + 1.0f) - 1.0f) * 0.5f);
-        while ((Q + 1) * (Q + 2) / 2 <= t) ++Q;
-        while (Q * (Q + 1) / 2 > t) --Q;
-        const int P = t - Q * (Q + 1) / 2;
-        const int r0 = pr[2 * P], r1 = pr[2 * P + 1], c0 = pr[2 * Q], c1 = pr[2 * Q + 1];
-        const dd cP = cs[2 * P], sP = cs[2 * P + 1], cQ = cs[2 * Q], sQ = cs[2 * Q + 1];
-        const bool v1 = r1 < k, w1 = c1 < k;  // r0, c0 < k always (the dummy index is the larger)
-        dd b00 = upper(A, r0, c0), b01 = w1 ? upper(A, r0, c1) : dd{0.0, 0.0};
-        dd b10 = v1 ? upper(A, r1, c0) : dd{0.0, 0.0}, b11 = v1 && w1 ? upper(A, r1, c1) : dd{0.0, 0.0};
-        if (!(sQ.hi == 0.0 && sQ.lo == 0.0)) {  // B J_Q
-          const dd mQ = dd_neg(sQ);
-          const dd t00 = A_::dot2(b00, cQ, b01, mQ), t01 = A_::dot2(b00, sQ, b01, cQ);
-          const dd t10 = A_::dot2(b10, cQ, b11, mQ), t11 = A_::dot2(b10, sQ, b11, cQ);
-          b00 = t00; b01 = t01; b10 = t10; b11 = t11;
-        }
-        if (!(sP.hi == 0.0 && sP.lo == 0.0)) {  // J_P^T (B J_Q)
-          const dd mP = dd_neg(sP);
-          const dd t00 = A_::dot2(cP, b00, mP, b10), t10 = A_::dot2(sP, b00, cP, b10);
-          const dd t01 = A_::dot2(cP, b01, mP, b11), t11 = A_::dot2(sP, b01, cP, b11);
-          b00 = t00; b01 = t01; b10 = t10; b11 = t11;
-        }
-        auto put = [&](int r, int c, dd v) { A2[max(r, c) * k + min(r, c)] = v; };
-        put(r0, c0, b00);
-        if (w1) put(r0, c1, b01);
-        if (P == Q) {
-          if (v1) put(r1, c1, b11);  // (r1, c0) is the mirror of (r0, c1)
-        } else {
-          if (v1) put(r1, c0, b10);
-          if (v1 && w1) put(r1, c1, b11);
-        }
-      }
-      // U <- U J, columns lo_Q, hi_Q of row m
-      for (int t = tid; t < npairs * k; t += kThreads) {
-        const int q = t % npairs, m = t / npairs;
-        const int a = pr[2 * q], b = pr[2 * q + 1];
-        const dd c = cs[2 * q], sn = cs[2 * q + 1];
-        if (b >= k || (sn.hi == 0.0 && sn.lo == 0.0)) continue;
-        const dd x = U[a * k + m], y = U[b * k + m];
-        U[a * k + m] = A_::dot2(c, x, dd_neg(sn), y);
-        U[b * k + m] = A_::dot2(sn, x, c, y);
-      }
-      __syncthreads();
-      dd* sw = A;
+      const typename N::Vec sw = A;
       A = A2;
       A2 = sw;
     }
@@ -565,105 +737,110 @@ __device__ __forceinline__ void svqb_small_body(int k, const double* Mh, const d
     __syncthreads();
     if (sweep == 39 && tid == 0) st->sweeps = 40;
   }
-  // the upper triangle holds the result: mirror it (the diagonal is eigenvalues)
-  for (int t = tid; t < k * k; t += kThreads) {
-    const int i = t % k, j = t / k;
-    if (i > j) A[t] = A[i * k + j];
-  }
-  __syncthreads();
   if (rotated) {
     // Column a of U: its largest-magnitude entry (lowest row on ties) made
     // positive; its place in the ascending order of the eigenvalues (ties by
-    // index) gives the column of Z it lands in.  Normalized double-doubles
-    // compare exactly as (hi, lo) pairs.
-    auto lt = [](dd x, dd y) { return x.hi < y.hi || (x.hi == y.hi && x.lo < y.lo); };
-    auto mag = [](dd x) { return x.hi < 0.0 ? dd_neg(x) : x; };
-    for (int a = tid; a < k; a += kThreads) {
-      dd* u = U + a * k;
+    // index) gives the column of Z it lands in.
+    auto mag = [](T x) { return N::is_neg(x) ? N::neg(x) : x; };
+    for (int a = tid; a < k; a += kJacThreads) {
       int mb = 0;
-      for (int m = 1; m < k; ++m)
-        if (lt(mag(u[mb]), mag(u[m]))) mb = m;
-      if (u[mb].hi < 0.0)
-        for (int m = 0; m < k; ++m) u[m] = dd_neg(u[m]);
-      const dd la = A[a * k + a];
+      T best = mag(U.get(a * k));
+      for (int m = 1; m < k; ++m) {
+        const T x = mag(U.get(a * k + m));
+        if (N::less(best, x)) {
+          best = x;
+          mb = m;
+        }
+      }
+      if (N::is_neg(U.get(a * k + mb)))
+        for (int m = 0; m < k; ++m) U.set(a * k + m, N::neg(U.get(a * k + m)));
+      const T la = A.get(tri(a, a));
       int pos = 0;
       for (int b = 0; b < k; ++b) {
-        const dd lb = A[b * k + b];
-        pos += lt(lb, la) || (!lt(la, lb) && b < a);
+        const T lb = A.get(tri(b, b));
+        pos += N::less(lb, la) || (!N::less(la, lb) && b < a);
       }
       perm[pos] = a;  // pos < k; with a NaN eigenvalue two columns may collide, the rest keep the identity
     }
     __syncthreads();
   }
-  // w_l = lambda_l^{-1/2} for kept eigenvalues; Z = U diag(w) U^T into A's storage.
+  // w_l = lambda_l^{-1/2} for kept eigenvalues (in cs, which has at least k entries)
+  __shared__ double lam[KMAX];
   __shared__ double lmax_s, lmin_s;
   __shared__ int rank_s;
-  dd* w = cs;  // reuse: k entries needed, cs has 2*(k/2+1) >= k
+  for (int i = tid; i < k; i += kJacThreads) {
+    double lo;
+    N::to(A.get(tri(i, i)), lam[i], lo);
+  }
+  __syncthreads();
   if (tid == 0) {
     double lmax = 0.0;
-    for (int i = 0; i < k; ++i) lmax = fmax(lmax, A[i * k + i].hi);
+    for (int i = 0; i < k; ++i) lmax = lam[i] > lmax ? lam[i] : lmax;
+    const double cut = tol * lmax;
     int rank = 0;
     double lmin = lmax;
-    for (int i = 0; i < k; ++i) {
-      const dd l = A[i * k + i];
-      if (lmax > 0.0 && l.hi > tol * lmax) {
-        w[i] = A_::div(dd{1.0, 0.0}, A_::sqrt(l));
+    for (int i = 0; i < k; ++i)
+      if (lmax > 0.0 && lam[i] > cut) {
         ++rank;
-        lmin = fmin(lmin, l.hi);
-      } else {
-        w[i] = dd{0.0, 0.0};
+        lmin = lam[i] < lmin ? lam[i] : lmin;
       }
-    }
     lmax_s = lmax;
     lmin_s = lmin;
     rank_s = rank;
   }
   __syncthreads();
-  if (rotated) {  // Z(:, j) = D u_a w_a with a = perm[j]
-    for (int t = tid; t < k * k; t += kThreads) {
-      const int i = t % k, a = perm[t / k];
-      A[t] = A_::mul(A_::mul(dv[i], U[a * k + i]), w[a]);
-    }
-    __syncthreads();
-  } else {  // one triangle, mirrored, so that Z is exactly symmetric
-    for (int t = tid; t < k * k; t += kThreads) {
-      const int i = t % k, j = t / k;
-      if (i > j) continue;
-      dd v = dd{0.0, 0.0};
-      for (int l = 0; l < k; ++l) v = A_::fma(A_::mul(U[l * k + i], w[l]), U[l * k + j], v);
-      A[t] = v;
-    }
-    __syncthreads();
-    for (int t = tid; t < k * k; t += kThreads) {
-      const int i = t % k, j = t / k;
-      if (i > j) A[t] = A[i * k + j];
-    }
-    __syncthreads();
-  }
-  for (int t = tid; t < k * k; t += kThreads) {
-    const int i = t % k, j = t / k;
-    ws->Zh[j * KMAX + i] = A[t].hi;
-    ws->Zl[j * KMAX + i] = A[t].lo;
-  }
+  for (int i = tid; i < k; i += kJacThreads)
+    cs.set(i, lmax_s > 0.0 && lam[i] > tol * lmax_s ? N::rsqrt(A.get(tri(i, i))) : N::zero());
   __syncthreads();
-  // T <- T Z (full product); T = Z on the first pass.  U's storage is free now.
-  for (int t = tid; t < k * k; t += kThreads) {
-    const int i = t % k, j = t / k;
-    dd v = dd{0.0, 0.0};
-    if (pass == 0) {
-      v = A[t];
-    } else {
-      for (int l = 0; l < k; ++l) v = A_::fma(dd{ws->Th[l * KMAX + i], ws->Tl[l * KMAX + i]}, A[j * k + l], v);
+  auto out_z = [&](int i, int j, T v, bool last) {  // Z, and T = Z when there is no earlier transform
+    double h, l;
+    N::to(v, h, l);
+    ws->Zh[j * KMAX + i] = h;
+    ws->Zl[j * KMAX + i] = l;
+    if (!last) return;
+    ws->Th[j * KMAX + i] = h;
+    ws->Tl[j * KMAX + i] = l;
+    if (Zh_u) Zh_u[(size_t)j * ldz + i] = h;
+    if (Zl_u) Zl_u[(size_t)j * ldz + i] = l;
+  };
+  if (rotated) {  // Z(:, j) = D u_a w_a with a = perm[j] (one pass)
+    for (int t = tid; t < k * k; t += kJacThreads) {
+      const int i = t % k, j = t / k, a = perm[j];
+      out_z(i, j, N::mul(N::mul(dv.get(i), U.get(a * k + i)), cs.get(a)), true);
     }
-    U[t] = v;
-  }
-  __syncthreads();
-  for (int t = tid; t < k * k; t += kThreads) {
-    const int i = t % k, j = t / k;
-    ws->Th[j * KMAX + i] = U[t].hi;
-    ws->Tl[j * KMAX + i] = U[t].lo;
-    if (Zh_u) Zh_u[(size_t)j * ldz + i] = U[t].hi;
-    if (Zl_u) Zl_u[(size_t)j * ldz + i] = U[t].lo;
+  } else {
+    // Z = U diag(w) U^T = (U diag(w)^{1/2}) (U diag(w)^{1/2})^T: one triangle,
+    // mirrored, so that Z is exactly symmetric (into A2)
+    for (int t = tid; t < k * k; t += kJacThreads) U.set(t, N::mul(U.get(t), N::sqrt(cs.get(t / k))));
+    __syncthreads();
+    for (int t = tid; t < nt; t += kJacThreads) {
+      int i, j;
+      untri(t, i, j);
+      T v = N::zero();
+      for (int l = 0; l < k; ++l) v = N::fma(U.get(l * k + i), U.get(l * k + j), v);
+      A2.set(t, v);
+      out_z(i, j, v, pass == 0);
+      if (i != j) out_z(j, i, v, pass == 0);
+    }
+    if (pass != 0) {  // T <- T Z (the old T into U)
+      __syncthreads();
+      for (int t = tid; t < k * k; t += kJacThreads) {
+        const size_t e = (size_t)(t / k) * KMAX + t % k;
+        U.set(t, N::from(ws->Th[e], ws->Tl[e]));
+      }
+      __syncthreads();
+      for (int t = tid; t < k * k; t += kJacThreads) {
+        const int i = t % k, j = t / k;
+        T v = N::zero();
+        for (int l = 0; l < k; ++l) v = N::fma(U.get(l * k + i), A2.get(sym(l, j)), v);
+        double h, lo;
+        N::to(v, h, lo);
+        ws->Th[j * KMAX + i] = h;
+        ws->Tl[j * KMAX + i] = lo;
+        if (Zh_u) Zh_u[(size_t)j * ldz + i] = h;
+        if (Zl_u) Zl_u[(size_t)j * ldz + i] = lo;
+      }
+    }
   }
   if (tid == 0) {
     st->rank = rank_s;
@@ -677,20 +854,23 @@ __device__ __forceinline__ void svqb_small_body(int k, const double* Mh, const d
 // ----------------------------------------------------- kernel wrappers
 
 template <int MODE>
+using Num = std::conditional_t<MODE == MODE_DD, Wide, F64>;
+
+template <int MODE>
 __global__ void __launch_bounds__(kThreads) chol_small_kernel(int k, const double* Mh, const double* Ml, int ldm,
                                                               SmallWs* ws, double* Rh_u, double* Rl_u, int ldr,
                                                               DevStatus* st, SmallGates g, int pass, int passes,
                                                               double thr, int* info_user) {
-  chol_small_body<MODE>(k, Mh, Ml, ldm, ws, Rh_u, Rl_u, ldr, st, g, pass, passes, thr, info_user);
+  chol_small_body<Num<MODE>>(k, Mh, Ml, ldm, ws, Rh_u, Rl_u, ldr, st, g, pass, passes, thr, info_user);
 }
 
 template <int MODE>
-__global__ void __launch_bounds__(kThreads) svqb_small_kernel(int k, const double* Mh, const double* Ml, int ldm,
+__global__ void __launch_bounds__(kJacThreads, 1) svqb_small_kernel(int k, const double* Mh, const double* Ml, int ldm,
                                                               SmallWs* ws, double* Zh_u, double* Zl_u, int ldz,
                                                               double tol, DevStatus* st, SmallGates g, int pass,
-                                                              int passes, double thr, double eps, int* rank_user,
+                                                              int passes, double thr, int* rank_user,
                                                               bool rotated) {
-  svqb_small_body<MODE>(k, Mh, Ml, ldm, ws, Zh_u, Zl_u, ldz, tol, st, g, pass, passes, thr, eps, rank_user, rotated);
+  svqb_small_body<Num<MODE>>(k, Mh, Ml, ldm, ws, Zh_u, Zl_u, ldz, tol, st, g, pass, passes, thr, rank_user, rotated);
 }
 
 // One CTA per job: the factorization of pass `pass` of many independent
@@ -705,17 +885,17 @@ __global__ void __launch_bounds__(kThreads) chol_small_batched_kernel(const Smal
                                                                       double thr) {
   const SmallJob j = jobs[blockIdx.x];
   const int npass = passes == 1 ? 1 : 2;
-  chol_small_body<MODE>(j.k, j.ws->Mh, j.ws->Ml, KMAX, j.ws, j.Oh, j.Ol, j.ldo, j.st, job_gates(j, pass, npass), pass,
+  chol_small_body<Num<MODE>>(j.k, j.ws->Mh, j.ws->Ml, KMAX, j.ws, j.Oh, j.Ol, j.ldo, j.st, job_gates(j, pass, npass), pass,
                         passes, thr, j.out);
 }
 
 template <int MODE>
-__global__ void __launch_bounds__(kThreads) svqb_small_batched_kernel(const SmallJob* jobs, int pass, int passes,
-                                                                      double thr, double eps) {
+__global__ void __launch_bounds__(kJacThreads, 1) svqb_small_batched_kernel(const SmallJob* jobs, int pass, int passes,
+                                                                      double thr) {
   const SmallJob j = jobs[blockIdx.x];
   const int npass = passes == 1 ? 1 : 2;
-  svqb_small_body<MODE>(j.k, j.ws->Mh, j.ws->Ml, KMAX, j.ws, j.Oh, j.Ol, j.ldo, j.tol, j.st,
-                        job_gates(j, pass, npass), pass, passes, thr, eps, j.out, false);
+  svqb_small_body<Num<MODE>>(j.k, j.ws->Mh, j.ws->Ml, KMAX, j.ws, j.Oh, j.Ol, j.ldo, j.tol, j.st,
+                        job_gates(j, pass, npass), pass, passes, thr, j.out, false);
 }
 
 __global__ void status_init_batched_kernel(const SmallJob* jobs, int njobs) {
@@ -809,13 +989,18 @@ cudaError_t launch_status_init(DevStatus* s, int k, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-size_t chol_smem(int k) { return 3 * (size_t)k * k * sizeof(dd); }
+size_t pivchol_smem(int k) { return 3 * (size_t)k * k * sizeof(dd); }
+size_t chol_smem(bool wide, int k) { return 3 * (size_t)(k * (k + 1) / 2) * (wide ? Wide::kBytes : F64::kBytes); }
+size_t svqb_smem(bool wide, int k) {
+  const size_t n = (size_t)k * (k + 1) + (size_t)k * k + 2 * (size_t)((k + 1) / 2) + k;
+  return n * (wide ? Wide::kBytes : F64::kBytes);
+}
 
 cudaError_t launch_pivchol_small(Mode mode, int k, const double* Mh, const double* Ml, int ldm, SmallWs* ws,
                                  double* R_hi, double* R_lo, int ldr, double tol, DevStatus* s, SmallGates g,
                                  int pass, int passes, int* info_user, int* rank_user, int* perm_user,
                                  cudaStream_t st) {
-  const size_t smem = chol_smem(k);
+  const size_t smem = pivchol_smem(k);
   cudaError_t e;
   if (mode == MODE_DD) {
     e = set_dyn_smem(pivchol_small_kernel<MODE_DD>, smem);
@@ -830,15 +1015,10 @@ cudaError_t launch_pivchol_small(Mode mode, int k, const double* Mh, const doubl
   }
   return cudaGetLastError();
 }
-size_t svqb_smem(int k) {
-  return 3 * (size_t)k * k * sizeof(dd) + (2 * (size_t)(k / 2 + 1) + k) * sizeof(dd) +
-         (2 * (size_t)(k / 2 + 1) + k) * sizeof(int);
-}
-
 cudaError_t launch_chol_small(Mode mode, int k, const double* Mh, const double* Ml, int ldm, SmallWs* ws,
                               double* R_hi, double* R_lo, int ldr, DevStatus* s, SmallGates g, int pass, int passes,
                               int* info_user, cudaStream_t st) {
-  const size_t smem = chol_smem(k);
+  const size_t smem = chol_smem(mode == MODE_DD, k);
   cudaError_t e;
   if (mode == MODE_DD) {
     e = set_dyn_smem(chol_small_kernel<MODE_DD>, smem);
@@ -857,21 +1037,21 @@ cudaError_t launch_chol_small(Mode mode, int k, const double* Mh, const double* 
 cudaError_t launch_svqb_small(Mode mode, int k, const double* Mh, const double* Ml, int ldm, SmallWs* ws,
                               double* Z_hi, double* Z_lo, int ldz, double tol, DevStatus* s, SmallGates g, int pass,
                               int passes, int* rank_user, cudaStream_t st, bool rotated) {
-  const size_t smem = svqb_smem(k);
+  const size_t smem = svqb_smem(mode == MODE_DD, k);
   if (rotated) passes = 1;
   cudaError_t e;
   if (mode == MODE_DD) {
     if (tol < 0) tol = k * 0x1p-104;
     e = set_dyn_smem(svqb_small_kernel<MODE_DD>, smem);
     if (e != cudaSuccess) return e;
-    svqb_small_kernel<MODE_DD><<<1, kThreads, smem, st>>>(k, Mh, Ml, ldm, ws, Z_hi, Z_lo, ldz, tol, s, g, pass,
-                                                         passes, 1e7, kJacobiEpsDD, rank_user, rotated);
+    svqb_small_kernel<MODE_DD><<<1, kJacThreads, smem, st>>>(k, Mh, Ml, ldm, ws, Z_hi, Z_lo, ldz, tol, s, g, pass,
+                                                         passes, 1e7, rank_user, rotated);
   } else {
     if (tol < 0) tol = k * 0x1p-52;
     e = set_dyn_smem(svqb_small_kernel<MODE_FP64>, smem);
     if (e != cudaSuccess) return e;
-    svqb_small_kernel<MODE_FP64><<<1, kThreads, smem, st>>>(k, Mh, Ml, ldm, ws, Z_hi, Z_lo, ldz, tol, s, g, pass,
-                                                           passes, 1e4, kJacobiEpsFP64, rank_user, rotated);
+    svqb_small_kernel<MODE_FP64><<<1, kJacThreads, smem, st>>>(k, Mh, Ml, ldm, ws, Z_hi, Z_lo, ldz, tol, s, g, pass,
+                                                           passes, 1e4, rank_user, rotated);
   }
   return cudaGetLastError();
 }
@@ -888,7 +1068,7 @@ cudaError_t launch_small_batched(bool chol, Mode mode, int njobs, int kmax, cons
   const bool ddm = mode == MODE_DD;
   cudaError_t e;
   if (chol) {
-    const size_t smem = chol_smem(kmax);
+    const size_t smem = chol_smem(ddm, kmax);
     auto kern = ddm ? chol_small_batched_kernel<MODE_DD> : chol_small_batched_kernel<MODE_FP64>;
     e = set_dyn_smem(kern, smem);
     if (e != cudaSuccess) return e;
@@ -900,12 +1080,12 @@ cudaError_t launch_small_batched(bool chol, Mode mode, int njobs, int kmax, cons
     // Asking for more than half of an SM's shared memory keeps one such CTA
     // per SM (the jobs are ordered widest first, so the first wave spreads
     // the widest over the SMs).
-    size_t smem = svqb_smem(kmax);
+    size_t smem = svqb_smem(ddm, kmax);
     if (kmax >= 16) smem = std::max<size_t>(smem, 116 * 1024);
     auto kern = ddm ? svqb_small_batched_kernel<MODE_DD> : svqb_small_batched_kernel<MODE_FP64>;
     e = set_dyn_smem(kern, smem);
     if (e != cudaSuccess) return e;
-    kern<<<njobs, kThreads, smem, st>>>(jobs, pass, passes, ddm ? 1e7 : 1e4, ddm ? kJacobiEpsDD : kJacobiEpsFP64);
+    kern<<<njobs, kJacThreads, smem, st>>>(jobs, pass, passes, ddm ? 1e7 : 1e4);
   }
   return cudaGetLastError();
 }

@@ -1,5 +1,6 @@
 """The tensor-core Gram engine at the edges of its tiles: column counts on
-either side of its 8-, 16-, 32- and 64-column tiles, row counts on either side
+either side of its 8-, 16-, 32- and 64-column tiles and of the narrow products
+that the integer limbs keep, row counts on either side
 of a K step, of a panel and of a row chunk, TMA and element-wise loads, and
 values on either side of the near window (25 binades below the alignment
 exponent), zeros and growing exponents among them.
@@ -34,7 +35,8 @@ def check(eo, ctx, x, y, odd_ld=False):
 
 
 @pytest.mark.parametrize("odd_ld", [False, True])
-@pytest.mark.parametrize("kx,ky", [(9, 1), (16, 8), (17, 9), (32, 16), (33, 8), (64, 17), (3, 40), (16, 0), (17, 0), (64, 0)])
+@pytest.mark.parametrize("kx,ky", [(9, 1), (16, 8), (17, 9), (32, 16), (33, 8), (64, 17), (3, 40), (16, 0), (17, 0), (64, 0),
+                                   (4, 0), (5, 0), (8, 0), (8, 3), (8, 4), (5, 7)])
 def test_column_tiles(eo, ctx, kx, ky, odd_ld):
     x = synth.gaussian(12_345, kx, 900 + kx)
     check(eo, ctx, x, synth.gaussian(12_345, ky, 950 + ky) if ky else x, odd_ld)
@@ -48,7 +50,7 @@ def test_row_edges(eo, ctx, n, kx, ky):
 
 
 @pytest.mark.parametrize("kind", ["zeros", "below", "grow", "zero column", "mixed"])
-@pytest.mark.parametrize("kx,ky", [(20, 12), (64, 16), (30, 5), (16, 0), (10, 0), (12, 9)])
+@pytest.mark.parametrize("kx,ky", [(20, 12), (64, 16), (30, 5), (16, 0), (10, 0), (12, 9), (5, 0), (8, 8)])
 @pytest.mark.parametrize("odd_ld", [False, True])
 def test_special_panels(eo, ctx, kind, kx, ky, odd_ld):
     n = 30_011
