@@ -119,6 +119,7 @@ __device__ void finish_gates(const SmallGates& g, int run_update, int want_next)
 struct F64 {
   typedef double T;
   static constexpr size_t kBytes = 8;
+  static constexpr bool kOneSided = false;
   struct Vec {
     double* p;
     __device__ __forceinline__ T get(int i) const { return p[i]; }
@@ -175,6 +176,7 @@ struct F64 {
 
 struct Wide {
   typedef wide T;
+  static constexpr bool kOneSided = true;  // Jacobi on the Cholesky factor where it can
   static constexpr size_t kBytes = 20;  // significand, exponent and sign in arrays of their own
   struct Vec {
     u128* m;
@@ -597,6 +599,249 @@ __global__ void __launch_bounds__(kThreads)
   }
 }
 
+// ------------------------------------------------- one-sided Jacobi
+
+// x c >> 128 for signed x and 0 <= c < 2^128 (below the exact value by at most 3).
+__device__ __forceinline__ i128 smulhi128(i128 x, u128 c) {
+  return (i128)(mulhi128((u128)x, c) - (x < 0 ? c : (u128)0));
+}
+__device__ __forceinline__ i128 sar128(i128 x, int n) {  // n >= 0
+  return n < 127 ? x >> n : (x < 0 ? (i128)-1 : (i128)0);
+}
+__device__ __forceinline__ i128 shfl_sum(i128 v) {  // over the warp
+#pragma unroll
+  for (int m = 16; m >= 1; m >>= 1) {
+    const unsigned long long h = __shfl_xor_sync(0xffffffffu, (unsigned long long)((u128)v >> 64), m);
+    const unsigned long long l = __shfl_xor_sync(0xffffffffu, (unsigned long long)(u128)v, m);
+    v += (i128)(((u128)h << 64) | l);
+  }
+  return v;
+}
+// v 2^x as a wide number
+__device__ __forceinline__ wide wide_int(i128 v, int x) {
+  const bool neg = v < 0;
+  return wide_norm(neg ? (u128)-v : (u128)v, x + 127, neg ? 1 : 0);
+}
+// A column of up to 64 entries, two per lane, in units 2^(E - 125): shifted so
+// that its largest magnitude lies in [2^121, 2^122) (so that its norm is below
+// 2^125); from units 2^x.  Returns E.
+__device__ __forceinline__ int settle(i128 (&v)[2], int x) {
+  auto top = [](i128 a) { return (unsigned)((u128)(a < 0 ? ~a : a) >> 95); };
+  auto low = [](i128 a) { return (unsigned)((u128)(a < 0 ? ~a : a) >> 63); };
+  unsigned t = __reduce_max_sync(0xffffffffu, max(top(v[0]), top(v[1])));
+  int z;
+  if (t) {
+    z = __clz((int)t) - 5;  // |largest| in [2^(126 - clz), 2^(127 - clz))
+  } else {
+    t = __reduce_max_sync(0xffffffffu, max(low(v[0]), low(v[1])));
+    z = t ? __clz((int)t) + 27 : 59;  // (a column that cancels further is settled again by its next rotation)
+  }
+#pragma unroll
+  for (int q = 0; q < 2; ++q) v[q] = z >= 0 ? (i128)((u128)v[q] << z) : v[q] >> -z;
+  return x - z + 125;
+}
+
+// Eigenvalues and vectors of a positive semidefinite M (A, packed; destroyed) by
+// one-sided Jacobi on its Cholesky factor with diagonal pivoting (Drmac and
+// Veselic): M = L L^T, and rotations V that make the columns of L V orthogonal
+// give the eigenvectors as its normalized columns, their squared norms as the
+// eigenvalues (into A's diagonal; zero for the columns beyond the rank).
+// Against the two-sided form on M it needs about half the sweeps on a graded
+// spectrum, no second matrix to update, and no exponent per entry: a column is
+// 128-bit fixed point with one exponent (errors 2^-118 of its norm).  One warp
+// takes a pair of columns through a whole rotation (three sums over the rows,
+// the angle, the update), so that a step has one barrier.
+// False (with M's triangle to be loaded again) when M is not semidefinite to
+// rounding, or its diagonal spans more than 100 binades, where small entries
+// need exponents of their own.
+__device__ bool onesided_jacobi(int k, const Wide::Vec A, const Wide::Vec U, DevStatus* st) {
+  __shared__ int E[KMAX], ref[KMAX], pos[KMAX], col[KMAX];
+  __shared__ wide inv;
+  __shared__ int piv, state, rot_count;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  if (tid < k) {
+    ref[tid] = A.get(tri(tid, tid)).e;
+    pos[tid] = k;  // step at which the row was eliminated
+    col[tid] = -1;  // row eliminated at a step (-1: none)
+  }
+  if (tid == 0) state = 0;
+  __syncthreads();
+  {
+    int lo = 1 << 30, hi = -(1 << 30);  // exponents of the nonzero diagonal entries
+    for (int i = lane; i < k; i += 32) {
+      if (ref[i] == kWideZero) continue;
+      lo = min(lo, ref[i]);
+      hi = max(hi, ref[i]);
+    }
+    lo = __reduce_min_sync(0xffffffffu, lo);
+    hi = __reduce_max_sync(0xffffffffu, hi);
+    if (hi - lo > 100) return false;
+  }
+  // M = L L^T in the order of the largest remaining diagonal entries: column
+  // `step` of L is A(:, p) / sqrt(d) over the rows not eliminated before.  An
+  // entry that rounding alone may have left is dropped (no column).
+  for (int step = 0; step < k; ++step) {
+    if (warp == 0) {
+      unsigned long long best = 0;  // exponent and leading bits, then the index from the top
+      for (int i = lane; i < k; i += 32) {
+        if (pos[i] != k) continue;
+        const wide d = A.get(tri(i, i));
+        const bool good = !wide_is_zero(d) && d.s == 0;
+        const unsigned long long key = good ? ((unsigned long long)(unsigned)(d.e + (1 << 29)) << 32) |
+                                                  ((unsigned)(d.m >> 96) & ~63u) | (unsigned)(63 - i)
+                                            : (unsigned long long)(63 - i) + 1;
+        best = key > best ? key : best;
+      }
+#pragma unroll
+      for (int m = 16; m >= 1; m >>= 1) {
+        const unsigned long long o = __shfl_xor_sync(0xffffffffu, best, m);
+        best = o > best ? o : best;
+      }
+      const bool good = best >> 32;
+      const int p = 63 - (int)((good ? best : best - 1) & 63ull);
+      const wide d = A.get(tri(p, p));
+      const bool ok = good && Wide::pivot_ok(d, ref[p]);
+      if (lane == 0) {
+        piv = ok ? p : -1;
+        pos[p] = step;
+        if (ok) {
+          inv = wide_recip(d);
+          col[step] = p;
+        } else if (d.s && !wide_is_zero(d) && d.e > ref[p] - 100) {
+          state = 1;  // a negative diagonal entry: not semidefinite
+        }
+      }
+    }
+    __syncthreads();
+    if (state) return false;
+    const int p = piv;
+    if (p >= 0) {
+      const wide w = inv;
+      for (int t = tid; t < k * (k + 1) / 2; t += kJacThreads) {
+        int a, b;
+        untri(t, a, b);
+        if (pos[a] == k && pos[b] == k)
+          A.set(t, wide_sub(A.get(t), wide_mul(wide_mul(A.get(sym(a, p)), w), A.get(sym(b, p)))));
+      }
+    }
+    __syncthreads();
+  }
+  // L's columns in fixed point, rows in M's order (U's significands)
+  i128* W = reinterpret_cast<i128*>(U.m);
+  for (int l = warp; l < k; l += kJacThreads / 32) {
+    const int p = col[l];
+    wide x[2] = {wide_zero(), wide_zero()};
+    if (p >= 0) {
+      const wide r = wide_rsqrt(A.get(tri(p, p)));
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        const int i = lane + 32 * q;
+        if (i < k && pos[i] >= l) x[q] = wide_mul(A.get(sym(i, p)), r);
+      }
+    }
+    const int top = __reduce_max_sync(0xffffffffu, max(x[0].e, x[1].e));
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const int i = lane + 32 * q;
+      const i128 v = (i128)shr128(x[q].m, p >= 0 ? min(128, 6 + top - x[q].e) : 128);
+      if (i < k) W[l * k + i] = x[q].s ? -v : v;
+    }
+    if (lane == 0) E[l] = p >= 0 ? top + 4 : 0;
+  }
+  __syncthreads();
+  const int kk = k + (k & 1), npairs = kk / 2;
+  for (int sweep = 0; sweep < 40; ++sweep) {
+    if (tid == 0) rot_count = 0;
+    __syncthreads();
+    for (int step = 0; step < kk - 1; ++step) {
+      for (int pr = warp; pr < npairs; pr += kJacThreads / 32) {
+        // round-robin pairing: player 0 fixed, the others rotate by `step`
+        auto player = [&](int at) { return at == 0 ? 0 : 1 + (at - 1 + step) % (kk - 1); };
+        const int a = player(pr), b = player(kk - 1 - pr);
+        const int lo = min(a, b), hi = max(a, b);
+        if (hi >= k) continue;
+        i128 x[2], y[2];
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+          const int i = lane + 32 * q;
+          x[q] = i < k ? W[lo * k + i] : (i128)0;
+          y[q] = i < k ? W[hi * k + i] : (i128)0;
+        }
+        const int ex = E[lo], ey = E[hi];
+        // sums of squares and products, units 2^(2 E - 250 + 128)
+        i128 sxx = 0, syy = 0, sxy = 0;
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+          if (q && k <= 32) break;
+          const u128 ax = (u128)(x[q] < 0 ? -x[q] : x[q]), ay = (u128)(y[q] < 0 ? -y[q] : y[q]);
+          sxx += (i128)mulhi128(ax, ax);
+          syy += (i128)mulhi128(ay, ay);
+          const i128 m = (i128)mulhi128(ax, ay);
+          sxy += (x[q] < 0) != (y[q] < 0) ? -m : m;
+        }
+        sxx = shfl_sum(sxx);
+        syy = shfl_sum(syy);
+        sxy = shfl_sum(sxy);
+        wide c, sn;
+        if (!Wide::rotation(wide_int(sxx, 2 * ex - 122), wide_int(syy, 2 * ey - 122), wide_int(sxy, ex + ey - 122), c, sn))
+          continue;
+        if (lane == 0) atomicAdd(&rot_count, 1);
+        // x' = c x - s y, y' = s x + c y: the high halves of the products, in units 2^(E - 124) (c) and 2^(E + es - 124) (s)
+        const u128 cf = c.m >> -c.e;  // c 2^127 (c.e is 0 or -1)
+        const int mx = max(ex, ey + sn.e), my = max(ey, ex + sn.e);
+        i128 nx[2], ny[2];
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+          const i128 sy = smulhi128(y[q], sn.m), sx = smulhi128(x[q], sn.m);
+          nx[q] = sar128(smulhi128(x[q], cf), mx - ex) + sar128(sn.s ? sy : -sy, mx - ey - sn.e);
+          ny[q] = sar128(smulhi128(y[q], cf), my - ey) + sar128(sn.s ? -sx : sx, my - ex - sn.e);
+        }
+        const int fx = settle(nx, mx - 124), fy = settle(ny, my - 124);
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+          const int i = lane + 32 * q;
+          if (i < k) {
+            W[lo * k + i] = nx[q];
+            W[hi * k + i] = ny[q];
+          }
+        }
+        if (lane == 0) {
+          E[lo] = fx;
+          E[hi] = fy;
+        }
+      }
+      __syncthreads();
+    }
+    if (rot_count == 0) {
+      if (tid == 0) st->sweeps = sweep + 1;
+      break;
+    }
+    __syncthreads();
+    if (sweep == 39 && tid == 0) st->sweeps = 40;
+  }
+  // eigenvalues and normalized columns
+  for (int l = warp; l < k; l += kJacThreads / 32) {
+    i128 x[2], sxx = 0;
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const int i = lane + 32 * q;
+      x[q] = i < k ? W[l * k + i] : (i128)0;
+      const u128 ax = (u128)(x[q] < 0 ? -x[q] : x[q]) << 2;  // (a norm below 2^127)
+      sxx += (i128)mulhi128(ax, ax);
+    }
+    const wide lam = wide_int(shfl_sum(sxx), 2 * E[l] - 126);
+    const wide r = wide_is_zero(lam) ? wide_zero() : wide_rsqrt(lam);
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const int i = lane + 32 * q;
+      if (i < k) U.set(l * k + i, wide_mul(wide_int(x[q], E[l] - 125), r));
+    }
+    if (lane == 0) A.set(tri(l, l), lam);
+  }
+  __syncthreads();
+  return true;
+}
+
 // --------------------------------------------------------------- SVQB
 
 template <class N>
@@ -629,7 +874,6 @@ __device__ __forceinline__ void svqb_small_body(int k, const double* Mh, const d
     }
     return;
   }
-  for (int t = tid; t < k * k; t += kJacThreads) U.set(t, t % k == t / k ? N::one() : N::zero());
   if (rotated) {  // the Jacobi runs on D M D (unit diagonal; a zero diagonal gives d_i = 0)
     for (int i = tid; i < k; i += kJacThreads) {
       const T m = A.get(tri(i, i));
@@ -644,98 +888,118 @@ __device__ __forceinline__ void svqb_small_body(int k, const double* Mh, const d
     }
   }
   __syncthreads();
-  // Sweeps of the parallel (round-robin) ordering.  Per step: (1) each pair's
-  // rotation (N::rotation: the angle in a short format, c and s orthogonal to
-  // full precision; the remainder of a_pq is removed by later sweeps); (2) A' =
-  // J^T A J by 2x2 blocks of pairs on the upper triangle, into the second
-  // buffer, and U <- U J in place.  The warps take units of (2) from a counter:
-  // first 16 blocks a unit (a pair of lanes per block: each multiplies a row by
-  // J_Q, then, after an exchange, a column by J_P^T), then 64 entries of U.
-  const int nblk = npairs * (npairs + 1) / 2, ablk = (nblk + 15) / 16, uent = 2 * npairs * k, nunits = ablk + (uent + 63) / 64;
-  for (int sweep = 0; sweep < 40; ++sweep) {
-    if (tid == 0) rot_count = 0;
-    __syncthreads();
-    for (int step = 0; step < kk - 1; ++step) {
-      // round-robin pairing: player 0 fixed, the others rotate by `step`
-      if (tid < npairs) {
-        auto player = [&](int pos) { return pos == 0 ? 0 : 1 + (pos - 1 + step) % (kk - 1); };
-        const int a = player(tid), b = player(kk - 1 - tid);
-        const int lo = min(a, b), hi = max(a, b);
-        T c = N::one(), sn = N::zero();
-        const bool rot = hi < k && N::rotation(A.get(tri(lo, lo)), A.get(tri(hi, hi)), A.get(tri(lo, hi)), c, sn);
-        if (rot) atomicAdd(&rot_count, 1);
-        rotates[tid] = rot;
-        cs.set(2 * tid, c);
-        cs.set(2 * tid + 1, sn);
-        pr[2 * tid] = lo;
-        pr[2 * tid + 1] = hi;
-      }
-      if (tid == kJacThreads - 1) next_unit = 0;
+  auto twosided = [&]() {
+    // Sweeps of the parallel (round-robin) ordering.  Per step: (1) each pair's
+    // rotation (N::rotation: the angle in a short format, c and s orthogonal to
+    // full precision; the remainder of a_pq is removed by later sweeps); (2) A' =
+    // J^T A J by 2x2 blocks of pairs on the upper triangle, into the second
+    // buffer, and U <- U J in place.  The warps take units of (2) from a counter:
+    // first 16 blocks a unit (a pair of lanes per block: each multiplies a row by
+    // J_Q, then, after an exchange, a column by J_P^T), then 64 entries of U.
+    const int nblk = npairs * (npairs + 1) / 2, ablk = (nblk + 15) / 16, uent = 2 * npairs * k, nunits = ablk + (uent + 63) / 64;
+    for (int sweep = 0; sweep < 40; ++sweep) {
+      if (tid == 0) rot_count = 0;
       __syncthreads();
-      for (;;) {
-        int unit = 0;
-        if (lane == 0) unit = atomicAdd(&next_unit, 1);
-        unit = __shfl_sync(0xffffffffu, unit, 0);
-        if (unit >= nunits) break;
-        if (unit < ablk) {
-          // A2 = J^T A J, block (P, Q) of rows {lo_P, hi_P} and columns {lo_Q, hi_Q}, P <= Q
-          const int b = unit * 16 + (lane >> 1), r = lane & 1;
-          const bool act = b < nblk;
-          int P, Q;
-          untri(act ? b : 0, P, Q);
-          const int r0 = pr[2 * P], r1 = pr[2 * P + 1], c0 = pr[2 * Q], c1 = pr[2 * Q + 1];
-          const bool v1 = r1 < k, w1 = c1 < k;  // r0, c0 < k always (the dummy index is the larger)
-          const int row = r ? r1 : r0;
-          const bool have = !r || v1;
-          T t0 = have ? A.get(sym(row, c0)) : N::zero();
-          T t1 = have && w1 ? A.get(sym(row, c1)) : N::zero();
-          if (rotates[Q]) {  // row r of B J_Q
-            const T c = cs.get(2 * Q), sn = cs.get(2 * Q + 1);
-            const T x = N::dot2(t0, c, t1, N::neg(sn));
-            t1 = N::dot2(t0, sn, t1, c);
-            t0 = x;
-          }
-          const T other = N::shfl_xor(r ? t0 : t1, 1);
-          T y0 = r ? other : t0, y1 = r ? t1 : other;  // column r
-          if (rotates[P]) {  // J_P^T (B J_Q)
-            const T c = cs.get(2 * P), sn = cs.get(2 * P + 1);
-            const T x = N::dot2(c, y0, N::neg(sn), y1);
-            y1 = N::dot2(sn, y0, c, y1);
-            y0 = x;
-          }
-          if (act && (!r || w1)) {
-            const int col = r ? c1 : c0;
-            A2.set(sym(r0, col), y0);
-            if (v1 && (P != Q || r)) A2.set(sym(r1, col), y1);  // (P = Q: (r1, c0) is the mirror of (r0, c1))
-          }
-        } else {
-          // U <- U J, columns lo_Q, hi_Q of row m: a pair of lanes per row and pair
-          for (int h = 0; h < 2; ++h) {
-            const int t = (unit - ablk) * 64 + h * 32 + lane;
-            const int q = (t >> 1) / k, m = (t >> 1) % k, r = t & 1;
-            const bool act = t < uent && rotates[q] != 0;
-            T v = N::zero();
-            if (act) {
-              const T c = cs.get(2 * q), sn = cs.get(2 * q + 1);
-              const T x = U.get(pr[2 * q] * k + m), y = U.get(pr[2 * q + 1] * k + m);
-              v = r ? N::dot2(sn, x, c, y) : N::dot2(c, x, N::neg(sn), y);
+      for (int step = 0; step < kk - 1; ++step) {
+        // round-robin pairing: player 0 fixed, the others rotate by `step`
+        if (tid < npairs) {
+          auto player = [&](int pos) { return pos == 0 ? 0 : 1 + (pos - 1 + step) % (kk - 1); };
+          const int a = player(tid), b = player(kk - 1 - tid);
+          const int lo = min(a, b), hi = max(a, b);
+          T c = N::one(), sn = N::zero();
+          const bool rot = hi < k && N::rotation(A.get(tri(lo, lo)), A.get(tri(hi, hi)), A.get(tri(lo, hi)), c, sn);
+          if (rot) atomicAdd(&rot_count, 1);
+          rotates[tid] = rot;
+          cs.set(2 * tid, c);
+          cs.set(2 * tid + 1, sn);
+          pr[2 * tid] = lo;
+          pr[2 * tid + 1] = hi;
+        }
+        if (tid == kJacThreads - 1) next_unit = 0;
+        __syncthreads();
+        for (;;) {
+          int unit = 0;
+          if (lane == 0) unit = atomicAdd(&next_unit, 1);
+          unit = __shfl_sync(0xffffffffu, unit, 0);
+          if (unit >= nunits) break;
+          if (unit < ablk) {
+            // A2 = J^T A J, block (P, Q) of rows {lo_P, hi_P} and columns {lo_Q, hi_Q}, P <= Q
+            const int b = unit * 16 + (lane >> 1), r = lane & 1;
+            const bool act = b < nblk;
+            int P, Q;
+            untri(act ? b : 0, P, Q);
+            const int r0 = pr[2 * P], r1 = pr[2 * P + 1], c0 = pr[2 * Q], c1 = pr[2 * Q + 1];
+            const bool v1 = r1 < k, w1 = c1 < k;  // r0, c0 < k always (the dummy index is the larger)
+            const int row = r ? r1 : r0;
+            const bool have = !r || v1;
+            T t0 = have ? A.get(sym(row, c0)) : N::zero();
+            T t1 = have && w1 ? A.get(sym(row, c1)) : N::zero();
+            if (rotates[Q]) {  // row r of B J_Q
+              const T c = cs.get(2 * Q), sn = cs.get(2 * Q + 1);
+              const T x = N::dot2(t0, c, t1, N::neg(sn));
+              t1 = N::dot2(t0, sn, t1, c);
+              t0 = x;
             }
-            __syncwarp();  // both lanes have read the entries that they replace
-            if (act) U.set(pr[2 * q + r] * k + m, v);
+            const T other = N::shfl_xor(r ? t0 : t1, 1);
+            T y0 = r ? other : t0, y1 = r ? t1 : other;  // column r
+            if (rotates[P]) {  // J_P^T (B J_Q)
+              const T c = cs.get(2 * P), sn = cs.get(2 * P + 1);
+              const T x = N::dot2(c, y0, N::neg(sn), y1);
+              y1 = N::dot2(sn, y0, c, y1);
+              y0 = x;
+            }
+            if (act && (!r || w1)) {
+              const int col = r ? c1 : c0;
+              A2.set(sym(r0, col), y0);
+              if (v1 && (P != Q || r)) A2.set(sym(r1, col), y1);  // (P = Q: (r1, c0) is the mirror of (r0, c1))
+            }
+          } else {
+            // U <- U J, columns lo_Q, hi_Q of row m: a pair of lanes per row and pair
+            for (int h = 0; h < 2; ++h) {
+              const int t = (unit - ablk) * 64 + h * 32 + lane;
+              const int q = (t >> 1) / k, m = (t >> 1) % k, r = t & 1;
+              const bool act = t < uent && rotates[q] != 0;
+              T v = N::zero();
+              if (act) {
+                const T c = cs.get(2 * q), sn = cs.get(2 * q + 1);
+                const T x = U.get(pr[2 * q] * k + m), y = U.get(pr[2 * q + 1] * k + m);
+                v = r ? N::dot2(sn, x, c, y) : N::dot2(c, x, N::neg(sn), y);
+              }
+              __syncwarp();  // both lanes have read the entries that they replace
+              if (act) U.set(pr[2 * q + r] * k + m, v);
+            }
           }
         }
+        __syncthreads();
+        const typename N::Vec sw = A;
+        A = A2;
+        A2 = sw;
       }
+      if (rot_count == 0) {
+        if (tid == 0) st->sweeps = sweep + 1;
+        break;
+      }
+      __syncthreads();
+      if (sweep == 39 && tid == 0) st->sweeps = 40;
+    }
+  };
+  // M itself (or D M D) is kept in A2 in case the one-sided form declines it
+  bool done = false;
+  if constexpr (N::kOneSided) {
+    for (int t = tid; t < nt; t += kJacThreads) A2.set(t, A.get(t));
+    __syncthreads();
+    done = onesided_jacobi(k, A, U, st);
+    if (!done) {
       __syncthreads();
       const typename N::Vec sw = A;
       A = A2;
       A2 = sw;
     }
-    if (rot_count == 0) {
-      if (tid == 0) st->sweeps = sweep + 1;
-      break;
-    }
+  }
+  if (!done) {
+    for (int t = tid; t < k * k; t += kJacThreads) U.set(t, t % k == t / k ? N::one() : N::zero());
     __syncthreads();
-    if (sweep == 39 && tid == 0) st->sweeps = 40;
+    twosided();
   }
   if (rotated) {
     // Column a of U: its largest-magnitude entry (lowest row on ties) made
