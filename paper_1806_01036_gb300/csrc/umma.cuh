@@ -3,13 +3,6 @@
 // loads and stores, shared-memory matrix descriptors and tcgen05.mma, and the
 // 7-bit digits of an FP64 value aligned to a group exponent.
 //
-// Digits: a value x aligned to the exponent A of its group (A >= the biased
-// exponent of every member) is the integer X = floor(|x| 2^(1127 - A)) < 2^105
-// = sum_{s=0}^{14} D_s 2^(98 - 7s).  The row kernels (umma_rowprod.cu) use
-// plain digits D_s in [0, 127], each the FP16 subnormal +-D_s 2^-24 whose bit
-// pattern is the digit with the value's sign, so products of two digits are
-// exact and FP32 sums of fewer than 2^24 units of 2^-48 are exact.  The Gram
-// kernel (umma_gram.cu) has balanced 8-bit digits of its own.
 #pragma once
 
 #include <cuda.h>
@@ -23,7 +16,6 @@ namespace umma {
 
 using namespace fx;
 
-constexpr int NS = 15;  // digits per value
 constexpr unsigned long long kWaitNs = 2000000000ull;  // bound of every mbarrier wait
 
 // ------------------------------------------------------------ PTX helpers
@@ -252,13 +244,27 @@ __device__ __forceinline__ void tma_load_2d(unsigned dst, const CUtensorMap* map
 }
 
 // ------------------------------------------------------------ digits
-// X = floor(|x| 2^(1127 - A)) < 2^105 as four 32-bit words (w[0] least
-// significant); A >= align_exp(x).  X = m 2^t with m the 53-bit significand.
-__device__ __forceinline__ void xwords(double x, int A, unsigned (&w)[4]) {
+// A value x aligned to the exponent A of its group (A >= the biased exponent
+// of every member) is held as X = floor(|x| 2^(1132 - A)) < 2^110, written with
+// 14 balanced base-256 digits, X = sum_s D_s 2^(104 - 8s): the fields of X +
+// bias, less 128, D_s in [-128, 127] for s >= 1, and D_0 in [0, 64].  A digit is the FP16
+// integer sign(x) D_s: the field is put into the significand of the FP16 1024
+// (bit pattern 0x6400 | f) and one f16x2 FMA takes the offset off and the sign
+// on.  Fields are bytes, so two values' digits are cut with one byte
+// permutation or one masked merge.  A value within kNearBits binades of A has a zero low word, and
+// its digits 10..13 are zero.
+constexpr int kNear = 10, kAll = 14;  // digits of a near value, of any value
+constexpr int kNearBits = 25;
+__device__ __forceinline__ unsigned abs_hi(double x) { return hi32(x) & 0x7fffffffu; }
+// Smallest |x| high word of a near value (at least the smallest normal).
+__device__ __forceinline__ unsigned near_floor(int A) { return (unsigned)max(A - kNearBits, 1) << 20; }
+
+// X = m 2^t (m the 53-bit significand) as four 32-bit words (w[0] least significant).
+__device__ __forceinline__ void any_value_words(double x, int A, unsigned (&w)[4]) {
   const unsigned hi = hi32(x), lo = lo32(x);
   const int e = (hi >> 20) & 0x7ff;
   const unsigned mh = (hi & 0xfffffu) | (e ? 0x100000u : 0u);
-  const int t = 52 - A + max(e, 1);
+  const int t = 57 - A + max(e, 1);
   if (t >= 0) {
     const int bo = t & 31;
     const unsigned s0 = lo << bo, s1 = __funnelshift_l(lo, mh, bo), s2 = __funnelshift_l(mh, 0u, bo);
@@ -278,26 +284,6 @@ __device__ __forceinline__ void xwords(double x, int A, unsigned (&w)[4]) {
   }
 }
 
-// X for a normal value within 20 binades of A (its exponent e >= A - 20,
-// so t = 52 - A + e is in [32, 52]): the significand shifted by t - 32
-// lands in words 1..3 and word 0 is zero.  cA = 52 - A.  The shift amount
-// is taken from the low five bits of (hi >> 20) + cA: the sign bit above
-// the exponent field adds a multiple of 32, and the funnel shifts use the
-// amount modulo 32.
-__device__ __forceinline__ void xwords_near(double x, int cA, unsigned (&w)[4]) {
-  const unsigned hi = hi32(x), lo = lo32(x);
-  const unsigned bo = (hi >> 20) + (unsigned)cA;
-  const unsigned mh = (hi & 0xfffffu) | 0x100000u;
-  w[0] = 0u;
-  w[1] = __funnelshift_l(0u, lo, bo);
-  w[2] = __funnelshift_l(lo, mh, bo);
-  w[3] = __funnelshift_l(mh, 0u, bo);
-}
-// Smallest |x| high word that xwords_near accepts for alignment exponent A:
-// exponent at least max(A - 20, 1) (zeros and subnormals take xwords).
-__device__ __forceinline__ unsigned near_floor(int A) { return (unsigned)max(A - 20, 1) << 20; }
-__device__ __forceinline__ unsigned abs_hi(double x) { return hi32(x) & 0x7fffffffu; }
-
 // 8-byte asynchronous copy global -> shared; src_bytes 0 writes zeros.
 __device__ __forceinline__ void cp_async8z(unsigned dst, const void* src, unsigned src_bytes) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(dst), "l"(src), "r"(src_bytes) : "memory");
@@ -308,36 +294,6 @@ __device__ __forceinline__ void cp_async4z(unsigned dst, const void* src, unsign
 }
 __device__ __forceinline__ void cp_async_commit_group() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 
-// A pair of values (a, b) interleaved in 16-bit lanes: Z[k] holds bits
-// 16k .. 16k + 15 of a in its low half and of b in its high half (k = 0..6),
-// Z8[k] the same for bits 16k + 8 .. 16k + 23 (k = 0..5).  Every 7-bit digit
-// field of both values then lies inside one lane of one word.
-struct PairLanes {
-  unsigned Z[7], Z8[6];
-};
-__device__ __forceinline__ PairLanes pair_lanes(const unsigned (&a)[4], const unsigned (&b)[4]) {
-  PairLanes p;
-#pragma unroll
-  for (int k = 0; k < 7; ++k) p.Z[k] = __byte_perm(a[k >> 1], b[k >> 1], (k & 1) ? 0x7632 : 0x5410);
-#pragma unroll
-  for (int k = 0; k < 6; ++k) p.Z8[k] = __byte_perm(p.Z[k], p.Z[k + 1], 0x6341);
-  return p;
-}
-// Digit word of slab S for the pair: (D_S(a) | sign a) | ((D_S(b) | sign b) << 16),
-// both halves FP16 subnormals +-D 2^-24 (signs: bit 15 and bit 31).
-template <int S>
-__device__ __forceinline__ unsigned pair_word(const PairLanes& p, unsigned signs) {
-  constexpr int q = 98 - 7 * S, k = q >> 4, o = q & 15;
-  constexpr bool low = o <= 9;
-  constexpr int sh = low ? o : o - 8;
-  const unsigned z = low ? p.Z[k] : p.Z8[k];
-  // the shift as a high-half multiplication (the FMA pipe), then one
-  // three-input logic operation (z & 0x007f007f) | signs (the ALU)
-  unsigned zs = z, w;
-  if constexpr (sh > 0) asm("mul.hi.u32 %0, %1, %2;" : "=r"(zs) : "r"(z), "n"(1u << (32 - sh)));
-  asm("lop3.b32 %0, %1, %2, %3, 0xEA;" : "=r"(w) : "r"(zs), "n"(0x007f007fu), "r"(signs));
-  return w;
-}
 // The FP16 exponent field of 1024 in both halves, as a register (so that
 // the digit's mask and this constant fit one three-input logic operation).
 __device__ __forceinline__ unsigned exp1024x2() {
@@ -350,5 +306,71 @@ __device__ __forceinline__ unsigned hfma2(unsigned a, unsigned b, unsigned c) {
   asm("fma.rn.f16x2 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(c));
   return d;
 }
+// Bias of the balanced digits: 128 in each of the digit places 1..13 (bits
+// 0..103); the top digit is not negative and takes none.
+constexpr unsigned kB = 0x80808080u, kBTop = 0x80u;
+
+// Words 1..3 of X + bias for a value within kNearBits binades of A (X's word 0
+// is zero): the significand times 2^bo, bo = t - 32 with X = m 2^t, t = 57 - A
+// + e, so bo is in [0, 25].  bo has the sign bit (above the exponent field)
+// added as 2^11; shifts take their amount modulo 32.  cA = 25 - A.
+// ZERO: a value that is zero gives X = 0 (else the implicit bit would stand).
+template <bool ZERO>
+__device__ __forceinline__ void near_words(double x, int cA, unsigned& w1, unsigned& w2, unsigned& w3) {
+  const unsigned hi = hi32(x), lo = lo32(x);
+  const unsigned bo = (hi >> 20) + (unsigned)cA;
+  unsigned mh = (hi & 0xfffffu) | 0x100000u;
+  if (ZERO) mh = ((hi & 0x7fffffffu) | lo) ? mh : 0u;
+  w1 = __funnelshift_l(0u, lo, bo);
+  w2 = __funnelshift_l(lo, mh, bo);
+  w3 = __funnelshift_l(mh, 0u, bo);
+  asm("add.cc.u32 %0, %0, %3;\n\t"
+      "addc.cc.u32 %1, %1, %3;\n\t"
+      "addc.u32 %2, %2, %4;"
+      : "+r"(w1), "+r"(w2), "+r"(w3)
+      : "n"(kB), "n"(kBTop));
+}
+
+// X + bias of any value (A >= its exponent), four words.
+__device__ __forceinline__ void any_words(double x, int A, unsigned (&w)[4]) {
+  any_value_words(x, A, w);
+  asm("add.cc.u32 %0, %0, %4;\n\t"
+      "addc.cc.u32 %1, %1, %4;\n\t"
+      "addc.cc.u32 %2, %2, %4;\n\t"
+      "addc.u32 %3, %3, %5;"
+      : "+r"(w[0]), "+r"(w[1]), "+r"(w[2]), "+r"(w[3])
+      : "n"(kB), "n"(kBTop));
+}
+
+// f16x2 factors (+-1, +-1) of a pair's digit FMA sign (1024 + f) + addend,
+// with the addends -sign 1152 (f - 128) and, for the top digit, -sign 1024.
+struct Sign2 {
+  unsigned mul, add;
+};
+__device__ __forceinline__ unsigned hmul2(unsigned a, unsigned b) {
+  unsigned d;
+  asm("mul.rn.f16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
+  return d;
+}
+__device__ __forceinline__ Sign2 sign2(double a, double b) {
+  Sign2 s;
+  asm("lop3.b32 %0, %1, %2, %3, 0xEA;"
+      : "=r"(s.mul)
+      : "r"(__byte_perm(hi32(a), hi32(b), 0x7632)), "n"(0x80008000u), "r"(0x3C003C00u));
+  s.add = hmul2(s.mul, 0xE480E480u);
+  return s;
+}
+__device__ __forceinline__ Sign2 top(Sign2 s) { return Sign2{s.mul, hmul2(s.mul, 0xE400E400u)}; }
+// Both digits of a byte-interleaved lane word z = [lo a, hi a, lo b, hi b].
+__device__ __forceinline__ unsigned digit_lo(unsigned z, unsigned e1024, Sign2 s) {
+  unsigned f;
+  asm("lop3.b32 %0, %1, %2, %3, 0xEA;" : "=r"(f) : "r"(z), "n"(0x00ff00ffu), "r"(e1024));  // (z & m) | 1024
+  return hfma2(f, s.mul, s.add);
+}
+__device__ __forceinline__ unsigned digit_hi(unsigned z, unsigned e1024, Sign2 s) {
+  return hfma2(__byte_perm(z, e1024, 0x7371), s.mul, s.add);  // [z1, 0x64, z3, 0x64]
+}
+
+
 }  // namespace umma
 }  // namespace eo

@@ -104,7 +104,6 @@ constexpr int kWarps = kConvWarps + 1;      // all drain TMEM (4 per lane quarte
 constexpr int kThreads = 32 * kWarps;
 constexpr int kIssuer = 32 * kConvWarps;    // the thread that issues the MMAs
 constexpr int kLanes = 128;                   // MMA M = TMEM lanes
-constexpr int kNear = 10, kAll = 14;          // digit slabs of a near panel, of any panel
 constexpr int kDiag = 14;                     // last digit diagonal kept
 constexpr int kOffsetDigits = 2148;
 // Running sums grow by at most 2^24 per drain: exact in 32 bits for 127.
@@ -116,7 +115,6 @@ constexpr size_t kSmemCap = 225 * 1024;
 #ifndef EO_GRAM_HEADROOM
 #define EO_GRAM_HEADROOM 2
 #endif
-constexpr int kNearBits = 25;  // values within this many binades of A have a zero low word
 
 // Digit pairs per row that a column block of any lane block collects at most,
 // with ns digits per value: pairs (s, t) = (J q + j, c - J q), all < ns.
@@ -183,71 +181,6 @@ __device__ __forceinline__ double widen(float f) {
   const unsigned e = (b >> 23) & 0xffu;
   if (e == 0u || e == 255u) return (double)f;
   return __hiloint2double((int)((b & 0x80000000u) | ((e + 896u) << 20) | ((b & 0x7fffffu) >> 3)), (int)(b << 29));
-}
-
-// Bias of the balanced digits: 128 in each of the digit places 1..13 (bits
-// 0..103); the top digit is not negative and takes none.
-constexpr unsigned kB = 0x80808080u, kBTop = 0x80u;
-
-// Words 1..3 of X + bias for a value within kNearBits binades of A (X's word 0
-// is zero): the significand times 2^bo, bo = t - 32 with X = m 2^t, t = 57 - A
-// + e, so bo is in [0, 25].  bo has the sign bit (above the exponent field)
-// added as 2^11; shifts take their amount modulo 32.  cA = 25 - A.
-// ZERO: a value that is zero gives X = 0 (else the implicit bit would stand).
-template <bool ZERO>
-__device__ __forceinline__ void near_words(double x, int cA, unsigned& w1, unsigned& w2, unsigned& w3) {
-  const unsigned hi = hi32(x), lo = lo32(x);
-  const unsigned bo = (hi >> 20) + (unsigned)cA;
-  unsigned mh = (hi & 0xfffffu) | 0x100000u;
-  if (ZERO) mh = ((hi & 0x7fffffffu) | lo) ? mh : 0u;
-  w1 = __funnelshift_l(0u, lo, bo);
-  w2 = __funnelshift_l(lo, mh, bo);
-  w3 = __funnelshift_l(mh, 0u, bo);
-  asm("add.cc.u32 %0, %0, %3;\n\t"
-      "addc.cc.u32 %1, %1, %3;\n\t"
-      "addc.u32 %2, %2, %4;"
-      : "+r"(w1), "+r"(w2), "+r"(w3)
-      : "n"(kB), "n"(kBTop));
-}
-
-// X + bias of any value (A >= its exponent), four words.
-__device__ __forceinline__ void any_words(double x, int A, unsigned (&w)[4]) {
-  xwords(x, A - 5, w);  // floor(|x| 2^(1127 - (A - 5)))
-  asm("add.cc.u32 %0, %0, %4;\n\t"
-      "addc.cc.u32 %1, %1, %4;\n\t"
-      "addc.cc.u32 %2, %2, %4;\n\t"
-      "addc.u32 %3, %3, %5;"
-      : "+r"(w[0]), "+r"(w[1]), "+r"(w[2]), "+r"(w[3])
-      : "n"(kB), "n"(kBTop));
-}
-
-// f16x2 factors (+-1, +-1) of a pair's digit FMA sign (1024 + f) + addend,
-// with the addends -sign 1152 (f - 128) and, for the top digit, -sign 1024.
-struct Sign2 {
-  unsigned mul, add;
-};
-__device__ __forceinline__ unsigned hmul2(unsigned a, unsigned b) {
-  unsigned d;
-  asm("mul.rn.f16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
-  return d;
-}
-__device__ __forceinline__ Sign2 sign2(double a, double b) {
-  Sign2 s;
-  asm("lop3.b32 %0, %1, %2, %3, 0xEA;"
-      : "=r"(s.mul)
-      : "r"(__byte_perm(hi32(a), hi32(b), 0x7632)), "n"(0x80008000u), "r"(0x3C003C00u));
-  s.add = hmul2(s.mul, 0xE480E480u);
-  return s;
-}
-__device__ __forceinline__ Sign2 top(Sign2 s) { return Sign2{s.mul, hmul2(s.mul, 0xE400E400u)}; }
-// Both digits of a byte-interleaved lane word z = [lo a, hi a, lo b, hi b].
-__device__ __forceinline__ unsigned digit_lo(unsigned z, unsigned e1024, Sign2 s) {
-  unsigned f;
-  asm("lop3.b32 %0, %1, %2, %3, 0xEA;" : "=r"(f) : "r"(z), "n"(0x00ff00ffu), "r"(e1024));  // (z & m) | 1024
-  return hfma2(f, s.mul, s.add);
-}
-__device__ __forceinline__ unsigned digit_hi(unsigned z, unsigned e1024, Sign2 s) {
-  return hfma2(__byte_perm(z, e1024, 0x7371), s.mul, s.add);  // [z1, 0x64, z3, 0x64]
 }
 
 __device__ __forceinline__ void st_digits(unsigned addr, unsigned a, unsigned b, unsigned c, unsigned d) {
@@ -706,7 +639,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       // a nonzero value (normal or not) below the window
       const int A = max(te, 1);
       bool below = false;
-      const unsigned floor = (unsigned)max(A - kNearBits, 1) << 20;
+      const unsigned floor = near_floor(A);
 #pragma unroll
       for (int i = 0; i < 8; ++i) below |= valid && (abs_hi(u[i]) | lo32(u[i])) != 0u && abs_hi(u[i]) < floor;
       all = bar_any(below);

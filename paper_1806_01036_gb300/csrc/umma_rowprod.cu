@@ -10,34 +10,47 @@
 // Digits (umma.cuh): a row of the streamed matrix (V or X) is aligned to its
 // own largest exponent A_r, a column j of the small matrix (C or Z) to
 // B_j = its largest exponent + 1 (room for the low part); both are cut into
-// fifteen 7-bit digits.  A tile is 128 rows = the 128 TMEM lanes; the K
-// dimension is the kin columns of the row (kin <= 64), the N dimension the
-// digit slab t and the output column j (16 columns, padded).  One MMA
-// multiplies digit slab s of the tile (M = 128, K = 16) by the slabs
-// t = 0 .. 14 - s of the small matrix (N = 16 (15 - s)) and writes at TMEM
-// column offset 16 s: column block d of a lane collects the digit diagonal
-// d = s + t of its row.  A diagonal sum has at most kin x 15 products of
-// magnitude <= 127^2, below 2^24 for kin <= 64, so the FP32 accumulators are
-// exact over the whole row: a tile needs no drains, only an epilogue that
-// combines its 15 diagonals per output in 128-bit integers,
-//   h = sum_d S_d 2^(7 (14 - d)),   sum_i v_i c_ij ~= h 2^(A_r + B_j - 2156),
-// and rounds y - h 2^(...) (or h 2^(...)) to FP64 in integer arithmetic.
+// fourteen balanced 8-bit digits, of which the last four are zero for a row
+// whose values lie within 25 binades ("near", nearly always).  A tile is 128
+// rows = the 128 TMEM lanes; the K dimension is the kin columns of the row
+// (kin <= 64), the N dimension the digit slab t and the output column j (16
+// columns, padded).  One MMA multiplies digit slab s of the tile (M = 128, K =
+// 16) by the slabs t = 0 .. 13 - s of the small matrix (N = 16 (14 - s)) and
+// writes at TMEM column offset 16 s: column block d of a lane collects the
+// digit diagonal d = s + t of its row.  A diagonal sum has at most kin x 14
+// products of magnitude <= 2^14, below 2^24 for kin <= 64, so the FP32
+// accumulators are exact over the whole row: a tile needs no drains, only an
+// epilogue that combines its 14 diagonals per output in 128-bit integers,
+//   h = sum_d S_d 2^(8 (13 - d)),   sum_i v_i c_ij ~= h 2^(A_r + B_j - 2160),
+// and rounds y - h 2^(...) (or h 2^(...)) to FP64 in integer arithmetic.  The
+// dropped pairs (d >= 14: thirteen of weight 2^96 units^2 and fewer of smaller
+// weights, max|v| >= 2^109 units, max|c| >= 2^108) are below 2^-103 max|v_i|
+// max|c_ij| per product.
 //
-// Pipeline (one CTA per SM, tiles round-robin): the 16 converter warps hold
-// a tile's values in registers (8 rows x 4 column groups per warp,
-// coalesced along rows), fetched a tile ahead (staged through shared memory
-// with cp.async for kin <= 32, loaded into registers after the previous
-// tile's digits are stored for kin <= 64), find each row's exponent by
-// shuffles, and write the digits in three groups of five slabs into two
-// alternating shared-memory buffers; one warp issues the group's MMAs and
-// commits them to an mbarrier per buffer; TMEM holds two accumulators, so
-// the epilogue of tile i - 1 (tcgen05.ld, exact rounding, stores) runs
-// while the tensor cores work on tile i (with two blocks of 16 output
-// columns, one accumulator each: see the kernel).  The projection's Y of a tile is
-// prefetched into L2 a tile ahead and loaded before its epilogue reads
-// TMEM.  Every wait is bounded (the outputs of a CTA whose wait ran out are
-// NaN).  Each tile's loads precede its own stores, and no tile is written
+// Pipeline (one CTA per SM, tiles round-robin): the 16 converter warps hold a
+// tile's values in registers (8 rows x 4 column groups per warp, coalesced
+// along rows), fetched a tile ahead (staged through shared memory with cp.async
+// for kin <= 32, loaded into registers after the previous tile's digits are
+// stored for kin <= 64), find each row's exponent by shuffles, agree at the
+// barrier that ends the previous tile whether every value of the tile is near,
+// and write the digits in two groups of five slabs (a third of four for a tile
+// that is not near) into two alternating shared-memory buffers; one warp issues
+// the group's MMAs and commits them to an mbarrier per buffer; TMEM holds two
+// accumulators, so the epilogue of tile i - 1 (tcgen05.ld, exact rounding,
+// stores) runs while the tensor cores work on tile i (with two blocks of 16
+// output columns, one accumulator each: see the kernel).  The projection's Y of
+// a tile is prefetched into L2 a tile ahead and loaded before its epilogue
+// reads TMEM.  Every wait is bounded (the outputs of a CTA whose wait ran out
+// are NaN).  Each tile's loads precede its own stores, and no tile is written
 // by another CTA, so the update may run in place.
+//
+// Bound by instruction issue on the integer pipe (conversion and epilogue);
+// memory needs a third of the time.  8-bit digits in byte places (ten near
+// slabs, 14 diagonals) against 7-bit ones (twelve, 15), Y - V C of 4e6 rows:
+// 64 x 16 1.645 -> 1.507 ms, 32 x 32 2.135 -> 1.933, 32 x 16 1.230 -> 1.090,
+// 16 x 16 1.017 -> 0.907, 20 x 4 0.969 -> 0.811.
+#include <cuda_fp16.h>
+
 #include <algorithm>
 #include <cstdlib>
 
@@ -56,15 +69,11 @@ constexpr int kConvThreads = 32 * kConvWarps;
 constexpr int kThreads = kConvThreads + 32;  // plus one MMA-issuing warp
 constexpr int kRows = 128;                   // rows per tile (MMA M, TMEM lanes)
 constexpr int kOut = 16;                     // output columns of the MMA (padded)
-// Digit slabs per group (three groups per tile).
-template <int W>
-constexpr int kGroupSlabs = 5;
-template <int W>
-constexpr int kGroups = NS / kGroupSlabs<W>;
-constexpr int kScaleProd = 2156;             // value of h: h 2^(A_r + B_j - 2156)
-constexpr unsigned kAccCols = 256;           // TMEM columns per accumulator (240 used)
+constexpr int kGroup = 5;                    // digit slabs per group
+constexpr int kGroupsNear = 2, kGroupsAll = 3;
+constexpr int kScaleProd = 2160;             // value of h: h 2^(A_r + B_j - 2160)
+constexpr unsigned kAccCols = 256;           // TMEM columns per accumulator (224 used)
 constexpr size_t kMinSmem = 120 * 1024;      // keeps one CTA per SM (TMEM: 512 columns)
-
 
 // With kin <= 32 the digit buffers leave room below the shared-memory floor
 // that keeps one CTA per SM: every converter thread then stages its own
@@ -77,24 +86,15 @@ constexpr size_t kMinSmem = 120 * 1024;      // keeps one CTA per SM (TMEM: 512 
 // previous tile's epilogue.
 template <int W>
 constexpr bool kStageValues = W <= 8;
-#ifndef EO_ROW_NEAR
-#define EO_ROW_NEAR(W) ((W) >= 8)
-#endif
 
-// Diagonal d of a tile sums (d + 1) kin <= (d + 1) 4 W digit products of
-// magnitude <= 127^2.  Diagonals d <= kRoundDiag stay below 2^22 units, so
-// their integer value comes out of one FP32 add (the bit pattern of
-// 1.5 2^23 + S_d is 0x4B400000 + S_d) instead of a float-to-int conversion.
+// Diagonal d of a tile sums at most (d + 1) kin <= (d + 1) 4 W digit products of
+// magnitude <= 2^14.  Diagonals d <= kRoundDiag stay below 2^22, so their
+// integer value comes out of one FP32 add (the bit pattern of 1.5 2^23 + S_d is
+// 0x4B400000 + S_d) instead of a float-to-int conversion.
 template <int W>
-constexpr int kRoundDiag = (int)(4194303 / (4 * W * 127 * 127)) - 1;
-static_assert(kRoundDiag<4> >= 14 && kRoundDiag<8> == 7 && kRoundDiag<16> == 3, "diagonal bounds");
-// What those patterns add to chain c (diagonals 5c .. 5c + 4, weights 128^(5c + 4 - d)).
-template <int W>
-__host__ __device__ constexpr long long chain_offset(int c) {
-  long long o = 0;
-  for (int d = 5 * c; d < 5 * c + 5; ++d) o = o * 128 + (d <= kRoundDiag<W> ? 0x4B400000ll : 0ll);
-  return o;
-}
+constexpr int kRoundDiag = 4194303 / (4 * W * 16384) - 1;
+static_assert(kRoundDiag<4> >= 13 && kRoundDiag<8> == 6 && kRoundDiag<16> == 2, "diagonal bounds");
+
 __device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 
 __device__ __forceinline__ void st_shared_v4(unsigned addr, unsigned a, unsigned b, unsigned c, unsigned d) {
@@ -104,36 +104,22 @@ __device__ __forceinline__ void st_shared_v2(unsigned addr, unsigned a, unsigned
   asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(addr), "r"(a), "r"(b) : "memory");
 }
 
-// Three groups of four TMEM columns (this warp's 32 lanes), loaded and waited for in one step.
-__device__ __forceinline__ void tmem_ld3x4(unsigned a0, unsigned a1, unsigned a2, unsigned (&v)[3][4]) {
+// Two groups of four TMEM columns (this warp's 32 lanes), loaded and waited for in one step.
+__device__ __forceinline__ void tmem_ld2x4(unsigned a0, unsigned a1, unsigned (&v)[2][4]) {
   asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%12];\n"
-      "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%4,%5,%6,%7}, [%13];\n"
-      "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%8,%9,%10,%11}, [%14];\n"
+      "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%8];\n"
+      "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%4,%5,%6,%7}, [%9];\n"
       "tcgen05.wait::ld.sync.aligned;\n"
       : "=r"(v[0][0]), "=r"(v[0][1]), "=r"(v[0][2]), "=r"(v[0][3]), "=r"(v[1][0]), "=r"(v[1][1]), "=r"(v[1][2]),
-        "=r"(v[1][3]), "=r"(v[2][0]), "=r"(v[2][1]), "=r"(v[2][2]), "=r"(v[2][3])
-      : "r"(a0), "r"(a1), "r"(a2)
+        "=r"(v[1][3])
+      : "r"(a0), "r"(a1)
       : "memory");
 }
 
-// Digit words of slab S for W values of one row (two values per word, low
-// half first), stored at dst (W = 16: two 16-byte chunks 128 bytes apart;
-// W = 8: one chunk; W = 4: half a chunk).
-// near: every value of the warp had its X's low 32 bits zero (within 20
-// binades of its row's exponent), so the digits of slabs 11..14 (bits
-// 0..27) are zero and are stored as such without being extracted.
-template <int S, int W>
-__device__ __forceinline__ void store_slab(unsigned dst, const PairLanes (&P)[W / 2], const unsigned (&sg)[W / 2],
-                                           bool near) {
-  unsigned w[W / 2];
-  if (S >= 11 && near) {
-#pragma unroll
-    for (int m = 0; m < W / 2; ++m) w[m] = 0u;
-  } else {
-#pragma unroll
-    for (int m = 0; m < W / 2; ++m) w[m] = pair_word<S>(P[m], sg[m]);
-  }
+// The words of one slab for W values of a row, stored at dst (W = 16: two
+// 16-byte chunks 128 bytes apart; W = 8: one chunk; W = 4: half a chunk).
+template <int W>
+__device__ __forceinline__ void st_slab(unsigned dst, const unsigned (&w)[W / 2]) {
   if constexpr (W == 16) {
     st_shared_v4(dst, w[0], w[1], w[2], w[3]);
     st_shared_v4(dst + 128u, w[4], w[5], w[6], w[7]);
@@ -144,36 +130,71 @@ __device__ __forceinline__ void store_slab(unsigned dst, const PairLanes (&P)[W 
   }
 }
 
-template <int G, int W, int J = 0>
-__device__ __forceinline__ void store_group(unsigned dst, unsigned slab_bytes, const PairLanes (&P)[W / 2],
-                                            const unsigned (&sg)[W / 2], bool near) {
-  if constexpr (J < kGroupSlabs<W>) {
-    store_slab<G * kGroupSlabs<W> + J, W>(dst + J * slab_bytes, P, sg, near);
-    store_group<G, W, J + 1>(dst, slab_bytes, P, sg, near);
+// Lane words of W near values: z[m][i] holds digits 2i (high bytes) and 2i + 1
+// (low bytes) of the pair m.
+template <int W, bool ZERO>
+__device__ __forceinline__ void near_lanes(const double (&v)[W], int A, unsigned (&z)[W / 2][5], unsigned (&sg)[W / 2]) {
+#pragma unroll
+  for (int m = 0; m < W / 2; ++m) {
+    unsigned a1, a2, a3, b1, b2, b3;
+    near_words<ZERO>(v[2 * m], 25 - A, a1, a2, a3);
+    near_words<ZERO>(v[2 * m + 1], 25 - A, b1, b2, b3);
+    sg[m] = sign2(v[2 * m], v[2 * m + 1]).mul;
+    z[m][0] = __byte_perm(a3, b3, 0x5410);
+    z[m][1] = __byte_perm(a2, b2, 0x7632);
+    z[m][2] = __byte_perm(a2, b2, 0x5410);
+    z[m][3] = __byte_perm(a1, b1, 0x7632);
+    z[m][4] = __byte_perm(a1, b1, 0x5410);
   }
 }
-
-// store_group for a group index known at run time
+// Group G (slabs 5 G .. 5 G + 4) of near values.
+template <int G, int W>
+__device__ __forceinline__ void store_near(unsigned dst, unsigned slab_bytes, const unsigned (&z)[W / 2][5],
+                                           const unsigned (&sg)[W / 2], unsigned e1024) {
+#pragma unroll
+  for (int j = 0; j < kGroup; ++j) {
+    const int s = G * kGroup + j;
+    unsigned w[W / 2];
+#pragma unroll
+    for (int m = 0; m < W / 2; ++m) {
+      const Sign2 f{sg[m], hmul2(sg[m], s == 0 ? 0xE400E400u : 0xE480E480u)};
+      w[m] = s % 2 == 0 ? digit_hi(z[m][s / 2], e1024, f) : digit_lo(z[m][s / 2], e1024, f);
+    }
+    st_slab<W>(dst + (unsigned)j * slab_bytes, w);
+  }
+}
+// Group g of any values (rare: the words are formed anew for every slab).
 template <int W>
-__device__ __forceinline__ void store_group_rt(int g, unsigned dst, unsigned slab_bytes, const PairLanes (&P)[W / 2],
-                                               const unsigned (&sg)[W / 2], bool near) {
-  switch (g) {
-    case 0: store_group<0, W>(dst, slab_bytes, P, sg, near); break;
-    case 1: store_group<1, W>(dst, slab_bytes, P, sg, near); break;
-    case 2: store_group<2, W>(dst, slab_bytes, P, sg, near); break;
-    case 3: if constexpr (kGroups<W> > 3) store_group<3, W>(dst, slab_bytes, P, sg, near); break;
-    default: if constexpr (kGroups<W> > 4) store_group<4, W>(dst, slab_bytes, P, sg, near); break;
+__device__ __noinline__ void store_any(int g, unsigned dst, unsigned slab_bytes, const double* v, int A) {
+  const unsigned e1024 = exp1024x2();
+#pragma unroll 1
+  for (int j = 0; j < kGroup; ++j) {
+    const int s = g * kGroup + j;
+    if (s >= kAll) break;
+    unsigned w[W / 2];
+#pragma unroll 1
+    for (int m = 0; m < W / 2; ++m) {
+      unsigned a[4], b[4];
+      any_words(v[2 * m], A, a);
+      any_words(v[2 * m + 1], A, b);
+      const int q = 104 - 8 * s;  // the digit's place
+      const unsigned fa = (a[q >> 5] >> (q & 31)) & 255u, fb = (b[q >> 5] >> (q & 31)) & 255u;
+      Sign2 f = sign2(v[2 * m], v[2 * m + 1]);
+      if (s == 0) f = top(f);
+      w[m] = hfma2(fa | (fb << 16) | e1024, f.mul, f.add);
+    }
+    st_slab<W>(dst + (unsigned)j * slab_bytes, w);
   }
 }
 
-// x 2^(1127 - A) as a signed 128-bit integer, truncated toward zero.
+// x 2^(1132 - A) as a signed 128-bit integer, truncated toward zero.
 __device__ __forceinline__ i128 fixed_trunc(double x, int A) {
   const unsigned hi = hi32(x), lo = lo32(x);
   int be = (hi >> 20) & 0x7ff;
   unsigned mh = hi & 0xfffffu;
   if (be) mh |= 0x100000u; else be = 1;
   const unsigned long long m = ((unsigned long long)mh << 32) | lo;
-  const int t = 52 - (A - be);
+  const int t = 57 - (A - be);
   u128 X;
   if (t >= 0) X = (u128)m << t;
   else if (t > -64) X = (u128)(m >> (-t));
@@ -181,13 +202,13 @@ __device__ __forceinline__ i128 fixed_trunc(double x, int A) {
   return (hi >> 31) ? -(i128)X : (i128)X;
 }
 
-// The general exact rounding (rare inputs the branch-free forms leave),
-// kept out of line so that the kernels' code stays small.
 // Outputs of a thread rounded side by side (measured on 4e6 rows: one at a
 // time for kin = 64, where two already cost spills at 96 registers; two
 // for the narrower products).
 template <int W>
 constexpr int kRoundPair = W >= 16 ? 1 : 2;
+// The general exact rounding (rare inputs the branch-free forms leave),
+// kept out of line so that the kernels' code stays small.
 __device__ __noinline__ double round_general(int update, double y, i128 h, int S) {
   return update ? w_to_double(h, S) : sub_round(y, h, S);
 }
@@ -211,15 +232,14 @@ __global__ void __launch_bounds__(kThreads, 1)
   constexpr int KC = KP / 16;             // MMAs (K = 16) per slab
   constexpr unsigned SBO = 16u * KP;      // bytes between 8-row groups of an operand
   constexpr unsigned SLAB_A = 16u * SBO;  // one digit slab of the tile (128 rows)
-  constexpr unsigned B_BYTES = 32u * SBO; // 16 slabs x 16 columns (one block of outputs)
+  constexpr unsigned B_BYTES = 2u * kAll * SBO;  // 14 slabs x 16 columns (one block of outputs)
   constexpr int NOUT = kOut * KO;
   static_assert(KO == 1 || (KO == 2 && W <= 8), "two output blocks only for kin <= 32");
 
   extern __shared__ __align__(128) unsigned char smem[];
   unsigned char* bdig = smem;                                  // the small matrix's digits
   unsigned char* adig = smem + KO * B_BYTES;                   // two group buffers of 5 slabs
-  constexpr int GS = kGroupSlabs<W>, NG = kGroups<W>;
-  int* Arow = reinterpret_cast<int*>(adig + 2 * GS * SLAB_A);  // [2][128] row exponents
+  int* Arow = reinterpret_cast<int*>(adig + 2 * kGroup * SLAB_A);  // [2][128] row exponents
   int* Rbad = Arow + 2 * kRows;                                // [2][128] non-finite rows
   int* Bexp = Rbad + 2 * kRows;                                // [NOUT] column exponents
   int* Bbad = Bexp + NOUT;                                     // [NOUT] non-finite columns
@@ -227,6 +247,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   __shared__ __align__(8) unsigned long long full_bar[2], ready_bar[2], tfree_bar;
   __shared__ unsigned tmem_base;
   __shared__ int bad;
+  __shared__ int far[2];  // far[i & 1] = i: the CTA's tile i needs all digits (set before the arrivals for its first group)
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int64_t ntiles = (n + kRows - 1) / kRows;
@@ -241,6 +262,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     mbar_init(smem_u32(&tfree_bar), kConvThreads);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     bad = 0;
+    far[0] = far[1] = -1;
   }
   if (tid < NOUT) {
     const int j = tid;
@@ -264,14 +286,13 @@ __global__ void __launch_bounds__(kThreads, 1)
       const double h = Bh[(size_t)j * ldb + i], l = Bl ? Bl[(size_t)j * ldb + i] : 0.0;
       x = fixed_trunc(h, Bexp[j]) + fixed_trunc(l, Bexp[j]);
     }
-    const unsigned sign = x < 0 ? 0x8000u : 0u;
-    const u128 U = x < 0 ? (u128)(-x) : (u128)x;  // < 2^104
-    for (int t = 0; t < 16; ++t) {
-      const unsigned dgt = t < NS ? ((unsigned)(U >> (98 - 7 * t)) & 127u) | sign : 0u;
+    const bool neg = x < 0;
+    const u128 U = (neg ? (u128)(-x) : (u128)x) + (((u128)0x8080808080ull << 64) | 0x8080808080808080ull);  // < 2^110 + bias
+    for (int t = 0; t < kAll; ++t) {
+      const int f = (int)((unsigned)(U >> (104 - 8 * t)) & 255u) - (t ? 128 : 0);
       const int R = t * kOut + j % kOut;
-      *reinterpret_cast<unsigned short*>(bdig + (j / kOut) * B_BYTES + (R >> 3) * SBO + (i >> 3) * 128 +
-                                         (R & 7) * 16 + (i & 7) * 2) =
-          (unsigned short)dgt;
+      *reinterpret_cast<__half*>(bdig + (j / kOut) * B_BYTES + (R >> 3) * SBO + (i >> 3) * 128 + (R & 7) * 16 +
+                                 (i & 7) * 2) = __int2half_rn(neg ? -f : f);
     }
   }
   fence_proxy_async();
@@ -295,18 +316,21 @@ __global__ void __launch_bounds__(kThreads, 1)
             tc_fence_after();
           }
         }
+        int ng = kGroupsNear;
 #pragma unroll 1
-        for (int g = 0; g < NG; ++g, ++G) {
+        for (int g = 0; g < ng; ++g, ++G) {
           const int b = G & 1;
           if (!mbar_wait(rb0 + 8u * b, (unsigned)(G >> 1) & 1u, &bad)) {
             ok = false;
             break;
           }
+          if (g == 0 && *reinterpret_cast<volatile int*>(&far[i & 1]) == (int)i) ng = kGroupsAll;
           tc_fence_after();
-          const unsigned abuf = adig_s + (unsigned)b * GS * SLAB_A;
-          for (int sg = 0; sg < GS; ++sg) {
-            const int s = g * GS + sg;
-            const unsigned idesc = idesc_f16(kRows, kOut * (NS - s));
+          const unsigned abuf = adig_s + (unsigned)b * kGroup * SLAB_A;
+          const int ns = min(kGroup, kAll - g * kGroup);
+          for (int sg = 0; sg < ns; ++sg) {
+            const int s = g * kGroup + sg;
+            const unsigned idesc = idesc_f16(kRows, kOut * (kAll - s));
 #pragma unroll
             for (int h = 0; h < KO; ++h)
 #pragma unroll
@@ -368,64 +392,40 @@ __global__ void __launch_bounds__(kThreads, 1)
                       : 0.0;
       }
       i128 h[4];
-      if constexpr (kRoundDiag<W> >= NS - 1) {
-        // every diagonal below 2^22 units: q_m = S_2m 128 + S_2m+1 in 32 bits
-        // (m = 0..6; the FP32 bit patterns carry the offset 0x4B400000, taken
-        // off once per pair), r = q_a 2^14 + q_b in 64 bits, and
-        // h = r_0 2^77 + r_1 2^49 + r_2 2^21 + r_3 with r_3 = q_6 2^7 + S_14.
-        unsigned qa[4];
-        long long ra[4];
+      // S_d of an accumulator: from the bit pattern of one FP32 add below 2^22
+      // (the offset is taken off), else converted
+      auto integer = [](unsigned v, int d) -> int {
+        return d <= kRoundDiag<W> ? (int)(__float_as_uint(__uint_as_float(v) + 0x1.8p23f) - 0x4B400000u)
+                                  : __float2int_rn(__uint_as_float(v));
+      };
+      {
+        // pairs q_m = S_2m 256 + S_2m+1 (m = 0..6): in 32 bits when every diagonal
+        // is below 2^22, else in 64; fours r = q_a 2^16 + q_b in 64 bits (below 2^50);
+        // h = r_0 2^80 + r_1 2^48 + r_2 2^16 + q_6
+        long long r[4];
 #pragma unroll
-        for (int d0 = 0; d0 < NS; d0 += 3) {
-          unsigned v[3][4];
-          tmem_ld3x4(tb + (unsigned)(d0 * kOut), tb + (unsigned)((d0 + 1) * kOut), tb + (unsigned)((d0 + 2) * kOut), v);
+        for (int m = 0; m < 7; ++m) {
+          unsigned v[2][4];
+          tmem_ld2x4(tb + (unsigned)(2 * m * kOut), tb + (unsigned)((2 * m + 1) * kOut), v);
 #pragma unroll
-          for (int u = 0; u < 3; ++u) {
-            const int d = d0 + u, m = d / 2;
-#pragma unroll
-            for (int y = 0; y < 4; ++y) {
-              const unsigned b = __float_as_uint(fmaf(__uint_as_float(v[u][y]), 0x1p48f, 0x1.8p23f));
-              if (d == NS - 1) {
-                h[y] += (i128)(ra[y] + (long long)(int)(b - 0x4B400000u));
-              } else if (d % 2 == 0) {
-                qa[y] = b;
-              } else {
-                const long long q = (long long)(int)((qa[y] << 7) + b - 129u * 0x4B400000u);
-                if (m % 2 == 0) ra[y] = q << (m == 6 ? 7 : 14);
-                else if (m == 1) h[y] = (i128)(ra[y] + q) << 77;
-                else h[y] += (i128)(ra[y] + q) << (m == 3 ? 49 : 21);
-              }
+          for (int y = 0; y < 4; ++y) {
+            long long q;
+            if constexpr (kRoundDiag<W> >= kAll - 1) {
+              const unsigned x0 = __float_as_uint(__uint_as_float(v[0][y]) + 0x1.8p23f);
+              const unsigned x1 = __float_as_uint(__uint_as_float(v[1][y]) + 0x1.8p23f);
+              q = (long long)(int)(x0 * 256u + x1 - 257u * 0x4B400000u);
+            } else {
+              q = (long long)integer(v[0][y], 2 * m) * 256 + integer(v[1][y], 2 * m + 1);
+            }
+            if (m % 2 == 0) {
+              r[y] = m == 6 ? q : q * 65536;
+              if (m == 6) h[y] += (i128)q;
+            } else if (m == 1) {
+              h[y] = (i128)(r[y] + q) << 80;
+            } else {
+              h[y] += (i128)(r[y] + q) << (m == 3 ? 48 : 16);
             }
           }
-        }
-      } else {
-        // h = p0 2^70 + p1 2^35 + p2 with p_c = sum over the five diagonals
-        // d = 5c .. 5c + 4 of S_d 2^(7 (5c + 4 - d)) (|p_c| < 2^53: 64-bit chains)
-        long long p[3][4];
-#pragma unroll
-        for (int d0 = 0; d0 < NS; d0 += 3) {
-          unsigned v[3][4];
-          tmem_ld3x4(tb + (unsigned)(d0 * kOut), tb + (unsigned)((d0 + 1) * kOut), tb + (unsigned)((d0 + 2) * kOut), v);
-#pragma unroll
-          for (int u = 0; u < 3; ++u) {
-            const int d = d0 + u, c = d / 5;
-#pragma unroll
-            for (int y = 0; y < 4; ++y) {
-              // S_d = accumulator x 2^48; diagonals below 2^22 units come out of
-              // the FP32 add of 1.5 2^23 as its bit pattern 0x4B400000 + S_d
-              // (the offsets are taken off the chains below)
-              const long long sd = d <= kRoundDiag<W>
-                                       ? (long long)__float_as_uint(fmaf(__uint_as_float(v[u][y]), 0x1p48f, 0x1.8p23f))
-                                       : (long long)__float2int_rn(__uint_as_float(v[u][y]) * 0x1p48f);
-              p[c][y] = (d % 5 == 0) ? sd : p[c][y] * 128 + sd;
-            }
-          }
-        }
-#pragma unroll
-        for (int y = 0; y < 4; ++y) {
-#pragma unroll
-          for (int c = 0; c < 3; ++c) p[c][y] -= chain_offset<W>(c);
-          h[y] = ((i128)p[0][y] << 70) + ((i128)p[1][y] << 35) + (i128)p[2][y];
         }
       }
       const int64_t grow = T * kRows + L;
@@ -468,26 +468,21 @@ __global__ void __launch_bounds__(kThreads, 1)
         v[k] = (T < ntiles && gr < n && col < kin) ? A[(size_t)col * lda + gr] : 0.0;
       }
     };
-    double vn[W];  // without staging: the values of the tile to come
-    if constexpr (!kStageValues<W>) load_direct(blockIdx.x, vn);
-
-    int G = 0;
-    int64_t Tprev = -1, iprev = 0;
-    for (int64_t T = blockIdx.x, i = 0; T < ntiles; T += gridDim.x, ++i) {
-      double v[W];
-      if constexpr (kStageValues<W>) {
-        asm volatile("cp.async.wait_all;" ::: "memory");  // this tile's copies, issued a tile ago
+    double v[W];  // the values of the tile to come
+    // takes the staged values of the tile that prefetch was last called for
+    auto take = [&]() {
+      asm volatile("cp.async.wait_all;" ::: "memory");
 #pragma unroll
-        for (int k = 0; k < W; ++k) v[k] = stg[k * kConvThreads + tid];
-        prefetch(T + gridDim.x);  // the next tile's values into the same slots, while this one runs
-      } else {
-#pragma unroll
-        for (int k = 0; k < W; ++k) v[k] = vn[k];
-      }
-      // the row's exponent: max of the |x| high words over the four threads
-      // of the row (a row of subnormals and zeros has exponent field 0 and
-      // is aligned to 1, the subnormals' own exponent)
-      unsigned key = 0, low = 0xffffffffu;  // largest and smallest |x| high word
+      for (int k = 0; k < W; ++k) v[k] = stg[k * kConvThreads + tid];
+    };
+    // The row's exponent: max of the |x| high words over the four threads of
+    // the row (a row of subnormals and zeros has exponent field 0 and is aligned
+    // to 1, the subnormals' own exponent); whether this thread's values hold a
+    // zero; whether one of them is nonzero and below the near window.
+    int Ar = 1;
+    bool nonfinite = false, zeros = false;
+    auto look = [&]() -> bool {
+      unsigned key = 0, low = 0xffffffffu;
 #pragma unroll
       for (int k = 0; k < W; ++k) {
         key = max(key, abs_hi(v[k]));
@@ -496,40 +491,57 @@ __global__ void __launch_bounds__(kThreads, 1)
       key = max(key, __shfl_xor_sync(0xffffffffu, key, 8));
       key = max(key, __shfl_xor_sync(0xffffffffu, key, 16));
       const int e = (int)(key >> 20);
-      const int Ar = max(e, 1);
+      Ar = max(e, 1);
+      nonfinite = e == 2047;
+      const unsigned floor = near_floor(Ar);
+      bool below = false;
+      zeros = __any_sync(0xffffffffu, low < floor);
+      if (zeros) {
+#pragma unroll
+        for (int k = 0; k < W; ++k) below |= abs_hi(v[k]) < floor && (abs_hi(v[k]) | lo32(v[k])) != 0u;
+      }
+      return below;
+    };
+    const unsigned e1024 = exp1024x2();
+    bool all = false;  // the tile to come needs all digits
+    {
+      bool below;
+      if constexpr (kStageValues<W>) {
+        take();
+        below = look();
+        prefetch(blockIdx.x + (int64_t)gridDim.x);
+      } else {
+        load_direct(blockIdx.x, v);
+        below = look();
+      }
+      all = bar_conv_or<kConvThreads>(below);
+    }
+
+    int G = 0;
+    int64_t Tprev = -1, iprev = 0;
+    for (int64_t T = blockIdx.x, i = 0; T < ntiles; T += gridDim.x, ++i) {
       if (cg == 0) {
         Arow[(i & 1) * kRows + r] = Ar;
-        Rbad[(i & 1) * kRows + r] = e == 2047;
+        Rbad[(i & 1) * kRows + r] = nonfinite;
       }
-      PairLanes P[W / 2];  // the W values as interleaved pairs
-      unsigned sg[W / 2];
-      // every value of the warp normal and within 20 binades of its row's
-      // exponent (nearly always): the aligned words without selects
-      const bool near = EO_ROW_NEAR(W) && __all_sync(0xffffffffu, low >= near_floor(Ar));
-#pragma unroll
-      for (int m = 0; m < W / 2; ++m) {
-        unsigned xa[4], xb[4];
-        if (near) {
-          xwords_near(v[2 * m], 52 - Ar, xa);
-          xwords_near(v[2 * m + 1], 52 - Ar, xb);
-        } else {
-          xwords(v[2 * m], Ar, xa);
-          xwords(v[2 * m + 1], Ar, xb);
-        }
-        P[m] = pair_lanes(xa, xb);
-        sg[m] = ((hi32(v[2 * m]) >> 31) << 15) | (hi32(v[2 * m + 1]) & 0x80000000u);
+      if (all && tid == 0) *reinterpret_cast<volatile int*>(&far[i & 1]) = (int)i;
+      const int ng = all ? kGroupsAll : kGroupsNear;
+      unsigned z[W / 2][5], sg[W / 2];
+      if (!all) {
+        if (zeros) near_lanes<W, true>(v, Ar, z, sg);
+        else near_lanes<W, false>(v, Ar, z, sg);
       }
-
-      // NG groups of GS slabs into the alternating buffers
-#pragma unroll
-      for (int g = 0; g < NG; ++g, ++G) {
+      // groups of slabs into the alternating buffers
+      auto group = [&](int g, auto store) {
         const int b = G & 1;
         if constexpr (KO > 1) {
-          if (g == NG - 1 && Tprev >= 0) {
-            // one accumulator per output block: the previous tile's MMAs are
-            // done (its last group was waited for before group 1 of this tile
-            // was stored), so its epilogue reads them here and releases them
-            // to this tile's MMAs
+          if (g == ng - 1 && Tprev >= 0) {
+            // one accumulator per output block: the previous tile's epilogue
+            // reads them here and releases them to this tile's MMAs (which are
+            // not issued before, so no group of this tile may be waited for).
+            // The previous tile's last group is G - 2 at a tile's second group:
+            // waited for here, or before this tile's second group was stored
+            if (g == 1) mbar_wait(fb0 + 8u * b, (unsigned)((G - 2) >> 1) & 1u, &bad);
             tc_fence_after();
 #pragma unroll 1
             for (int ob = 0; ob < KO; ++ob) epilogue_block(Tprev, iprev, ob);
@@ -538,17 +550,30 @@ __global__ void __launch_bounds__(kThreads, 1)
           }
         }
         if (G >= 2) mbar_wait(fb0 + 8u * b, (unsigned)((G - 2) >> 1) & 1u, &bad);  // MMAs of group G - 2 done
-        store_group_rt<W>(g, adig_s + (unsigned)b * GS * SLAB_A + dofs, SLAB_A, P, sg, near);
+        store(adig_s + (unsigned)b * kGroup * SLAB_A + dofs);
         fence_proxy_async();
         mbar_arrive(rb0 + 8u * b);
+        ++G;
+      };
+      if (!all) {
+        group(0, [&](unsigned dst) { store_near<0, W>(dst, SLAB_A, z, sg, e1024); });
+        group(1, [&](unsigned dst) { store_near<1, W>(dst, SLAB_A, z, sg, e1024); });
+      } else {
+        double u[W];
+#pragma unroll
+        for (int k = 0; k < W; ++k) u[k] = v[k];
+#pragma unroll 1
+        for (int g = 0; g < kGroupsAll; ++g) group(g, [&](unsigned dst) { store_any<W>(g, dst, SLAB_A, u, Ar); });
       }
-      if constexpr (!kStageValues<W>) load_direct(T + gridDim.x, vn);
+      // the next tile's values: in flight during the epilogue
+      if constexpr (!kStageValues<W>) load_direct(T + gridDim.x, v);
       if (!update && tid < 8 * kout) {  // Y of this tile, read by its epilogue a tile from now: into L2
         const int64_t g0 = T * kRows + (tid & 7) * 16;  // 16 rows = one 128-byte line per thread
         if (g0 < n) prefetch_l2(Yin + (size_t)(tid >> 3) * ldyin + g0);
       }
-      // the previous tile's MMAs completed (its last group was waited for before
-      // this tile's second group was written): its epilogue overlaps this tile's MMAs
+      // the previous tile's MMAs completed (all but its last group were waited
+      // for before this tile's groups were written, the last one here): its
+      // epilogue overlaps this tile's MMAs
       if constexpr (KO == 1) {
         if (Tprev >= 0) {
           tc_fence_after();
@@ -556,7 +581,17 @@ __global__ void __launch_bounds__(kThreads, 1)
           tc_fence_before();
         }
       }
-      bar_conv<kConvThreads>();  // row exponents of buffer (i - 1) & 1 are free again
+      bool below;
+      if constexpr (kStageValues<W>) {
+        take();
+        below = look();  // (reads every value before their slots are refilled)
+        prefetch(T + 2 * (int64_t)gridDim.x);
+      } else {
+        below = look();
+      }
+      // every warp has read buffer (i - 1) & 1 of the row exponents, and the
+      // next tile's kind is agreed on
+      all = bar_conv_or<kConvThreads>(below);
       Tprev = T;
       iprev = i;
     }
@@ -585,7 +620,7 @@ template <int W, int KO>
 size_t smem_bytes() {
   constexpr int KP = 4 * W;
   const size_t sbo = 16u * KP;
-  const size_t b = KO * 32 * sbo, a = 2 * kGroupSlabs<W> * 16 * sbo, small = (4 * kRows + 2 * kOut * KO) * sizeof(int);
+  const size_t b = KO * 2 * kAll * sbo, a = 2 * kGroup * 16 * sbo, small = (4 * kRows + 2 * kOut * KO) * sizeof(int);
   const size_t stage = kStageValues<W> ? (size_t)W * kConvThreads * sizeof(double) : 0;
   return std::max(b + a + small + stage, kMinSmem);
 }
@@ -613,10 +648,10 @@ bool umma_rowprod_supported(int kin, int kout) {
   if (e && e[0] == 'i') return false;
   if (kin < 1 || kin > 64 || kout < 1 || kout > 2 * kOut || (kout > kOut && kin > 32)) return false;
   // Small products run faster on the integer limbs: a tile's fixed cost
-  // (15 digit slabs, 16 padded outputs) dominates below kin max(kout, 4) =
-  // 128 (measured on 4e6 rows: kin = kout = 4 0.38 vs 1.29 ms, kin = 10,
-  // kout = 4 0.64 vs 1.30 ms; equal at 16 x 8; kin = 64, kout = 16 7.05 vs
-  // 2.35 ms the other way).  EO_DD_ROW_ENGINE=umma keeps the tensor cores.
+  // (its digit slabs, 16 padded outputs) dominates below kin max(kout, 4) =
+  // 128 (measured on 4e6 rows: kin = kout = 4 0.27 vs 0.59 ms, kin = 10,
+  // kout = 4 0.62 vs 0.60 ms; 16 x 8 1.31 vs 0.68, 16 x 16 2.32 vs 0.91 ms the
+  // other way).  EO_DD_ROW_ENGINE=umma keeps the tensor cores.
   if (!(e && e[0] == 'u') && kin * std::max(kout, 4) < 128) return false;
   return true;
 }
