@@ -403,6 +403,84 @@ FX_HD double sub_round_fast(double y, i128 w, int S, bool& ok) {
   return o;
 }
 
+// ---- the same two roundings on 32-bit words, for results whose low bits are
+// neither all zeros nor all ones (any but about 2^-25 of them, when the result
+// is not exact).  Variable 128-bit shifts, the carry chain of a negation and
+// the tie logic are most of the forms above; here words are selected and
+// funnel-shifted, a negative value is complemented instead of negated and a
+// truncation is left standing, both of which move the value by less than 64
+// units of a 32-bit word below the rounding bits, and ok is cleared when that
+// word is within 64 of wrapping (ties and exact results among them).
+FX_HD unsigned funnel_l(unsigned lo, unsigned hi, int s) {  // high word of (hi:lo) << (s mod 32)
+#ifdef __CUDA_ARCH__
+  return __funnelshift_l(lo, hi, (unsigned)s);
+#else
+  s &= 31;
+  return s ? (hi << s) | (lo >> (32 - s)) : hi;
+#endif
+}
+FX_HD int clz32(unsigned v) {
+#ifdef __CUDA_ARCH__
+  return __clz((int)v);
+#else
+  return v ? __builtin_clz(v) : 32;
+#endif
+}
+FX_HD unsigned word(u128 v, int i) { return (unsigned)(v >> (32 * i)); }
+FX_HD u128 from_words(unsigned w3, unsigned w2, unsigned w1, unsigned w0) {
+  return (u128)(((unsigned long long)w3 << 32) | w2) << 64 | (((unsigned long long)w1 << 32) | w0);
+}
+
+// (r + f) 2^S (0 <= f < 1, f = 0 if |r| < 2^92) with the sign flipped if flip
+// has its top bit set.
+FX_HD double w_to_double_lean(u128 r, int S, unsigned flip, bool& ok) {
+  const unsigned neg = (unsigned)((int)word(r, 3) >> 31);
+  const unsigned u3 = word(r, 3) ^ neg, u2 = word(r, 2) ^ neg, u1 = word(r, 1) ^ neg, u0 = word(r, 0) ^ neg;
+  const bool top = u3 != 0u;
+  const unsigned a = top ? u3 : u2, b = top ? u2 : u1, c = top ? u1 : u0, d = top ? u0 : neg;
+  const int lz = clz32(a);
+  const unsigned t2 = funnel_l(b, a, lz), t1 = funnel_l(c, b, lz), t0 = funnel_l(d, c, lz);
+  const int be1 = S + (top ? 1149 : 1117) - lz;  // biased exponent - 1
+  ok = a != 0u && (unsigned)be1 < 2045u && t0 + 64u >= 128u;
+  const unsigned hi = (t2 >> 11) + ((unsigned)be1 << 20);
+  const unsigned long long bits = (((unsigned long long)hi << 32) | funnel_l(t1, t2, 21)) + ((t1 >> 10) & 1u);
+  return from_bits(bits ^ ((unsigned long long)((neg ^ flip) & 0x80000000u) << 32));
+}
+
+// Does y dominate the grid 2^S by more than 2^72 of its units in its last place?
+FX_HD bool dominates(double y, int S) { return (int)((hi32(y) >> 20) & 0x7ffu) - 1075 - S > 72; }
+
+// y - w 2^S with w = raw - K; |w| < 2^122.  FAR: y may dominate the grid.
+template <bool FAR>
+FX_HD double sub_round_lean(double y, u128 raw, u128 K, int S, bool& ok) {
+  const unsigned hi = hi32(y), lo = lo32(y);
+  // sign(y) (y - w 2^S) = (|y| + g 2^S), g = -w for y >= 0 (the complement of
+  // raw - K - 1), w for y < 0
+  const unsigned pos = ~(unsigned)((int)hi >> 31);
+  u128 g = raw - from_words(word(K, 3), word(K, 2), word(K, 1), word(K, 0) + (pos & 1u));
+  unsigned g3 = word(g, 3) ^ pos, g2 = word(g, 2) ^ pos, g1 = word(g, 1) ^ pos, g0 = word(g, 0) ^ pos;
+  const int be = (int)((hi >> 20) & 0x7ffu);
+  const unsigned mh = (hi & 0xfffffu) | 0x100000u;
+  int d = be - 1075 - S;  // |y| = m 2^(S + d)
+  if (FAR) {  // y dominating: its last bit at 41 to 72 of a frame some words up
+    const int k = d > 72 ? (d - 41) >> 5 : 0;
+    const unsigned sx = (unsigned)((int)g3 >> 31);
+    g0 = k == 0 ? g0 : k == 1 ? g1 : k == 2 ? g2 : k == 3 ? g3 : sx;
+    g1 = k == 0 ? g1 : k == 1 ? g2 : k == 2 ? g3 : sx;
+    g2 = k == 0 ? g2 : k == 1 ? g3 : sx;
+    g3 = k == 0 ? g3 : sx;
+    d -= 32 * k;
+    S += 32 * k;
+  }
+  const unsigned m0 = lo << (d & 31), m1 = funnel_l(lo, mh, d), m2 = funnel_l(mh, 0u, d);
+  const bool w0 = d < 32, w1 = d < 64;
+  const u128 ym = from_words(w0 ? 0u : w1 ? m2 : m1, w0 ? m2 : w1 ? m1 : m0, w0 ? m1 : w1 ? m0 : 0u, w0 ? m0 : 0u);
+  bool okr;
+  const double o = w_to_double_lean(ym + from_words(g3, g2, g1, g0), S, hi, okr);
+  ok = okr && (unsigned)(be - 1) < 2046u && (unsigned)d <= 72u;
+  return o;
+}
+
 // 256-bit signed accumulator for sums of 128-bit terms.
 struct Acc256 {
   u128 lo;

@@ -20,7 +20,7 @@
 // digit diagonal d = s + t of its row.  A diagonal sum has at most kin x 14
 // products of magnitude <= 2^14, below 2^24 for kin <= 64, so the FP32
 // accumulators are exact over the whole row: a tile needs no drains, only an
-// epilogue that combines its 14 diagonals per output in 128-bit integers,
+// epilogue that combines its 14 diagonals per output in 32-bit words,
 //   h = sum_d S_d 2^(8 (13 - d)),   sum_i v_i c_ij ~= h 2^(A_r + B_j - 2160),
 // and rounds y - h 2^(...) (or h 2^(...)) to FP64 in integer arithmetic.  The
 // dropped pairs (d >= 14: thirteen of weight 2^96 units^2 and fewer of smaller
@@ -44,15 +44,21 @@
 // are NaN).  Each tile's loads precede its own stores, and no tile is written
 // by another CTA, so the update may run in place.
 //
-// Bound by instruction issue on the integer pipe (conversion and epilogue);
-// memory needs a third of the time.  8-bit digits in byte places (ten near
-// slabs, 14 diagonals) against 7-bit ones (twelve, 15), Y - V C of 4e6 rows:
-// 64 x 16 1.645 -> 1.507 ms, 32 x 32 2.135 -> 1.933, 32 x 16 1.230 -> 1.090,
-// 16 x 16 1.017 -> 0.907, 20 x 4 0.969 -> 0.811.
+// Bound by the integer pipe (62% busy over a kernel, saturated inside the
+// conversion and the epilogue): 131 instructions an output and 40 to 60 a
+// value; memory needs a third of the time.  Y - V C of 4e6 rows, with 7-bit
+// digits and 128-bit roundings (280 instructions an output), then with 8-bit
+// digits in byte places (ten near slabs and 14 diagonals, not twelve and 15),
+// then with the diagonals combined in words and the lean roundings of fx.cuh,
+// the outputs dealt evenly to the warps:
+//   64 x 16 1.645 -> 1.507 -> 1.224 ms, 32 x 32 2.135 -> 1.933 -> 1.396,
+//   32 x 16 1.230 -> 1.090 -> 0.829, 16 x 16 1.017 -> 0.907 -> 0.651,
+//   20 x 4 0.969 -> 0.811 -> 0.601, 8 x 8 0.774 -> 0.687 -> 0.500.
 #include <cuda_fp16.h>
 
 #include <algorithm>
 #include <cstdlib>
+#include <type_traits>
 
 #include "common.cuh"
 #include "fx.cuh"
@@ -87,13 +93,23 @@ constexpr size_t kMinSmem = 120 * 1024;      // keeps one CTA per SM (TMEM: 512 
 template <int W>
 constexpr bool kStageValues = W <= 8;
 
-// Diagonal d of a tile sums at most (d + 1) kin <= (d + 1) 4 W digit products of
-// magnitude <= 2^14.  Diagonals d <= kRoundDiag stay below 2^22, so their
-// integer value comes out of one FP32 add (the bit pattern of 1.5 2^23 + S_d is
-// 0x4B400000 + S_d) instead of a float-to-int conversion.
+// An accumulator S of magnitude below 2^22 becomes an integer with one FP32
+// add: the bit pattern of 1.5 2^23 + S is 0x4B400000 + S, and two of them
+// combine modulo 2^32 to S_2m 256 + S_2m+1 + kPairOffset, which stays in
+// [0, 2^32) below 2^22.  A diagonal of kin <= 16 columns sums at most 14 x 16
+// products of magnitude <= 2^14, below 2^22; wider rows pass 2^22 hardly ever,
+// and the sum of the squares of the diagonals tells when one could.
+constexpr unsigned kPairOffset = 0x8B400000u;
 template <int W>
-constexpr int kRoundDiag = 4194303 / (4 * W * 16384) - 1;
-static_assert(kRoundDiag<4> >= 13 && kRoundDiag<8> == 6 && kRoundDiag<16> == 2, "diagonal bounds");
+constexpr bool kSmallDiag = 4 * W * kAll * 16384 < 4194304;
+constexpr float kSquares = 0x1p42f;  // the rounded sum of 14 squares; each |S| < 2^21.1
+// The pairs' offsets in h: kPairOffset 2^(16 m), m = 0..6, modulo 2^128.
+constexpr u128 offset_sum() {
+  u128 k = 0;
+  for (int m = 0; m < 7; ++m) k += (u128)kPairOffset << (16 * m);
+  return k;
+}
+constexpr u128 kOffset = offset_sum();
 
 __device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 
@@ -104,16 +120,48 @@ __device__ __forceinline__ void st_shared_v2(unsigned addr, unsigned a, unsigned
   asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(addr), "r"(a), "r"(b) : "memory");
 }
 
-// Two groups of four TMEM columns (this warp's 32 lanes), loaded and waited for in one step.
-__device__ __forceinline__ void tmem_ld2x4(unsigned a0, unsigned a1, unsigned (&v)[2][4]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%8];\n"
-      "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%4,%5,%6,%7}, [%9];\n"
-      "tcgen05.wait::ld.sync.aligned;\n"
-      : "=r"(v[0][0]), "=r"(v[0][1]), "=r"(v[0][2]), "=r"(v[0][3]), "=r"(v[1][0]), "=r"(v[1][1]), "=r"(v[1][2]),
-        "=r"(v[1][3])
-      : "r"(a0), "r"(a1)
-      : "memory");
+// N groups of four TMEM columns (this warp's 32 lanes), 16 columns apart from column a on.
+template <int N>
+__device__ __forceinline__ void tmem_ld4(unsigned a, unsigned (&v)[N][4]) {
+#pragma unroll
+  for (int i = 0; i < N; ++i)
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(v[i][0]), "=r"(v[i][1]), "=r"(v[i][2]), "=r"(v[i][3])
+                 : "r"(a + (unsigned)(i * kOut))
+                 : "memory");
+}
+// Completes the loads into v (named, so that no use can move above the wait).
+template <int N>
+__device__ __forceinline__ void tmem_wait4(unsigned (&v)[N][4]) {
+  static_assert(N == 2 || N == 4, "groups per load");
+  if constexpr (N == 4)
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+r"(v[0][0]), "+r"(v[0][1]), "+r"(v[0][2]), "+r"(v[0][3]), "+r"(v[1][0]), "+r"(v[1][1]), "+r"(v[1][2]),
+                   "+r"(v[1][3]), "+r"(v[2][0]), "+r"(v[2][1]), "+r"(v[2][2]), "+r"(v[2][3]), "+r"(v[3][0]), "+r"(v[3][1]),
+                   "+r"(v[3][2]), "+r"(v[3][3])
+                 :
+                 : "memory");
+  else
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+r"(v[0][0]), "+r"(v[0][1]), "+r"(v[0][2]), "+r"(v[0][3]), "+r"(v[1][0]), "+r"(v[1][1]), "+r"(v[1][2]),
+                   "+r"(v[1][3])
+                 :
+                 : "memory");
+}
+// h + kOffset of four outputs whose diagonals reach 2^22 (rare), from the columns tb, tb + 16, ..
+__device__ __noinline__ void combine_any(unsigned tb, u128* h) {
+  for (int y = 0; y < 4; ++y) h[y] = kOffset;
+#pragma unroll 1
+  for (int m = 0; m < 7; ++m) {
+    unsigned v[2][4];
+    tmem_ld4(tb + (unsigned)(2 * m * kOut), v);
+    tmem_wait4(v);
+    for (int y = 0; y < 4; ++y) {
+      const long long q =
+          (long long)__float2int_rn(__uint_as_float(v[0][y])) * 256 + __float2int_rn(__uint_as_float(v[1][y]));
+      h[y] += (u128)(i128)q << (16 * (6 - m));
+    }
+  }
 }
 
 // The words of one slab for W values of a row, stored at dst (W = 16: two
@@ -202,14 +250,18 @@ __device__ __forceinline__ i128 fixed_trunc(double x, int A) {
   return (hi >> 31) ? -(i128)X : (i128)X;
 }
 
-// Outputs of a thread rounded side by side (measured on 4e6 rows: one at a
-// time for kin = 64, where two already cost spills at 96 registers; two
-// for the narrower products).
+// Outputs of a thread rounded side by side: one at a time where the next
+// tile's values stand in registers meanwhile (kin = 64).
 template <int W>
-constexpr int kRoundPair = W >= 16 ? 1 : 2;
-// The general exact rounding (rare inputs the branch-free forms leave),
+constexpr int kRoundSide = W >= 16 ? 1 : 4;
+// Added to the exponent of a row or a column with a non-finite value, and to a
+// row's when a wait has run out: no lean rounding takes it, and the general one
+// answers NaN.
+constexpr int kNaNExp = 1 << 24;
+// The general exact rounding (rare inputs the lean forms leave),
 // kept out of line so that the kernels' code stays small.
-__device__ __noinline__ double round_general(int update, double y, i128 h, int S) {
+__device__ __noinline__ double round_general(bool update, double y, i128 h, int S) {
+  if (S >= kNaNExp / 2) return __longlong_as_double(0x7ff8000000000000ll);
   return update ? w_to_double(h, S) : sub_round(y, h, S);
 }
 
@@ -222,9 +274,9 @@ __device__ __noinline__ double round_general(int update, double y, i128 h, int S
 // accumulators, release them (tfree) and then store group 2, and the MMAs of
 // tile i wait for that release, so the inputs are converted once for all 32
 // outputs.
-template <int W, int KO = 1>
+template <bool UPDATE, int W, int KO = 1>
 __global__ void __launch_bounds__(kThreads, 1)
-    umma_rowprod_kernel(int update, int64_t n, int kin, const double* A, int64_t lda, int kout,
+    umma_rowprod_kernel(int64_t n, int kin, const double* A, int64_t lda, int kout,
                         const double* __restrict__ Bh, const double* __restrict__ Bl, int ldb, int tri,
                         const double* Yin, int64_t ldyin, double* Out, int64_t ldo, const int* gate) {
   if (gate && *gate == 0) return;
@@ -240,10 +292,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   unsigned char* bdig = smem;                                  // the small matrix's digits
   unsigned char* adig = smem + KO * B_BYTES;                   // two group buffers of 5 slabs
   int* Arow = reinterpret_cast<int*>(adig + 2 * kGroup * SLAB_A);  // [2][128] row exponents
-  int* Rbad = Arow + 2 * kRows;                                // [2][128] non-finite rows
-  int* Bexp = Rbad + 2 * kRows;                                // [NOUT] column exponents
-  int* Bbad = Bexp + NOUT;                                     // [NOUT] non-finite columns
-  double* stg = reinterpret_cast<double*>(Bbad + NOUT);        // [W][512] staged values (kin <= 32)
+  int* Bexp = Arow + 2 * kRows;                                // [NOUT] column exponents
+  double* stg = reinterpret_cast<double*>(Bexp + NOUT);        // [W][512] staged values (kin <= 32)
   __shared__ __align__(8) unsigned long long full_bar[2], ready_bar[2], tfree_bar;
   __shared__ unsigned tmem_base;
   __shared__ int bad;
@@ -275,14 +325,13 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (ae == 2047 || (Bl && align_exp(Bl[(size_t)j * ldb + i]) == 2047)) nf = 1;
       }
     }
-    Bexp[j] = e + 1;  // one binade of headroom: |h + l| may round up past the largest h
-    Bbad[j] = nf;
+    Bexp[j] = e + 1 + (nf ? kNaNExp : 0);  // one binade of headroom: |h + l| may round up past the largest h
   }
   __syncthreads();
   for (int e = tid; e < NOUT * KP; e += kThreads) {  // block j / 16: B row R = t * 16 + j % 16 (slab t), K index i
     const int j = e / KP, i = e % KP;
     i128 x = 0;
-    if (j < kout && i < kin && !(tri && i > j) && !Bbad[j]) {
+    if (j < kout && i < kin && !(tri && i > j) && Bexp[j] < kNaNExp) {
       const double h = Bh[(size_t)j * ldb + i], l = Bl ? Bl[(size_t)j * ldb + i] : 0.0;
       x = fixed_trunc(h, Bexp[j]) + fixed_trunc(l, Bexp[j]);
     }
@@ -356,117 +405,151 @@ __global__ void __launch_bounds__(kThreads, 1)
     // digit offset of (row r, column c0) within a slab
     const unsigned dofs = (unsigned)(r >> 3) * SBO + (unsigned)(c0 >> 3) * 128u + (unsigned)(r & 7) * 16u +
                           (unsigned)(c0 & 7) * 2u;
-    // epilogue mapping: TMEM lane quarter warp % 4, outputs 4 (warp / 4) .. + 3
+    // epilogue mapping: TMEM lane quarter warp % 4; the kout outputs of a block
+    // are dealt to the four warps of a quarter, ny = ceil(kout / 4) to each
     const int eq = warp & 3, ep = warp >> 2;
     const int L = eq * 32 + lane;
-    const unsigned tq = taddr + ((unsigned)(eq * 32) << 16) + (unsigned)(ep * 4);
+    const unsigned tq = taddr + ((unsigned)(eq * 32) << 16);
 
-    // value k of this thread for tile T into its staging slots (zeros beyond the matrix)
-    const unsigned stg_s = smem_u32(stg);
+    // the values of tile T into this thread's staging slots (zeros beyond the
+    // matrix: nothing is read there)
+    const int nv = min(max(kin - c0, 0), W);  // columns of this thread
+    const unsigned stg_s = smem_u32(stg) + (unsigned)(tid * 8);
     auto prefetch = [&](int64_t T) {
       const int64_t gr = T * kRows + r;
+      const int in = gr < n ? nv : 0;  // (T >= ntiles: gr >= n)
+      const double* src = A + (in > 0 ? (size_t)c0 * lda + gr : 0);
 #pragma unroll
       for (int k = 0; k < W; ++k) {
-        const int col = c0 + k;
-        const bool ok = T < ntiles && gr < n && col < kin;
-        cp_async8z(stg_s + (unsigned)((k * kConvThreads + tid) * 8), ok ? A + (size_t)col * lda + gr : A,
-                   ok ? 8u : 0u);
+        cp_async8z(stg_s + (unsigned)(k * kConvThreads * 8), src, k < in ? 8u : 0u);
+        if (k + 1 < in) src += lda;
       }
       cp_async_commit_group();
     };
     if constexpr (kStageValues<W>) prefetch(blockIdx.x);
 
-    // outputs 16 ob + 4 ep .. + 3 (output block ob) of tile T (the index is
-    // written out at each use: a variable for it costs a register at the
-    // 96-register limit of the kin = 64 kernel, and it spills)
-    auto epilogue_block = [&](int64_t T, int64_t i, int ob) {
-      if (ob * kOut + ep * 4 >= kout) return;  // all four outputs of this warp are padding (warp-uniform)
-      const unsigned tb = tq + (unsigned)(KO > 1 ? ob : (int)(i & 1)) * kAccCols;
-      double yv[4];
-      {
-        const int64_t grow = T * kRows + L;
-#pragma unroll
-        for (int y = 0; y < 4; ++y)
-          yv[y] = (!update && ob * kOut + ep * 4 + y < kout && grow < n)
-                      ? Yin[(size_t)(ob * kOut + ep * 4 + y) * ldyin + grow]
-                      : 0.0;
-      }
-      i128 h[4];
-      // S_d of an accumulator: from the bit pattern of one FP32 add below 2^22
-      // (the offset is taken off), else converted
-      auto integer = [](unsigned v, int d) -> int {
-        return d <= kRoundDiag<W> ? (int)(__float_as_uint(__uint_as_float(v) + 0x1.8p23f) - 0x4B400000u)
-                                  : __float2int_rn(__uint_as_float(v));
-      };
-      {
-        // pairs q_m = S_2m 256 + S_2m+1 (m = 0..6): in 32 bits when every diagonal
-        // is below 2^22, else in 64; fours r = q_a 2^16 + q_b in 64 bits (below 2^50);
-        // h = r_0 2^80 + r_1 2^48 + r_2 2^16 + q_6
-        long long r[4];
-#pragma unroll
-        for (int m = 0; m < 7; ++m) {
-          unsigned v[2][4];
-          tmem_ld2x4(tb + (unsigned)(2 * m * kOut), tb + (unsigned)((2 * m + 1) * kOut), v);
-#pragma unroll
-          for (int y = 0; y < 4; ++y) {
-            long long q;
-            if constexpr (kRoundDiag<W> >= kAll - 1) {
-              const unsigned x0 = __float_as_uint(__uint_as_float(v[0][y]) + 0x1.8p23f);
-              const unsigned x1 = __float_as_uint(__uint_as_float(v[1][y]) + 0x1.8p23f);
-              q = (long long)(int)(x0 * 256u + x1 - 257u * 0x4B400000u);
-            } else {
-              q = (long long)integer(v[0][y], 2 * m) * 256 + integer(v[1][y], 2 * m + 1);
-            }
-            if (m % 2 == 0) {
-              r[y] = m == 6 ? q : q * 65536;
-              if (m == 6) h[y] += (i128)q;
-            } else if (m == 1) {
-              h[y] = (i128)(r[y] + q) << 80;
-            } else {
-              h[y] += (i128)(r[y] + q) << (m == 3 ? 48 : 16);
-            }
-          }
-        }
-      }
+    // outputs j0 .. j0 + ny - 1 of this warp (output block ob) of tile T
+    auto epilogue_ny = [&](auto NYc, int64_t T, int64_t i, int ob) {
+      constexpr int ny = decltype(NYc)::value;
+      const int j0 = ob * kOut + ep * ny;
+      if (j0 >= kout) return;  // all outputs of this warp are padding (warp-uniform)
+      const unsigned tb = tq + (unsigned)(KO > 1 ? ob : (int)(i & 1)) * kAccCols + (unsigned)(ep * ny);
       const int64_t grow = T * kRows + L;
-      const int Ar = Arow[(i & 1) * kRows + L];
-      const bool rbad = Rbad[(i & 1) * kRows + L] != 0;
-      // the four roundings without branches (independent, so they
-      // interleave); the rare inputs they leave (not ok) take the general
-      // rounding out of line
+      double yv[ny];
+      {
+        const double* Yp = Yin + (size_t)j0 * ldyin + grow;
 #pragma unroll
-      for (int y0 = 0; y0 < 4; y0 += kRoundPair<W>) {
-        double o[kRoundPair<W>];
-        bool ok[kRoundPair<W>];
-        if (update) {
+        for (int y = 0; y < ny; ++y)
+          yv[y] = (!UPDATE && j0 + y < kout && grow < n) ? Yp[(size_t)y * ldyin] : 0.0;
+      }
+      // pairs q_m = S_2m 256 + S_2m+1 + kPairOffset (m = 0..6) in 32 bits;
+      // h + kOffset = sum_m q_m 2^(16 (6 - m)): the even pairs are its words, the
+      // odd ones lie half a word up
+      u128 h[ny];
+      {
+        unsigned q[ny][7];
+        float squares[ny] = {};
+        // (two buffers of loads cost the kin = 64 kernel more spills than they hide)
+        constexpr int kBuf = W < 16 ? 2 : 1;
+        unsigned v[kBuf][4][4], vl[2][4];
+        auto pairs = [&](int m, const unsigned(&a)[4], const unsigned(&b)[4]) {
 #pragma unroll
-          for (int u = 0; u < kRoundPair<W>; ++u)
-            o[u] = w_to_double_fast(h[y0 + u], Ar + Bexp[ob * kOut + ep * 4 + y0 + u] - kScaleProd, ok[u]);
-        } else {
+          for (int y = 0; y < ny; ++y) {
+            const float fa = __uint_as_float(a[y]), fb = __uint_as_float(b[y]);
+            q[y][m] = __float_as_uint(fa + 0x1.8p23f) * 256u + __float_as_uint(fb + 0x1.8p23f);
+            if constexpr (!kSmallDiag<W>) squares[y] = fmaf(fa, fa, fmaf(fb, fb, squares[y]));
+          }
+        };
+        tmem_ld4(tb, v[0]);
+        tmem_wait4(v[0]);
 #pragma unroll
-          for (int u = 0; u < kRoundPair<W>; ++u)
-            o[u] = sub_round_fast(yv[y0 + u], h[y0 + u], Ar + Bexp[ob * kOut + ep * 4 + y0 + u] - kScaleProd, ok[u]);
+        for (int t = 0; t < 3; ++t) {  // diagonals 4 t .. 4 t + 3
+          auto next = [&]() {
+            if (t < 2) tmem_ld4(tb + (unsigned)((4 * t + 4) * kOut), v[(t + 1) % kBuf]);
+            else tmem_ld4(tb + (unsigned)(12 * kOut), vl);
+          };
+          if (kBuf > 1) next();
+          pairs(2 * t, v[t % kBuf][0], v[t % kBuf][1]);
+          pairs(2 * t + 1, v[t % kBuf][2], v[t % kBuf][3]);
+          if (kBuf == 1) next();
+          if (t < 2) tmem_wait4(v[(t + 1) % kBuf]);
+          else tmem_wait4(vl);
         }
+        pairs(6, vl[0], vl[1]);
+        float most = 0.f;
 #pragma unroll
-        for (int u = 0; u < kRoundPair<W>; ++u) {
-          const int y = y0 + u, j = ob * kOut + ep * 4 + y;
-          if (j < kout && grow < n) {
-            if (!ok[u]) o[u] = round_general(update, yv[y], h[y], Ar + Bexp[j] - kScaleProd);
-            if (rbad || Bbad[j] || bad) o[u] = __longlong_as_double(0x7ff8000000000000ll);
-            Out[(size_t)j * ldo + grow] = o[u];
+        for (int y = 0; y < ny; ++y) {
+          h[y] = from_words(q[y][0], q[y][2], q[y][4], q[y][6]) +
+                 from_words(q[y][1] >> 16, funnel_l(q[y][3], q[y][1], 16), funnel_l(q[y][5], q[y][3], 16), q[y][5] << 16);
+          most = fmaxf(most, squares[y]);
+        }
+        if constexpr (!kSmallDiag<W>) {
+          if (__any_sync(0xffffffffu, most >= kSquares)) {
+            u128 g[4];
+            combine_any(tb, g);
+#pragma unroll
+            for (int y = 0; y < ny; ++y) h[y] = g[y];
           }
         }
+      }
+      const int Sr = Arow[(i & 1) * kRows + L] - kScaleProd + (bad ? kNaNExp : 0);
+      double* Op = Out + (size_t)j0 * ldo + grow;
+      // the roundings of kSide outputs side by side (no branches among them);
+      // what they do not take is rounded by the general functions
+      constexpr int kSide = kRoundSide<W> < ny ? kRoundSide<W> : ny;
+#pragma unroll
+      for (int y0 = 0; y0 < ny; y0 += kSide) {
+        double o[kSide];
+        unsigned left = 0;
+        auto round_side = [&](auto FAR) {
+#pragma unroll
+          for (int y = y0; y < y0 + kSide && y < ny; ++y) {
+            const int S = Sr + Bexp[j0 + y];
+            bool ok;
+            o[y - y0] = UPDATE ? w_to_double_lean(h[y] - kOffset, S, 0u, ok)
+                               : sub_round_lean<decltype(FAR)::value>(yv[y], h[y], kOffset, S, ok);
+            left |= ok || j0 + y >= kout || grow >= n ? 0u : 1u << y;
+          }
+        };
+        bool far_y = false;
+        if constexpr (!UPDATE) {
+#pragma unroll
+          for (int y = y0; y < y0 + kSide && y < ny; ++y) far_y |= dominates(yv[y], Sr + Bexp[j0 + y]);
+        }
+        if (!UPDATE && __any_sync(0xffffffffu, far_y)) round_side(std::true_type{});
+        else round_side(std::false_type{});
+        if (__any_sync(0xffffffffu, left != 0u)) {
+          u128 g[4];  // formed anew when several outputs' sums would have to be kept
+          if constexpr (kSide > 1) combine_any(tb, g);
+#pragma unroll
+          for (int y = y0; y < y0 + kSide && y < ny; ++y) {
+            if constexpr (kSide == 1) g[y] = h[y];
+            if (left >> y & 1u)
+              o[y - y0] = round_general(UPDATE, UPDATE ? 0.0 : Yin[(size_t)(j0 + y) * ldyin + grow],
+                                        (i128)(g[y] - kOffset), Sr + Bexp[j0 + y]);
+          }
+        }
+#pragma unroll
+        for (int y = y0; y < y0 + kSide && y < ny; ++y)
+          if (grow < n && j0 + y < kout) Op[(size_t)y * ldo] = o[y - y0];
+      }
+    };
+    auto epilogue_block = [&](int64_t T, int64_t i, int ob) {
+      switch (min((kout - ob * kOut + 3) >> 2, 4)) {
+        case 1: epilogue_ny(std::integral_constant<int, 1>{}, T, i, ob); break;
+        case 2: epilogue_ny(std::integral_constant<int, 2>{}, T, i, ob); break;
+        case 3: epilogue_ny(std::integral_constant<int, 3>{}, T, i, ob); break;
+        default: epilogue_ny(std::integral_constant<int, 4>{}, T, i, ob); break;
       }
     };
 
     // this thread's W values of row r of tile T (zero beyond the matrix)
     auto load_direct = [&](int64_t T, double (&v)[W]) {
       const int64_t gr = T * kRows + r;
+      const int in = gr < n ? nv : 0;
+      const double* src = A + (size_t)c0 * lda + gr;
 #pragma unroll
-      for (int k = 0; k < W; ++k) {
-        const int col = c0 + k;
-        v[k] = (T < ntiles && gr < n && col < kin) ? A[(size_t)col * lda + gr] : 0.0;
-      }
+      for (int k = 0; k < W; ++k) v[k] = k < in ? src[(size_t)k * lda] : 0.0;
     };
     double v[W];  // the values of the tile to come
     // takes the staged values of the tile that prefetch was last called for
@@ -521,8 +604,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     int64_t Tprev = -1, iprev = 0;
     for (int64_t T = blockIdx.x, i = 0; T < ntiles; T += gridDim.x, ++i) {
       if (cg == 0) {
-        Arow[(i & 1) * kRows + r] = Ar;
-        Rbad[(i & 1) * kRows + r] = nonfinite;
+        Arow[(i & 1) * kRows + r] = Ar + (nonfinite ? kNaNExp : 0);
       }
       if (all && tid == 0) *reinterpret_cast<volatile int*>(&far[i & 1]) = (int)i;
       const int ng = all ? kGroupsAll : kGroupsNear;
@@ -567,7 +649,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
       // the next tile's values: in flight during the epilogue
       if constexpr (!kStageValues<W>) load_direct(T + gridDim.x, v);
-      if (!update && tid < 8 * kout) {  // Y of this tile, read by its epilogue a tile from now: into L2
+      if (!UPDATE && tid < 8 * kout) {  // Y of this tile, read by its epilogue a tile from now: into L2
         const int64_t g0 = T * kRows + (tid & 7) * 16;  // 16 rows = one 128-byte line per thread
         if (g0 < n) prefetch_l2(Yin + (size_t)(tid >> 3) * ldyin + g0);
       }
@@ -620,23 +702,36 @@ template <int W, int KO>
 size_t smem_bytes() {
   constexpr int KP = 4 * W;
   const size_t sbo = 16u * KP;
-  const size_t b = KO * 2 * kAll * sbo, a = 2 * kGroup * 16 * sbo, small = (4 * kRows + 2 * kOut * KO) * sizeof(int);
+  const size_t b = KO * 2 * kAll * sbo, a = 2 * kGroup * 16 * sbo, small = (2 * kRows + kOut * KO) * sizeof(int);
   const size_t stage = kStageValues<W> ? (size_t)W * kConvThreads * sizeof(double) : 0;
   return std::max(b + a + small + stage, kMinSmem);
 }
 
-template <int W, int KO = 1>
-cudaError_t launch_w(bool update, int64_t n, int kin, const double* A, int64_t lda, int kout, const double* Bh,
-                     const double* Bl, int ldb, bool tri, const double* Yin, int64_t ldyin, double* Out, int64_t ldo,
-                     const int* gate, cudaStream_t st, int ctas) {
+template <bool UPDATE, int W, int KO>
+cudaError_t launch_w(int64_t n, int kin, const double* A, int64_t lda, int kout, const double* Bh, const double* Bl,
+                     int ldb, bool tri, const double* Yin, int64_t ldyin, double* Out, int64_t ldo, const int* gate,
+                     cudaStream_t st, int ctas) {
   const size_t smem = smem_bytes<W, KO>();
-  cudaError_t e = set_dyn_smem(umma_rowprod_kernel<W, KO>, smem);
+  cudaError_t e = set_dyn_smem(umma_rowprod_kernel<UPDATE, W, KO>, smem);
   if (e != cudaSuccess) return e;
   const int64_t ntiles = (n + kRows - 1) / kRows;
   const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(ntiles, ctas > 0 ? ctas : 152));
-  umma_rowprod_kernel<W, KO><<<grid, kThreads, smem, st>>>(update ? 1 : 0, n, kin, A, lda, kout, Bh, Bl, ldb,
-                                                                tri ? 1 : 0, Yin, ldyin, Out, ldo, gate);
+  umma_rowprod_kernel<UPDATE, W, KO><<<grid, kThreads, smem, st>>>(n, kin, A, lda, kout, Bh, Bl, ldb, tri ? 1 : 0, Yin,
+                                                                   ldyin, Out, ldo, gate);
   return cudaGetLastError();
+}
+
+template <bool UPDATE>
+cudaError_t launch_mode(int64_t n, int kin, const double* A, int64_t lda, int kout, const double* Bh, const double* Bl,
+                        int ldb, bool tri, const double* Yin, int64_t ldyin, double* Out, int64_t ldo, const int* gate,
+                        cudaStream_t st, int ctas) {
+  if (kout > kOut)  // two blocks of output columns (kin <= 32): the inputs converted once
+    return launch_w<UPDATE, 8, 2>(n, kin, A, lda, kout, Bh, Bl, ldb, tri, Yin, ldyin, Out, ldo, gate, st, ctas);
+  if (kin <= 16)
+    return launch_w<UPDATE, 4, 1>(n, kin, A, lda, kout, Bh, Bl, ldb, tri, Yin, ldyin, Out, ldo, gate, st, ctas);
+  if (kin <= 32)
+    return launch_w<UPDATE, 8, 1>(n, kin, A, lda, kout, Bh, Bl, ldb, tri, Yin, ldyin, Out, ldo, gate, st, ctas);
+  return launch_w<UPDATE, 16, 1>(n, kin, A, lda, kout, Bh, Bl, ldb, tri, Yin, ldyin, Out, ldo, gate, st, ctas);
 }
 
 }  // namespace
@@ -649,9 +744,8 @@ bool umma_rowprod_supported(int kin, int kout) {
   if (kin < 1 || kin > 64 || kout < 1 || kout > 2 * kOut || (kout > kOut && kin > 32)) return false;
   // Small products run faster on the integer limbs: a tile's fixed cost
   // (its digit slabs, 16 padded outputs) dominates below kin max(kout, 4) =
-  // 128 (measured on 4e6 rows: kin = kout = 4 0.27 vs 0.59 ms, kin = 10,
-  // kout = 4 0.62 vs 0.60 ms; 16 x 8 1.31 vs 0.68, 16 x 16 2.32 vs 0.91 ms the
-  // other way).  EO_DD_ROW_ENGINE=umma keeps the tensor cores.
+  // 128 (measured on 4e6 rows: kin = kout = 4 0.27 vs 0.43 ms, 16 x 8 1.31 vs
+  // 0.50, 16 x 16 2.32 vs 0.65 ms the other way).  EO_DD_ROW_ENGINE=umma keeps the tensor cores.
   if (!(e && e[0] == 'u') && kin * std::max(kout, 4) < 128) return false;
   return true;
 }
@@ -661,13 +755,8 @@ cudaError_t launch_umma_rowprod(bool update, int64_t n, int kin, const double* A
                                 int64_t ldyin, double* Out, int64_t ldo, const int* gate, cudaStream_t st,
                                 int ctas) {
   if (n <= 0) return cudaSuccess;
-  if (kout > kOut)  // two blocks of output columns (kin <= 32): the inputs converted once
-    return launch_w<8, 2>(update, n, kin, A, lda, kout, Bh, Bl, ldb, tri, Yin, ldyin, Out, ldo, gate, st, ctas);
-  if (kin <= 16)
-    return launch_w<4>(update, n, kin, A, lda, kout, Bh, Bl, ldb, tri, Yin, ldyin, Out, ldo, gate, st, ctas);
-  if (kin <= 32)
-    return launch_w<8>(update, n, kin, A, lda, kout, Bh, Bl, ldb, tri, Yin, ldyin, Out, ldo, gate, st, ctas);
-  return launch_w<16>(update, n, kin, A, lda, kout, Bh, Bl, ldb, tri, Yin, ldyin, Out, ldo, gate, st, ctas);
+  return update ? launch_mode<true>(n, kin, A, lda, kout, Bh, Bl, ldb, tri, Yin, ldyin, Out, ldo, gate, st, ctas)
+                : launch_mode<false>(n, kin, A, lda, kout, Bh, Bl, ldb, tri, Yin, ldyin, Out, ldo, gate, st, ctas);
 }
 
 }  // namespace eo

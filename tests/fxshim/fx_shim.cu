@@ -49,6 +49,27 @@ double fxs_w_to_double(long long wlo, long long whi, int S) { return w_to_double
 
 double fxs_sub_round(double y, long long wlo, long long whi, int S) { return sub_round(y, mk(wlo, whi), S); }
 
+double fxs_w_to_double_lean(long long wlo, long long whi, int S, int flip, int* ok) {
+  bool o = false;
+  const double r = w_to_double_lean((u128)mk(wlo, whi), S, flip ? 0x80000000u : 0u, o);
+  *ok = o;
+  return r;
+}
+
+double fxs_sub_round_lean(double y, long long wlo, long long whi, long long klo, long long khi, int S, int* ok) {
+  bool o = false;
+  const u128 K = (u128)mk(klo, khi);
+  const u128 raw = (u128)mk(wlo, whi) + K;
+  const double r = dominates(y, S) ? sub_round_lean<true>(y, raw, K, S, o) : sub_round_lean<false>(y, raw, K, S, o);
+  if (!dominates(y, S)) {  // the wider form takes the others as well
+    bool o2 = false;
+    const double r2 = sub_round_lean<true>(y, raw, K, S, o2);
+    if (o2 != o || (o && memcmp(&r, &r2, 8) != 0)) return r + 1;
+  }
+  *ok = o;
+  return r;
+}
+
 double fxs_w_to_double_fast(long long wlo, long long whi, int S, int* ok) {
   bool o = false;
   const double r = w_to_double_fast(mk(wlo, whi), S, o);
