@@ -447,6 +447,40 @@ FX_HD double w_to_double_lean(u128 r, int S, unsigned flip, bool& ok) {
   return from_bits(bits ^ ((unsigned long long)((neg ^ flip) & 0x80000000u) << 32));
 }
 
+// r 2^S rounded to FP32, the same way.
+FX_HD float w_to_float_lean(u128 r, int S, bool& ok) {
+  const unsigned neg = (unsigned)((int)word(r, 3) >> 31);
+  const unsigned u3 = word(r, 3) ^ neg, u2 = word(r, 2) ^ neg, u1 = word(r, 1) ^ neg, u0 = word(r, 0) ^ neg;
+  const bool top = u3 != 0u;
+  const unsigned a = top ? u3 : u2, b = top ? u2 : u1, c = top ? u1 : u0;
+  const int lz = clz32(a);
+  const unsigned t2 = funnel_l(b, a, lz), t1 = funnel_l(c, b, lz);
+  const int be1 = S + (top ? 253 : 221) - lz;  // biased exponent - 1
+  ok = a != 0u && (unsigned)be1 < 253u && t1 + 64u >= 128u;
+  const unsigned bits = ((t2 >> 8) + ((t2 >> 7) & 1u) + ((unsigned)be1 << 23)) | (neg & 0x80000000u);
+  float f;
+#ifdef __CUDA_ARCH__
+  f = __uint_as_float(bits);
+#else
+  memcpy(&f, &bits, 4);
+#endif
+  return f;
+}
+
+// x widened without the FP64 pipe (finite, zero and non-finite values alike).
+FX_HD double widen(float x) {
+  unsigned u;
+#ifdef __CUDA_ARCH__
+  u = __float_as_uint(x);
+#else
+  memcpy(&u, &x, 4);
+#endif
+  const unsigned m = u & 0x7fffffffu;
+  if (m - 0x00800000u >= 0x7f000000u && m != 0u) return (double)x;  // subnormal, Inf, NaN
+  const unsigned hi = (u & 0x80000000u) | (m ? (m >> 3) + (896u << 20) : 0u);
+  return from_bits(((unsigned long long)hi << 32) | (m << 29));
+}
+
 // Does y dominate the grid 2^S by more than 2^72 of its units in its last place?
 FX_HD bool dominates(double y, int S) { return (int)((hi32(y) >> 20) & 0x7ffu) - 1075 - S > 72; }
 

@@ -299,25 +299,25 @@ __global__ void copy_cols_kernel(int64_t n, int cols, const double* __restrict__
 }
 
 size_t fx_update_tmp_bytes(int64_t n, int k) {
-  if (k <= 16 || umma_rowprod_supported(k, k) || !umma_rowprod_supported(k, 16)) return 0;
+  if (k <= 16 || umma_rowprod_supported(n, k, k) || !umma_rowprod_supported(n, k, 16)) return 0;
   return (size_t)n * 16 * ((k + 15) / 16 - 1) * sizeof(double);
 }
 
 int fx_update_launches(int64_t n, int k, size_t tmp_bytes) {
-  if (umma_rowprod_supported(k, k)) return n > 0 ? 1 : 0;
+  if (umma_rowprod_supported(n, k, k)) return n > 0 ? 1 : 0;
   const size_t need = fx_update_tmp_bytes(n, k);
   if (n > 0 && need > 0 && tmp_bytes >= need) return (k + 15) / 16 + 1;
   return 1;
 }
 
 int fx_project_launches(int64_t n, int kv, int k) {
-  if (umma_rowprod_supported(kv, k)) return n > 0 ? 1 : 0;
-  if (umma_rowprod_supported(kv, 16)) return n > 0 ? (k + 15) / 16 : 0;
+  if (umma_rowprod_supported(n, kv, k)) return n > 0 ? 1 : 0;
+  if (k > 16 && umma_rowprod_supported(n, kv, 16)) return n > 0 ? (k + 15) / 16 : 0;
   return 1;
 }
 
 int fx_update_ctas(int64_t n, int k, int ctas) {
-  if (umma_rowprod_supported(k, k) || fx_update_tmp_bytes(n, k) > 0) {
+  if (umma_rowprod_supported(n, k, k) || fx_update_tmp_bytes(n, k) > 0) {
     const int64_t ntiles = (n + 127) / 128;  // 128-row tiles of the tensor-core engine
     return (int)std::max<int64_t>(1, std::min<int64_t>(ntiles, ctas > 0 ? ctas : 152));
   }
@@ -327,7 +327,7 @@ int fx_update_ctas(int64_t n, int k, int ctas) {
 
 cudaError_t launch_fx_update(int64_t n, int k, double* X, int64_t ldx, const double* Zh, const double* Zl, bool tri,
                              const int* gate, cudaStream_t st, int ctas, void* tmp, size_t tmp_bytes) {
-  if (umma_rowprod_supported(k, k))
+  if (umma_rowprod_supported(n, k, k))
     return launch_umma_rowprod(true, n, k, X, ldx, k, Zh, Zl, KMAX, tri, nullptr, 0, X, ldx, gate, st, ctas);
   const size_t need = fx_update_tmp_bytes(n, k);
   if (n > 0 && need > 0 && tmp && tmp_bytes >= need) {
@@ -357,9 +357,9 @@ cudaError_t launch_fx_update(int64_t n, int k, double* X, int64_t ldx, const dou
 cudaError_t launch_fx_project(int64_t n, int kv, const double* V, int64_t ldv, int k, const double* Y, int64_t ldy,
                               double* Yout, int64_t ldyo, const double* C_hi, const double* C_lo, int ldc,
                               const int* gate, cudaStream_t st) {
-  if (umma_rowprod_supported(kv, k))
+  if (umma_rowprod_supported(n, kv, k))
     return launch_umma_rowprod(false, n, kv, V, ldv, k, C_hi, C_lo, ldc, false, Y, ldy, Yout, ldyo, gate, st);
-  if (umma_rowprod_supported(kv, 16)) {
+  if (k > 16 && umma_rowprod_supported(n, kv, 16)) {
     // groups of 16 columns: each reads V and its own columns of Y and writes
     // the same columns of Yout, so groups never disturb one another (in place too)
     for (int c0 = 0; c0 < k; c0 += 16) {

@@ -54,6 +54,11 @@
 //   64 x 16 1.645 -> 1.507 -> 1.224 ms, 32 x 32 2.135 -> 1.933 -> 1.396,
 //   32 x 16 1.230 -> 1.090 -> 0.829, 16 x 16 1.017 -> 0.907 -> 0.651,
 //   20 x 4 0.969 -> 0.811 -> 0.601, 8 x 8 0.774 -> 0.687 -> 0.500.
+// A launch's fixed part is about 8 us (64 x 16 on 1e4 rows: 14.4).
+//
+// FP32 updates (kin <= 32) take the same path with seven near slabs (24 bits
+// and the near window); their outputs are rounded from the exact sum to FP32.
+// 2e6 x 32: 4.0 ms on the FP64 pipe -> 0.57 ms.
 #include <cuda_fp16.h>
 
 #include <algorithm>
@@ -77,6 +82,9 @@ constexpr int kRows = 128;                   // rows per tile (MMA M, TMEM lanes
 constexpr int kOut = 16;                     // output columns of the MMA (padded)
 constexpr int kGroup = 5;                    // digit slabs per group
 constexpr int kGroupsNear = 2, kGroupsAll = 3;
+// Slabs of a near tile: FP32 values have 24 bits, with the near window 49 of the 110.
+template <typename Real>
+constexpr int kNearOf = std::is_same_v<Real, float> ? 7 : kNear;
 constexpr int kScaleProd = 2160;             // value of h: h 2^(A_r + B_j - 2160)
 constexpr unsigned kAccCols = 256;           // TMEM columns per accumulator (224 used)
 constexpr size_t kMinSmem = 120 * 1024;      // keeps one CTA per SM (TMEM: 512 columns)
@@ -195,12 +203,12 @@ __device__ __forceinline__ void near_lanes(const double (&v)[W], int A, unsigned
     z[m][4] = __byte_perm(a1, b1, 0x5410);
   }
 }
-// Group G (slabs 5 G .. 5 G + 4) of near values.
-template <int G, int W>
+// Group G of near values: N slabs from 5 G on.
+template <int G, int N, int W>
 __device__ __forceinline__ void store_near(unsigned dst, unsigned slab_bytes, const unsigned (&z)[W / 2][5],
                                            const unsigned (&sg)[W / 2], unsigned e1024) {
 #pragma unroll
-  for (int j = 0; j < kGroup; ++j) {
+  for (int j = 0; j < N; ++j) {
     const int s = G * kGroup + j;
     unsigned w[W / 2];
 #pragma unroll
@@ -274,11 +282,11 @@ __device__ __noinline__ double round_general(bool update, double y, i128 h, int 
 // accumulators, release them (tfree) and then store group 2, and the MMAs of
 // tile i wait for that release, so the inputs are converted once for all 32
 // outputs.
-template <bool UPDATE, int W, int KO = 1>
+template <typename Real, bool UPDATE, int W, int KO>
 __global__ void __launch_bounds__(kThreads, 1)
-    umma_rowprod_kernel(int64_t n, int kin, const double* A, int64_t lda, int kout,
+    umma_rowprod_kernel(int64_t n, int kin, const Real* A, int64_t lda, int kout,
                         const double* __restrict__ Bh, const double* __restrict__ Bl, int ldb, int tri,
-                        const double* Yin, int64_t ldyin, double* Out, int64_t ldo, const int* gate) {
+                        const Real* Yin, int64_t ldyin, Real* Out, int64_t ldo, const int* gate) {
   if (gate && *gate == 0) return;
   constexpr int KP = 4 * W;
   constexpr int KC = KP / 16;             // MMAs (K = 16) per slab
@@ -287,13 +295,15 @@ __global__ void __launch_bounds__(kThreads, 1)
   constexpr unsigned B_BYTES = 2u * kAll * SBO;  // 14 slabs x 16 columns (one block of outputs)
   constexpr int NOUT = kOut * KO;
   static_assert(KO == 1 || (KO == 2 && W <= 8), "two output blocks only for kin <= 32");
+  static_assert(std::is_same_v<Real, double> || (UPDATE && kStageValues<W>), "FP32: the update for kin <= 32");
+  constexpr int NEAR = kNearOf<Real>;
 
   extern __shared__ __align__(128) unsigned char smem[];
   unsigned char* bdig = smem;                                  // the small matrix's digits
   unsigned char* adig = smem + KO * B_BYTES;                   // two group buffers of 5 slabs
   int* Arow = reinterpret_cast<int*>(adig + 2 * kGroup * SLAB_A);  // [2][128] row exponents
   int* Bexp = Arow + 2 * kRows;                                // [NOUT] column exponents
-  double* stg = reinterpret_cast<double*>(Bexp + NOUT);        // [W][512] staged values (kin <= 32)
+  Real* stg = reinterpret_cast<Real*>(Bexp + NOUT);            // [W][512] staged values (kin <= 32)
   __shared__ __align__(8) unsigned long long full_bar[2], ready_bar[2], tfree_bar;
   __shared__ unsigned tmem_base;
   __shared__ int bad;
@@ -314,18 +324,23 @@ __global__ void __launch_bounds__(kThreads, 1)
     bad = 0;
     far[0] = far[1] = -1;
   }
-  if (tid < NOUT) {
-    const int j = tid;
-    int e = 0, nf = 0;
+  // column exponents, a warp to a column (one round of loads: a thread to a
+  // column, one load after another, made a launch of 64 x 16 10 us longer)
+  for (int j = warp; j < NOUT; j += kThreads / 32) {
+    int e = 0;
+    bool nf = false;
     if (j < kout) {
-      for (int i = 0; i < kin; ++i) {
+      for (int i = lane; i < kin; i += 32) {
         if (tri && i > j) continue;
         const int ae = align_exp(Bh[(size_t)j * ldb + i]);
         e = max(e, ae);
-        if (ae == 2047 || (Bl && align_exp(Bl[(size_t)j * ldb + i]) == 2047)) nf = 1;
+        nf |= ae == 2047 || (Bl && align_exp(Bl[(size_t)j * ldb + i]) == 2047);
       }
     }
-    Bexp[j] = e + 1 + (nf ? kNaNExp : 0);  // one binade of headroom: |h + l| may round up past the largest h
+    e = (int)__reduce_max_sync(0xffffffffu, (unsigned)e);
+    nf = __any_sync(0xffffffffu, nf);
+    // one binade of headroom: |h + l| may round up past the largest h
+    if (lane == 0) Bexp[j] = e + 1 + (nf ? kNaNExp : 0);
   }
   __syncthreads();
   for (int e = tid; e < NOUT * KP; e += kThreads) {  // block j / 16: B row R = t * 16 + j % 16 (slab t), K index i
@@ -365,7 +380,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             tc_fence_after();
           }
         }
-        int ng = kGroupsNear;
+        int ng = kGroupsNear, nslabs = NEAR;
 #pragma unroll 1
         for (int g = 0; g < ng; ++g, ++G) {
           const int b = G & 1;
@@ -373,10 +388,10 @@ __global__ void __launch_bounds__(kThreads, 1)
             ok = false;
             break;
           }
-          if (g == 0 && *reinterpret_cast<volatile int*>(&far[i & 1]) == (int)i) ng = kGroupsAll;
+          if (g == 0 && *reinterpret_cast<volatile int*>(&far[i & 1]) == (int)i) ng = kGroupsAll, nslabs = kAll;
           tc_fence_after();
           const unsigned abuf = adig_s + (unsigned)b * kGroup * SLAB_A;
-          const int ns = min(kGroup, kAll - g * kGroup);
+          const int ns = min(kGroup, nslabs - g * kGroup);
           for (int sg = 0; sg < ns; ++sg) {
             const int s = g * kGroup + sg;
             const unsigned idesc = idesc_f16(kRows, kOut * (kAll - s));
@@ -414,14 +429,16 @@ __global__ void __launch_bounds__(kThreads, 1)
     // the values of tile T into this thread's staging slots (zeros beyond the
     // matrix: nothing is read there)
     const int nv = min(max(kin - c0, 0), W);  // columns of this thread
-    const unsigned stg_s = smem_u32(stg) + (unsigned)(tid * 8);
+    const unsigned stg_s = smem_u32(stg) + (unsigned)(tid * sizeof(Real));
     auto prefetch = [&](int64_t T) {
       const int64_t gr = T * kRows + r;
       const int in = gr < n ? nv : 0;  // (T >= ntiles: gr >= n)
-      const double* src = A + (in > 0 ? (size_t)c0 * lda + gr : 0);
+      const Real* src = A + (in > 0 ? (size_t)c0 * lda + gr : 0);
 #pragma unroll
       for (int k = 0; k < W; ++k) {
-        cp_async8z(stg_s + (unsigned)(k * kConvThreads * 8), src, k < in ? 8u : 0u);
+        const unsigned dst = stg_s + (unsigned)(k * kConvThreads * sizeof(Real));
+        if constexpr (sizeof(Real) == 8) cp_async8z(dst, src, k < in ? 8u : 0u);
+        else cp_async4z(dst, src, k < in ? 4u : 0u);
         if (k + 1 < in) src += lda;
       }
       cp_async_commit_group();
@@ -437,7 +454,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       const int64_t grow = T * kRows + L;
       double yv[ny];
       {
-        const double* Yp = Yin + (size_t)j0 * ldyin + grow;
+        const Real* Yp = Yin + (size_t)j0 * ldyin + grow;
 #pragma unroll
         for (int y = 0; y < ny; ++y)
           yv[y] = (!UPDATE && j0 + y < kout && grow < n) ? Yp[(size_t)y * ldyin] : 0.0;
@@ -493,21 +510,22 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
       }
       const int Sr = Arow[(i & 1) * kRows + L] - kScaleProd + (bad ? kNaNExp : 0);
-      double* Op = Out + (size_t)j0 * ldo + grow;
+      Real* Op = Out + (size_t)j0 * ldo + grow;
       // the roundings of kSide outputs side by side (no branches among them);
       // what they do not take is rounded by the general functions
       constexpr int kSide = kRoundSide<W> < ny ? kRoundSide<W> : ny;
 #pragma unroll
       for (int y0 = 0; y0 < ny; y0 += kSide) {
-        double o[kSide];
+        Real o[kSide];
         unsigned left = 0;
         auto round_side = [&](auto FAR) {
 #pragma unroll
           for (int y = y0; y < y0 + kSide && y < ny; ++y) {
             const int S = Sr + Bexp[j0 + y];
             bool ok;
-            o[y - y0] = UPDATE ? w_to_double_lean(h[y] - kOffset, S, 0u, ok)
-                               : sub_round_lean<decltype(FAR)::value>(yv[y], h[y], kOffset, S, ok);
+            if constexpr (!UPDATE) o[y - y0] = sub_round_lean<decltype(FAR)::value>(yv[y], h[y], kOffset, S, ok);
+            else if constexpr (sizeof(Real) == 8) o[y - y0] = w_to_double_lean(h[y] - kOffset, S, 0u, ok);
+            else o[y - y0] = w_to_float_lean(h[y] - kOffset, S, ok);
             left |= ok || j0 + y >= kout || grow >= n ? 0u : 1u << y;
           }
         };
@@ -525,7 +543,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           for (int y = y0; y < y0 + kSide && y < ny; ++y) {
             if constexpr (kSide == 1) g[y] = h[y];
             if (left >> y & 1u)
-              o[y - y0] = round_general(UPDATE, UPDATE ? 0.0 : Yin[(size_t)(j0 + y) * ldyin + grow],
+              o[y - y0] = (Real)round_general(UPDATE, UPDATE ? 0.0 : Yin[(size_t)(j0 + y) * ldyin + grow],
                                         (i128)(g[y] - kOffset), Sr + Bexp[j0 + y]);
           }
         }
@@ -547,7 +565,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     auto load_direct = [&](int64_t T, double (&v)[W]) {
       const int64_t gr = T * kRows + r;
       const int in = gr < n ? nv : 0;
-      const double* src = A + (size_t)c0 * lda + gr;
+      const Real* src = A + (size_t)c0 * lda + gr;
 #pragma unroll
       for (int k = 0; k < W; ++k) v[k] = k < in ? src[(size_t)k * lda] : 0.0;
     };
@@ -556,7 +574,10 @@ __global__ void __launch_bounds__(kThreads, 1)
     auto take = [&]() {
       asm volatile("cp.async.wait_all;" ::: "memory");
 #pragma unroll
-      for (int k = 0; k < W; ++k) v[k] = stg[k * kConvThreads + tid];
+      for (int k = 0; k < W; ++k) {
+        if constexpr (sizeof(Real) == 8) v[k] = stg[k * kConvThreads + tid];
+        else v[k] = widen(stg[k * kConvThreads + tid]);
+      }
     };
     // The row's exponent: max of the |x| high words over the four threads of
     // the row (a row of subnormals and zeros has exponent field 0 and is aligned
@@ -638,8 +659,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         ++G;
       };
       if (!all) {
-        group(0, [&](unsigned dst) { store_near<0, W>(dst, SLAB_A, z, sg, e1024); });
-        group(1, [&](unsigned dst) { store_near<1, W>(dst, SLAB_A, z, sg, e1024); });
+        group(0, [&](unsigned dst) { store_near<0, kGroup, W>(dst, SLAB_A, z, sg, e1024); });
+        group(1, [&](unsigned dst) { store_near<1, NEAR - kGroup, W>(dst, SLAB_A, z, sg, e1024); });
       } else {
         double u[W];
 #pragma unroll
@@ -707,17 +728,17 @@ size_t smem_bytes() {
   return std::max(b + a + small + stage, kMinSmem);
 }
 
-template <bool UPDATE, int W, int KO>
-cudaError_t launch_w(int64_t n, int kin, const double* A, int64_t lda, int kout, const double* Bh, const double* Bl,
-                     int ldb, bool tri, const double* Yin, int64_t ldyin, double* Out, int64_t ldo, const int* gate,
+template <typename Real, bool UPDATE, int W, int KO>
+cudaError_t launch_w(int64_t n, int kin, const Real* A, int64_t lda, int kout, const double* Bh, const double* Bl,
+                     int ldb, bool tri, const Real* Yin, int64_t ldyin, Real* Out, int64_t ldo, const int* gate,
                      cudaStream_t st, int ctas) {
   const size_t smem = smem_bytes<W, KO>();
-  cudaError_t e = set_dyn_smem(umma_rowprod_kernel<UPDATE, W, KO>, smem);
+  cudaError_t e = set_dyn_smem(umma_rowprod_kernel<Real, UPDATE, W, KO>, smem);
   if (e != cudaSuccess) return e;
   const int64_t ntiles = (n + kRows - 1) / kRows;
   const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(ntiles, ctas > 0 ? ctas : 152));
-  umma_rowprod_kernel<UPDATE, W, KO><<<grid, kThreads, smem, st>>>(n, kin, A, lda, kout, Bh, Bl, ldb, tri ? 1 : 0, Yin,
-                                                                   ldyin, Out, ldo, gate);
+  umma_rowprod_kernel<Real, UPDATE, W, KO><<<grid, kThreads, smem, st>>>(n, kin, A, lda, kout, Bh, Bl, ldb, tri ? 1 : 0,
+                                                                      Yin, ldyin, Out, ldo, gate);
   return cudaGetLastError();
 }
 
@@ -726,28 +747,32 @@ cudaError_t launch_mode(int64_t n, int kin, const double* A, int64_t lda, int ko
                         int ldb, bool tri, const double* Yin, int64_t ldyin, double* Out, int64_t ldo, const int* gate,
                         cudaStream_t st, int ctas) {
   if (kout > kOut)  // two blocks of output columns (kin <= 32): the inputs converted once
-    return launch_w<UPDATE, 8, 2>(n, kin, A, lda, kout, Bh, Bl, ldb, tri, Yin, ldyin, Out, ldo, gate, st, ctas);
+    return launch_w<double, UPDATE, 8, 2>(n, kin, A, lda, kout, Bh, Bl, ldb, tri, Yin, ldyin, Out, ldo, gate, st, ctas);
   if (kin <= 16)
-    return launch_w<UPDATE, 4, 1>(n, kin, A, lda, kout, Bh, Bl, ldb, tri, Yin, ldyin, Out, ldo, gate, st, ctas);
+    return launch_w<double, UPDATE, 4, 1>(n, kin, A, lda, kout, Bh, Bl, ldb, tri, Yin, ldyin, Out, ldo, gate, st, ctas);
   if (kin <= 32)
-    return launch_w<UPDATE, 8, 1>(n, kin, A, lda, kout, Bh, Bl, ldb, tri, Yin, ldyin, Out, ldo, gate, st, ctas);
-  return launch_w<UPDATE, 16, 1>(n, kin, A, lda, kout, Bh, Bl, ldb, tri, Yin, ldyin, Out, ldo, gate, st, ctas);
+    return launch_w<double, UPDATE, 8, 1>(n, kin, A, lda, kout, Bh, Bl, ldb, tri, Yin, ldyin, Out, ldo, gate, st, ctas);
+  return launch_w<double, UPDATE, 16, 1>(n, kin, A, lda, kout, Bh, Bl, ldb, tri, Yin, ldyin, Out, ldo, gate, st, ctas);
 }
 
 }  // namespace
 
 cudaError_t umma_rowprod_take_wait_record(unsigned* out) { return take_wait_record(out); }
 
-bool umma_rowprod_supported(int kin, int kout) {
+bool umma_rowprod_supported(int64_t n, int kin, int kout) {
   const char* e = getenv("EO_DD_ROW_ENGINE");
   if (e && e[0] == 'i') return false;
   if (kin < 1 || kin > 64 || kout < 1 || kout > 2 * kOut || (kout > kOut && kin > 32)) return false;
-  // Small products run faster on the integer limbs: a tile's fixed cost
-  // (its digit slabs, 16 padded outputs) dominates below kin max(kout, 4) =
-  // 128 (measured on 4e6 rows: kin = kout = 4 0.27 vs 0.43 ms, 16 x 8 1.31 vs
-  // 0.50, 16 x 16 2.32 vs 0.65 ms the other way).  EO_DD_ROW_ENGINE=umma keeps the tensor cores.
-  if (!(e && e[0] == 'u') && kin * std::max(kout, 4) < 128) return false;
-  return true;
+  if (e && e[0] == 'u') return true;  // (for comparisons: the tensor cores wherever they can run)
+  // Small products run faster on the integer limbs, whose cost follows
+  // kin kout, while a tile here costs its digits and at least one output for
+  // every warp.  Measured, integer limbs vs tiles: on 1e6 rows 4 x 4 68 vs
+  // 111 us, 8 x 4 105 vs 120, 10 x 4 163 vs 121, 8 x 8 205 vs 139, 16 x 8 336
+  // vs 139, 16 x 16 587 vs 177.  Rows of up to 8 entries stay in the
+  // registers of a thread there, which starts quicker: 8 x 8 on 1e4 rows 8.3
+  // vs 10.3 us, equal on 2e4, on 4e4 16.5 vs 14.4 (16 x 4, 2e3 rows: 12.4 vs 10.3).
+  const int entries = kin * std::max(kout, 4);
+  return entries >= 128 || (entries >= 40 && (kin > 8 || n >= 32768));
 }
 
 cudaError_t launch_umma_rowprod(bool update, int64_t n, int kin, const double* A, int64_t lda, int kout,
@@ -757,6 +782,14 @@ cudaError_t launch_umma_rowprod(bool update, int64_t n, int kin, const double* A
   if (n <= 0) return cudaSuccess;
   return update ? launch_mode<true>(n, kin, A, lda, kout, Bh, Bl, ldb, tri, Yin, ldyin, Out, ldo, gate, st, ctas)
                 : launch_mode<false>(n, kin, A, lda, kout, Bh, Bl, ldb, tri, Yin, ldyin, Out, ldo, gate, st, ctas);
+}
+
+cudaError_t launch_umma_update_f32(int64_t n, int k, float* X, int64_t ldx, const double* Zh, const double* Zl, int ldz,
+                                   bool tri, const int* gate, cudaStream_t st) {
+  if (n <= 0) return cudaSuccess;
+  const float* none = nullptr;
+  if (k > kOut) return launch_w<float, true, 8, 2>(n, k, X, ldx, k, Zh, Zl, ldz, tri, none, 0, X, ldx, gate, st, 0);
+  return launch_w<float, true, 4, 1>(n, k, X, ldx, k, Zh, Zl, ldz, tri, none, 0, X, ldx, gate, st, 0);
 }
 
 }  // namespace eo

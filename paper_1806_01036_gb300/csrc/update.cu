@@ -15,6 +15,14 @@ namespace eo {
 namespace {
 
 constexpr int kThreads = 128;
+// FP32 blocks of 9 to 32 columns run on the tensor-core digits from 16384 rows
+// on: exact sums rounded once, where the loop below is bound by the FP64 pipe.
+// One CholQR pass with this kernel and with the digits, 2e6 rows: 8 columns
+// 632 vs 562 us, 9 1219 vs 815, 16 1398 vs 503, 32 5944 vs 1318; 20,000 rows:
+// 8 59 vs 57 us, 9 73 vs 67, 32 182 vs 168; below, the digits' start costs what
+// they save (1e4 rows, 16 columns: 73 vs 75).  (The digits' groups of more than
+// 32 columns would need scratch that the FP32 mode does not reserve.)
+bool f32_digits(int64_t n, int k) { return k >= 9 && k <= 32 && n >= 16384; }
 
 template <int MODE, typename T, int KM>
 __global__ void __launch_bounds__(kThreads) update_kernel(int64_t n, int k, T* X, int64_t ldx,
@@ -84,7 +92,10 @@ cudaError_t launch_update(Mode mode, int64_t n, int k, void* X, int64_t ldx, con
                           bool tri, const int* gate, cudaStream_t st) {
   switch (mode) {
     case MODE_DD: return launch_k<MODE_DD, double>(n, k, X, ldx, Zh, Zl, tri, gate, st);
-    case MODE_F32: return launch_k<MODE_F32, float>(n, k, X, ldx, Zh, Zl, tri, gate, st);
+    case MODE_F32:
+      if (f32_digits(n, k))
+        return launch_umma_update_f32(n, k, static_cast<float*>(X), ldx, Zh, Zl, KMAX, tri, gate, st);
+      return launch_k<MODE_F32, float>(n, k, X, ldx, Zh, Zl, tri, gate, st);
     default: return launch_k<MODE_FP64, double>(n, k, X, ldx, Zh, Zl, tri, gate, st);
   }
 }

@@ -56,6 +56,15 @@ double fxs_w_to_double_lean(long long wlo, long long whi, int S, int flip, int* 
   return r;
 }
 
+float fxs_w_to_float_lean(long long wlo, long long whi, int S, int* ok) {
+  bool o = false;
+  const float r = w_to_float_lean((u128)mk(wlo, whi), S, o);
+  *ok = o;
+  return r;
+}
+
+double fxs_widen(float x) { return widen(x); }
+
 double fxs_sub_round_lean(double y, long long wlo, long long whi, long long klo, long long khi, int S, int* ok) {
   bool o = false;
   const u128 K = (u128)mk(klo, khi);

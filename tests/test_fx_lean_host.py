@@ -99,3 +99,35 @@ def test_lean_difference_rounding(fx):
                 must += 1
                 assert ok.value, (y, w, S)
     assert must > 3000
+
+
+def test_lean_single_rounding_and_widening(fx):
+    fx.fxs_w_to_float_lean.restype = C.c_float
+    fx.fxs_w_to_float_lean.argtypes = [C.c_longlong, C.c_longlong, C.c_int, C.c_void_p]
+    fx.fxs_widen.restype = C.c_double
+    fx.fxs_widen.argtypes = [C.c_float]
+    g = np.random.default_rng(33)
+    ok = C.c_int(0)
+    must = 0
+    for _ in range(20000):
+        w = rand_w(g)
+        S = int(g.integers(-240, 120))
+        got = np.float32(fx.fxs_w_to_float_lean(*split_w(w), S, C.byref(ok)))
+        exact = F(w) * F(2) ** S
+        if ok.value:
+            assert 2.0 ** -126 <= abs(got) < np.inf
+            err = abs(F(float(got)) - exact)
+            for side in (np.float32(np.inf), np.float32(-np.inf)):
+                other = np.nextafter(got, side)
+                if np.isfinite(other):
+                    assert err <= abs(F(float(other)) - exact), (w, S)
+        v = abs(w) << 128 >> max(abs(w).bit_length() + 128 - 64, 0)  # the 64 leading bits
+        if abs(w) >= 2 ** 64 and F(2) ** -125 <= abs(exact) < F(2) ** 126 and 1 << 12 < v % 2 ** 32 < 2 ** 32 - (1 << 12):
+            must += 1
+            assert ok.value, (w, S)
+    assert must > 4000
+    for x in (0.0, -0.0, 1.0, -1.5, 1e-45, -1e-40, 1.17549435e-38, 3.4028235e38, float("inf"), -float("inf")):
+        assert _bits(fx.fxs_widen(x)) == _bits(float(np.float32(x)))
+    assert np.isnan(fx.fxs_widen(float("nan")))
+    for x in g.standard_normal(500).astype(np.float32) * np.float32(2.0) ** g.integers(-60, 60, 500).astype(np.float32):
+        assert fx.fxs_widen(float(x)) == float(x)

@@ -71,3 +71,30 @@ def test_tiles_of_both_kinds(eo, ctx, monkeypatch, kind, kv, k):
         v[g.integers(0, n, 40)] = 0.0
         v[g.integers(0, n, 40), 0] = -0.0
     check(eo, ctx, monkeypatch, np.asfortranarray(v), k, 2400 + k)
+
+
+@pytest.mark.parametrize("n,k", [(16384, 9), (16383, 16), (20_011, 16), (20_011, 17), (152 * 128 + 1, 32), (20_000, 8),
+                                 (20_000, 33)])
+@pytest.mark.parametrize("spread", [0, 60])
+def test_f32_update(eo, ctx, n, k, spread):
+    """Q = X R^-1 of an FP32 block, on either side of the digit engine's sizes,
+    rows of widely different scale and a column far below the others (tiles
+    that need all digits) included.  Q is one FP32 rounding (2^-24 relative;
+    2^-23 allows for R^-1 formed here in FP64) of X R^-1, whose error is k 2^-48
+    of the row's and the column's largest values at most."""
+    import torch
+
+    g = synth.rng(2500 + k)
+    x = g.standard_normal((n, k))
+    if spread:
+        x *= np.ldexp(1.0, g.integers(-spread // 2, 1, n))[:, None]
+        x[:, k // 2] *= 2.0 ** -spread
+    x = x.astype(np.float32)
+    X = torch.from_numpy(np.ascontiguousarray(x.T)).cuda().t()
+    rh, rl, info = eo.cholqr(ctx, X, passes=1, prec=eo.F32)
+    assert int(info) == 0
+    z = np.linalg.inv((rh + rl).cpu().numpy())
+    want = x.astype(np.float64) @ z
+    err = np.abs(X.cpu().numpy().astype(np.float64) - want)
+    row_max = np.max(np.abs(x), axis=1)[:, None].astype(np.float64) * np.max(np.abs(z), axis=0)[None, :]
+    assert np.all(err <= 2.0 ** -23 * np.abs(want) + k * 2.0 ** -48 * row_max)
