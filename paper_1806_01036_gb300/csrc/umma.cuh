@@ -145,30 +145,9 @@ __device__ __forceinline__ void mma_commit(unsigned bar) {
                : "memory");
 }
 
-// Three column groups of NY consecutive TMEM columns (this warp's 32 lanes),
-// loaded and waited for in one step.
-template <int NY>
-__device__ __forceinline__ void tmem_ld3(unsigned a0, unsigned a1, unsigned a2, unsigned (&v)[3][NY]) {
-  if constexpr (NY == 4) {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%12];\n"
-        "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%4,%5,%6,%7}, [%13];\n"
-        "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%8,%9,%10,%11}, [%14];\n"
-        "tcgen05.wait::ld.sync.aligned;\n"
-        : "=r"(v[0][0]), "=r"(v[0][1]), "=r"(v[0][2]), "=r"(v[0][3]), "=r"(v[1][0]), "=r"(v[1][1]), "=r"(v[1][2]),
-          "=r"(v[1][3]), "=r"(v[2][0]), "=r"(v[2][1]), "=r"(v[2][2]), "=r"(v[2][3])
-        : "r"(a0), "r"(a1), "r"(a2)
-        : "memory");
-  } else {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x2.b32 {%0,%1}, [%6];\n"
-        "tcgen05.ld.sync.aligned.32x32b.x2.b32 {%2,%3}, [%7];\n"
-        "tcgen05.ld.sync.aligned.32x32b.x2.b32 {%4,%5}, [%8];\n"
-        "tcgen05.wait::ld.sync.aligned;\n"
-        : "=r"(v[0][0]), "=r"(v[0][1]), "=r"(v[1][0]), "=r"(v[1][1]), "=r"(v[2][0]), "=r"(v[2][1])
-        : "r"(a0), "r"(a1), "r"(a2)
-        : "memory");
-  }
+// One TMEM column of this warp's 32 lanes (the caller waits).
+__device__ __forceinline__ void tmem_ld1(unsigned a, unsigned& v) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(v) : "r"(a) : "memory");
 }
 
 __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }

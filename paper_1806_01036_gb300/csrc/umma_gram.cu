@@ -169,19 +169,9 @@ struct Plan : Geo<KXP_, KYP_, SHARED_> {
   static constexpr int pairs_near = group_pairs(B::J, kNear, B::NQN), pairs_all = group_pairs(B::J, kAll, B::NQA);
   static constexpr size_t smem = B::bytes(P) + 1024;
   static_assert(FK >= 1 && P * pairs_near <= kPairRows && 16 * FK * pairs_all <= kPairRows, "a step fits the accumulators");
-  static_assert(2 * (size_t)dig_bytes >= (SHARED_ ? 2u : 1u) * (size_t)kLanes * KYP_ * 16, "final sums fit the digit buffers");
+  static_assert(2 * (size_t)dig_bytes >= (SHARED_ ? 2u : 1u) * (size_t)(kLanes + 1) * KYP_ * 16, "final sums fit the digit buffers");
   static_assert(dig_bytes % 16 == 0 && B::LAA / 16 < (1u << 14), "descriptor strides");
 };
-
-// An FP32 value widened to FP64 exactly in integer arithmetic (the FP64
-// conversion unit is slow on this GPU); zeros, subnormals, infinities and
-// NaNs (the exponent field 0 or 255) take the conversion instruction.
-__device__ __forceinline__ double widen(float f) {
-  const unsigned b = __float_as_uint(f);
-  const unsigned e = (b >> 23) & 0xffu;
-  if (e == 0u || e == 255u) return (double)f;
-  return __hiloint2double((int)((b & 0x80000000u) | ((e + 896u) << 20) | ((b & 0x7fffffu) >> 3)), (int)(b << 29));
-}
 
 __device__ __forceinline__ void st_digits(unsigned addr, unsigned a, unsigned b, unsigned c, unsigned d) {
   asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
@@ -252,41 +242,69 @@ __device__ __forceinline__ void drain(unsigned ta, int q) {
 
 // Running sums of this thread's TMEM lane (NY columns of every column block,
 // from address ts) -> the totals (units 2^(Ax + Ay - 2148)).
-// With h = sum_d S_d 2^(8 (14 - d)) the value is h 2^(Ax + Ay - 2168); h = H 2^24
-// + l (H: diagonals 0..11) and the total takes floor(h 2^-20) = H 2^4 + floor(l
-// 2^-20).  Rare, and out of line: its 128-bit sums would cost the panel loop
-// registers.  jl: the lane's digit phase (column block c holds diagonal c + jl).
-template <class G>
+// With h = sum_d S_d 2^(8 (14 - d)) the value is h 2^(Ax + Ay - 2168), and the
+// total takes floor(h 2^-20).  jl: the lane's digit phase (column block c holds
+// diagonal c + jl), so h = 2^(-8 jl) sum_c S_c 2^(8 (14 - c)) over c <= 14 - jl:
+// four sums of neighbouring blocks in 64 bits each, five words, one shift.
+// (Horner's rule on 128-bit integers took 12,000 to 18,000 cycles, most of a
+// product of few rows.)  Out of line: its registers would cost the panel loop.
+// LAST: the accumulators (256 columns before) are added in, not drained first.
+template <class G, bool LAST>
 __device__ __noinline__ void fold(unsigned ts, int jl, i128* tot) {
   constexpr int KYP = G::KYP, NY = KYP / 4;
+  const int sh = 8 * jl + 20;
 #pragma unroll 1
-  for (int part = 0; part < (G::SHARED ? 2 : 1); ++part) {  // SHARED: U from blocks c < J, V from the others
-    i128 h[NY];
-    long long l[NY];
+  for (int y = 0; y < NY; ++y) {  // (one column at a time: few registers)
+    unsigned s[kDiag + 1];
 #pragma unroll
-    for (int y = 0; y < NY; ++y) {
-      h[y] = 0;
-      l[y] = 0;
-    }
-    // Horner over the diagonals d = c + jl; a block outside the part adds zero
-#pragma unroll 1
-    for (int c0 = 0; c0 <= kDiag; c0 += 3) {
-      unsigned s[3][NY];
-      tmem_ld3<NY>(ts + c0 * KYP, ts + (c0 + 1) * KYP, ts + (c0 + 2) * KYP, s);
+    for (int c = 0; c <= kDiag; ++c) tmem_ld1(ts + (unsigned)(c * KYP + y), s[c]);
+    if constexpr (LAST) {
+      unsigned f[kDiag + 1];
 #pragma unroll
-      for (int u = 0; u < 3; ++u) {
-        const int c = c0 + u, d = c + jl;
-        const bool in = !G::SHARED || (c < G::J) == (part == 0);
+      for (int c = 0; c <= kDiag; ++c) tmem_ld1(ts - 256u + (unsigned)(c * KYP + y), f[c]);
+      asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-        for (int y = 0; y < NY; ++y) {
-          const int x = in ? (int)s[u][y] : 0;
-          if (d <= 11) h[y] = (h[y] << 8) + (i128)x;
-          else if (d <= kDiag) l[y] = l[y] * 256 + x;
-        }
+      for (int c = 0; c <= kDiag; ++c) {  // no use moves above the wait
+        asm volatile("" : "+r"(s[c]), "+r"(f[c]));
+        s[c] += (unsigned)__float2int_rn(__uint_as_float(f[c]));
       }
+    } else {
+      asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+      for (int c = 0; c <= kDiag; ++c) asm volatile("" : "+r"(s[c]));
     }
 #pragma unroll
-    for (int y = 0; y < NY; ++y) tot[part * NY + y] += (h[y] << 4) + (i128)(l[y] >> 20);
+    for (int part = 0; part < (G::SHARED ? 2 : 1); ++part) {  // SHARED: U from blocks c < J, V from the others
+      // S_c 2^24 + S_c+1 2^16 + S_c+2 2^8 + S_c+3, a block outside the part or past the last diagonal as zero
+      auto quad = [&](int c0) {
+        long long r = 0;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int c = c0 + u;
+          if (c < 0 || (G::SHARED && (c < G::J) != (part == 0))) continue;
+          const int x = c <= kDiag - (G::J - 1) || c + jl <= kDiag ? (int)s[c] : 0;  // (jl < J)
+          asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(r) : "r"(x), "r"(1 << (24 - 8 * u)));
+        }
+        return r;
+      };
+      unsigned w[7];
+      long long t = quad(11);
+      w[0] = (unsigned)t;
+      t = (t >> 32) + quad(7);
+      w[1] = (unsigned)t;
+      t = (t >> 32) + quad(3);
+      w[2] = (unsigned)t;
+      t = (t >> 32) + quad(-1);
+      w[3] = (unsigned)t;
+      w[4] = (unsigned)(t >> 32);
+      w[5] = w[6] = (unsigned)((int)w[4] >> 31);
+      unsigned a[5], o[4];
+#pragma unroll
+      for (int i = 0; i < 5; ++i) a[i] = sh < 32 ? w[i] : sh < 64 ? w[i + 1] : w[i + 2 < 7 ? i + 2 : 6];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) o[i] = __funnelshift_r(a[i], a[i + 1], (unsigned)sh);
+      tot[part * NY + y] += (i128)from_words(o[3], o[2], o[1], o[0]);
+    }
   }
 }
 
@@ -320,10 +338,9 @@ __global__ void __launch_bounds__(kThreads, 1)
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
-  // ---- set-up: TMEM (accumulators in columns 0..255, running sums in 256..511),
-  // barriers, zero digits (padded columns and slabs stay zero), exponents
+  // ---- set-up: TMEM (accumulators in columns 0..255, running sums in 256..511), barriers
   if (warp == 0) tmem_alloc(smem_u32(&tmem_base), 512);
-  if (tid == 0) {
+  if (tid == kIssuer) {  // (the thread that fetches, so that the first copies need no CTA barrier)
     for (int b = 0; b < 2; ++b) {
       mbar_init(smem_u32(&full_bar[b]), 1);
       mbar_init(smem_u32(&stage_bar[b]), 1);
@@ -334,14 +351,6 @@ __global__ void __launch_bounds__(kThreads, 1)
     flag = 0;
     bad = 0;
   }
-  for (int c = tid; c < 2 * G::COLS; c += kThreads) Erun[c] = 0;  // Erun and Enew
-  for (unsigned e = tid; e < 2 * G::dig_bytes / 16; e += kThreads)
-    reinterpret_cast<uint4*>(dig)[e] = make_uint4(0u, 0u, 0u, 0u);
-  fence_proxy_async();
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  const unsigned taddr = tmem_base;
 
   const int64_t r0 = (int64_t)blockIdx.y * rows_per_chunk;
   const int64_t r1 = min(n, r0 + rows_per_chunk);
@@ -404,6 +413,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   // Panel p's values (zeros past the chunk).  The units of an item differ in
   // bits 4 and 5 of their address only (the swizzle's), as an exclusive or.
   double v[8];
+  // rows of this thread's item that panel p has (8 or more but in the chunk's last panel)
+  auto rows_left = [&](int p) { return (int)min(r1 - (r0 + (int64_t)p * P + 8 * kc), (int64_t)8); };
   const unsigned item_s = stage_s + (mine ? unit(0, 0) : 0u);
   auto load = [&](int p) {
     if constexpr (TMA) mbar_wait(sb0 + 8u * (unsigned)(p & 1), (unsigned)(p >> 1) & 1u, &bad);
@@ -421,7 +432,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
     }
     if (TMA && p + 1 == npan) {  // (the copies zero-fill rows past the chunk, but not the tensor map)
-      const int64_t left = r1 - (r0 + (int64_t)p * P + 8 * kc);
+      const int left = rows_left(p);
 #pragma unroll
       for (int m = 0; m < 8; ++m)
         if (m >= left) v[m] = 0.0;
@@ -435,16 +446,42 @@ __global__ void __launch_bounds__(kThreads, 1)
     wlo = (unsigned)f << 21;
     wrange = ((unsigned)(A + 1) << 21) - wlo;
   };
-  auto outside = [&]() {
+  // (rows past the chunk's end do not count: its last panel masks zeros)
+  auto outside = [&](int p) {
     unsigned k = 0;
+    if (p + 1 < npan) {
 #pragma unroll
-    for (int m = 0; m < 8; ++m) k = max(k, 2u * hi32(v[m]) - wlo);
+      for (int m = 0; m < 8; ++m) k = max(k, 2u * hi32(v[m]) - wlo);
+    } else {
+      const int left = rows_left(p);
+#pragma unroll
+      for (int m = 0; m < 8; ++m) k = max(k, m < left ? 2u * hi32(v[m]) - wlo : 0u);
+    }
     return k >= wrange;
   };
   if (npan > 0) {
     fetch(0);
     if (!TMA || npan > 1) fetch(1);
   }
+
+  // zero digits (padded columns and slabs stay zero) and exponents, while the first copies fly
+  for (int c = tid; c < 2 * G::COLS; c += kThreads) Erun[c] = 0;  // Erun and Enew
+  if (kx < KXP || (!SHARED && ky - y0 < KYP)) {
+    for (unsigned e = tid; e < 2 * G::dig_bytes / 16; e += kThreads)
+      reinterpret_cast<uint4*>(dig)[e] = make_uint4(0u, 0u, 0u, 0u);
+  } else if constexpr (G::SAN > kNear) {  // the slabs past the last digit of every K chunk (the others are stored)
+    constexpr unsigned per = (G::SAN - kNear) * KXP;
+    for (unsigned e = tid; e < 2 * (P / 8) * per; e += kThreads) {
+      const unsigned c = e / per, u = e % per;  // chunk of the two buffers
+      reinterpret_cast<uint4*>(dig + (c / (P / 8)) * G::dig_bytes + (c % (P / 8)) * G::LAN)[kNear * KXP + u] =
+          make_uint4(0u, 0u, 0u, 0u);
+    }
+  }
+  fence_proxy_async();
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const unsigned taddr = tmem_base;
 
   // ---- drains: this thread's TMEM lane: lane block jl (digit phase), X column xl
   const int Lq = (warp & 3) * 32, L = Lq + lane;
@@ -523,7 +560,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     drain<KYP>(tq, warp >> 2);
     if (full) {  // all of the lane quarter's blocks are drained
       asm volatile("bar.sync %0, 128;" ::"r"(1 + (warp & 3)) : "memory");
-      fold<G>(tsum, jl, tot);
+      fold<G, false>(tsum, jl, tot);
       asm volatile("bar.sync %0, 128;" ::"r"(1 + (warp & 3)) : "memory");
       zero_blocks(tq + 256u);
     }
@@ -567,9 +604,26 @@ __global__ void __launch_bounds__(kThreads, 1)
   // MMAs and the copies of panel p + 1's successor at that point instead.
   const bool conv = warp < kConvWarps;
   const unsigned rb0 = smem_u32(&ready_bar[0]);
-  if (npan > 0) {
-    if (conv) load(0);
-    if (tid == 0) spec[0] = 0;  // no exponents yet
+  if (npan > 0) {  // the columns' exponents from panel 0
+    if (conv) {
+      load(0);
+      unsigned m = 0;  // largest magnitude
+#pragma unroll
+      for (int i = 0; i < 8; ++i) m = max(m, abs_hi(v[i]));
+      const int e = (int)(m >> 20);  // (subnormals set none: an alignment exponent is at least 1)
+      if (valid && e > 0) {
+        if (e == 2047) flag = 1;
+        // (finite exponents stay below 2047, so that an Inf or NaN always raises)
+        atomicMax(&Enew[slot], e == 2047 ? e : min(e + EO_GRAM_HEADROOM, 2046));
+      }
+    }
+    __syncthreads();
+    if (tid < G::COLS) Erun[tid] = Enew[tid];
+    if (valid) {
+      te = Enew[slot];
+      set_window();
+    }
+    if (conv && outside(0)) *reinterpret_cast<volatile int*>(&spec[0]) = 0;
   }
   __syncthreads();
   if (TMA && npan > 2) fetch(2);  // (TMA: panel 0's values are in registers)
@@ -579,11 +633,12 @@ __global__ void __launch_bounds__(kThreads, 1)
     Sign2 sg[4];
     bool off = false;
     if (conv) {
-      near_lanes<false>(v, max(te, 1), z, sg);
+      if (p + 1 < npan) near_lanes<false>(v, max(te, 1), z, sg);
+      else near_lanes<true>(v, max(te, 1), z, sg);  // rows past the chunk's end
       if constexpr (!TMA) fetch(p + 2);
       if (p + 1 < npan) {
         load(p + 1);
-        off = outside();
+        off = outside(p + 1);
       }
     }
     if (p > 0) {
@@ -700,7 +755,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       // exponents may have grown
       if (conv && p + 1 < npan) {
         load(p + 1);
-        off = outside();
+        off = outside(p + 1);
       } else {
 #pragma unroll
         for (int i = 0; i < 8; ++i) v[i] = 0.0;
@@ -722,7 +777,10 @@ __global__ void __launch_bounds__(kThreads, 1)
   issue();
   if (step > 0) {
     if (warp == 0) mbar_wait_final(fb0 + 8u * (unsigned)((step - 1) & 1), (unsigned)((step - 1) >> 1) & 1u, &bad);
-    empty(step, true);
+    wait_step(step - 1);
+    tc_fence_after();  // (the drains' running sums: before the barrier above)
+    fold<G, true>(tsum, jl, tot);
+    tc_fence_before();
   }
   __syncthreads();
   if (warp == 0) {
@@ -731,17 +789,20 @@ __global__ void __launch_bounds__(kThreads, 1)
   }
 
   // sum the lane blocks (digit phase j) of every output and write the partials
-  i128* red = reinterpret_cast<i128*>(dig);  // kParts x 128 lanes x KYP entries (the MMAs are done)
+  // (lanes next to one another, and a lane of padding: neither the stores nor
+  // the loads of a column or of its transpose meet in a bank)
+  constexpr int kRow = kLanes + 1;
+  i128* red = reinterpret_cast<i128*>(dig);  // kParts x KYP x 129 entries (the MMAs are done)
   for (int q = 0; q < kParts; ++q)
-    for (int y = 0; y < NY; ++y) red[(q * kLanes + L) * KYP + yq + y] = tot[q * NY + y];
+    for (int y = 0; y < NY; ++y) red[(q * KYP + yq + y) * kRow + L] = tot[q * NY + y];
   __syncthreads();
   for (int e = tid; e < KXP * KYP; e += kThreads) {
-    const int i = e / KYP, yo = e % KYP, j = y0 + yo;
+    const int i = e % KXP, yo = e / KXP, j = y0 + yo;
     if (i >= kx || j >= ky) continue;
     i128 w = 0;
     for (int b = 0; b < J; ++b) {
-      w += red[(b * KXP + i) * KYP + yo];
-      if constexpr (SHARED) w += red[(kLanes + b * KXP + i) * KYP + yo] + red[(kLanes + b * KXP + yo) * KYP + i];
+      w += red[yo * kRow + b * KXP + i];
+      if constexpr (SHARED) w += red[(KYP + yo) * kRow + b * KXP + i] + red[(KYP + i) * kRow + b * KXP + yo];
     }
     FxPart o;
     o.wl = (long long)(unsigned long long)(u128)w;
@@ -772,9 +833,20 @@ UPlan make_plan(int kx, int ky, bool sym) {
 
 constexpr int kMinRows = 64;  // rows of the smallest row chunk
 
+// A symmetric product with more than 16 columns runs as column strips of 16
+// (below), from kStripRows rows on; with fewer, as one launch of X^T X: it
+// converts more, but the strips run one after another, each with its fixed part
+// (set-up, first panel, last fold: 10 us and the reduction's 5 to 9).
+// Measured, one launch vs strips: 2e4 rows of 32 columns 32 vs 57 us, of 64 49
+// vs 114; 1e5 rows 61 vs 81, 131 vs 161; 2e5 rows 101 vs 98, 234 vs 253.
+constexpr int64_t kStripRows = 160000;
+bool use_strips(int64_t n, int kx, bool sym) { return sym && kx > 16 && n >= kStripRows; }
+
 int num_chunks(int64_t n, const UPlan& p) {
   const int64_t by_rows = (n + kMinRows - 1) / kMinRows;
-  const int64_t want = std::max<int64_t>(1, (152 + p.nty - 1) / p.nty);  // one CTA per SM
+  // one CTA per SM, none left over for a second wave (three tiles with 51
+  // chunks: a symmetric product of 48 columns on 1e5 rows took 156 us, on 64 131)
+  const int64_t want = std::max<int64_t>(1, 152 / p.nty);
   const int64_t need = (n + (1ll << 22) - 1) >> 22;                       // <= 2^22 rows per chunk
   return (int)std::max<int64_t>(1, std::min(by_rows, std::max(want, need)));
 }
@@ -913,7 +985,11 @@ template <typename T>
 cudaError_t launch_gram_t(int64_t n, int kx, const T* X, int64_t ldx, int ky, const T* Y, int64_t ldy, bool sym,
                           void* scratch, double* G_hi, double* G_lo, int ldg, const int* gate, cudaStream_t st,
                           int ctas) {
-  if (!sym) return launch_one(n, kx, X, ldx, ky, Y, ldy, scratch, G_hi, G_lo, ldg, gate, st, ctas, false, 0, false);
+  if (!use_strips(n, kx, sym)) {
+    const T* B = sym ? X : Y;
+    return launch_one(n, kx, X, ldx, sym ? kx : ky, B, sym ? ldx : ldy, scratch, G_hi, G_lo, ldg, gate, st, ctas, sym, 0,
+                      sym);
+  }
   for (int c0 = 0; c0 < kx; c0 += 16) {
     const int c1 = std::min(kx, c0 + 16);
     cudaError_t e = launch_one(n, c1, X, ldx, c1 - c0, X + (size_t)c0 * ldx, ldx, scratch, G_hi, G_lo, ldg, gate, st,
@@ -926,7 +1002,8 @@ cudaError_t launch_gram_t(int64_t n, int kx, const T* X, int64_t ldx, int ky, co
 }  // namespace
 
 size_t umma_gram_scratch_bytes(int64_t n, int kx, int ky, bool sym) {
-  if (!sym) return (size_t)num_chunks(n, make_plan(kx, ky, false)) * (size_t)kx * ky * sizeof(FxPart);
+  if (sym) ky = kx;
+  if (!use_strips(n, kx, sym)) return (size_t)num_chunks(n, make_plan(kx, ky, sym)) * (size_t)kx * ky * sizeof(FxPart);
   size_t b = 0;  // the column strips (one after another: the largest)
   for (int c0 = 0; c0 < kx; c0 += 16) {
     const int c1 = std::min(kx, c0 + 16);
@@ -936,8 +1013,8 @@ size_t umma_gram_scratch_bytes(int64_t n, int kx, int ky, bool sym) {
 }
 
 int umma_gram_ctas(int64_t n, int kx, int ky, bool sym, int ctas) {
-  if (!sym) {
-    const UPlan plan = make_plan(kx, ky, false);
+  if (!use_strips(n, kx, sym)) {
+    const UPlan plan = make_plan(kx, sym ? kx : ky, sym);
     return plan.nty * capped_chunks(n, plan, ctas);
   }
   int c = 0;
@@ -951,13 +1028,12 @@ int umma_gram_ctas(int64_t n, int kx, int ky, bool sym, int ctas) {
 
 int umma_gram_launches(int64_t n, int kx, const double* X, int64_t ldx, int ky, const double* Y, int64_t ldy,
                        bool sym) {
-  (void)n;
   (void)X;
   (void)ldx;
   (void)ky;
   (void)Y;
   (void)ldy;
-  return sym ? 2 * ((kx + 15) / 16) : 2;
+  return use_strips(n, kx, sym) ? 2 * ((kx + 15) / 16) : 2;
 }
 
 cudaError_t launch_umma_gram(int64_t n, int kx, const double* X, int64_t ldx, int ky, const double* Y, int64_t ldy,
