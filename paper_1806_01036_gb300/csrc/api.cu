@@ -105,23 +105,27 @@ __global__ void copy_small_kernel(int rows, int cols, const double* sh, const do
 // Engine of a compensated Gram product: the tcgen05 digit engine
 // (umma_gram.cu) or, for narrow products, the integer limbs (fxgram.cu), whose
 // work grows with the entries while a 16-column tile of the digit engine costs
-// the same for any columns in it.  Measured (us, limbs / digits): symmetric,
-// 4e6 rows, k = 4 207 / 280, 5 370 / 281, 8 473 / 282, and 1e6 rows, k = 4 75 /
-// 97, 5 117 / 97; X^T Y, 4e6 rows, 8 x 2 426 / 487, 8 x 4 513 / 488, 8 x 8 745 /
-// 488, 4 x 4 302 / 488; equal within the launches' time at 1e5 rows.
-// EO_DD_GRAM_ENGINE=int|umma overrides the choice (both engines give results
-// within the same bound).
-static bool use_umma_gram(int kx, int ky, bool sym) {
+// the same for any columns in it (a symmetric product of up to 8 columns fills
+// the tile with parts of its rows) and has the longer start.  Measured (us,
+// limbs / digits): symmetric, 4e6 rows, k = 1 90 / 33, 4 201 / 90, 8 468 / 145;
+// 1e6 rows, k = 2 45 / 39, 4 68 / 35; 3e5 rows, k = 4 33 / 39; 1e5 rows, k = 8
+// 36 / 29; 2e4 rows, k = 8 25 / 25.  X^T Y, 4e6 rows, 8 x 2 426 / 487, 8 x 4 513
+// / 488, 8 x 8 745 / 488, 4 x 4 302 / 488; equal within the launches' time at
+// 1e5 rows.  EO_DD_GRAM_ENGINE=int|umma overrides the choice (both engines give
+// results within the same bound).
+static bool use_umma_gram(int64_t n, int kx, int ky, bool sym) {
   const char* e = getenv("EO_DD_GRAM_ENGINE");
   if (e && e[0] == 'u') return true;
   if (e && e[0] == 'i') return false;
-  return std::max(kx, ky) > 8 || (sym ? kx >= 5 : kx * ky >= 32);
+  if (std::max(kx, ky) > 8) return true;
+  if (!sym) return kx * ky >= 32;
+  return n >= (kx >= 5 ? 32768 : (kx >= 3 ? 524288 : 1048576));
 }
 
 // Kernels one launch_dd_gram call launches.
 static uint64_t dd_gram_launches(int64_t n, int kx, const double* X, int64_t ldx, int ky, const double* Y,
                                  int64_t ldy, bool sym) {
-  return use_umma_gram(kx, sym ? kx : ky, sym) ? (uint64_t)umma_gram_launches(n, kx, X, ldx, ky, Y, ldy, sym)
+  return use_umma_gram(n, kx, sym ? kx : ky, sym) ? (uint64_t)umma_gram_launches(n, kx, X, ldx, ky, Y, ldy, sym)
                                           : kGramLaunches;
 }
 
@@ -132,13 +136,13 @@ size_t dd_gram_scratch(int64_t n, int kx, int ky, bool sym) {
 cudaError_t launch_dd_gram(int64_t n, int kx, const double* X, int64_t ldx, int ky, const double* Y, int64_t ldy,
                            bool sym, void* scratch, double* G_hi, double* G_lo, int ldg, const int* gate,
                            cudaStream_t st, int ctas) {
-  if (use_umma_gram(kx, sym ? kx : ky, sym))
+  if (use_umma_gram(n, kx, sym ? kx : ky, sym))
     return launch_umma_gram(n, kx, X, ldx, ky, Y, ldy, sym, scratch, G_hi, G_lo, ldg, gate, st, ctas);
   return launch_fx_gram(n, kx, X, ldx, ky, Y, ldy, sym, scratch, G_hi, G_lo, ldg, gate, st, ctas);
 }
 
 int dd_gram_ctas(int64_t n, int kx, int ky, bool sym, int ctas) {
-  return use_umma_gram(kx, sym ? kx : ky, sym) ? umma_gram_ctas(n, kx, ky, sym, ctas) : fx_gram_ctas(n, kx, ky, sym, ctas);
+  return use_umma_gram(n, kx, sym ? kx : ky, sym) ? umma_gram_ctas(n, kx, ky, sym, ctas) : fx_gram_ctas(n, kx, ky, sym, ctas);
 }
 
 // EO_F32 Gram products with 16 or more columns on one side run on the

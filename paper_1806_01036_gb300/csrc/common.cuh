@@ -122,6 +122,8 @@ bool umma_gram_f32_supported(const float* X, const float* Y, int kx, int ky, boo
 cudaError_t launch_umma_gram_f32(int64_t n, int kx, const float* X, int64_t ldx, int ky, const float* Y,
                                  int64_t ldy, bool sym, void* scratch, double* G_hi, double* G_lo, int ldg,
                                  const int* gate, cudaStream_t st);
+cudaError_t launch_fx_gram_part(int64_t n, int k, const double* X, int64_t ldx, FxPart* parts, const int* gate,
+                                cudaStream_t st);
 int fx_gram_ctas(int64_t n, int kx, int ky, bool sym, int ctas);
 cudaError_t launch_fx_gram(int64_t n, int kx, const double* X, int64_t ldx, int ky, const double* Y, int64_t ldy,
                            bool sym, void* scratch, double* G_hi, double* G_lo, int ldg, const int* gate,

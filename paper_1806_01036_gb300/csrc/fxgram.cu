@@ -485,6 +485,18 @@ int fx_gram_ctas(int64_t n, int kx, int ky, bool sym, int ctas) {
   return plan.groups * num_chunks(n, plan, ctas);
 }
 
+// One partial of X^T X over few rows (n <= 256) at parts.
+cudaError_t launch_fx_gram_part(int64_t n, int k, const double* X, int64_t ldx, FxPart* parts, const int* gate,
+                                cudaStream_t st) {
+  const GramPlan plan = make_plan(k, k, true);
+  const int64_t rpc = (n + plan.P - 1) / plan.P * plan.P;
+  const size_t smem = plan_smem(plan);
+  cudaError_t e = set_dyn_smem(fx_gram_partial_kernel, smem);
+  if (e != cudaSuccess) return e;
+  fx_gram_partial_kernel<<<dim3(plan.groups, 1), kThreads, smem, st>>>(n, k, X, ldx, k, X, ldx, plan, rpc, parts, gate);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_fx_gram(int64_t n, int kx, const double* X, int64_t ldx, int ky, const double* Y, int64_t ldy,
                            bool sym, void* scratch, double* G_hi, double* G_lo, int ldg, const int* gate,
                            cudaStream_t st, int ctas) {

@@ -222,6 +222,15 @@ __device__ __forceinline__ void tma_load_2d(unsigned dst, const CUtensorMap* map
       : "memory");
 }
 
+// 3-D box at (x, 0, 0).
+__device__ __forceinline__ void tma_load_3d(unsigned dst, const CUtensorMap* map, int x, unsigned bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %3}], [%4];" ::"r"(
+          dst),
+      "l"(reinterpret_cast<unsigned long long>(map)), "r"(x), "r"(0), "r"(bar)
+      : "memory");
+}
+
 // ------------------------------------------------------------ digits
 // A value x aligned to the exponent A of its group (A >= the biased exponent
 // of every member) is held as X = floor(|x| 2^(1132 - A)) < 2^110, written with

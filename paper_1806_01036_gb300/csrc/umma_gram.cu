@@ -88,6 +88,7 @@
 #include <algorithm>
 #include <cstdlib>
 #include <mutex>
+#include <type_traits>
 
 #include "common.cuh"
 #include "fx.cuh"
@@ -308,17 +309,25 @@ __device__ __noinline__ void fold(unsigned ts, int jl, i128* tot) {
   }
 }
 
+// The 16-column tile of a symmetric product whose columns are parts of rows.
+struct PackPlan : Plan<16, 16, true> {};
+
 // ------------------------------------------------------------ kernel
+// PackPlan: a symmetric product of kx <= 2^lg <= 8 columns.  The rows are
+// 16 >> lg parts of part_rows (n = part_rows here), and column c of part g is
+// column g 2^lg + c of the 16-column tile, so that every lane converts; the
+// diagonal blocks of the tile's product are the parts' products, whose sum is
+// written.
 template <class G, typename T, bool TMA>
 __global__ void __launch_bounds__(kThreads, 1)
     umma_gram_partial_kernel(int64_t n, int kx, const T* __restrict__ X, int64_t ldx, int ky,
                              const T* __restrict__ Y, int64_t ldy, int64_t rows_per_chunk,
                              const __grid_constant__ CUtensorMap tmx, const __grid_constant__ CUtensorMap tmy,
-                             FxPart* __restrict__ parts, const int* gate) {
+                             FxPart* __restrict__ parts, const int* gate, int lg, int64_t part_rows) {
   static_assert(sizeof(T) == 8 || !TMA, "FP32 operands are copied by the converter threads");
   if (gate && *gate == 0) return;
   constexpr int KXP = G::KXP, KYP = G::KYP, J = G::J, P = G::P;
-  constexpr bool SHARED = G::SHARED;
+  constexpr bool SHARED = G::SHARED, PACK = std::is_same_v<G, PackPlan>;
   // Y columns of one draining thread (four warps share a TMEM lane quarter)
   constexpr int NY = KYP / 4;
   constexpr int kParts = SHARED ? 2 : 1;  // totals per output of a lane: U (and V)
@@ -364,7 +373,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   const bool isb = !SHARED && cg * 16 >= KXP;  // of the Y operand (uniform over the warp)
   const int lc = slot - (isb ? KXP : 0);
   const bool mine = warp < kConvWarps && kc < P / 8 && slot < G::COLS;  // the thread has an item
-  const bool valid = mine && (isb ? y0 + lc < ky : lc < kx);
+  const int cx = PACK ? lc & ((1 << lg) - 1) : lc;  // column of X
+  const bool valid = mine && (isb ? y0 + lc < ky : cx < kx);
   const unsigned dst_near = dig_s + (isb ? G::b_off + (unsigned)kc * G::LBN : (unsigned)kc * G::LAN) + (unsigned)lc * 16u;
   const unsigned e1024 = exp1024x2();
 
@@ -376,7 +386,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   // into its own place, element by element.
   constexpr unsigned xbox = KXP * 128u, ybox = KYP * 128u;
   const unsigned stage_s = smem_u32(stage), sb0 = smem_u32(&stage_bar[0]);
-  const T* src = valid ? (isb ? Y + (size_t)(y0 + lc) * ldy : X + (size_t)lc * ldx) + r0 + 8 * kc : nullptr;
+  const T* src = valid ? (isb ? Y + (size_t)(y0 + lc) * ldy : X + (size_t)cx * ldx + (PACK ? (lc >> lg) * part_rows : 0)) + r0 + 8 * kc : nullptr;
   const unsigned item = (isb ? (P / 16) * xbox : 0u) + (unsigned)(kc >> 1) * (isb ? ybox : xbox) + (unsigned)lc * 128u;
   // 16-byte unit u (rows 2u, 2u + 1) of the item
   auto unit = [&](int p, int u) {
@@ -390,7 +400,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         fence_proxy_async();
         mbar_arrive_expect_tx(bar, G::copy_bytes);
         for (int h = 0; h < P / 16; ++h) {
-          tma_load_2d(dst + (unsigned)h * xbox, &tmx, xr + 16 * h, 0, bar);
+          if (PACK) tma_load_3d(dst + (unsigned)h * xbox, &tmx, xr + 16 * h, bar);
+          else tma_load_2d(dst + (unsigned)h * xbox, &tmx, xr + 16 * h, 0, bar);
           if (!SHARED) tma_load_2d(dst + (P / 16) * xbox + (unsigned)h * ybox, &tmy, xr + 16 * h, y0, bar);
         }
       }
@@ -466,7 +477,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 
   // zero digits (padded columns and slabs stay zero) and exponents, while the first copies fly
   for (int c = tid; c < 2 * G::COLS; c += kThreads) Erun[c] = 0;  // Erun and Enew
-  if (kx < KXP || (!SHARED && ky - y0 < KYP)) {
+  if (kx < (PACK ? 1 << lg : KXP) || (!SHARED && ky - y0 < KYP)) {
     for (unsigned e = tid; e < 2 * G::dig_bytes / 16; e += kThreads)
       reinterpret_cast<uint4*>(dig)[e] = make_uint4(0u, 0u, 0u, 0u);
   } else if constexpr (G::SAN > kNear) {  // the slabs past the last digit of every K chunk (the others are stored)
@@ -796,9 +807,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   for (int q = 0; q < kParts; ++q)
     for (int y = 0; y < NY; ++y) red[(q * KYP + yq + y) * kRow + L] = tot[q * NY + y];
   __syncthreads();
-  for (int e = tid; e < KXP * KYP; e += kThreads) {
-    const int i = e % KXP, yo = e / KXP, j = y0 + yo;
-    if (i >= kx || j >= ky) continue;
+  auto output = [&](int i, int yo) {  // columns i and yo of the tile
     i128 w = 0;
     for (int b = 0; b < J; ++b) {
       w += red[yo * kRow + b * KXP + i];
@@ -810,7 +819,35 @@ __global__ void __launch_bounds__(kThreads, 1)
     o.s = max(Erun[i], 1) + max(Erun[(SHARED ? 0 : KXP) + yo], 1) - kOffsetDigits;
     o.flag = flag | bad;
     o.pad = 0;
-    parts[(size_t)blockIdx.y * ((size_t)kx * ky) + (size_t)j * kx + i] = o;
+    return o;
+  };
+  FxPart* mine_parts = parts + (size_t)blockIdx.y * ((size_t)kx * ky);
+  if constexpr (PACK) {  // the parts' blocks, aligned to the largest scale
+    FxPart* blocks = reinterpret_cast<FxPart*>(stage);  // (the copies are done)
+    const int kc2 = 1 << lg;
+    for (int e = tid; e < 16 << lg; e += kThreads) {
+      const int i = e & 15, yo = (i & -kc2) + (e >> 4);
+      blocks[e] = output(i, yo);
+    }
+    __syncthreads();
+    for (int e = tid; e < kx * kx; e += kThreads) {
+      const int i = e % kx, j = e / kx;
+      FxPart o = blocks[j * 16 + i];
+      for (int g = kc2; g < 16; g += kc2) o.s = max(o.s, blocks[j * 16 + g + i].s);
+      i128 w = 0;
+      for (int g = 0; g < 16; g += kc2) {
+        const FxPart& b = blocks[j * 16 + g + i];
+        w += w_shift((i128)(((u128)(unsigned long long)b.wh << 64) | (unsigned long long)b.wl), o.s - b.s);
+      }
+      o.wl = (long long)(unsigned long long)(u128)w;
+      o.wh = (long long)(w >> 64);
+      mine_parts[j * kx + i] = o;
+    }
+  } else {
+    for (int e = tid; e < KXP * KYP; e += kThreads) {
+      const int i = e % KXP, yo = e / KXP, j = y0 + yo;
+      if (i < kx && j < ky) mine_parts[(size_t)j * kx + i] = output(i, yo);
+    }
   }
 }
 
@@ -887,6 +924,20 @@ bool make_map(CUtensorMap* m, const double* A, int64_t n, int k, int64_t ld, int
              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// The same for a matrix in parts of q rows, one above the other: boxes of 16
+// rows x kc columns x all parts.
+bool make_parts_map(CUtensorMap* m, const double* A, int64_t q, int k, int64_t ld, int kc, int parts) {
+  PFN_cuTensorMapEncodeTiled_v12000 enc = encode_tiled();
+  if (!enc) return false;
+  const cuuint64_t dims[3] = {(cuuint64_t)q, (cuuint64_t)k, (cuuint64_t)parts};
+  const cuuint64_t strides[2] = {(cuuint64_t)ld * 8u, (cuuint64_t)q * 8u};
+  const cuuint32_t box[3] = {16u, (cuuint32_t)kc, (cuuint32_t)parts};
+  const cuuint32_t estr[3] = {1u, 1u, 1u};
+  return enc(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 3, const_cast<double*>(A), dims, strides, box, estr,
+             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 struct Maps {
   CUtensorMap x, y;
 };
@@ -894,11 +945,12 @@ struct Maps {
 template <class G, typename T, bool TMA>
 cudaError_t launch_kernel(const UPlan& plan, int chunks, int64_t n, int kx, const T* X, int64_t ldx, int ky,
                           const T* Y, int64_t ldy, int64_t rpc, const Maps& maps, FxPart* parts, const int* gate,
-                          cudaStream_t st) {
+                          cudaStream_t st, int lg = 0, int64_t part_rows = 0) {
   cudaError_t e = set_dyn_smem(umma_gram_partial_kernel<G, T, TMA>, G::smem);
   if (e != cudaSuccess) return e;
   umma_gram_partial_kernel<G, T, TMA>
-      <<<dim3(plan.nty, chunks), kThreads, G::smem, st>>>(n, kx, X, ldx, ky, Y, ldy, rpc, maps.x, maps.y, parts, gate);
+      <<<dim3(plan.nty, chunks), kThreads, G::smem, st>>>(n, kx, X, ldx, ky, Y, ldy, rpc, maps.x, maps.y, parts, gate,
+                                                       lg, part_rows);
   return cudaGetLastError();
 }
 
@@ -981,10 +1033,52 @@ cudaError_t launch_one(int64_t n, int kx, const T* X, int64_t ldx, int ky, const
   return launch_fx_reduce(kx, ky, sym, chunks, parts, G_hi, G_lo, ldg, gate, st, jo);
 }
 
+// Symmetric products of up to 8 columns: the rows in 16 >> lg parts side by side
+// as the columns of the 16-column tile, so that its lanes all have a value; the
+// fewer than 16 rows a part that are left over go through the integer limbs, a
+// launch of 8 us that pays from kPackRows rows on.  Measured: 32e6 rows of 4
+// columns 1.43 ms (limbs; 2.1 on a padded tile) -> 0.49; 4e6 rows of 8 columns
+// 282 us (padded tile) -> 145.
+int pack_lg(int kx) { return kx <= 1 ? 0 : (kx <= 2 ? 1 : (kx <= 4 ? 2 : 3)); }
+constexpr int64_t kPackRows = 300000;
+int64_t part_rows_of(int64_t n, int kx);
+bool use_pack(int64_t n, int kx, bool sym) {
+  return sym && kx <= 8 && n >= 256 && (n >= kPackRows || n == (16 >> pack_lg(kx)) * part_rows_of(n, kx));
+}
+int64_t part_rows_of(int64_t n, int kx) { return n / (16 * (16 >> pack_lg(kx))) * 16; }
+
+cudaError_t launch_packed(int64_t n, int kx, const double* X, int64_t ldx, void* scratch, double* G_hi, double* G_lo,
+                          int ldg, const int* gate, cudaStream_t st, int ctas) {
+  const int lg = pack_lg(kx), np = 16 >> lg;
+  const int64_t q = part_rows_of(n, kx), rest = n - np * q;
+  const UPlan plan = make_plan(kx, kx, true);
+  const int chunks = capped_chunks(q, plan, ctas);
+  int64_t rpc = (q + chunks - 1) / chunks;
+  rpc = std::max<int64_t>(16, (rpc + 15) / 16 * 16);
+  FxPart* parts = static_cast<FxPart*>(scratch);
+  alignas(64) Maps maps{};
+  using P = PackPlan;
+  const char* lm = getenv("EO_DD_GRAM_LOADS");
+  const bool tma = (uintptr_t)X % 16 == 0 && ldx % 2 == 0 && n < (1ll << 31) - 1024 && !(lm && lm[0] == 'd') &&
+                   make_parts_map(&maps.x, X, q, kx, ldx, 1 << lg, np);
+  cudaError_t e =
+      tma ? launch_kernel<P, double, true>(plan, chunks, q, kx, X, ldx, kx, X, ldx, rpc, maps, parts, gate, st, lg, q)
+          : launch_kernel<P, double, false>(plan, chunks, q, kx, X, ldx, kx, X, ldx, rpc, maps, parts, gate, st, lg, q);
+  if (e != cudaSuccess) return e;
+  if (rest > 0) {
+    e = launch_fx_gram_part(rest, kx, X + np * q, ldx, parts + (size_t)chunks * kx * kx, gate, st);
+    if (e != cudaSuccess) return e;
+  }
+  return launch_fx_reduce(kx, kx, true, chunks + (rest > 0 ? 1 : 0), parts, G_hi, G_lo, ldg, gate, st, 0);
+}
+
 template <typename T>
 cudaError_t launch_gram_t(int64_t n, int kx, const T* X, int64_t ldx, int ky, const T* Y, int64_t ldy, bool sym,
                           void* scratch, double* G_hi, double* G_lo, int ldg, const int* gate, cudaStream_t st,
                           int ctas) {
+  if constexpr (sizeof(T) == 8) {
+    if (use_pack(n, kx, sym)) return launch_packed(n, kx, X, ldx, scratch, G_hi, G_lo, ldg, gate, st, ctas);
+  }
   if (!use_strips(n, kx, sym)) {
     const T* B = sym ? X : Y;
     return launch_one(n, kx, X, ldx, sym ? kx : ky, B, sym ? ldx : ldy, scratch, G_hi, G_lo, ldg, gate, st, ctas, sym, 0,
@@ -1001,18 +1095,25 @@ cudaError_t launch_gram_t(int64_t n, int kx, const T* X, int64_t ldx, int ky, co
 
 }  // namespace
 
+// Symmetric: the largest of all forms and of all column counts up to kx, so that
+// scratch for the largest of several products holds each of them.
 size_t umma_gram_scratch_bytes(int64_t n, int kx, int ky, bool sym) {
   if (sym) ky = kx;
-  if (!use_strips(n, kx, sym)) return (size_t)num_chunks(n, make_plan(kx, ky, sym)) * (size_t)kx * ky * sizeof(FxPart);
-  size_t b = 0;  // the column strips (one after another: the largest)
-  for (int c0 = 0; c0 < kx; c0 += 16) {
+  size_t b = (size_t)num_chunks(n, make_plan(kx, ky, sym)) * (size_t)kx * ky;
+  if (!sym) return b * sizeof(FxPart);
+  for (int c0 = 0; c0 < kx; c0 += 16) {  // the column strips, one after another
     const int c1 = std::min(kx, c0 + 16);
-    b = std::max(b, (size_t)num_chunks(n, make_plan(c1, c1 - c0, c0 == 0)) * (size_t)c1 * (c1 - c0) * sizeof(FxPart));
+    b = std::max(b, (size_t)num_chunks(n, make_plan(c1, c1 - c0, c0 == 0)) * (size_t)c1 * (c1 - c0));
   }
-  return b;
+  for (int k = 1; k <= std::min(kx, 8); ++k) {  // rows in parts
+    const size_t chunks = num_chunks(part_rows_of(n, k), make_plan(k, k, true));
+    b = std::max(b, (chunks + 1) * (size_t)k * k);
+  }
+  return b * sizeof(FxPart);
 }
 
 int umma_gram_ctas(int64_t n, int kx, int ky, bool sym, int ctas) {
+  if (use_pack(n, kx, sym)) n = part_rows_of(n, kx);
   if (!use_strips(n, kx, sym)) {
     const UPlan plan = make_plan(kx, sym ? kx : ky, sym);
     return plan.nty * capped_chunks(n, plan, ctas);
@@ -1033,6 +1134,7 @@ int umma_gram_launches(int64_t n, int kx, const double* X, int64_t ldx, int ky, 
   (void)ky;
   (void)Y;
   (void)ldy;
+  if (use_pack(n, kx, sym)) return n % (16 * (16 >> pack_lg(kx))) ? 3 : 2;
   return use_strips(n, kx, sym) ? 2 * ((kx + 15) / 16) : 2;
 }
 

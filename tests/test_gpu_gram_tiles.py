@@ -72,3 +72,36 @@ def test_special_panels(eo, ctx, kind, kx, ky, odd_ld):
         if kind == "zero column":
             a[:, k - 1] = 0.0
     check(eo, ctx, x, y, odd_ld)
+
+
+@pytest.mark.parametrize("kind", ["plain", "mixed"])
+@pytest.mark.parametrize("n", [256, 4096, 4097, 300_000, 300_255, 152 * 240 * 16])
+@pytest.mark.parametrize("k", [1, 2, 3, 4, 7, 8])
+@pytest.mark.parametrize("odd_ld", [False, True])
+def test_rows_in_parts(eo, ctx, monkeypatch, kind, n, k, odd_ld):
+    """Symmetric products of up to 8 columns on the tensor cores: the rows in
+    parts side by side, with and without rows left over, chunks of one panel and
+    of several."""
+    monkeypatch.setenv("EO_DD_GRAM_ENGINE", "umma")
+    g = synth.rng(1500 + k + n % 97)
+    x = synth.gaussian(n, k, 1600 + k)
+    if kind == "mixed":
+        x[n // 3:] *= 2.0 ** -9  # the parts' exponents differ
+        x[g.random(x.shape) < 1e-3] = 0.0
+        r, c = g.integers(0, n, 40), g.integers(0, k, 40)
+        x[r, c] *= 2.0 ** -g.integers(18, 140, 40).astype(float)
+        x[g.integers(0, n, 4), g.integers(0, k, 4)] = 5e-324
+        for i in range(4):
+            x[g.integers(0, n), g.integers(0, k)] *= 2.0 ** (7 * (i + 1))
+    check(eo, ctx, x, x, odd_ld)
+
+
+def test_rows_in_parts_non_finite(eo, ctx, monkeypatch):
+    import torch
+
+    monkeypatch.setenv("EO_DD_GRAM_ENGINE", "umma")
+    for row in (0, 4095, 2500):
+        x = synth.gaussian(4096, 4, 1700)
+        x[row, 2] = np.inf if row else np.nan
+        gh, _ = eo.gram(ctx, torch.from_numpy(np.ascontiguousarray(x.T)).cuda().t())
+        assert bool(torch.isnan(gh[2, 2]))
