@@ -24,7 +24,11 @@ constexpr int kThreads = 128;
 // 32 columns would need scratch that the FP32 mode does not reserve.)
 bool f32_digits(int64_t n, int k) { return k >= 9 && k <= 32 && n >= 16384; }
 
-template <int MODE, typename T, int KM>
+// Bound by the FP64 pipe (2 FMA a clock and SM).  TRI: the triangle written out
+// (k <= KM <= 32, FP64 accumulation).  A loop whose FMAs past the diagonal are
+// predicated off spends the pipe's time on them all the same: 500,000 x 16, one
+// update, 240 -> 118 us (its FMAs alone: 116).  The sums keep their order.
+template <int MODE, typename T, int KM, bool TRI>
 __global__ void __launch_bounds__(kThreads) update_kernel(int64_t n, int k, T* X, int64_t ldx,
                                                           const double* __restrict__ Zh, const double* __restrict__ Zl,
                                                           int tri, const int* gate) {
@@ -41,24 +45,35 @@ __global__ void __launch_bounds__(kThreads) update_kernel(int64_t n, int k, T* X
     double x[KM];  // the whole row stays in registers, so q_j may overwrite x_j at once
 #pragma unroll
     for (int i = 0; i < KM; ++i) x[i] = i < k ? (double)X[(size_t)i * ldx + r] : 0.0;
-#pragma unroll 1
-    for (int j = 0; j < k; ++j) {
-      const int iend = tri ? j + 1 : k;
-      double q;
-      if (MODE == MODE_DD) {
-        dd s = dd{0.0, 0.0};
+    if constexpr (TRI) {
 #pragma unroll
-        for (int i = 0; i < KM; ++i)
-          if (i < iend) dd_fma_acc_dd(s, Zs[j * k + i], x[i]);
-        q = __dadd_rn(s.hi, s.lo);
-      } else {
+      for (int j = 0; j < KM; ++j) {
+        if (j >= k) break;
         double s = 0.0;
 #pragma unroll
-        for (int i = 0; i < KM; ++i)
-          if (i < iend) s = __fma_rn(x[i], Zs[j * k + i].hi, s);
-        q = s;
+        for (int i = 0; i <= j; ++i) s = __fma_rn(x[i], Zs[j * k + i].hi, s);
+        X[(size_t)j * ldx + r] = (T)s;
       }
-      X[(size_t)j * ldx + r] = (T)q;
+    } else {
+#pragma unroll 1
+      for (int j = 0; j < k; ++j) {
+        const int iend = tri ? j + 1 : k;
+        double q;
+        if (MODE == MODE_DD) {
+          dd s = dd{0.0, 0.0};
+#pragma unroll
+          for (int i = 0; i < KM; ++i)
+            if (i < iend) dd_fma_acc_dd(s, Zs[j * k + i], x[i]);
+          q = __dadd_rn(s.hi, s.lo);
+        } else {
+          double s = 0.0;
+#pragma unroll
+          for (int i = 0; i < KM; ++i)
+            if (i < iend) s = __fma_rn(x[i], Zs[j * k + i].hi, s);
+          q = s;
+        }
+        X[(size_t)j * ldx + r] = (T)q;
+      }
     }
   }
 }
@@ -72,16 +87,20 @@ cudaError_t launch_k(int64_t n, int k, void* X, int64_t ldx, const double* Zh, c
   const int t = tri ? 1 : 0;
   const size_t smem = (size_t)k * k * sizeof(dd);
   cudaError_t e = cudaSuccess;
+  constexpr bool kTri = MODE != MODE_DD;
   if (k <= 8) {
-    update_kernel<MODE, T, 8><<<blocks, kThreads, smem, st>>>(n, k, x, ldx, Zh, Zl, t, gate);
+    if (kTri && tri) update_kernel<MODE, T, 8, kTri><<<blocks, kThreads, smem, st>>>(n, k, x, ldx, Zh, Zl, t, gate);
+    else update_kernel<MODE, T, 8, false><<<blocks, kThreads, smem, st>>>(n, k, x, ldx, Zh, Zl, t, gate);
   } else if (k <= 16) {
-    update_kernel<MODE, T, 16><<<blocks, kThreads, smem, st>>>(n, k, x, ldx, Zh, Zl, t, gate);
+    if (kTri && tri) update_kernel<MODE, T, 16, kTri><<<blocks, kThreads, smem, st>>>(n, k, x, ldx, Zh, Zl, t, gate);
+    else update_kernel<MODE, T, 16, false><<<blocks, kThreads, smem, st>>>(n, k, x, ldx, Zh, Zl, t, gate);
   } else if (k <= 32) {
-    update_kernel<MODE, T, 32><<<blocks, kThreads, smem, st>>>(n, k, x, ldx, Zh, Zl, t, gate);
+    if (kTri && tri) update_kernel<MODE, T, 32, kTri><<<blocks, kThreads, smem, st>>>(n, k, x, ldx, Zh, Zl, t, gate);
+    else update_kernel<MODE, T, 32, false><<<blocks, kThreads, smem, st>>>(n, k, x, ldx, Zh, Zl, t, gate);
   } else {
-    e = set_dyn_smem(update_kernel<MODE, T, 64>, smem);
+    e = set_dyn_smem(update_kernel<MODE, T, 64, false>, smem);
     if (e != cudaSuccess) return e;
-    update_kernel<MODE, T, 64><<<blocks, kThreads, smem, st>>>(n, k, x, ldx, Zh, Zl, t, gate);
+    update_kernel<MODE, T, 64, false><<<blocks, kThreads, smem, st>>>(n, k, x, ldx, Zh, Zl, t, gate);
   }
   return cudaGetLastError();
 }
