@@ -223,40 +223,64 @@ struct Wide {
   // entry is what rounding left of an exact zero.
   static __device__ __forceinline__ bool pivot_ok(T d, int ref) { return !wide_is_zero(d) && d.s == 0 && d.e > ref - 118; }
   static __device__ __forceinline__ int scale_of(T a) { return a.e; }
-  // The rotation that zeroes apq, whether |apq| > 2^-100 sqrt(|app aqq|): the
-  // tangent t from FP32 (24 bits: the remainder of apq is left to later
-  // sweeps), then c = (1 + t^2)^(-1/2) and s = t c to 2^-119, so that the
-  // rotation is orthogonal to that precision.
-  static __device__ __forceinline__ bool rotation(T app, T aqq, T apq, T& c, T& sn) {
+  // A rotation: c 2^127 and the tangent +-mt 2^(te - 23), 2^23 <= mt < 2^24.
+  struct Turn {
+    u128 c;
+    unsigned mt;
+    int te, s;
+  };
+  // Leading bits of u 2^(x - 127): f in [1, 2], the binary exponent e.
+  static __device__ __forceinline__ void leading(u128 u, int x, float& f, int& e) {
+    unsigned long long h = (unsigned long long)(u >> 64), l = (unsigned long long)u;
+    if (h == 0ull) {
+      h = l;
+      l = 0ull;
+      x -= 64;
+    }
+    const int z = clz64(h);
+    f = (float)(unsigned)(((h << z) | ((l >> 1) >> (63 - z))) >> 32) * 0x1p-31f;
+    e = x - z;
+  }
+  // Whether |apq| > 2^-100 sqrt(|app aqq|) (leading bits and exponents, all nonzero).
+  static __device__ __forceinline__ bool apart(float fpp, int epp, float fqq, int eqq, float fpq, int epq) {
     static_assert(kJacobiEpsDD == 0x1p-100, "the test below");
-    if (wide_is_zero(apq)) return false;
-    const float fpq = wide_top(apq);
-    const int D = 2 * apq.e - app.e - aqq.e + 200;  // log2 of apq^2 2^200 / (app aqq), up to the significands
-    if (D < -2 || (D <= 2 && !(ldexpf(fpq * fpq, D) > wide_top(app) * wide_top(aqq)))) return false;
-    const wide d = wide_sub(aqq, app);
-    const int x = d.e - apq.e - 1;  // th = d / (2 apq) = +-(top d / top apq) 2^x
+    const int D = 2 * epq - epp - eqq + 200;  // log2 of apq^2 2^200 / (app aqq), up to the leading bits
+    return D >= -2 && (D > 2 || ldexpf(fpq * fpq, D) > fpp * fqq);
+  }
+  // The rotation that zeroes apq, d = aqq - app: the tangent t from FP32 (24
+  // bits: the remainder of apq is left to later sweeps), then c = (1 + t^2)^(-1/2)
+  // to 2^-119, so that with s = t c the rotation is orthogonal to that precision.
+  static __device__ __forceinline__ Turn turn(float fpq, int epq, int spq, bool dzero, float fd, int ed, int sd) {
+    const int x = ed - epq - 1;  // th = d / (2 apq) = +-(fd / fpq) 2^x
     float t;
     int te = 0;  // |t| 2^te
-    if (wide_is_zero(d) || x < -40) {
+    if (dzero || x < -40) {
       t = 1.0f;
     } else if (x > 40) {
-      t = fpq / wide_top(d);  // 1 / (2 th)
+      t = fpq / fd;  // 1 / (2 th)
       te = -x - 1;
     } else {
-      const float th = ldexpf(wide_top(d) / fpq, x);
+      const float th = ldexpf(fd / fpq, x);
       t = 1.0f / (th + sqrtf(fmaf(th, th, 1.0f)));
     }
     const float g = te < -20 ? 1.0f : fmaf(ldexpf(t, te), ldexpf(t, te), 1.0f);  // 1 + t^2
     const unsigned bits = __float_as_uint(t);                                       // t in (2^-43, 2)
     const unsigned mt = (bits & 0x7fffffu) | 0x800000u;
     te += (int)(bits >> 23) - 127;
-    const wide tw{(u128)mt << 104, te, wide_is_zero(d) ? 0 : d.s ^ apq.s};
     // 1 + t^2 = G 2^-126: t^2 = mt^2 2^(2 te - 46) (te <= 0, or t = 1 up to its rounding)
     const unsigned long long q = (unsigned long long)mt * mt;
     const int sh = 80 + 2 * te;
     const u128 t2 = sh >= 0 ? (u128)q << sh : shr128((u128)q, -sh);
-    c = wide_norm(rsqrt_fixed(((u128)1 << 126) + t2, g), 0, 0);
-    sn = wide_mul(tw, c);
+    return Turn{rsqrt_fixed(((u128)1 << 126) + t2, g), mt, te, dzero ? 0 : sd ^ spq};
+  }
+  static __device__ __forceinline__ bool rotation(T app, T aqq, T apq, T& c, T& sn) {
+    if (wide_is_zero(apq)) return false;
+    const float fpq = wide_top(apq);
+    if (!apart(wide_top(app), app.e, wide_top(aqq), aqq.e, fpq, apq.e)) return false;
+    const wide d = wide_sub(aqq, app);
+    const Turn r = turn(fpq, apq.e, apq.s, wide_is_zero(d), wide_top(d), d.e, d.s);
+    c = wide_norm(r.c, 0, 0);
+    sn = wide_mul(wide{(u128)r.mt << 104, r.te, r.s}, c);
     return true;
   }
 };
@@ -622,23 +646,96 @@ __device__ __forceinline__ wide wide_int(i128 v, int x) {
   const bool neg = v < 0;
   return wide_norm(neg ? (u128)-v : (u128)v, x + 127, neg ? 1 : 0);
 }
-// A column of up to 64 entries, two per lane, in units 2^(E - 125): shifted so
+// A column of up to 32 NQ entries, NQ per lane, in units 2^(E - 125): shifted so
 // that its largest magnitude lies in [2^121, 2^122) (so that its norm is below
 // 2^125); from units 2^x.  Returns E.
-__device__ __forceinline__ int settle(i128 (&v)[2], int x) {
+template <int NQ>
+__device__ __forceinline__ int settle(i128 (&v)[NQ], int x) {
   auto top = [](i128 a) { return (unsigned)((u128)(a < 0 ? ~a : a) >> 95); };
   auto low = [](i128 a) { return (unsigned)((u128)(a < 0 ? ~a : a) >> 63); };
-  unsigned t = __reduce_max_sync(0xffffffffu, max(top(v[0]), top(v[1])));
+  unsigned t = __reduce_max_sync(0xffffffffu, max(top(v[0]), top(v[NQ - 1])));
   int z;
   if (t) {
     z = __clz((int)t) - 5;  // |largest| in [2^(126 - clz), 2^(127 - clz))
   } else {
-    t = __reduce_max_sync(0xffffffffu, max(low(v[0]), low(v[1])));
+    t = __reduce_max_sync(0xffffffffu, max(low(v[0]), low(v[NQ - 1])));
     z = t ? __clz((int)t) + 27 : 59;  // (a column that cancels further is settled again by its next rotation)
   }
 #pragma unroll
-  for (int q = 0; q < 2; ++q) v[q] = z >= 0 ? (i128)((u128)v[q] << z) : v[q] >> -z;
+  for (int q = 0; q < NQ; ++q) v[q] = z >= 0 ? (i128)((u128)v[q] << z) : v[q] >> -z;
   return x - z + 125;
+}
+
+// v mt 2^-24, mt < 2^24, rounded down.
+__device__ __forceinline__ i128 smul24(i128 v, unsigned mt) {
+  const i128 h = (i128)(long long)(v >> 64) * (long long)mt;
+  const u128 l = (u128)(unsigned long long)v * mt;
+  return (i128)((u128)h << 40) + (i128)(l >> 24);
+}
+
+// One warp makes two columns of up to 32 NQ entries (units 2^(ex - 125) and
+// 2^(ey - 125)) orthogonal; false if they already are.  With s = t c the columns
+// become c (x - t y) and c (y + t x): t has 24 bits, so a product by t is a
+// quarter of a product by c.
+template <int NQ>
+__device__ __forceinline__ bool rotate_pair(int k, i128* wx, i128* wy, int& Ex, int& Ey, int lane) {
+  i128 x[NQ], y[NQ];
+#pragma unroll
+  for (int q = 0; q < NQ; ++q) {
+    const int i = lane + 32 * q;
+    x[q] = i < k ? wx[i] : (i128)0;
+    y[q] = i < k ? wy[i] : (i128)0;
+  }
+  const int ex = Ex, ey = Ey;
+  // sums of squares and products, units 2^(2 E - 250 + 128)
+  i128 sxx = 0, syy = 0, sxy = 0;
+#pragma unroll
+  for (int q = 0; q < NQ; ++q) {
+    const u128 ax = (u128)(x[q] < 0 ? -x[q] : x[q]), ay = (u128)(y[q] < 0 ? -y[q] : y[q]);
+    sxx += (i128)mulhi128(ax, ax);
+    syy += (i128)mulhi128(ay, ay);
+    const i128 m = (i128)mulhi128(ax, ay);
+    sxy += (x[q] < 0) != (y[q] < 0) ? -m : m;
+  }
+  sxx = shfl_sum(sxx);
+  syy = shfl_sum(syy);
+  sxy = shfl_sum(sxy);
+  if (sxy == 0 || sxx == 0 || syy == 0) return false;
+  float fxx, fyy, fxy, fd;
+  int exx, eyy, exy, ed;
+  Wide::leading((u128)sxx, 2 * ex - 122, fxx, exx);
+  Wide::leading((u128)syy, 2 * ey - 122, fyy, eyy);
+  Wide::leading((u128)(sxy < 0 ? -sxy : sxy), ex + ey - 122, fxy, exy);
+  if (!Wide::apart(fxx, exx, fyy, eyy, fxy, exy)) return false;
+  // the difference in the units of the larger exponent
+  const int top = max(ex, ey);
+  const i128 d = (i128)shr128((u128)syy, 2 * (top - ey)) - (i128)shr128((u128)sxx, 2 * (top - ex));
+  Wide::leading((u128)(d < 0 ? -d : d), 2 * top - 122, fd, ed);
+  const Wide::Turn r = Wide::turn(fxy, exy, sxy < 0 ? 1 : 0, d == 0, fd, ed, d < 0 ? 1 : 0);
+  // t y and t x in units 2^(E + te - 124); the columns in units 2^(mx - 125), 2^(my - 125) before the product by c / 2
+  const int mx = max(ex, ey + r.te + 1), my = max(ey, ex + r.te + 1);
+  i128 nx[NQ], ny[NQ];
+#pragma unroll
+  for (int q = 0; q < NQ; ++q) {
+    const i128 ty = sar128(smul24(y[q], r.mt), mx - ey - r.te - 1), tx = sar128(smul24(x[q], r.mt), my - ex - r.te - 1);
+    nx[q] = smulhi128(sar128(x[q], mx - ex) + (r.s ? ty : -ty), r.c);
+    ny[q] = smulhi128(sar128(y[q], my - ey) + (r.s ? -tx : tx), r.c);
+  }
+  const int fx = settle(nx, mx - 124), fy = settle(ny, my - 124);
+#pragma unroll
+  for (int q = 0; q < NQ; ++q) {
+    const int i = lane + 32 * q;
+    if (i < k) {
+      wx[i] = nx[q];
+      wy[i] = ny[q];
+    }
+  }
+  __syncwarp();
+  if (lane == 0) {
+    Ex = fx;
+    Ey = fy;
+  }
+  return true;
 }
 
 // Eigenvalues and vectors of a positive semidefinite M (A, packed; destroyed) by
@@ -650,7 +747,11 @@ __device__ __forceinline__ int settle(i128 (&v)[2], int x) {
 // spectrum, no second matrix to update, and no exponent per entry: a column is
 // 128-bit fixed point with one exponent (errors 2^-118 of its norm).  One warp
 // takes a pair of columns through a whole rotation (three sums over the rows,
-// the angle, the update), so that a step has one barrier.
+// the angle, the update), so that a step has one barrier.  Bound by the issue of
+// its integer instructions, one CTA on one SM: about 1000 a warp and step (2000
+// with products by sine and cosine in 128 bits and the angle on wide numbers).
+// SVQB step of k = 32: 9.3 ms with double-doubles on the FP64 pipe, 2.5 ms
+// two-sided on wide numbers, 1.35 in this form, 0.95 with the 24-bit tangent.
 // False (with M's triangle to be loaded again) when M is not semidefinite to
 // rounding, or its diagonal spans more than 100 binades, where small entries
 // need exponents of their own.
@@ -760,54 +861,9 @@ __device__ bool onesided_jacobi(int k, const Wide::Vec A, const Wide::Vec U, Dev
         const int a = player(pr), b = player(kk - 1 - pr);
         const int lo = min(a, b), hi = max(a, b);
         if (hi >= k) continue;
-        i128 x[2], y[2];
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-          const int i = lane + 32 * q;
-          x[q] = i < k ? W[lo * k + i] : (i128)0;
-          y[q] = i < k ? W[hi * k + i] : (i128)0;
-        }
-        const int ex = E[lo], ey = E[hi];
-        // sums of squares and products, units 2^(2 E - 250 + 128)
-        i128 sxx = 0, syy = 0, sxy = 0;
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-          if (q && k <= 32) break;
-          const u128 ax = (u128)(x[q] < 0 ? -x[q] : x[q]), ay = (u128)(y[q] < 0 ? -y[q] : y[q]);
-          sxx += (i128)mulhi128(ax, ax);
-          syy += (i128)mulhi128(ay, ay);
-          const i128 m = (i128)mulhi128(ax, ay);
-          sxy += (x[q] < 0) != (y[q] < 0) ? -m : m;
-        }
-        sxx = shfl_sum(sxx);
-        syy = shfl_sum(syy);
-        sxy = shfl_sum(sxy);
-        wide c, sn;
-        if (!Wide::rotation(wide_int(sxx, 2 * ex - 122), wide_int(syy, 2 * ey - 122), wide_int(sxy, ex + ey - 122), c, sn))
-          continue;
-        if (lane == 0) atomicAdd(&rot_count, 1);
-        // x' = c x - s y, y' = s x + c y: the high halves of the products, in units 2^(E - 124) (c) and 2^(E + es - 124) (s)
-        const u128 cf = c.m >> -c.e;  // c 2^127 (c.e is 0 or -1)
-        const int mx = max(ex, ey + sn.e), my = max(ey, ex + sn.e);
-        i128 nx[2], ny[2];
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-          const i128 sy = smulhi128(y[q], sn.m), sx = smulhi128(x[q], sn.m);
-          nx[q] = sar128(smulhi128(x[q], cf), mx - ex) + sar128(sn.s ? sy : -sy, mx - ey - sn.e);
-          ny[q] = sar128(smulhi128(y[q], cf), my - ey) + sar128(sn.s ? -sx : sx, my - ex - sn.e);
-        }
-        const int fx = settle(nx, mx - 124), fy = settle(ny, my - 124);
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-          const int i = lane + 32 * q;
-          if (i < k) {
-            W[lo * k + i] = nx[q];
-            W[hi * k + i] = ny[q];
-          }
-        }
-        if (lane == 0) {
-          E[lo] = fx;
-          E[hi] = fy;
+        if (k <= 32 ? rotate_pair<1>(k, W + lo * k, W + hi * k, E[lo], E[hi], lane)
+                    : rotate_pair<2>(k, W + lo * k, W + hi * k, E[lo], E[hi], lane)) {
+          if (lane == 0) atomicAdd(&rot_count, 1);
         }
       }
       __syncthreads();
