@@ -750,8 +750,8 @@ __device__ __forceinline__ bool rotate_pair(int k, i128* wx, i128* wy, int& Ex, 
 // the angle, the update), so that a step has one barrier.  Bound by the issue of
 // its integer instructions, one CTA on one SM: about 1000 a warp and step (2000
 // with products by sine and cosine in 128 bits and the angle on wide numbers).
-// SVQB step of k = 32: 9.3 ms with double-doubles on the FP64 pipe, 2.5 ms
-// two-sided on wide numbers, 1.35 in this form, 0.95 with the 24-bit tangent.
+// SVQB step of k = 32: about 10 ms with double-doubles on the FP64 pipe, 1.35 in
+// this form, 0.95 with the 24-bit tangent.
 // False (with M's triangle to be loaded again) when M is not semidefinite to
 // rounding, or its diagonal spans more than 100 binades, where small entries
 // need exponents of their own.
@@ -1394,8 +1394,8 @@ cudaError_t launch_small_batched(bool chol, Mode mode, int njobs, int kmax, cons
     if (e != cudaSuccess) return e;
     kern<<<njobs, kThreads, smem, st>>>(jobs, pass, passes, ddm ? 1e7 : 1e4);
   } else {
-    // A DD Jacobi eigensolve of 16 or more columns keeps one SM's FP64 pipe
-    // busy on its own (a k = 32 one takes 7-11 ms alone): when several share
+    // A DD Jacobi eigensolve of 16 or more columns fills most of an SM's issue
+    // slots on its own (a k = 32 one takes 1 ms alone): when several share
     // an SM they all slow down and the launch ends with the last of them.
     // Asking for more than half of an SM's shared memory keeps one such CTA
     // per SM (the jobs are ordered widest first, so the first wave spreads
