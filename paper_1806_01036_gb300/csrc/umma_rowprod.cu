@@ -55,6 +55,10 @@
 //   32 x 16 1.230 -> 1.090 -> 0.829, 16 x 16 1.017 -> 0.907 -> 0.651,
 //   20 x 4 0.969 -> 0.811 -> 0.601, 8 x 8 0.774 -> 0.687 -> 0.500.
 // A launch's fixed part is about 8 us (64 x 16 on 1e4 rows: 14.4).
+// Tiles that need all digits are no rare case for updates: a block whose columns
+// span more than 25 binades has nothing else.  One CholQR pass on 4e6 rows, columns
+// of one scale / over 10 decades, 7-bit digits first: 8 columns 1.19 / 1.19 -> 0.65 /
+// 0.83 ms, 16 1.44 / 1.44 -> 0.93 / 1.12, 32 4.01 / 4.08 -> 2.51 / 3.10.
 //
 // FP32 updates (kin <= 32) take the same path with seven near slabs (24 bits
 // and the near window); their outputs are rounded from the exact sum to FP32.
@@ -128,6 +132,12 @@ __device__ __forceinline__ void st_shared_v2(unsigned addr, unsigned a, unsigned
   asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(addr), "r"(a), "r"(b) : "memory");
 }
 
+// h + kOffset from its pairs: the even pairs are its words, the odd ones lie half a word up.
+__device__ __forceinline__ u128 pairs_sum(const unsigned (&q)[7]) {
+  return from_words(q[0], q[2], q[4], q[6]) +
+         from_words(q[1] >> 16, funnel_l(q[3], q[1], 16), funnel_l(q[5], q[3], 16), q[5] << 16);
+}
+
 // N groups of four TMEM columns (this warp's 32 lanes), 16 columns apart from column a on.
 template <int N>
 __device__ __forceinline__ void tmem_ld4(unsigned a, unsigned (&v)[N][4]) {
@@ -156,8 +166,28 @@ __device__ __forceinline__ void tmem_wait4(unsigned (&v)[N][4]) {
                  :
                  : "memory");
 }
-// h + kOffset of four outputs whose diagonals reach 2^22 (rare), from the columns tb, tb + 16, ..
+// h + kOffset of four outputs from the columns tb, tb + 16, .., out of line: for
+// diagonals that reach 2^22 (rare), and for outputs that the lean roundings left.
 __device__ __noinline__ void combine_any(unsigned tb, u128* h) {
+  unsigned q[4][7];
+  float most = 0.f;
+#pragma unroll
+  for (int m = 0; m < 7; ++m) {
+    unsigned v[2][4];
+    tmem_ld4(tb + (unsigned)(2 * m * kOut), v);
+    tmem_wait4(v);
+#pragma unroll
+    for (int y = 0; y < 4; ++y) {
+      const float a = __uint_as_float(v[0][y]), b = __uint_as_float(v[1][y]);
+      q[y][m] = __float_as_uint(a + 0x1.8p23f) * 256u + __float_as_uint(b + 0x1.8p23f);
+      most = fmaxf(most, fmaxf(fabsf(a), fabsf(b)));
+    }
+  }
+  if (!__any_sync(0xffffffffu, most >= 0x1p21f)) {
+#pragma unroll
+    for (int y = 0; y < 4; ++y) h[y] = pairs_sum(q[y]);
+    return;
+  }
   for (int y = 0; y < 4; ++y) h[y] = kOffset;
 #pragma unroll 1
   for (int m = 0; m < 7; ++m) {
@@ -165,9 +195,9 @@ __device__ __noinline__ void combine_any(unsigned tb, u128* h) {
     tmem_ld4(tb + (unsigned)(2 * m * kOut), v);
     tmem_wait4(v);
     for (int y = 0; y < 4; ++y) {
-      const long long q =
+      const long long r =
           (long long)__float2int_rn(__uint_as_float(v[0][y])) * 256 + __float2int_rn(__uint_as_float(v[1][y]));
-      h[y] += (u128)(i128)q << (16 * (6 - m));
+      h[y] += (u128)(i128)r << (16 * (6 - m));
     }
   }
 }
@@ -219,28 +249,80 @@ __device__ __forceinline__ void store_near(unsigned dst, unsigned slab_bytes, co
     st_slab<W>(dst + (unsigned)j * slab_bytes, w);
   }
 }
-// Group g of any values (rare: the words are formed anew for every slab).
-template <int W>
-__device__ __noinline__ void store_any(int g, unsigned dst, unsigned slab_bytes, const double* v, int A) {
-  const unsigned e1024 = exp1024x2();
-#pragma unroll 1
+// Lane words of any two values: y[i] holds digits 2i (high bytes) and 2i + 1 (low bytes).
+__device__ __forceinline__ void any_lanes(double va, double vb, int A, unsigned (&y)[7], unsigned& sg) {
+  unsigned a[4], b[4];
+  any_words(va, A, a);
+  any_words(vb, A, b);
+  sg = sign2(va, vb).mul;
+  y[0] = __byte_perm(a[3], b[3], 0x5410);
+#pragma unroll
+  for (int j = 0; j < 3; ++j) {
+    y[1 + 2 * j] = __byte_perm(a[2 - j], b[2 - j], 0x7632);
+    y[2 + 2 * j] = __byte_perm(a[2 - j], b[2 - j], 0x5410);
+  }
+}
+// Group G of any values from their lane words: slabs 5 G .. min(5 G + 4, 13).
+template <int G, int W>
+__device__ __forceinline__ void store_any(unsigned dst, unsigned slab_bytes, const unsigned (&y)[W / 2][7],
+                                          const unsigned (&sg)[W / 2], unsigned e1024) {
+#pragma unroll
   for (int j = 0; j < kGroup; ++j) {
-    const int s = g * kGroup + j;
+    const int s = G * kGroup + j;
     if (s >= kAll) break;
     unsigned w[W / 2];
-#pragma unroll 1
+#pragma unroll
     for (int m = 0; m < W / 2; ++m) {
-      unsigned a[4], b[4];
-      any_words(v[2 * m], A, a);
-      any_words(v[2 * m + 1], A, b);
-      const int q = 104 - 8 * s;  // the digit's place
-      const unsigned fa = (a[q >> 5] >> (q & 31)) & 255u, fb = (b[q >> 5] >> (q & 31)) & 255u;
-      Sign2 f = sign2(v[2 * m], v[2 * m + 1]);
-      if (s == 0) f = top(f);
-      w[m] = hfma2(fa | (fb << 16) | e1024, f.mul, f.add);
+      const Sign2 f{sg[m], hmul2(sg[m], s == 0 ? 0xE400E400u : 0xE480E480u)};
+      w[m] = s % 2 == 0 ? digit_hi(y[m][s / 2], e1024, f) : digit_lo(y[m][s / 2], e1024, f);
     }
     st_slab<W>(dst + (unsigned)j * slab_bytes, w);
   }
+}
+// A tile with all digits, 16 values (v) a thread: their lane words would not fit
+// the registers, so they are cut eight at a time, groups 0 and 1 together once
+// both buffers are free (the MMAs of groups G - 2 and G - 1 done), and the lowest
+// words are kept for group 2.  Out of line, waits and arrivals included.
+__device__ __noinline__ void store_any16(const double* v, int A, unsigned dst, unsigned slab_bytes, unsigned fb0,
+                                         unsigned rb0, int G, volatile int* bad) {
+  const unsigned e1024 = exp1024x2();
+  const unsigned b = G & 1, buffer = kGroup * slab_bytes;
+  if (G >= 2) {
+    mbar_wait(fb0 + 8u * b, (unsigned)((G - 2) >> 1) & 1u, bad);
+    mbar_wait(fb0 + 8u * (b ^ 1u), (unsigned)((G - 1) >> 1) & 1u, bad);
+  }
+  unsigned keep[2][4][3];
+#pragma unroll 1
+  for (int h = 0; h < 2; ++h) {
+    unsigned y[4][7], sg[4];
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+      any_lanes(v[8 * h + 2 * m], v[8 * h + 2 * m + 1], A, y[m], sg[m]);
+      keep[h][m][0] = y[m][5];
+      keep[h][m][1] = y[m][6];
+      keep[h][m][2] = sg[m];
+    }
+    const unsigned at = dst + (unsigned)h * 128u;
+    store_any<0, 8>(at + b * buffer, slab_bytes, y, sg, e1024);
+    store_any<1, 8>(at + (b ^ 1u) * buffer, slab_bytes, y, sg, e1024);
+  }
+  fence_proxy_async();
+  mbar_arrive(rb0 + 8u * b);
+  mbar_arrive(rb0 + 8u * (b ^ 1u));
+  mbar_wait(fb0 + 8u * b, (unsigned)(G >> 1) & 1u, bad);  // group 0's MMAs
+#pragma unroll 1
+  for (int h = 0; h < 2; ++h) {
+    unsigned y[4][7], sg[4];
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+      y[m][5] = keep[h][m][0];
+      y[m][6] = keep[h][m][1];
+      sg[m] = keep[h][m][2];
+    }
+    store_any<2, 8>(dst + (unsigned)h * 128u + b * buffer, slab_bytes, y, sg, e1024);
+  }
+  fence_proxy_async();
+  mbar_arrive(rb0 + 8u * b);
 }
 
 // x 2^(1132 - A) as a signed 128-bit integer, truncated toward zero.
@@ -270,6 +352,9 @@ constexpr int kNaNExp = 1 << 24;
 // kept out of line so that the kernels' code stays small.
 __device__ __noinline__ double round_general(bool update, double y, i128 h, int S) {
   if (S >= kNaNExp / 2) return __longlong_as_double(0x7ff8000000000000ll);
+  bool ok;
+  const double o = update ? w_to_double_fast(h, S, ok) : sub_round_fast(y, h, S, ok);
+  if (ok) return o;
   return update ? w_to_double(h, S) : sub_round(y, h, S);
 }
 
@@ -496,8 +581,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         float most = 0.f;
 #pragma unroll
         for (int y = 0; y < ny; ++y) {
-          h[y] = from_words(q[y][0], q[y][2], q[y][4], q[y][6]) +
-                 from_words(q[y][1] >> 16, funnel_l(q[y][3], q[y][1], 16), funnel_l(q[y][5], q[y][3], 16), q[y][5] << 16);
+          h[y] = pairs_sum(q[y]);
           most = fmaxf(most, squares[y]);
         }
         if constexpr (!kSmallDiag<W>) {
@@ -661,12 +745,23 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (!all) {
         group(0, [&](unsigned dst) { store_near<0, kGroup, W>(dst, SLAB_A, z, sg, e1024); });
         group(1, [&](unsigned dst) { store_near<1, NEAR - kGroup, W>(dst, SLAB_A, z, sg, e1024); });
+      } else if constexpr (W <= 8) {
+        unsigned y[W / 2][7];
+#pragma unroll
+        for (int m = 0; m < W / 2; ++m) any_lanes(v[2 * m], v[2 * m + 1], Ar, y[m], sg[m]);
+#pragma unroll 1
+        for (int g = 0; g < kGroupsAll; ++g)
+          group(g, [&](unsigned dst) {
+            if (g == 0) store_any<0, W>(dst, SLAB_A, y, sg, e1024);
+            else if (g == 1) store_any<1, W>(dst, SLAB_A, y, sg, e1024);
+            else store_any<2, W>(dst, SLAB_A, y, sg, e1024);
+          });
       } else {
         double u[W];
 #pragma unroll
         for (int k = 0; k < W; ++k) u[k] = v[k];
-#pragma unroll 1
-        for (int g = 0; g < kGroupsAll; ++g) group(g, [&](unsigned dst) { store_any<W>(g, dst, SLAB_A, u, Ar); });
+        store_any16(u, Ar, adig_s + dofs, SLAB_A, fb0, rb0, G, &bad);
+        G += kGroupsAll;
       }
       // the next tile's values: in flight during the epilogue
       if constexpr (!kStageValues<W>) load_direct(T + gridDim.x, v);
