@@ -51,14 +51,17 @@
 // digits in byte places (ten near slabs and 14 diagonals, not twelve and 15),
 // then with the diagonals combined in words and the lean roundings of fx.cuh,
 // the outputs dealt evenly to the warps:
-//   64 x 16 1.645 -> 1.507 -> 1.224 ms, 32 x 32 2.135 -> 1.933 -> 1.396,
+//   64 x 16 1.645 -> 1.507 -> 1.269 ms, 32 x 32 2.135 -> 1.933 -> 1.396,
 //   32 x 16 1.230 -> 1.090 -> 0.829, 16 x 16 1.017 -> 0.907 -> 0.651,
 //   20 x 4 0.969 -> 0.811 -> 0.601, 8 x 8 0.774 -> 0.687 -> 0.500.
 // A launch's fixed part is about 8 us (64 x 16 on 1e4 rows: 14.4).
 // Tiles that need all digits are no rare case for updates: a block whose columns
 // span more than 25 binades has nothing else.  One CholQR pass on 4e6 rows, columns
 // of one scale / over 10 decades, 7-bit digits first: 8 columns 1.19 / 1.19 -> 0.65 /
-// 0.83 ms, 16 1.44 / 1.44 -> 0.93 / 1.12, 32 4.01 / 4.08 -> 2.51 / 3.10.
+// 0.83 ms, 16 1.44 / 1.44 -> 0.94 / 1.12, 32 4.01 / 4.08 -> 2.51 / 3.10; Y - V C
+// with 64 such columns of V 1.645 / 1.88 -> 1.269 / 1.96 (group 2 after the previous
+// tile's epilogue; before it 1.22 / 2.11, with the third group's words formed anew
+// 1.15 / 2.42: the more the rare path holds, the more the common one spills).
 //
 // FP32 updates (kin <= 32) take the same path with seven near slabs (24 bits
 // and the near window); their outputs are rounded from the exact sum to FP32.
@@ -282,25 +285,25 @@ __device__ __forceinline__ void store_any(unsigned dst, unsigned slab_bytes, con
 // A tile with all digits, 16 values (v) a thread: their lane words would not fit
 // the registers, so they are cut eight at a time, groups 0 and 1 together once
 // both buffers are free (the MMAs of groups G - 2 and G - 1 done), and the lowest
-// words are kept for group 2.  Out of line, waits and arrivals included.
+// words are kept for group 2 (store_any16_last, after the previous tile's
+// epilogue, which covers group 0's MMAs).  Out of line, waits and arrivals included.
 __device__ __noinline__ void store_any16(const double* v, int A, unsigned dst, unsigned slab_bytes, unsigned fb0,
-                                         unsigned rb0, int G, volatile int* bad) {
+                                         unsigned rb0, int G, volatile int* bad, unsigned* keep) {
   const unsigned e1024 = exp1024x2();
   const unsigned b = G & 1, buffer = kGroup * slab_bytes;
   if (G >= 2) {
     mbar_wait(fb0 + 8u * b, (unsigned)((G - 2) >> 1) & 1u, bad);
     mbar_wait(fb0 + 8u * (b ^ 1u), (unsigned)((G - 1) >> 1) & 1u, bad);
   }
-  unsigned keep[2][4][3];
 #pragma unroll 1
   for (int h = 0; h < 2; ++h) {
     unsigned y[4][7], sg[4];
 #pragma unroll
     for (int m = 0; m < 4; ++m) {
       any_lanes(v[8 * h + 2 * m], v[8 * h + 2 * m + 1], A, y[m], sg[m]);
-      keep[h][m][0] = y[m][5];
-      keep[h][m][1] = y[m][6];
-      keep[h][m][2] = sg[m];
+      keep[(4 * h + m) * 3] = y[m][5];
+      keep[(4 * h + m) * 3 + 1] = y[m][6];
+      keep[(4 * h + m) * 3 + 2] = sg[m];
     }
     const unsigned at = dst + (unsigned)h * 128u;
     store_any<0, 8>(at + b * buffer, slab_bytes, y, sg, e1024);
@@ -309,15 +312,21 @@ __device__ __noinline__ void store_any16(const double* v, int A, unsigned dst, u
   fence_proxy_async();
   mbar_arrive(rb0 + 8u * b);
   mbar_arrive(rb0 + 8u * (b ^ 1u));
+}
+// Group 2 of the tile whose group 0 was G.
+__device__ __noinline__ void store_any16_last(const unsigned* keep, unsigned dst, unsigned slab_bytes, unsigned fb0,
+                                              unsigned rb0, int G, volatile int* bad) {
+  const unsigned e1024 = exp1024x2();
+  const unsigned b = G & 1, buffer = kGroup * slab_bytes;
   mbar_wait(fb0 + 8u * b, (unsigned)(G >> 1) & 1u, bad);  // group 0's MMAs
 #pragma unroll 1
   for (int h = 0; h < 2; ++h) {
     unsigned y[4][7], sg[4];
 #pragma unroll
     for (int m = 0; m < 4; ++m) {
-      y[m][5] = keep[h][m][0];
-      y[m][6] = keep[h][m][1];
-      sg[m] = keep[h][m][2];
+      y[m][5] = keep[(4 * h + m) * 3];
+      y[m][6] = keep[(4 * h + m) * 3 + 1];
+      sg[m] = keep[(4 * h + m) * 3 + 2];
     }
     store_any<2, 8>(dst + (unsigned)h * 128u + b * buffer, slab_bytes, y, sg, e1024);
   }
@@ -714,6 +723,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (all && tid == 0) *reinterpret_cast<volatile int*>(&far[i & 1]) = (int)i;
       const int ng = all ? kGroupsAll : kGroupsNear;
       unsigned z[W / 2][5], sg[W / 2];
+      [[maybe_unused]] unsigned keep[24];  // (kin = 64, all digits: for group 2)
       if (!all) {
         if (zeros) near_lanes<W, true>(v, Ar, z, sg);
         else near_lanes<W, false>(v, Ar, z, sg);
@@ -760,7 +770,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         double u[W];
 #pragma unroll
         for (int k = 0; k < W; ++k) u[k] = v[k];
-        store_any16(u, Ar, adig_s + dofs, SLAB_A, fb0, rb0, G, &bad);
+        store_any16(u, Ar, adig_s + dofs, SLAB_A, fb0, rb0, G, &bad, keep);
         G += kGroupsAll;
       }
       // the next tile's values: in flight during the epilogue
@@ -778,6 +788,9 @@ __global__ void __launch_bounds__(kThreads, 1)
           epilogue_block(Tprev, iprev, 0);
           tc_fence_before();
         }
+      }
+      if constexpr (W > 8) {
+        if (all) store_any16_last(keep, adig_s + dofs, SLAB_A, fb0, rb0, G - kGroupsAll, &bad);
       }
       bool below;
       if constexpr (kStageValues<W>) {
