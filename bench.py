@@ -233,7 +233,9 @@ class Clocks:
                 "samples": len(sm)}
 
 
-DIGIT_PAIRS = 120  # FP16 digit-pair products per multiply-add of the compensated tensor-core kernels
+# FP16 digit-pair products per multiply-add of the compensated Gram on the tensor cores: ten digits a value (the
+# near window), pairs of digit places s + t <= 14
+DIGIT_PAIRS = 90
 
 
 def gram_traffic(n, kv, k):
@@ -363,7 +365,7 @@ def run_eo(a):
     # measured copy bandwidth and `achieved` counts the algorithmic bytes
     # (V and Y read once, Y~ written once; V^T Y: V and Y read once) over the
     # launch's CUDA-event time.  The tensor-core view of the Gram
-    # (algorithmic flops against the FP16 dense peak / 120 digit pairs per
+    # (algorithmic flops against the FP16 dense peak / 90 digit pairs per
     # multiply-add) is kept beside it.
     hbm_peak, peak_kind = peak_hbm()
     tc_peak, tc_kind = peak_tensor()

@@ -54,7 +54,7 @@ typedef enum {
   EO_DD = 1,     /* FP64 data, compensated accumulation (>= double-double accuracy),
                     results rounded once; the sums are formed exactly in fixed
                     point, on the tensor cores or the integer pipe (see below)     */
-  EO_F32 = 2,    /* FP32 data (float*), FP64 accumulation of the exact products    */
+  EO_F32 = 2,    /* FP32 data (float*), FP64 or exact sums of the exact products   */
   EO_DD_EFT = 3  /* as EO_DD, but the sums use the paper's FP64 error-free
                     transformations (TwoProd + TwoSum) on the FP64 pipe           */
 } eo_prec;
@@ -62,8 +62,8 @@ typedef enum {
 /* EO_DD accuracy: each group of values summed against another (a column of a
  * block of rows, a row of V or X, a column of C or Z) is aligned to an
  * exponent at or above its largest and held as a 104-bit integer (four
- * 26-bit limbs; the ten most significant limb products are kept) or, in Gram
- * products with more than 8 columns on one side, as a 110-bit integer of
+ * 26-bit limbs; the ten most significant limb products are kept: narrow
+ * products) or, on the tensor cores, as a 110-bit integer of
  * fourteen 8-bit digits whose products are summed on the tensor cores (FP16
  * integer digits, exact FP32 sums; the digit pairs of weight 2^-112 of the
  * largest and above are kept; a column's alignment exponent sits up to two

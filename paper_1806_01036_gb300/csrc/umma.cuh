@@ -1,8 +1,7 @@
 // umma.cuh — building blocks of the tcgen05 digit kernels (umma_gram.cu,
 // umma_rowprod.cu): inline PTX for mbarriers, TMA, tensor-memory allocation,
 // loads and stores, shared-memory matrix descriptors and tcgen05.mma, and the
-// 7-bit digits of an FP64 value aligned to a group exponent.
-//
+// 8-bit digits of an FP64 value aligned to a group exponent.
 #pragma once
 
 #include <cuda.h>
@@ -235,12 +234,12 @@ __device__ __forceinline__ void tma_load_3d(unsigned dst, const CUtensorMap* map
 // A value x aligned to the exponent A of its group (A >= the biased exponent
 // of every member) is held as X = floor(|x| 2^(1132 - A)) < 2^110, written with
 // 14 balanced base-256 digits, X = sum_s D_s 2^(104 - 8s): the fields of X +
-// bias, less 128, D_s in [-128, 127] for s >= 1, and D_0 in [0, 64].  A digit is the FP16
-// integer sign(x) D_s: the field is put into the significand of the FP16 1024
+// bias, less 128, D_s in [-128, 127] for s >= 1, and D_0 in [0, 64].  A digit is
+// the FP16 integer sign(x) D_s: the field is put into the significand of the FP16 1024
 // (bit pattern 0x6400 | f) and one f16x2 FMA takes the offset off and the sign
 // on.  Fields are bytes, so two values' digits are cut with one byte
-// permutation or one masked merge.  A value within kNearBits binades of A has a zero low word, and
-// its digits 10..13 are zero.
+// permutation or one masked merge.  A value within kNearBits binades of A has a
+// zero low word, and its digits 10..13 are zero.
 constexpr int kNear = 10, kAll = 14;  // digits of a near value, of any value
 constexpr int kNearBits = 25;
 __device__ __forceinline__ unsigned abs_hi(double x) { return hi32(x) & 0x7fffffffu; }
