@@ -220,6 +220,16 @@ FX_HD int clz128(u128 u) {
   return h ? clz64(h) : 64 + clz64((unsigned long long)u);
 }
 
+// w 2^s with |w| < 2^(127 - spare), so that 2^spare of such integers of one s
+// add up in 128 bits: shifted down (floor) only when w is larger.
+FX_HD void make_room(i128& w, int& s, int spare) {
+  const int over = spare + 1 - clz128(w < 0 ? ~(u128)w : (u128)w);
+  if (over > 0) {
+    w >>= over;
+    s += over;
+  }
+}
+
 // Double with magnitude m * 2^e2 (2^52 <= m < 2^53, or m == 0) and the given sign.
 FX_HD double make_double(bool neg, unsigned long long m, int e2) {
   if (m == 0) return neg ? -0.0 : 0.0;

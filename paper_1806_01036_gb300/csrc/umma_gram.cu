@@ -827,7 +827,14 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int kc2 = 1 << lg;
     for (int e = tid; e < 16 << lg; e += kThreads) {
       const int i = e & 15, yo = (i & -kc2) + (e >> 4);
-      blocks[e] = output(i, yo);
+      FxPart o = output(i, yo);
+      // a part's total may take all 127 bits (2^22 rows of the largest values the
+      // exponents' headroom allows): room for the sum of all 16 >> lg parts
+      i128 w = (i128)(((u128)(unsigned long long)o.wh << 64) | (unsigned long long)o.wl);
+      make_room(w, o.s, 4 - lg);
+      o.wl = (long long)(unsigned long long)(u128)w;
+      o.wh = (long long)(w >> 64);
+      blocks[e] = o;
     }
     __syncthreads();
     for (int e = tid; e < kx * kx; e += kThreads) {

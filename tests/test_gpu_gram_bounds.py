@@ -1,0 +1,59 @@
+"""What the tensor-core Gram engine promises at the ends of its range: totals
+of many rows in one CTA, the error of short products, and columns whose first
+rows are subnormal."""
+import numpy as np
+import pytest
+
+import oracle
+import synth
+
+pytestmark = pytest.mark.gpu
+
+
+def dev(a):
+    import torch
+
+    return torch.from_numpy(np.ascontiguousarray(np.asarray(a).T)).cuda().t()
+
+
+@pytest.mark.parametrize("k", [1, 2, 4, 8])
+def test_many_rows_in_one_cta(eo, tmp_path, k):
+    """Products of up to 8 columns hold 16, 8, 4 or 2 parts of the rows side by
+    side.  One CTA over 2^26 / 2^25 / 2^24 / 2^23 rows, 2^22 a part, its first
+    panels at 1/4 and everything after them just below 2 (the two binades of
+    headroom of the alignment exponent used up): the parts' sums together pass
+    2^127 units.  The squared norms are summed exactly here, and q = x / |x| is
+    rounded once (2 ulps)."""
+    import torch
+
+    np_ = 16 >> {1: 0, 2: 1, 4: 2, 8: 3}[k]
+    q = 1 << 22
+    n = np_ * q
+    v = 2.0 - 2.0 ** -52
+    x = torch.full((k, np_, q), v, dtype=torch.float64, device="cuda")
+    x[:, :, :512] = 0.25
+    if k > 1:  # signs of a Hadamard pattern (period 8) make the columns orthogonal
+        s = torch.ones((k, 8), dtype=torch.float64)
+        for c in range(k):
+            for r in range(8):
+                s[c, r] = -1.0 if bin(c & r).count("1") % 2 else 1.0
+        x = (x.view(k, -1, 8) * s.cuda()[:, None, :]).view(k, np_, q)
+    x = x.view(k, n)
+    want = [0.25, v]
+    norm2 = np_ * (512 * 0.25 ** 2 + (q - 512) * v * v)
+    props = torch.cuda.get_device_properties(0)
+    path = tmp_path / "tiles.txt"
+    path.write_text("%d %d %d 1 0 %s/%d\n" % (k, n.bit_length() - 1, eo.DD, props.name.replace(" ", "_"),
+                                             props.multi_processor_count))
+    c = eo.Context(0)
+    c.tune_cache(str(path))
+    b = eo.Batch(c, [x.t()], passes=1, prec=eo.DD)
+    assert b.tile(0)[0] == 1
+    b.run()
+    torch.cuda.synchronize()
+    assert int(b.out[0]) == k
+    for at, w in ((0, want[0]), (511, want[0]), (512, want[1]), (n - 1, want[1])):
+        got = x[:, at].abs().cpu().numpy()
+        assert np.all(np.abs(got * np.sqrt(norm2) / w - 1) <= 2.0 ** -50), (at, got)
+    b.close()
+    c.close()
