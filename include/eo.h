@@ -68,7 +68,7 @@ typedef enum {
  * integer digits, exact FP32 sums; the digit pairs of weight 2^-112 of the
  * largest and above are kept; a column's alignment exponent sits up to two
  * binades above its largest, so that it rarely has to grow).  Each product then carries an
- * error below 2^-101 max|x| max|y| (integer limbs) or 2^-96 max|x| max|y|
+ * error below 2^-101 max|x| max|y| (integer limbs) or 2^-103 max|x| max|y|
  * (tensor-core digits), the sums of the kept products are exact, and every
  * result is rounded once.  Exact sums are
  * associative: the order of the partial sums does not matter, and the same
@@ -122,7 +122,7 @@ EO_API eo_status eo_selftest_wait_timeout(eo_ctx* ctx, double seconds);
  *   symmetric and both triangles are written).  FP64 data, or float data in
  *   EO_F32 mode.  G_hi (required) / G_lo: kx-by-ky with leading dimension ldg.
  * EO_DD: every G_ij is the double-double rounding of the sum of the exact
- * products (error below 2^-104 |G_ij| + n 2^-96 max|x_i| max|y_j|, see the
+ * products (error below 2^-104 |G_ij| + n 2^-101 max|x_i| max|y_j|, see the
  * accuracy note above); results are bitwise reproducible.
  */
 EO_API eo_status eo_gram(eo_ctx* ctx, int64_t n, int kx, const void* X, int64_t ldx, int ky, const void* Y, int64_t ldy,

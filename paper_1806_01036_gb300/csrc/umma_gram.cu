@@ -34,19 +34,23 @@
 //  * before an accumulator can exceed 2^24 in magnitude (group_pairs below)
 //    the accumulators are read back (tcgen05.ld), converted to integers,
 //    added to 32-bit running sums per (lane, column) kept in TMEM and set
-//    back to zero.  The running sums are folded into a 128-bit total W in the
-//    units of the integer engine (value = W 2^(Ax + Ay - 2148)) every
+//    back to zero.  The running sums are folded into a total of 128 + 20 bits in
+//    the units of the integer engine (2^(Ax + Ay - 2148)) and 2^-20 of them every
 //    kFoldDrains drains, before an alignment exponent grows, and at the end.
-//    The row-chunk partials go through the same exact, order-free reduction
-//    (fx_gram_reduce).
+//    The lanes' totals are added with all their bits; a row chunk's partial is
+//    their sum rounded down once, to the finest unit that 127 bits hold, and the
+//    partials go through the same exact, order-free reduction (fx_gram_reduce).
 //
 // Error per product x y: the dropped digit pairs (d >= 15, twelve of weight
 // 2^88 and fewer of smaller weights, each product at most 2^14) sum to less
 // than 2^105.7 units^2 (units of 2^(Ax - 1132), 2^(Ay - 1132)), and a value
-// more than 57 binades below A is truncated by less than one unit, 2^110 for
-// a product; with max|x| >= 2^(109 - h) units for a headroom h the error is
-// below 2^(2h - 107) max|x| max|y| (h = 2: 2^-103), under the 2^-96 that
-// include/eo.h states.
+// more than 57 binades below A is truncated by less than one unit, which with
+// max|x| >= 2^(109 - h) units for a headroom h is 2^(h - 109) max|x| max|y| of a
+// product.  Together, with the same for y: below 2^-105.7 max|x| max|y| (h = 2).
+// A growth and a chunk's rounding add one unit of 2^-20 each, 2^-118 max|x|
+// max|y| (or 2^-126 of the chunk's sum if that is more).  (Totals that dropped
+// the 20 bits lane by lane, 24 times an entry of a symmetric tile, were off by
+// 2^-96.2 max|x| max|y| on two rows.)
 //
 // Pipeline per CTA (one per SM, 16 warps of 128 registers): the values of a
 // panel of P rows arrive by TMA (two panels ahead, 16-row boxes with 128-byte
@@ -170,7 +174,7 @@ struct Plan : Geo<KXP_, KYP_, SHARED_> {
   static constexpr int pairs_near = group_pairs(B::J, kNear, B::NQN), pairs_all = group_pairs(B::J, kAll, B::NQA);
   static constexpr size_t smem = B::bytes(P) + 1024;
   static_assert(FK >= 1 && P * pairs_near <= kPairRows && 16 * FK * pairs_all <= kPairRows, "a step fits the accumulators");
-  static_assert(2 * (size_t)dig_bytes >= (SHARED_ ? 2u : 1u) * (size_t)(kLanes + 1) * KYP_ * 16, "final sums fit the digit buffers");
+  static_assert(2 * (size_t)dig_bytes >= (SHARED_ ? 2u : 1u) * (size_t)(kLanes + 1) * KYP_ * 20, "final sums fit the digit buffers");
   static_assert(dig_bytes % 16 == 0 && B::LAA / 16 < (1u << 14), "descriptor strides");
 };
 
@@ -244,16 +248,17 @@ __device__ __forceinline__ void drain(unsigned ta, int q) {
 // Running sums of this thread's TMEM lane (NY columns of every column block,
 // from address ts) -> the totals (units 2^(Ax + Ay - 2148)).
 // With h = sum_d S_d 2^(8 (14 - d)) the value is h 2^(Ax + Ay - 2168), and the
-// total takes floor(h 2^-20).  jl: the lane's digit phase (column block c holds
-// diagonal c + jl), so h = 2^(-8 jl) sum_c S_c 2^(8 (14 - c)) over c <= 14 - jl:
+// total takes h 2^-20 with all its bits (h may reach 2^146 in a chunk, so its low
+// 20 bits are a word of their own).  jl: the lane's digit phase (column block c
+// holds diagonal c + jl), so h = 2^(-8 jl) sum_c S_c 2^(8 (14 - c)) over c <= 14 - jl:
 // four sums of neighbouring blocks in 64 bits each, five words, one shift.
 // (Horner's rule on 128-bit integers took 12,000 to 18,000 cycles, most of a
 // product of few rows.)  Out of line: its registers would cost the panel loop.
 // LAST: the accumulators (256 columns before) are added in, not drained first.
 template <class G, bool LAST>
-__device__ __noinline__ void fold(unsigned ts, int jl, i128* tot) {
+__device__ __noinline__ void fold(unsigned ts, int jl, Total* tot) {
   constexpr int KYP = G::KYP, NY = KYP / 4;
-  const int sh = 8 * jl + 20;
+  const int sh = 8 * jl + kLowBits;
 #pragma unroll 1
   for (int y = 0; y < NY; ++y) {  // (one column at a time: few registers)
     unsigned s[kDiag + 1];
@@ -299,12 +304,15 @@ __device__ __noinline__ void fold(unsigned ts, int jl, i128* tot) {
       w[3] = (unsigned)t;
       w[4] = (unsigned)(t >> 32);
       w[5] = w[6] = (unsigned)((int)w[4] >> 31);
+      // h: bits 8 jl up (the ones below are zero), its low bits and the rest
+      const unsigned low = __funnelshift_r(sh - kLowBits < 32 ? w[0] : w[1], sh - kLowBits < 32 ? w[1] : w[2],
+                                           (unsigned)(sh - kLowBits)) & ((1u << kLowBits) - 1u);
       unsigned a[5], o[4];
 #pragma unroll
       for (int i = 0; i < 5; ++i) a[i] = sh < 32 ? w[i] : sh < 64 ? w[i + 1] : w[i + 2 < 7 ? i + 2 : 6];
 #pragma unroll
       for (int i = 0; i < 4; ++i) o[i] = __funnelshift_r(a[i], a[i + 1], (unsigned)sh);
-      tot[part * NY + y] += (i128)from_words(o[3], o[2], o[1], o[0]);
+      total_add(tot[part * NY + y], (i128)from_words(o[3], o[2], o[1], o[0]), low);
     }
   }
 }
@@ -501,10 +509,10 @@ __global__ void __launch_bounds__(kThreads, 1)
   const unsigned tq = taddr + ((unsigned)Lq << 16);             // the lane quarter's columns
   const unsigned tsum = tq + (unsigned)yq + 256u;               // the running sums of its columns
   // the exact totals; touched once per fold, so they are kept out of registers
-  i128 totals[kParts * NY];
-  i128* tot = totals;
+  Total totals[kParts * NY];
+  Total* tot = totals;
   asm volatile("" : "+l"(tot)::"memory");
-  for (int y = 0; y < kParts * NY; ++y) tot[y] = 0;
+  for (int y = 0; y < kParts * NY; ++y) tot[y] = Total{0, 0u};
 
   // the running sums and, first, the accumulators at zero (this warp's share of the column blocks)
   auto zero_blocks = [&](unsigned t) {
@@ -691,7 +699,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             const int cy = ysb + yq + y;
             const int dx = Erun[xl] ? Enew[xl] - Erun[xl] : 0;
             const int dy = Erun[cy] ? Enew[cy] - Erun[cy] : 0;
-            for (int q = 0; q < kParts; ++q) tot[q * NY + y] = w_shift(tot[q * NY + y], dx + dy);
+            for (int q = 0; q < kParts; ++q) total_shift(tot[q * NY + y], dx + dy);
           }
         }
         __syncthreads();
@@ -804,19 +812,37 @@ __global__ void __launch_bounds__(kThreads, 1)
   // the loads of a column or of its transpose meet in a bank)
   constexpr int kRow = kLanes + 1;
   i128* red = reinterpret_cast<i128*>(dig);  // kParts x KYP x 129 entries (the MMAs are done)
+  unsigned* redl = reinterpret_cast<unsigned*>(red + kParts * KYP * kRow);  // and their low bits
   for (int q = 0; q < kParts; ++q)
-    for (int y = 0; y < NY; ++y) red[(q * KYP + yq + y) * kRow + L] = tot[q * NY + y];
+    for (int y = 0; y < NY; ++y) {
+      const int at = (q * KYP + yq + y) * kRow + L;
+      red[at] = tot[q * NY + y].hi;
+      redl[at] = tot[q * NY + y].lo;
+    }
   __syncthreads();
-  auto output = [&](int i, int yo) {  // columns i and yo of the tile
+  // Columns i and yo of the tile: the lanes' totals are added with all their bits
+  // and rounded down once.  (A part's total may take all 127 bits: 2^22 rows of
+  // the largest values the exponents' headroom allows.  PACK: with room for the
+  // sum of the 16 >> lg parts.)
+  auto output = [&](int i, int yo) {
     i128 w = 0;
+    unsigned l = 0;  // (24 terms below 2^20)
+    auto add = [&](int at) {
+      w += red[at];
+      l += redl[at];
+    };
     for (int b = 0; b < J; ++b) {
-      w += red[yo * kRow + b * KXP + i];
-      if constexpr (SHARED) w += red[(KYP + yo) * kRow + b * KXP + i] + red[(KYP + i) * kRow + b * KXP + yo];
+      add(yo * kRow + b * KXP + i);
+      if constexpr (SHARED) {
+        add((KYP + yo) * kRow + b * KXP + i);
+        add((KYP + i) * kRow + b * KXP + yo);
+      }
     }
     FxPart o;
+    o.s = max(Erun[i], 1) + max(Erun[(SHARED ? 0 : KXP) + yo], 1) - kOffsetDigits;
+    w = total_narrow(w + (i128)(l >> kLowBits), l & ((1u << kLowBits) - 1u), PACK ? 4 - lg : 0, o.s);
     o.wl = (long long)(unsigned long long)(u128)w;
     o.wh = (long long)(w >> 64);
-    o.s = max(Erun[i], 1) + max(Erun[(SHARED ? 0 : KXP) + yo], 1) - kOffsetDigits;
     o.flag = flag | bad;
     o.pad = 0;
     return o;
@@ -827,14 +853,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int kc2 = 1 << lg;
     for (int e = tid; e < 16 << lg; e += kThreads) {
       const int i = e & 15, yo = (i & -kc2) + (e >> 4);
-      FxPart o = output(i, yo);
-      // a part's total may take all 127 bits (2^22 rows of the largest values the
-      // exponents' headroom allows): room for the sum of all 16 >> lg parts
-      i128 w = (i128)(((u128)(unsigned long long)o.wh << 64) | (unsigned long long)o.wl);
-      make_room(w, o.s, 4 - lg);
-      o.wl = (long long)(unsigned long long)(u128)w;
-      o.wh = (long long)(w >> 64);
-      blocks[e] = o;
+      blocks[e] = output(i, yo);
     }
     __syncthreads();
     for (int e = tid; e < kx * kx; e += kThreads) {

@@ -28,3 +28,16 @@ void tots_sum(int spare, const long long* w, const int* s, long long* out, int* 
   *s_out = top;
 }
 }
+
+extern "C" {
+
+// m terms w + lo 2^-20, added; shifted down by sh; narrowed with room for 2^spare.
+void tots_total(int m, const long long* w, const unsigned* lo, int sh, int spare, long long* out, int* s_out) {
+  Total t{0, 0u};
+  for (int i = 0; i < m; ++i) total_add(t, mk(w + 2 * i), lo[i]);
+  total_shift(t, sh);
+  int s = 0;
+  put(total_narrow(t.hi, t.lo, spare, s), out);
+  *s_out = s;
+}
+}

@@ -57,3 +57,24 @@ def test_many_rows_in_one_cta(eo, tmp_path, k):
         assert np.all(np.abs(got * np.sqrt(norm2) / w - 1) <= 2.0 ** -50), (at, got)
     b.close()
     c.close()
+
+
+@pytest.mark.parametrize("n", [1, 2, 4, 16, 63, 64, 65, 300])
+@pytest.mark.parametrize("k", [1, 3, 4, 8, 12, 16, 17, 40])
+def test_short_products(eo, ctx, monkeypatch, n, k):
+    """Values over 20 binades below a column maximum of 1.  A product is off by
+    less than 2^-105.7 (the dropped digit pairs and truncated values, see
+    umma_gram.cu) and the result is rounded to a double-double (2^-106)."""
+    monkeypatch.setenv("EO_DD_GRAM_ENGINE", "umma")
+    g = synth.rng(3100 + 17 * n + k)
+
+    def block(c):
+        x = g.uniform(0.5, 1.0, (n, c)) * np.ldexp(1.0, -g.integers(0, 21, (n, c)))
+        return np.asfortranarray(x / x.max(0) * np.where(g.random((n, c)) < 0.5, -1.0, 1.0))
+
+    x = block(k)
+    for y in (None, block(max(1, k // 2))):
+        gh, gl = eo.gram(ctx, dev(x), None if y is None else dev(y))
+        rh, rl = oracle.gram(x, y)
+        err = np.abs((gh.cpu().numpy() - rh) + (gl.cpu().numpy() - rl))
+        assert np.all(err <= 2.0 ** -105 * np.abs(rh) + n * 2.0 ** -105), float(np.log2(err.max() / n))

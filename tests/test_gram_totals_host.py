@@ -58,3 +58,27 @@ def test_sum_of_parts(lib, spare):
         assert abs(got - want) <= 2 * m * unit
         assert so.value <= max(s) + spare
         assert so.value == max(s) or max(abs(F(x)) * F(2) ** e for x, e in zip(v, s)) >= 2 ** (126 - spare) * unit / 2 ** spare
+
+
+@pytest.mark.parametrize("spare", [0, 1, 4])
+def test_totals_keep_their_low_bits(lib, spare):
+    """The sum of terms w + lo 2^-20 is exact, its shift rounds down by less than
+    2^-20, and narrowing it drops only what 127 - spare bits cannot hold."""
+    g = random.Random(11)
+    for trial in range(3000):
+        m = g.randint(1, 6)
+        bits = g.choice([0, 1, 40, 90, 106, 107, 110, 123])
+        v = [g.getrandbits(bits) * g.choice([-1, 1]) if bits else 0 for _ in range(m)]
+        lo = [g.getrandbits(20) if trial % 3 else g.choice([0, (1 << 20) - 1]) for _ in range(m)]
+        sh = g.choice([0, 0, 1, 7, 19, 20, 21, 60, 126, 127, 300])
+        out, so = (C.c_longlong * 2)(), C.c_int()
+        lib.tots_total(m, (C.c_longlong * (2 * m))(*[t for x in v for t in words(x)]), (C.c_uint * m)(*lo), sh, spare,
+                       out, C.byref(so))
+        got = signed(out[0], out[1])
+        full = sum((x << 20) + l for x, l in zip(v, lo))  # units 2^-20
+        full = full >> sh if sh < 127 else 0
+        assert abs(got) <= 1 << (127 - spare)
+        assert -20 <= so.value <= spare
+        assert got == full >> (so.value + 20)
+        if so.value > -20:
+            assert abs(got) >= 1 << (126 - spare - 1)
