@@ -697,8 +697,9 @@ __global__ void __launch_bounds__(kThreads, 1)
           const int ysb = SHARED ? 0 : KXP;
           for (int y = 0; y < NY; ++y) {
             const int cy = ysb + yq + y;
-            const int dx = Erun[xl] ? Enew[xl] - Erun[xl] : 0;
-            const int dy = Erun[cy] ? Enew[cy] - Erun[cy] : 0;
+            // (a column of zeros and subnormals so far, exponent 0, stands on the grid of exponent 1)
+            const int dx = max(Enew[xl], 1) - max(Erun[xl], 1);
+            const int dy = max(Enew[cy], 1) - max(Erun[cy], 1);
             for (int q = 0; q < kParts; ++q) total_shift(tot[q * NY + y], dx + dy);
           }
         }

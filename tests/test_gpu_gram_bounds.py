@@ -78,3 +78,22 @@ def test_short_products(eo, ctx, monkeypatch, n, k):
         rh, rl = oracle.gram(x, y)
         err = np.abs((gh.cpu().numpy() - rh) + (gl.cpu().numpy() - rl))
         assert np.all(err <= 2.0 ** -105 * np.abs(rh) + n * 2.0 ** -105), float(np.log2(err.max() / n))
+
+
+@pytest.mark.parametrize("n,kx,ky", [(300_000, 16, 0), (300_000, 9, 5), (200_000, 40, 17), (1_200_000, 4, 0), (600_000, 8, 0)])
+def test_columns_that_begin_with_subnormals(eo, ctx, n, kx, ky):
+    """A column whose first panels hold subnormals only: they stand on the grid of
+    exponent 1 and are shifted like any others when the first normal value
+    raises the column's exponent."""
+    x = synth.gaussian(n, kx, 3300 + kx)
+    y = synth.gaussian(n, ky, 3400 + ky) if ky else None
+    for a in (x, y) if ky else (x,):
+        a[:600, -1] *= 2e-309
+        a[:600, 0] = 0.0
+        a[100:110, 0] = 5e-324
+    gh, gl = eo.gram(ctx, dev(x), None if y is None else dev(y))
+    rh, rl = oracle.gram(x, y)
+    y = x if y is None else y
+    err = np.abs((gh.cpu().numpy() - rh) + (gl.cpu().numpy() - rl))
+    tol = 2.0 ** -104 * np.abs(rh) + n * 2.0 ** -103 * np.outer(np.abs(x).max(0), np.abs(y).max(0))
+    assert np.all(err <= tol), float((err / tol).max())
