@@ -220,51 +220,11 @@ FX_HD int clz128(u128 u) {
   return h ? clz64(h) : 64 + clz64((unsigned long long)u);
 }
 
-// w 2^s with |w| < 2^(127 - spare), so that 2^spare of such integers of one s
-// add up in 128 bits: shifted down (floor) only when w is larger.
-FX_HD void make_room(i128& w, int& s, int spare) {
-  const int over = spare + 1 - clz128(w < 0 ? ~(u128)w : (u128)w);
-  if (over > 0) {
-    w >>= over;
-    s += over;
-  }
-}
-
-// An exact total hi + lo 2^-20 (0 <= lo < 2^20) of terms given the same way.
-constexpr int kLowBits = 20;
-struct Total {
-  i128 hi;
-  unsigned lo;
-};
-FX_HD void total_add(Total& t, i128 hi, unsigned lo) {
-  lo += t.lo;
-  t.hi += hi + (i128)(lo >> kLowBits);
-  t.lo = lo & ((1u << kLowBits) - 1u);
-}
-// t 2^-sh, rounded down.
-FX_HD void total_shift(Total& t, int sh) {
-  if (sh <= 0) return;
-  constexpr unsigned mask = (1u << kLowBits) - 1u;
-  if (sh >= 127) {
-    t.hi = 0;
-    t.lo = 0;
-    return;
-  }
-  t.lo = sh < kLowBits ? (((unsigned)t.hi << (kLowBits - sh)) & mask) | (t.lo >> sh)
-                       : (unsigned)(t.hi >> (sh - kLowBits)) & mask;
-  t.hi >>= sh;
-}
-// w + lo 2^-20 in units 2^s as one integer with |w| < 2^(127 - spare), rounded
-// down: as many of the low bits as there is room for.
-FX_HD i128 total_narrow(i128 w, unsigned lo, int spare, int& s) {
-  const int room = clz128(w < 0 ? ~(u128)w : (u128)w) - 1 - spare;
-  if (room <= 0) {
-    make_room(w, s, spare);
-    return w;
-  }
-  const int g = room < kLowBits ? room : kLowBits;
-  s -= g;
-  return (i128)((u128)w << g) | (i128)(lo >> (kLowBits - g));
+// Bits dropped from the sums of `rows` products, each below 2^124 (1 + 2^-7), so
+// that their total stays below 2^127: ceil(log2(rows)) - 2, none for four rows.
+FX_HD int fold_bits(unsigned rows) {
+  const int b = rows > 1u ? 64 - clz64(rows - 1u) : 0;
+  return b > 2 ? b - 2 : 0;
 }
 
 // Double with magnitude m * 2^e2 (2^52 <= m < 2^53, or m == 0) and the given sign.

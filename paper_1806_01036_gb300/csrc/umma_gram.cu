@@ -34,12 +34,13 @@
 //  * before an accumulator can exceed 2^24 in magnitude (group_pairs below)
 //    the accumulators are read back (tcgen05.ld), converted to integers,
 //    added to 32-bit running sums per (lane, column) kept in TMEM and set
-//    back to zero.  The running sums are folded into a total of 128 + 20 bits in
-//    the units of the integer engine (2^(Ax + Ay - 2148)) and 2^-20 of them every
-//    kFoldDrains drains, before an alignment exponent grows, and at the end.
-//    The lanes' totals are added with all their bits; a row chunk's partial is
-//    their sum rounded down once, to the finest unit that 127 bits hold, and the
-//    partials go through the same exact, order-free reduction (fx_gram_reduce).
+//    back to zero.  The running sums are folded into 128-bit totals every
+//    kFoldDrains drains, before an alignment exponent grows, and at the end.  A
+//    fold drops only the bits that the sum of the chunk's rows could push out of
+//    127 (fold_bits: 5 for 132 rows, 13 for 26,000, 20 for the 2^22 of the
+//    largest chunk; of all parts' rows when parts are added up): the unit is
+//    2^(Ax + Ay - 2168 + drop).  The row-chunk partials go through the same exact,
+//    order-free reduction (fx_gram_reduce).
 //
 // Error per product x y: the dropped digit pairs (d >= 15, twelve of weight
 // 2^88 and fewer of smaller weights, each product at most 2^14) sum to less
@@ -47,10 +48,11 @@
 // more than 57 binades below A is truncated by less than one unit, which with
 // max|x| >= 2^(109 - h) units for a headroom h is 2^(h - 109) max|x| max|y| of a
 // product.  Together, with the same for y: below 2^-105.7 max|x| max|y| (h = 2).
-// A growth and a chunk's rounding add one unit of 2^-20 each, 2^-118 max|x|
-// max|y| (or 2^-126 of the chunk's sum if that is more).  (Totals that dropped
-// the 20 bits lane by lane, 24 times an entry of a symmetric tile, were off by
-// 2^-96.2 max|x| max|y| on two rows.)
+// A fold rounds a lane's sum down by less than a unit, 2^(drop - 118) max|x|
+// max|y|, and an entry of a symmetric tile adds 24 lanes: spread over the rows
+// 2^-114 a product, and on the longest chunks, which fold many times, 2^-108.
+// (Always dropping 20 bits was off by 2^-96.2 on two rows; keeping them
+// in a word of its own per lane made a product of few rows 14.6 -> 17.5 us.)
 //
 // Pipeline per CTA (one per SM, 16 warps of 128 registers): the values of a
 // panel of P rows arrive by TMA (two panels ahead, 16-row boxes with 128-byte
@@ -110,7 +112,7 @@ constexpr int kThreads = 32 * kWarps;
 constexpr int kIssuer = 32 * kConvWarps;    // the thread that issues the MMAs
 constexpr int kLanes = 128;                   // MMA M = TMEM lanes
 constexpr int kDiag = 14;                     // last digit diagonal kept
-constexpr int kOffsetDigits = 2148;
+constexpr int kOffsetDigits = 2168;  // value of h: h 2^(Ax + Ay - 2168)
 // Running sums grow by at most 2^24 per drain: exact in 32 bits for 127.
 constexpr int kFoldDrains = 96;
 constexpr int kPairRows = 1024;  // digit products of magnitude <= 2^14 that an FP32 accumulator holds exactly
@@ -174,7 +176,7 @@ struct Plan : Geo<KXP_, KYP_, SHARED_> {
   static constexpr int pairs_near = group_pairs(B::J, kNear, B::NQN), pairs_all = group_pairs(B::J, kAll, B::NQA);
   static constexpr size_t smem = B::bytes(P) + 1024;
   static_assert(FK >= 1 && P * pairs_near <= kPairRows && 16 * FK * pairs_all <= kPairRows, "a step fits the accumulators");
-  static_assert(2 * (size_t)dig_bytes >= (SHARED_ ? 2u : 1u) * (size_t)(kLanes + 1) * KYP_ * 20, "final sums fit the digit buffers");
+  static_assert(2 * (size_t)dig_bytes >= (SHARED_ ? 2u : 1u) * (size_t)(kLanes + 1) * KYP_ * 16, "final sums fit the digit buffers");
   static_assert(dig_bytes % 16 == 0 && B::LAA / 16 < (1u << 14), "descriptor strides");
 };
 
@@ -246,19 +248,18 @@ __device__ __forceinline__ void drain(unsigned ta, int q) {
 }
 
 // Running sums of this thread's TMEM lane (NY columns of every column block,
-// from address ts) -> the totals (units 2^(Ax + Ay - 2148)).
+// from address ts) -> the totals.
 // With h = sum_d S_d 2^(8 (14 - d)) the value is h 2^(Ax + Ay - 2168), and the
-// total takes h 2^-20 with all its bits (h may reach 2^146 in a chunk, so its low
-// 20 bits are a word of their own).  jl: the lane's digit phase (column block c
-// holds diagonal c + jl), so h = 2^(-8 jl) sum_c S_c 2^(8 (14 - c)) over c <= 14 - jl:
+// total takes floor(h 2^-drop), sh = 8 jl + drop.  jl: the lane's digit phase
+// (column block c holds diagonal c + jl), so h = 2^(-8 jl) sum_c S_c 2^(8 (14 - c))
+// over c <= 14 - jl:
 // four sums of neighbouring blocks in 64 bits each, five words, one shift.
 // (Horner's rule on 128-bit integers took 12,000 to 18,000 cycles, most of a
 // product of few rows.)  Out of line: its registers would cost the panel loop.
 // LAST: the accumulators (256 columns before) are added in, not drained first.
 template <class G, bool LAST>
-__device__ __noinline__ void fold(unsigned ts, int jl, Total* tot) {
+__device__ __noinline__ void fold(unsigned ts, int jl, int sh, i128* tot) {
   constexpr int KYP = G::KYP, NY = KYP / 4;
-  const int sh = 8 * jl + kLowBits;
 #pragma unroll 1
   for (int y = 0; y < NY; ++y) {  // (one column at a time: few registers)
     unsigned s[kDiag + 1];
@@ -304,15 +305,12 @@ __device__ __noinline__ void fold(unsigned ts, int jl, Total* tot) {
       w[3] = (unsigned)t;
       w[4] = (unsigned)(t >> 32);
       w[5] = w[6] = (unsigned)((int)w[4] >> 31);
-      // h: bits 8 jl up (the ones below are zero), its low bits and the rest
-      const unsigned low = __funnelshift_r(sh - kLowBits < 32 ? w[0] : w[1], sh - kLowBits < 32 ? w[1] : w[2],
-                                           (unsigned)(sh - kLowBits)) & ((1u << kLowBits) - 1u);
       unsigned a[5], o[4];
 #pragma unroll
       for (int i = 0; i < 5; ++i) a[i] = sh < 32 ? w[i] : sh < 64 ? w[i + 1] : w[i + 2 < 7 ? i + 2 : 6];
 #pragma unroll
       for (int i = 0; i < 4; ++i) o[i] = __funnelshift_r(a[i], a[i + 1], (unsigned)sh);
-      total_add(tot[part * NY + y], (i128)from_words(o[3], o[2], o[1], o[0]), low);
+      tot[part * NY + y] += (i128)from_words(o[3], o[2], o[1], o[0]);
     }
   }
 }
@@ -509,10 +507,12 @@ __global__ void __launch_bounds__(kThreads, 1)
   const unsigned tq = taddr + ((unsigned)Lq << 16);             // the lane quarter's columns
   const unsigned tsum = tq + (unsigned)yq + 256u;               // the running sums of its columns
   // the exact totals; touched once per fold, so they are kept out of registers
-  Total totals[kParts * NY];
-  Total* tot = totals;
+  i128 totals[kParts * NY];
+  i128* tot = totals;
   asm volatile("" : "+l"(tot)::"memory");
-  for (int y = 0; y < kParts * NY; ++y) tot[y] = Total{0, 0u};
+  for (int y = 0; y < kParts * NY; ++y) tot[y] = 0;
+  // bits of h that a total drops: 127 hold the sum of the chunk's rows (PACK: of all parts)
+  const int drop = fold_bits((unsigned)rows_per_chunk * (PACK ? 16u >> lg : 1u));
 
   // the running sums and, first, the accumulators at zero (this warp's share of the column blocks)
   auto zero_blocks = [&](unsigned t) {
@@ -579,7 +579,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     drain<KYP>(tq, warp >> 2);
     if (full) {  // all of the lane quarter's blocks are drained
       asm volatile("bar.sync %0, 128;" ::"r"(1 + (warp & 3)) : "memory");
-      fold<G, false>(tsum, jl, tot);
+      fold<G, false>(tsum, jl, 8 * jl + drop, tot);
       asm volatile("bar.sync %0, 128;" ::"r"(1 + (warp & 3)) : "memory");
       zero_blocks(tq + 256u);
     }
@@ -700,7 +700,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             // (a column of zeros and subnormals so far, exponent 0, stands on the grid of exponent 1)
             const int dx = max(Enew[xl], 1) - max(Erun[xl], 1);
             const int dy = max(Enew[cy], 1) - max(Erun[cy], 1);
-            for (int q = 0; q < kParts; ++q) total_shift(tot[q * NY + y], dx + dy);
+            for (int q = 0; q < kParts; ++q) tot[q * NY + y] = w_shift(tot[q * NY + y], dx + dy);
           }
         }
         __syncthreads();
@@ -799,7 +799,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (warp == 0) mbar_wait_final(fb0 + 8u * (unsigned)((step - 1) & 1), (unsigned)((step - 1) >> 1) & 1u, &bad);
     wait_step(step - 1);
     tc_fence_after();  // (the drains' running sums: before the barrier above)
-    fold<G, true>(tsum, jl, tot);
+    fold<G, true>(tsum, jl, 8 * jl + drop, tot);
     tc_fence_before();
   }
   __syncthreads();
@@ -813,37 +813,19 @@ __global__ void __launch_bounds__(kThreads, 1)
   // the loads of a column or of its transpose meet in a bank)
   constexpr int kRow = kLanes + 1;
   i128* red = reinterpret_cast<i128*>(dig);  // kParts x KYP x 129 entries (the MMAs are done)
-  unsigned* redl = reinterpret_cast<unsigned*>(red + kParts * KYP * kRow);  // and their low bits
   for (int q = 0; q < kParts; ++q)
-    for (int y = 0; y < NY; ++y) {
-      const int at = (q * KYP + yq + y) * kRow + L;
-      red[at] = tot[q * NY + y].hi;
-      redl[at] = tot[q * NY + y].lo;
-    }
+    for (int y = 0; y < NY; ++y) red[(q * KYP + yq + y) * kRow + L] = tot[q * NY + y];
   __syncthreads();
-  // Columns i and yo of the tile: the lanes' totals are added with all their bits
-  // and rounded down once.  (A part's total may take all 127 bits: 2^22 rows of
-  // the largest values the exponents' headroom allows.  PACK: with room for the
-  // sum of the 16 >> lg parts.)
-  auto output = [&](int i, int yo) {
+  auto output = [&](int i, int yo) {  // columns i and yo of the tile
     i128 w = 0;
-    unsigned l = 0;  // (24 terms below 2^20)
-    auto add = [&](int at) {
-      w += red[at];
-      l += redl[at];
-    };
     for (int b = 0; b < J; ++b) {
-      add(yo * kRow + b * KXP + i);
-      if constexpr (SHARED) {
-        add((KYP + yo) * kRow + b * KXP + i);
-        add((KYP + i) * kRow + b * KXP + yo);
-      }
+      w += red[yo * kRow + b * KXP + i];
+      if constexpr (SHARED) w += red[(KYP + yo) * kRow + b * KXP + i] + red[(KYP + i) * kRow + b * KXP + yo];
     }
     FxPart o;
-    o.s = max(Erun[i], 1) + max(Erun[(SHARED ? 0 : KXP) + yo], 1) - kOffsetDigits;
-    w = total_narrow(w + (i128)(l >> kLowBits), l & ((1u << kLowBits) - 1u), PACK ? 4 - lg : 0, o.s);
     o.wl = (long long)(unsigned long long)(u128)w;
     o.wh = (long long)(w >> 64);
+    o.s = max(Erun[i], 1) + max(Erun[(SHARED ? 0 : KXP) + yo], 1) - kOffsetDigits + drop;
     o.flag = flag | bad;
     o.pad = 0;
     return o;
