@@ -67,11 +67,15 @@
 // accumulators when due, and arrives; the sixteenth warp then issues the
 // panel's MMAs and the copies of the panel after the next.  A warp that holds a
 // zero masks it (4e6 x 64 + 16 with a zero column 1.04 ms, with every tenth value
-// zero 1.04, dense 1.02; 2.76 when a zero sent the panel through the branch that
-// follows).  A panel that was seen to hold a value above its column's exponent or
-// one other than zero below the near window sends every warp through a slower
-// branch with barriers: exponents grow, and with a value below the window the
-// panel is stored and multiplied in parts with all 14 slabs.  Every wait is
+// zero 1.04, dense 1.02).  A panel that holds a value other than zero below the
+// near window is stored and multiplied with all 14 slabs, in steps that fit the
+// digit buffers; only the warps that hold such values cut the last four digits,
+// in a branch of its own, the others store zeros.  (One value in 100,000 / 10,000
+// / 1,000 below it: 1.07 / 1.30 / 1.79 ms; through barriers, a second read and a
+// second conversion of the panel by every warp, as a growth takes it, 1.13 / 1.80 /
+// 3.40; 15 7-bit slabs of a panel in one buffer took 1.42 / 1.43 / 1.51.)  A value
+// above its column's exponent sends every warp through a branch with barriers in
+// which the exponents grow.  Every wait is
 // bounded; a wait that runs out marks the partials non-finite, so the result
 // is NaN.  Operands that TMA cannot address (a base not 16-byte aligned, an
 // odd leading dimension, FP32) are copied by the converter threads with
@@ -177,7 +181,7 @@ struct Plan : Geo<KXP_, KYP_, SHARED_> {
   static constexpr unsigned b_off_all = B::LAA * (2 * FK);
   static constexpr int pairs_near = group_pairs(B::J, kNear, B::NQN), pairs_all = group_pairs(B::J, kAll, B::NQA);
   static constexpr size_t smem = B::bytes(P) + 1024;
-  static_assert(FK >= 1 && P * pairs_near <= kPairRows && 16 * FK * pairs_all <= kPairRows, "a step fits the accumulators");
+  static_assert(FK >= 1 && NF >= 2 && P * pairs_near <= kPairRows && 16 * FK * pairs_all <= kPairRows, "a step fits the accumulators");
   static_assert(2 * (size_t)dig_bytes >= (SHARED_ ? 2u : 1u) * (size_t)(kLanes + 1) * KYP_ * 16, "final sums fit the digit buffers");
   static_assert(dig_bytes % 16 == 0 && B::LAA / 16 < (1u << 14), "descriptor strides");
 };
@@ -201,6 +205,25 @@ __device__ __forceinline__ void store_near(unsigned dst, unsigned stride, const 
   }
 }
 
+// The fourteen slabs: lane words z of the first ten digits, `low` (null: zero) of the last four.
+__device__ __forceinline__ void store_all(unsigned dst, unsigned stride, const unsigned (&z)[4][5], const Sign2 (&sg)[4],
+                                          const unsigned* low, unsigned e1024) {
+  store_near(dst, stride, z, sg, e1024);
+#pragma unroll 1
+  for (int i = 0; i < 2; ++i) {
+    const unsigned at = dst + (unsigned)(kNear + 2 * i) * stride;
+    if (low) {
+      st_digits(at, digit_hi(low[i], e1024, sg[0]), digit_hi(low[2 + i], e1024, sg[1]), digit_hi(low[4 + i], e1024, sg[2]),
+                digit_hi(low[6 + i], e1024, sg[3]));
+      st_digits(at + stride, digit_lo(low[i], e1024, sg[0]), digit_lo(low[2 + i], e1024, sg[1]),
+                digit_lo(low[4 + i], e1024, sg[2]), digit_lo(low[6 + i], e1024, sg[3]));
+    } else {
+      st_digits(at, 0u, 0u, 0u, 0u);
+      st_digits(at + stride, 0u, 0u, 0u, 0u);
+    }
+  }
+}
+
 // Barrier 0 over the CTA, true if any thread passes true.
 __device__ __forceinline__ bool bar_any(bool v) { return __syncthreads_or(v ? 1 : 0) != 0; }
 
@@ -219,6 +242,24 @@ __device__ __forceinline__ void near_lanes(const double (&v)[8], int A, unsigned
     z[m][2] = __byte_perm(a2, b2, 0x5410);
     z[m][3] = __byte_perm(a1, b1, 0x7632);
     z[m][4] = __byte_perm(a1, b1, 0x5410);
+  }
+}
+
+// The same for any values, with the lane words of the last four digits in low.
+__device__ __forceinline__ void any_lanes(const double (&v)[8], int A, unsigned (&z)[4][5], Sign2 (&sg)[4], unsigned* low) {
+#pragma unroll
+  for (int m = 0; m < 4; ++m) {
+    unsigned a[4], b[4];
+    any_words(v[2 * m], A, a);
+    any_words(v[2 * m + 1], A, b);
+    sg[m] = sign2(v[2 * m], v[2 * m + 1]);
+    z[m][0] = __byte_perm(a[3], b[3], 0x5410);
+    z[m][1] = __byte_perm(a[2], b[2], 0x7632);
+    z[m][2] = __byte_perm(a[2], b[2], 0x5410);
+    z[m][3] = __byte_perm(a[1], b[1], 0x7632);
+    z[m][4] = __byte_perm(a[1], b[1], 0x5410);
+    low[2 * m] = __byte_perm(a[0], b[0], 0x7632);
+    low[2 * m + 1] = __byte_perm(a[0], b[0], 0x5410);
   }
 }
 
@@ -350,7 +391,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   __shared__ __align__(8) unsigned long long full_bar[2], stage_bar[2], ready_bar[2];
   __shared__ unsigned tmem_base;
   __shared__ int flag, bad;
-  // spec[p & 1] = p: panel p holds a value that is not near; written before the arrivals for panel p - 1
+  // spec[p & 1]: 2 p + 1 if panel p holds a value above its column's exponent, else 2 p if one other
+  // than zero below the near window (the largest wins); written before the arrivals for panel p - 1's last step
   __shared__ int spec[2];
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -465,21 +507,36 @@ __global__ void __launch_bounds__(kThreads, 1)
     wlo = (unsigned)f << 21;
     wrange = ((unsigned)(A + 1) << 21) - wlo;
   };
-  // Whether a value other than zero is outside it.  Zeros (rows past the chunk's
-  // end in its last panel among them) are cut by the warps that hold one, with a
-  // mask: `zeros`, over the warp.
-  bool zeros = false;
-  auto outside = [&]() {
+  // Whether a value lies above it.  Over the warp: `zeros`, a value that is zero
+  // (rows past the chunk's end in its last panel among them) or below it, `below`,
+  // one other than zero below it; the warp cuts its values accordingly.
+  bool zeros = false, below = false;
+  auto look = [&]() {
     unsigned k = 0;
 #pragma unroll
     for (int m = 0; m < 8; ++m) k = max(k, 2u * hi32(v[m]) - wlo);
     zeros = __any_sync(0xffffffffu, k >= wrange);
+    below = false;
     if (!zeros) return false;
-    bool off = false;
+    bool up = false, low = false;
 #pragma unroll
-    for (int m = 0; m < 8; ++m) off |= 2u * hi32(v[m]) - wlo >= wrange && ((hi32(v[m]) & 0x7fffffffu) | lo32(v[m])) != 0u;
-    return off;
+    for (int m = 0; m < 8; ++m) {
+      const unsigned a = hi32(v[m]) & 0x7fffffffu;
+      const bool out = 2u * hi32(v[m]) - wlo >= wrange && (a | lo32(v[m])) != 0u;
+      const bool above = 2u * a >= wlo;
+      up |= out && above;
+      low |= out && !above;
+    }
+    below = __any_sync(0xffffffffu, low);
+    return up;
   };
+  // the values of a panel that `below` holds for, and the lane words of their
+  // digits 10..13; touched rarely, so they are kept out of registers
+  struct {
+    double v[8];
+    unsigned low[8];
+  } rare_, *rare = &rare_;
+  asm volatile("" : "+l"(rare)::"memory");
   if (npan > 0) {
     fetch(0);
     if (!TMA || npan > 1) fetch(1);
@@ -622,11 +679,16 @@ __global__ void __launch_bounds__(kThreads, 1)
     dirty &= ~(1 << (step & 1));
   };
   // One panel: convert panel p (its values are in v), take panel p + 1's values
-  // and look whether they are near, then, once every warp has stored panel p - 1
-  // (ready), store the digits and arrive.  The last warp issues panel p - 1's
-  // MMAs and the copies of panel p + 1's successor at that point instead.
+  // and look whether they are near, then, once every warp has stored the step
+  // before (ready), store the digits and arrive.  The last warp issues that
+  // step's MMAs and the copies of panel p + 1's successor at that point instead.
   const bool conv = warp < kConvWarps;
   const unsigned rb0 = smem_u32(&ready_bar[0]);
+  auto wait_ready = [&](int s) { return mbar_wait(rb0 + 8u * (unsigned)(s & 1), (unsigned)(s >> 1) & 1u, &bad); };
+  auto arrive = [&]() {  // this warp's digits of the last step are stored
+    __syncwarp();
+    if (conv && lane == 0) mbar_arrive(rb0 + 8u * (unsigned)((step - 1) & 1));
+  };
   if (npan > 0) {  // the columns' exponents from panel 0
     if (conv) {
       load(0);
@@ -646,7 +708,10 @@ __global__ void __launch_bounds__(kThreads, 1)
       te = Enew[slot];
       set_window();
     }
-    if (conv && outside()) *reinterpret_cast<volatile int*>(&spec[0]) = 0;
+    if (conv) {
+      look();  // (nothing above: the exponents are the panel's)
+      if (below && lane == 0) atomicMax(&spec[0], 0);
+    }
   }
   __syncthreads();
   if (TMA && npan > 2) fetch(2);  // (TMA: panel 0's values are in registers)
@@ -654,41 +719,49 @@ __global__ void __launch_bounds__(kThreads, 1)
   for (int p = 0; p < npan; ++p) {
     unsigned z[4][5];
     Sign2 sg[4];
-    bool off = false;
+    bool up = false, cut_all = below;
     if (conv) {
+      if (below) {  // cut below, where every warp is known to take that branch
+#pragma unroll
+        for (int i = 0; i < 8; ++i) rare->v[i] = v[i];
+      }
       if (zeros) near_lanes<true>(v, max(te, 1), z, sg);
       else near_lanes<false>(v, max(te, 1), z, sg);
       if constexpr (!TMA) fetch(p + 2);
       if (p + 1 < npan) {
         load(p + 1);
-        off = outside();
+        up = look();
       }
     }
-    if (p > 0) {
-      if (!mbar_wait(rb0 + 8u * (unsigned)((p - 1) & 1), (unsigned)((p - 1) >> 1) & 1u, &bad)) break;
+    if (step > 0) {
+      if (!wait_ready(step - 1)) break;
       if (!conv) {
         // every warp has taken panel p's values: its staging buffer is free
         if (TMA && p + 2 < npan) fetch(p + 2);
-        issue();  // panel p - 1's
+        issue();  // the last step's
       }
     }
     int ks = P / 16, cost = P * G::pairs_near;
     bool all = false;
-    if (*reinterpret_cast<volatile int*>(&spec[p & 1]) == p) {
-      // Panel p holds a value that is not near: every warp comes here.
-      __syncthreads();
-      double u[8];
-      unsigned m = 0;  // largest magnitude
-      const int64_t pr = (int64_t)p * P;
+    // (Nobody writes this word for panel p + 2 before the last warp has read it:
+    // a converter that has something to write waits for MMAs first that the last
+    // warp issues after this, or stands in panel p's barriers.)
+    const int sp = *reinterpret_cast<volatile int*>(&spec[p & 1]);
+    if ((sp >> 1) == p) {
+      // Panel p is not near: every warp comes here.
+      const bool grow = sp & 1;
+      if (grow) {
+        __syncthreads();
+        double u[8];
+        unsigned m = 0;  // largest magnitude
+        const int64_t pr = (int64_t)p * P;
 #pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        u[i] = (valid && r0 + pr + 8 * kc + i < r1) ? (sizeof(T) == 8 ? (double)src[pr + i] : widen((float)src[pr + i])) : 0.0;
-        m = max(m, abs_hi(u[i]));
-      }
-      // exponents (subnormals never raise a column: its alignment exponent is at least 1)
-      const bool up = valid && m >= ((unsigned)te + 1u) << 20;
-      if (bar_any(up)) {
-        if (up) {
+        for (int i = 0; i < 8; ++i) {
+          u[i] = (valid && r0 + pr + 8 * kc + i < r1) ? (sizeof(T) == 8 ? (double)src[pr + i] : widen((float)src[pr + i])) : 0.0;
+          m = max(m, abs_hi(u[i]));
+        }
+        // exponents (subnormals never raise a column: its alignment exponent is at least 1)
+        if (valid && m >= ((unsigned)te + 1u) << 20) {
           const int e = (int)(m >> 20);
           if (e == 2047) flag = 1;
           // (finite exponents stay below 2047, so that an Inf or NaN always raises)
@@ -713,61 +786,46 @@ __global__ void __launch_bounds__(kThreads, 1)
           te = Enew[slot];
           set_window();
         }
-        __syncthreads();
-      }
-      // a nonzero value (normal or not) below the window
-      const int A = max(te, 1);
-      bool below = false;
-      const unsigned floor = near_floor(A);
+        // a nonzero value (normal or not) below the window
+        const unsigned floor = near_floor(max(te, 1));
+        cut_all = false;
 #pragma unroll
-      for (int i = 0; i < 8; ++i) below |= valid && (abs_hi(u[i]) | lo32(u[i])) != 0u && abs_hi(u[i]) < floor;
-      all = bar_any(below);
-      if (!all) {
-        unsigned y[4][5];
-        Sign2 sy[4];
-        near_lanes<true>(u, A, y, sy);
-        put(y, sy);
+        for (int i = 0; i < 8; ++i) {
+          cut_all |= valid && (abs_hi(u[i]) | lo32(u[i])) != 0u && abs_hi(u[i]) < floor;
+          rare->v[i] = u[i];
+        }
+        cut_all = __any_sync(0xffffffffu, cut_all);
+        all = bar_any(cut_all);
+        near_lanes<true>(u, max(te, 1), z, sg);
       } else {
-        Sign2 sy[4];
+        all = true;
+      }
+      if (!all) {
+        put(z, sg);
+      } else {
+        // All digits: the panel in NF steps, the items of a step's K chunks each.
+        if (cut_all) {
+          double u[8];
+#pragma unroll
+          for (int i = 0; i < 8; ++i) u[i] = rare->v[i];
+          any_lanes(u, max(te, 1), z, sg, rare->low);
+        }
 #pragma unroll 1
         for (int h = 0; h < G::NF; ++h) {
-          if (h) {  // the previous step's digits are stored: its MMAs
+          if (h) {  // the step before is stored: its MMAs
             finish_step(G::FK, true, 16 * G::FK * G::pairs_all);
-            __syncthreads();
+            arrive();
+            wait_ready(step - 1);
             issue();
           }
-          const unsigned db = (unsigned)(step & 1) * G::dig_bytes;
-          if (step >= 2) wait_step(step - 2);
           const int k = kc - h * 2 * G::FK;  // K chunk within the step
           if (mine && k >= 0 && k < 2 * G::FK) {
-            const unsigned dst =
-                dig_s + db + (isb ? G::b_off_all + (unsigned)k * G::LBA : (unsigned)k * G::LAA) + (unsigned)lc * 16u;
+            if (step >= 2) wait_step(step - 2);
+            const unsigned dst = dig_s + (unsigned)(step & 1) * G::dig_bytes +
+                                 (isb ? G::b_off_all + (unsigned)k * G::LBA : (unsigned)k * G::LAA) + (unsigned)lc * 16u;
             const unsigned st = 16u * (unsigned)(isb ? KYP : KXP);
-            unsigned y[4][7];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-              unsigned a[4], b[4];
-              any_words(u[2 * i], A, a);
-              any_words(u[2 * i + 1], A, b);
-              sy[i] = sign2(u[2 * i], u[2 * i + 1]);
-              y[i][0] = __byte_perm(a[3], b[3], 0x5410);
-#pragma unroll
-              for (int j = 0; j < 3; ++j) {
-                y[i][1 + 2 * j] = __byte_perm(a[2 - j], b[2 - j], 0x7632);
-                y[i][2 + 2 * j] = __byte_perm(a[2 - j], b[2 - j], 0x5410);
-              }
-            }
-#pragma unroll
-            for (int i = 0; i < 7; ++i) {
-              const Sign2 s0 = i ? sy[0] : top(sy[0]), s1 = i ? sy[1] : top(sy[1]);
-              const Sign2 s2 = i ? sy[2] : top(sy[2]), s3 = i ? sy[3] : top(sy[3]);
-              st_digits(dst + (unsigned)(2 * i) * st, digit_hi(y[0][i], e1024, s0), digit_hi(y[1][i], e1024, s1),
-                        digit_hi(y[2][i], e1024, s2), digit_hi(y[3][i], e1024, s3));
-              st_digits(dst + (unsigned)(2 * i + 1) * st, digit_lo(y[0][i], e1024, sy[0]), digit_lo(y[1][i], e1024, sy[1]),
-                        digit_lo(y[2][i], e1024, sy[2]), digit_lo(y[3][i], e1024, sy[3]));
-            }
-            if (!isb)
-              for (int s = kAll; s < G::SAA; ++s) st_digits(dst + (unsigned)s * st, 0u, 0u, 0u, 0u);
+            if (valid) store_all(dst, st, z, sg, cut_all ? rare->low : nullptr, e1024);
+            for (int s = valid ? kAll : 0; s < (isb ? kAll : G::SAA); ++s) st_digits(dst + (unsigned)s * st, 0u, 0u, 0u, 0u);
           }
           dirty |= 1 << (step & 1);
         }
@@ -779,7 +837,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       // exponents may have grown
       if (conv && p + 1 < npan) {
         load(p + 1);
-        off = outside();
+        up = look();
       } else {
 #pragma unroll
         for (int i = 0; i < 8; ++i) v[i] = 0.0;
@@ -788,11 +846,11 @@ __global__ void __launch_bounds__(kThreads, 1)
       put(z, sg);
     }
     finish_step(ks, all, cost);
-    if (conv) {
-      if (off) *reinterpret_cast<volatile int*>(&spec[(p + 1) & 1]) = p + 1;
-      __syncwarp();
-      if (lane == 0) mbar_arrive(rb0 + 8u * (unsigned)(p & 1));
+    if (conv && (up || below)) {
+      if (up) atomicMax(&spec[(p + 1) & 1], 2 * p + 3);
+      else if (lane == 0) atomicMax(&spec[(p + 1) & 1], 2 * p + 2);
     }
+    arrive();
   }
 
   if constexpr (!TMA) asm volatile("cp.async.wait_all;" ::: "memory");  // the last (empty) copies

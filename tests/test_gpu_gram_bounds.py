@@ -126,3 +126,39 @@ def test_zeros_cost_little(eo, ctx, n, kx, ky):
     rare = best(x)
     x[kx - 1] = 0.0
     assert max(rare, best(x)) <= 1.5 * dense
+
+
+@pytest.mark.parametrize("rate", [2e-5, 1e-3])
+@pytest.mark.parametrize("kx,ky", [(64, 16), (40, 9), (20, 4), (16, 16), (16, 0), (4, 0)])
+@pytest.mark.parametrize("odd_ld", [False, True])
+def test_panels_of_every_kind_in_turn(eo, ctx, kx, ky, rate, odd_ld):
+    """Many panels a CTA: near ones, ones with values below the near window (all
+    digits, in steps), with zeros, and with growing exponents, in random order."""
+    import torch
+
+    n = 500_003
+    g = synth.rng(3600 + kx)
+
+    def block(k, seed):
+        a = synth.gaussian(n, k, seed)
+        m = g.random(a.shape) < rate
+        a[m] *= np.ldexp(1.0, -g.integers(20, 110, int(m.sum())))
+        a[g.random(a.shape) < rate] = 0.0
+        for i in range(40):
+            a[g.integers(0, n), g.integers(0, k)] *= 2.0 ** g.integers(2, 9)
+        return a
+
+    def put(a):
+        ld = n + 1 if not odd_ld else n
+        t = torch.full((a.shape[1], ld), float("nan"), dtype=torch.float64, device="cuda")
+        t[:, :n] = torch.from_numpy(np.ascontiguousarray(a.T))
+        return t.t()[:n]
+
+    x = block(kx, 3700 + kx)
+    y = block(ky, 3800 + ky) if ky else None
+    gh, gl = eo.gram(ctx, put(x), None if y is None else put(y))
+    rh, rl = oracle.gram(x, y)
+    y = x if y is None else y
+    err = np.abs((gh.cpu().numpy() - rh) + (gl.cpu().numpy() - rl))
+    tol = 2.0 ** -104 * np.abs(rh) + n * 2.0 ** -103 * np.outer(np.abs(x).max(0), np.abs(y).max(0))
+    assert np.all(err <= tol), float((err / tol).max())
