@@ -224,9 +224,6 @@ __device__ __forceinline__ void store_all(unsigned dst, unsigned stride, const u
   }
 }
 
-// Barrier 0 over the CTA, true if any thread passes true.
-__device__ __forceinline__ bool bar_any(bool v) { return __syncthreads_or(v ? 1 : 0) != 0; }
-
 // Lane words of the eight values' near digits and their signs.
 template <bool ZERO>
 __device__ __forceinline__ void near_lanes(const double (&v)[8], int A, unsigned (&z)[4][5], Sign2 (&sg)[4]) {
@@ -393,7 +390,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   __shared__ int flag, bad;
   // spec[p & 1]: 2 p + 1 if panel p holds a value above its column's exponent, else 2 p if one other
   // than zero below the near window (the largest wins); written before the arrivals for panel p - 1's last step
-  __shared__ int spec[2];
+  __shared__ int spec[2], any_at;
+  __shared__ __align__(8) unsigned long long cta_bar;
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
@@ -406,6 +404,8 @@ __global__ void __launch_bounds__(kThreads, 1)
       mbar_init(smem_u32(&ready_bar[b]), kConvWarps);
       spec[b] = -1;
     }
+    any_at = -1;
+    mbar_init(smem_u32(&cta_bar), kWarps);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     flag = 0;
     bad = 0;
@@ -442,9 +442,11 @@ __global__ void __launch_bounds__(kThreads, 1)
   auto unit = [&](int p, int u) {
     return (unsigned)(p & 1) * G::stage_bytes + item + (((unsigned)(4 * (kc & 1) + u) ^ (unsigned)(lc & 7)) << 4);
   };
+  [[maybe_unused]] int fetched = 0;  // panels whose copies were issued (the thread that fetches)
   auto fetch = [&](int p) {
     if constexpr (TMA) {
       if (tid == kIssuer) {
+        fetched = p + 1;
         const unsigned bar = sb0 + 8u * (unsigned)(p & 1), dst = stage_s + (unsigned)(p & 1) * G::stage_bytes;
         const int xr = (int)(r0 + (int64_t)p * P);
         fence_proxy_async();
@@ -629,6 +631,15 @@ __global__ void __launch_bounds__(kThreads, 1)
     pend = 0;
   };
   // wait for the MMAs of step s (committed to its buffer's barrier)
+  // Barrier of the panel loop over all warps, bounded like every wait in it, so
+  // that warps which a wait that ran out has sent out of the loop hold up nobody.
+  int syncs = 0;
+  auto sync_all = [&]() {
+    __syncwarp();
+    if (lane == 0) mbar_arrive(smem_u32(&cta_bar));
+    mbar_wait(smem_u32(&cta_bar), (unsigned)syncs & 1u, &bad);
+    ++syncs;
+  };
   auto wait_step = [&](int s) { mbar_wait(fb0 + 8u * (unsigned)(s & 1), (unsigned)(s >> 1) & 1u, &bad); };
   // Empties the accumulators (after the MMAs of the steps before s) and, when
   // due or asked for, folds the running sums.
@@ -639,9 +650,13 @@ __global__ void __launch_bounds__(kThreads, 1)
     tc_fence_after();
     drain<KYP>(tq, warp >> 2);
     if (full) {  // all of the lane quarter's blocks are drained
-      asm volatile("bar.sync %0, 128;" ::"r"(1 + (warp & 3)) : "memory");
+      tc_fence_before();
+      sync_all();
+      tc_fence_after();
       fold<G, false>(tsum, jl, 8 * jl + drop, tot);
-      asm volatile("bar.sync %0, 128;" ::"r"(1 + (warp & 3)) : "memory");
+      tc_fence_before();
+      sync_all();
+      tc_fence_after();
       zero_blocks(tq + 256u);
     }
     tc_fence_before();
@@ -734,7 +749,8 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
     }
     if (step > 0) {
-      if (!wait_ready(step - 1)) break;
+      // (a wait that ran out: the whole warp leaves; nothing in the loop waits for it without a bound)
+      if (!__all_sync(0xffffffffu, wait_ready(step - 1))) break;
       if (!conv) {
         // every warp has taken panel p's values: its staging buffer is free
         if (TMA && p + 2 < npan) fetch(p + 2);
@@ -751,7 +767,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       // Panel p is not near: every warp comes here.
       const bool grow = sp & 1;
       if (grow) {
-        __syncthreads();
+        sync_all();
         double u[8];
         unsigned m = 0;  // largest magnitude
         const int64_t pr = (int64_t)p * P;
@@ -767,7 +783,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           // (finite exponents stay below 2047, so that an Inf or NaN always raises)
           atomicMax(&Enew[slot], e == 2047 ? e : min(e + EO_GRAM_HEADROOM, 2046));
         }
-        __syncthreads();
+        sync_all();
         if (used > 0) {
           empty(step, true);
           // totals onto the new grid: divide by 2^(growth of both columns' exponents)
@@ -780,7 +796,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             for (int q = 0; q < kParts; ++q) tot[q * NY + y] = w_shift(tot[q * NY + y], dx + dy);
           }
         }
-        __syncthreads();
+        sync_all();
         if (tid < G::COLS) Erun[tid] = Enew[tid];
         if (valid) {
           te = Enew[slot];
@@ -795,7 +811,9 @@ __global__ void __launch_bounds__(kThreads, 1)
           rare->v[i] = u[i];
         }
         cut_all = __any_sync(0xffffffffu, cut_all);
-        all = bar_any(cut_all);
+        if (cut_all && lane == 0) *reinterpret_cast<volatile int*>(&any_at) = p;
+        sync_all();
+        all = *reinterpret_cast<volatile int*>(&any_at) == p;
         near_lanes<true>(u, max(te, 1), z, sg);
       } else {
         all = true;
@@ -857,6 +875,11 @@ __global__ void __launch_bounds__(kThreads, 1)
   // the last step's MMAs, drain and fold
   __syncthreads();
   issue();
+  if (tid == kIssuer && *reinterpret_cast<volatile int*>(&bad)) {
+    // after a wait that ran out: this thread's own MMAs and copies end before TMEM and shared memory are released
+    if (step > 0) mbar_wait_final(fb0 + 8u * (unsigned)((step - 1) & 1), (unsigned)((step - 1) >> 1) & 1u, &bad);
+    for (int q = max(fetched - 2, 0); q < fetched; ++q) mbar_wait_final(sb0 + 8u * (unsigned)(q & 1), (unsigned)(q >> 1) & 1u, &bad);
+  }
   if (step > 0) {
     if (warp == 0) mbar_wait_final(fb0 + 8u * (unsigned)((step - 1) & 1), (unsigned)((step - 1) >> 1) & 1u, &bad);
     wait_step(step - 1);
