@@ -119,6 +119,7 @@ __device__ void finish_gates(const SmallGates& g, int run_update, int want_next)
 struct F64 {
   typedef double T;
   static constexpr size_t kBytes = 8;
+  static constexpr bool kLowParts = false;  // a given matrix's low parts are not read
   static constexpr bool kOneSided = false;
   struct Vec {
     double* p;
@@ -176,6 +177,7 @@ struct F64 {
 
 struct Wide {
   typedef wide T;
+  static constexpr bool kLowParts = true;
   static constexpr bool kOneSided = true;  // Jacobi on the Cholesky factor where it can
   static constexpr size_t kBytes = 20;  // significand, exponent and sign in arrays of their own
   struct Vec {
@@ -295,15 +297,15 @@ __device__ __forceinline__ void untri(int t, int& i, int& j) {  // the entry wit
   i = t - j * (j + 1) / 2;
 }
 
-// M's upper triangle into A; false (everywhere) if it has a NaN or Inf.  Ends with a barrier.
+// M's upper triangle into A; false (everywhere) if it has a NaN or Inf (in the parts that are read).  Ends with a barrier.
 template <class N>
-__device__ __forceinline__ bool load_upper(int k, const double* Mh, const double* Ml, int ldm, bool use_lo,
-                                           typename N::Vec A, int threads) {
+__device__ __forceinline__ bool load_upper(int k, const double* Mh, const double* Ml, int ldm, typename N::Vec A,
+                                           int threads) {
   bool ok = true;
   for (int t = threadIdx.x; t < k * (k + 1) / 2; t += threads) {
     int i, j;
     untri(t, i, j);
-    const double h = Mh[(size_t)j * ldm + i], l = Ml && use_lo ? Ml[(size_t)j * ldm + i] : 0.0;
+    const double h = Mh[(size_t)j * ldm + i], l = N::kLowParts && Ml ? Ml[(size_t)j * ldm + i] : 0.0;
     const bool fin = isfinite(h) && isfinite(l);
     ok = ok && fin;
     A.set(t, fin ? N::from(h, l) : N::zero());
@@ -330,7 +332,7 @@ __device__ __forceinline__ void chol_small_body(int k, const double* Mh, const d
   __shared__ T piv_inv;
   const int tid = threadIdx.x;
   if (tid == 0) flag = 0;
-  if (!load_upper<N>(k, Mh, Ml, ldm, true, A, kThreads) && tid == 0) flag = -1;
+  if (!load_upper<N>(k, Mh, Ml, ldm, A, kThreads) && tid == 0) flag = -1;
   // Square-root-free (L D L^T) elimination on the upper triangle: at step j
   // the pivot d_j = A(j,j) and the row A(j, j+1..) are those of the
   // standard algorithm before scaling, the Schur complement takes
@@ -922,7 +924,7 @@ __device__ __forceinline__ void svqb_small_body(int k, const double* Mh, const d
   __shared__ int rotates[KMAX / 2 + 1];
   __shared__ int rot_count, next_unit;
   const int tid = threadIdx.x, lane = tid & 31;
-  if (!load_upper<N>(k, Mh, Ml, ldm, true, A, kJacThreads)) {
+  if (!load_upper<N>(k, Mh, Ml, ldm, A, kJacThreads)) {
     if (tid == 0) {
       st->rank = -1;
       finish_gates(g, 0, 0);
