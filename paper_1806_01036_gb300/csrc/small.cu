@@ -755,7 +755,8 @@ __device__ __forceinline__ bool rotate_pair(int k, i128* wx, i128* wy, int& Ex, 
 // SVQB step of k = 32: about 10 ms with double-doubles on the FP64 pipe, 1.35 in
 // this form, 0.95 with the 24-bit tangent.
 // False (with M's triangle to be loaded again) when M is not semidefinite to
-// rounding, or its diagonal spans more than 100 binades, where small entries
+// rounding (a row that is dropped keeps an entry above 2^-100 of the diagonal's
+// scale, or its diagonal entry is negative by more), or its diagonal spans more than 100 binades, where small entries
 // need exponents of their own.
 __device__ bool onesided_jacobi(int k, const Wide::Vec A, const Wide::Vec U, DevStatus* st) {
   __shared__ int E[KMAX], ref[KMAX], pos[KMAX], col[KMAX];
@@ -804,6 +805,17 @@ __device__ bool onesided_jacobi(int k, const Wide::Vec A, const Wide::Vec U, Dev
       const int p = 63 - (int)((good ? best : best - 1) & 63ull);
       const wide d = A.get(tri(p, p));
       const bool ok = good && Wide::pivot_ok(d, ref[p]);
+      if (!ok) {
+        // nothing left of the row but rounding?  (of a semidefinite M a diagonal
+        // entry of zero leaves a row of zeros)
+        bool rest = false;
+        for (int i = lane; i < k; i += 32) {
+          if (pos[i] != k || i == p) continue;
+          const wide a = A.get(sym(i, p));
+          rest |= !wide_is_zero(a) && 2 * a.e > ref[i] + ref[p] - 200;
+        }
+        if (__any_sync(0xffffffffu, rest) && lane == 0) state = 1;
+      }
       if (lane == 0) {
         piv = ok ? p : -1;
         pos[p] = step;
