@@ -315,6 +315,20 @@ FX_HD double w_to_double(i128 w, int S) {
   return from_bits(((unsigned long long)neg << 63) | ((unsigned long long)be << 52) | (m & ((1ull << 52) - 1)));
 }
 
+// Nearest float to w * 2^S (ties to even), subnormals and overflow included: w
+// rounded to odd in 53 bits, which a second rounding to 24 bits or fewer
+// cannot tell from w itself.
+FX_HD float w_to_float(i128 w, int S) {
+  if (w == 0) return 0.0f;
+  const u128 u = w < 0 ? (u128)(-w) : (u128)w;
+  const int lz = clz128(u);
+  const u128 v = u << lz;  // top bit at 127
+  const unsigned long long t = (unsigned long long)(v >> 64);
+  const unsigned long long m = (t >> 11) | (unsigned long long)((t & 0x7ffull) != 0ull || (unsigned long long)v != 0ull);
+  const float f = (float)ldexp((double)m, S + 75 - lz);
+  return w < 0 ? -f : f;
+}
+
 // Double-double (hi, lo) nearest to w * 2^S: hi = RN(w 2^S), lo = RN(w 2^S - hi).
 FX_HD void w_to_dd(i128 w, int S, double& hi, double& lo) {
   if (w == 0) {

@@ -359,6 +359,9 @@ constexpr int kRoundSide = W >= 16 ? 1 : 4;
 constexpr int kNaNExp = 1 << 24;
 // The general exact rounding (rare inputs the lean forms leave),
 // kept out of line so that the kernels' code stays small.
+__device__ __noinline__ float round_general_f32(i128 h, int S) {
+  return S >= kNaNExp / 2 ? __int_as_float(0x7fc00000) : w_to_float(h, S);
+}
 __device__ __noinline__ double round_general(bool update, double y, i128 h, int S) {
   if (S >= kNaNExp / 2) return __longlong_as_double(0x7ff8000000000000ll);
   bool ok;
@@ -635,9 +638,12 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
           for (int y = y0; y < y0 + kSide && y < ny; ++y) {
             if constexpr (kSide == 1) g[y] = h[y];
-            if (left >> y & 1u)
-              o[y - y0] = (Real)round_general(UPDATE, UPDATE ? 0.0 : Yin[(size_t)(j0 + y) * ldyin + grow],
-                                        (i128)(g[y] - kOffset), Sr + Bexp[j0 + y]);
+            if (left >> y & 1u) {
+              const i128 w = (i128)(g[y] - kOffset);
+              const int S = Sr + Bexp[j0 + y];
+              if constexpr (sizeof(Real) == 4) o[y - y0] = round_general_f32(w, S);
+              else o[y - y0] = round_general(UPDATE, UPDATE ? 0.0 : Yin[(size_t)(j0 + y) * ldyin + grow], w, S);
+            }
           }
         }
 #pragma unroll
