@@ -65,7 +65,10 @@
 //
 // FP32 updates (kin <= 32) take the same path with seven near slabs (24 bits
 // and the near window); their outputs are rounded from the exact sum to FP32.
-// 2e6 x 32: 4.0 ms on the FP64 pipe -> 0.57 ms.
+// 2e6 x 32: 4.0 ms on the FP64 pipe -> 0.57 ms.  Rows with a non-finite value, or
+// with one that the 110 bits of the row's grid do not hold, are summed in FP64
+// (plain_rows), so an Inf or NaN reaches the outputs whose sums it is part of
+// (every row like that: 2e6 x 32 3.6 ms a call, all on the FP64 pipe 4.1).
 #include <cuda_fp16.h>
 
 #include <algorithm>
@@ -353,9 +356,9 @@ __device__ __forceinline__ i128 fixed_trunc(double x, int A) {
 // tile's values stand in registers meanwhile (kin = 64).
 template <int W>
 constexpr int kRoundSide = W >= 16 ? 1 : 4;
-// Added to the exponent of a row or a column with a non-finite value, and to a
-// row's when a wait has run out: no lean rounding takes it, and the general one
-// answers NaN.
+// Added to the exponent of a row or a column with a non-finite value (FP32 rows:
+// of one that plain_rows takes), and to a row's when a wait has run out: no lean
+// rounding takes it, and the general one answers NaN.
 constexpr int kNaNExp = 1 << 24;
 // The general exact rounding (rare inputs the lean forms leave),
 // kept out of line so that the kernels' code stays small.
@@ -368,6 +371,30 @@ __device__ __noinline__ double round_general(bool update, double y, i128 h, int 
   const double o = update ? w_to_double_fast(h, S, ok) : sub_round_fast(y, h, S, ok);
   if (ok) return o;
   return update ? w_to_double(h, S) : sub_round(y, h, S);
+}
+
+// FP32 rows that the digits do not hold (k <= KM), summed in FP64 as update.cu
+// does: the four lanes of a row (cg) read all of it before one of them stores, and
+// take every fourth output.  Called by whole warps; rare, so out of line.
+template <int KM, bool TRI>
+__device__ __noinline__ void plain_rows(int k, const float* A, int64_t lda, const double* __restrict__ B, int ldb,
+                                        float* Out, int64_t ldo, int cg, bool mine) {
+  double x[KM];
+#pragma unroll
+  for (int i = 0; i < KM; ++i) x[i] = mine && i < k ? (double)A[(size_t)i * lda] : 0.0;
+  __syncwarp();
+  if (!mine) return;
+#pragma unroll
+  for (int j4 = 0; j4 < KM; j4 += 4) {
+    const int j = j4 + cg;
+    if (j >= k) break;
+    const double* b = B + (size_t)j * ldb;
+    double s = 0.0;
+#pragma unroll
+    for (int i = 0; i < (TRI ? j4 + 4 : KM); ++i)
+      if (TRI ? i <= j : i < k) s = __fma_rn(x[i], b[i], s);
+    Out[(size_t)j * ldo] = (float)s;
+  }
 }
 
 // KP = 4 W: the K dimension (kin padded to 16, 32 or 64; padded columns
@@ -548,7 +575,8 @@ __global__ void __launch_bounds__(kThreads, 1)
       const int j0 = ob * kOut + ep * ny;
       if (j0 >= kout) return;  // all outputs of this warp are padding (warp-uniform)
       const unsigned tb = tq + (unsigned)(KO > 1 ? ob : (int)(i & 1)) * kAccCols + (unsigned)(ep * ny);
-      const int64_t grow = T * kRows + L;
+      // (FP32: a row of plain_rows stands beyond the matrix)
+      const int64_t grow = sizeof(Real) == 4 && Arow[(i & 1) * kRows + L] >= kNaNExp ? n : T * kRows + L;
       double yv[ny];
       {
         const Real* Yp = Yin + (size_t)j0 * ldyin + grow;
@@ -703,6 +731,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
         for (int k = 0; k < W; ++k) below |= abs_hi(v[k]) < floor && (abs_hi(v[k]) | lo32(v[k])) != 0u;
       }
+      if constexpr (sizeof(Real) == 4) below |= nonfinite;  // (looked at again where all digits are cut)
       return below;
     };
     const unsigned e1024 = exp1024x2();
@@ -724,7 +753,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     int64_t Tprev = -1, iprev = 0;
     for (int64_t T = blockIdx.x, i = 0; T < ntiles; T += gridDim.x, ++i) {
       if (cg == 0) {
-        Arow[(i & 1) * kRows + r] = Ar + (nonfinite ? kNaNExp : 0);
+        Arow[(i & 1) * kRows + r] = Ar + (nonfinite && sizeof(Real) == 8 ? kNaNExp : 0);
       }
       if (all && tid == 0) *reinterpret_cast<volatile int*>(&far[i & 1]) = (int)i;
       const int ng = all ? kGroupsAll : kGroupsNear;
@@ -763,6 +792,17 @@ __global__ void __launch_bounds__(kThreads, 1)
         group(1, [&](unsigned dst) { store_near<1, NEAR - kGroup, W>(dst, SLAB_A, z, sg, e1024); });
       } else if constexpr (W <= 8) {
         unsigned y[W / 2][7];
+        [[maybe_unused]] bool plain = false;  // FP32: the row goes through plain_rows
+        if constexpr (sizeof(Real) == 4) {
+          // (24 bits that begin more than 86 binades below the row's largest reach
+          // below the digits' last bit)
+          const unsigned last = (unsigned)max(Ar - 86, 0) << 20;
+#pragma unroll
+          for (int k = 0; k < W; ++k) plain |= abs_hi(v[k]) < last && abs_hi(v[k]) != 0u;
+          plain |= __shfl_xor_sync(0xffffffffu, plain, 8);
+          plain |= __shfl_xor_sync(0xffffffffu, plain, 16);
+          plain |= nonfinite;
+        }
 #pragma unroll
         for (int m = 0; m < W / 2; ++m) any_lanes(v[2 * m], v[2 * m + 1], Ar, y[m], sg[m]);
 #pragma unroll 1
@@ -772,6 +812,15 @@ __global__ void __launch_bounds__(kThreads, 1)
             else if (g == 1) store_any<1, W>(dst, SLAB_A, y, sg, e1024);
             else store_any<2, W>(dst, SLAB_A, y, sg, e1024);
           });
+        if constexpr (sizeof(Real) == 4) {
+          // (the tile's values stand in memory until its epilogue, which passes these rows over)
+          if (__any_sync(0xffffffffu, plain)) {
+            const int64_t gr = T * kRows + r;
+            if (tri) plain_rows<KP, true>(kin, A + gr, lda, Bh, ldb, Out + gr, ldo, cg, plain && gr < n);
+            else plain_rows<KP, false>(kin, A + gr, lda, Bh, ldb, Out + gr, ldo, cg, plain && gr < n);
+            if (plain && cg == 0) Arow[(i & 1) * kRows + r] = Ar + kNaNExp;
+          }
+        }
       } else {
         double u[W];
 #pragma unroll
