@@ -68,7 +68,8 @@
 // 2e6 x 32: 4.0 ms on the FP64 pipe -> 0.57 ms.  Rows with a non-finite value, or
 // with one that the 110 bits of the row's grid do not hold, are summed in FP64
 // (plain_rows), so an Inf or NaN reaches the outputs whose sums it is part of
-// (every row like that: 2e6 x 32 3.6 ms a call, all on the FP64 pipe 4.1).
+// (every row like that: 2e6 x 32 3.6 ms a call, all on the FP64 pipe 4.1), and
+// all rows are when the columns' norms differ by more than 2^40 (kUneven).
 #include <cuda_fp16.h>
 
 #include <algorithm>
@@ -373,6 +374,14 @@ __device__ __noinline__ double round_general(bool update, double y, i128 h, int 
   return update ? w_to_double(h, S) : sub_round(y, h, S);
 }
 
+// FP32: binades between the largest entries of Z's rows beyond which all rows go
+// through plain_rows.  Z = R^{-1} or M^{-1/2} of X = U D (columns of norm 1 times
+// their norms d_i) has rows of about 1 / d_i, times at most kappa(U) < 2^27 (the
+// largest that an FP64 Cholesky takes), while a digit sum is off by up to 2^-98
+// max_i |x_ri| max_i |z_ij| <= 2^-98 max d max_i |z_ij| <= 2^(40 + 27 - 98) of a column
+// of norm 1: below the FP32 rounding, and 2^-57 of it for a well-conditioned U.
+constexpr int kUneven = 40;
+
 // FP32 rows that the digits do not hold (k <= KM), summed in FP64 as update.cu
 // does: the four lanes of a row (cg) read all of it before one of them stores, and
 // take every fourth output.  Called by whole warps; rare, so out of line.
@@ -431,6 +440,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   __shared__ __align__(8) unsigned long long full_bar[2], ready_bar[2], tfree_bar;
   __shared__ unsigned tmem_base;
   __shared__ int bad;
+  // FP32: the largest exponent of each row of the small matrix; whether it is too uneven for the digits
+  [[maybe_unused]] __shared__ int zrow[32], uneven;
   __shared__ int far[2];  // far[i & 1] = i: the CTA's tile i needs all digits (set before the arrivals for its first group)
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -448,6 +459,11 @@ __global__ void __launch_bounds__(kThreads, 1)
     bad = 0;
     far[0] = far[1] = -1;
   }
+  if constexpr (sizeof(Real) == 4) {
+    if (tid < 32) zrow[tid] = 0;
+    if (tid == 0) uneven = 0;
+    __syncthreads();
+  }
   // column exponents, a warp to a column (one round of loads: a thread to a
   // column, one load after another, made a launch of 64 x 16 10 us longer)
   for (int j = warp; j < NOUT; j += kThreads / 32) {
@@ -458,6 +474,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (tri && i > j) continue;
         const int ae = align_exp(Bh[(size_t)j * ldb + i]);
         e = max(e, ae);
+        if constexpr (sizeof(Real) == 4) atomicMax(&zrow[i], ae);
         nf |= ae == 2047 || (Bl && align_exp(Bl[(size_t)j * ldb + i]) == 2047);
       }
     }
@@ -465,8 +482,19 @@ __global__ void __launch_bounds__(kThreads, 1)
     nf = __any_sync(0xffffffffu, nf);
     // one binade of headroom: |h + l| may round up past the largest h
     if (lane == 0) Bexp[j] = e + 1 + (nf ? kNaNExp : 0);
+    if constexpr (sizeof(Real) == 4) {
+      if (nf) uneven = 1;
+    }
   }
   __syncthreads();
+  if constexpr (sizeof(Real) == 4) {
+    if (warp == 0) {
+      const int e = lane < kin ? zrow[lane] : 0;
+      const int hi = (int)__reduce_max_sync(0xffffffffu, (unsigned)e);
+      const int lo = (int)__reduce_min_sync(0xffffffffu, e ? (unsigned)e : 4095u);
+      if (lane == 0 && hi - lo > kUneven) uneven = 1;
+    }
+  }
   for (int e = tid; e < NOUT * KP; e += kThreads) {  // block j / 16: B row R = t * 16 + j % 16 (slab t), K index i
     const int j = e / KP, i = e % KP;
     i128 x = 0;
@@ -491,7 +519,17 @@ __global__ void __launch_bounds__(kThreads, 1)
   const unsigned fb0 = smem_u32(&full_bar[0]), rb0 = smem_u32(&ready_bar[0]), tfb = smem_u32(&tfree_bar);
   const unsigned adig_s = smem_u32(adig), bdig_s = smem_u32(bdig);
 
-  if (warp == kConvWarps) {
+  if (sizeof(Real) == 4 && uneven) {
+    // ---------------- FP32, columns of X too uneven for the digits: every row in FP64
+    if constexpr (sizeof(Real) == 4) {
+      const int64_t r = (int64_t)warp * 8 + (lane & 7);
+      for (int64_t T = blockIdx.x; T < ntiles && warp < kConvWarps; T += gridDim.x) {
+        const int64_t gr = T * kRows + r;
+        if (tri) plain_rows<KP, true>(kin, A + gr, lda, Bh, ldb, Out + gr, ldo, lane >> 3, gr < n);
+        else plain_rows<KP, false>(kin, A + gr, lda, Bh, ldb, Out + gr, ldo, lane >> 3, gr < n);
+      }
+    }
+  } else if (warp == kConvWarps) {
     // ---------------- MMA issuer
     if (lane == 0) {
       int G = 0;  // groups issued

@@ -67,3 +67,29 @@ def test_values_far_below_their_row(eo, ctx, k):
     _, _, info = eo.cholqr(ctx, d, passes=1, prec=eo.F32, M=(dev(np.eye(k)), dev(np.zeros((k, k)))))
     assert int(info) == 0
     assert np.array_equal(d.cpu().numpy(), x)
+
+
+@pytest.mark.parametrize("method", ["cholqr", "svqb"])
+@pytest.mark.parametrize("decades", [-30, -24, -16, -8, 8, 16, 24, 30])
+@pytest.mark.parametrize("k", [9, 16, 32])
+def test_columns_of_widely_different_norms(eo, ctx, method, decades, k):
+    """Columns of norms spread over the FP32 range, falling and rising, otherwise
+    well conditioned.  Q is R^-1 of FP64 applied to X and rounded to FP32: every
+    entry to 2^-23 and 2^-30 of its column's largest (R^-1 is formed here in FP64).
+    SVQB's rank counts the eigenvalues above k 2^-52 of the largest."""
+    n = 20_000
+    s = 10.0 ** (np.linspace(0, decades, k) - min(decades, 0) * 0.5 - max(decades, 0) * 0.5)
+    x = (synth.conditioned(n, k, 3.0, 6900 + k) * s).astype(np.float32)
+    d = dev(x)
+    if method == "cholqr":
+        rh, _, info = eo.cholqr(ctx, d, passes=1, prec=eo.F32)
+        assert int(info) == 0
+        q = d.double().cpu().numpy()
+        want = fp64_update(x, np.linalg.inv(rh.cpu().numpy()), True)
+        assert np.max(np.abs(q.T @ q - np.eye(k))) <= 2.0 ** -18
+        assert np.all(np.abs(q - want) <= 2.0 ** -23 * np.abs(want) + 2.0 ** -30 * np.abs(want).max(0))
+    else:
+        _, _, rank = eo.svqb(ctx, d, passes=1, prec=eo.F32)
+        lam = np.linalg.svd(x.astype(np.float64), compute_uv=False) ** 2
+        assert int(rank) <= np.sum(lam > 0.5 * k * 2.0 ** -52 * lam[0]) and int(rank) >= np.sum(lam > 2 * k * 2.0 ** -52 * lam[0])
+        assert np.all(np.isfinite(d.cpu().numpy()))
