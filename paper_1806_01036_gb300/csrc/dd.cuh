@@ -9,11 +9,8 @@
 //   two_prod      TwoProd with a fused multiply-add (2 flops)
 //   dd_add        Joldes-Muller-Popescu 2017, "AccurateDWPlusDW"
 //   dd_mul        Joldes-Muller-Popescu 2017, "DWTimesDW3"
-//   dd_mul_d      Joldes-Muller-Popescu 2017, "DWTimesFP3"
-//   dd_div        Newton-Raphson (Karp-Markstein) correction of the FP64
-//                 quotient, carried out in DD, as the paper prescribes for
-//                 divisions and square roots
-//   dd_sqrt       one Newton-Raphson (Karp-Markstein) step from the FP64 root
+//   dd_sqrt       one Newton-Raphson (Karp-Markstein) step from the FP64 root,
+//                 as the paper prescribes for divisions and square roots
 // The explicit __dadd_rn/__dmul_rn/__fma_rn intrinsics keep the compiler from
 // contracting or reassociating any step.
 #pragma once
@@ -69,12 +66,6 @@ __device__ __forceinline__ dd dd_mul(dd x, dd y) {
   return fast_two_sum(c.hi, cl3);
 }
 
-__device__ __forceinline__ dd dd_mul_d(dd x, double y) {
-  dd c = two_prod(x.hi, y);
-  double cl3 = __fma_rn(x.lo, y, c.lo);
-  return fast_two_sum(c.hi, cl3);
-}
-
 // Accumulate the exact product a*b into the DD sum s (Ogita-Rump-Oishi Dot2
 // step: TwoProd, TwoSum of the high parts, low parts summed in FP64).
 __device__ __forceinline__ void dd_fma_acc(dd& s, double a, double b) {
@@ -97,20 +88,6 @@ __device__ __forceinline__ void dd_fma_acc_dd(dd& s, dd x, double b) {
 // Renormalize an accumulator so that |lo| <= ulp(hi)/2 (TwoSum: after
 // cancellation the low part of a Dot2 accumulator may exceed the high part).
 __device__ __forceinline__ dd dd_norm(dd s) { return two_sum(s.hi, s.lo); }
-
-// q = x / y: FP64 quotient, then two Newton-Raphson corrections
-// q <- q + (x - y q) / y with the residual evaluated in DD.
-__device__ __forceinline__ dd dd_div(dd x, dd y) {
-  double q0 = __ddiv_rn(x.hi, y.hi);
-  dd r = dd_sub(x, dd_mul_d(y, q0));
-  double q1 = __ddiv_rn(r.hi, y.hi);
-  dd q = fast_two_sum(q0, q1);
-  dd r2 = dd_sub(x, dd_mul(y, q));
-  double q2 = __ddiv_rn(r2.hi, y.hi);
-  return dd_add(q, dd_make(q2));
-}
-
-__device__ __forceinline__ dd dd_recip(dd y) { return dd_div(dd_make(1.0), y); }
 
 // sqrt(x) for x > 0: s = sqrt(x.hi), then s + (x - s^2) / (2 s) in DD.
 __device__ __forceinline__ dd dd_sqrt(dd x) {

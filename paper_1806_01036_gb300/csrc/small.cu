@@ -39,25 +39,20 @@ constexpr int kJacThreads = 512;
 constexpr double kJacobiEpsDD = 0x1p-100;
 constexpr double kJacobiEpsFP64 = 0x1p-48;
 
+// Double-double (or FP64) arithmetic of the pivoted Cholesky.
 template <int MODE>
 struct Ar {
-  static __device__ __forceinline__ dd add(dd a, dd b) { return dd{__dadd_rn(a.hi, b.hi), 0.0}; }
   static __device__ __forceinline__ dd sub(dd a, dd b) { return dd{__dsub_rn(a.hi, b.hi), 0.0}; }
   static __device__ __forceinline__ dd mul(dd a, dd b) { return dd{__dmul_rn(a.hi, b.hi), 0.0}; }
-  static __device__ __forceinline__ dd div(dd a, dd b) { return dd{__ddiv_rn(a.hi, b.hi), 0.0}; }
   static __device__ __forceinline__ dd sqrt(dd a) { return dd{__dsqrt_rn(a.hi), 0.0}; }
   static __device__ __forceinline__ dd fma(dd a, dd b, dd c) { return dd{__fma_rn(a.hi, b.hi, c.hi), 0.0}; }
   static __device__ __forceinline__ dd recip(dd a) { return dd{__drcp_rn(a.hi), 0.0}; }
-  static __device__ __forceinline__ dd dot2(dd a, dd x, dd b, dd y) { return add(mul(a, x), mul(b, y)); }
-  static __device__ __forceinline__ dd rsqrt(dd a) { return dd{__ddiv_rn(1.0, __dsqrt_rn(a.hi)), 0.0}; }
 };
 
 template <>
 struct Ar<MODE_DD> {
-  static __device__ __forceinline__ dd add(dd a, dd b) { return dd_add(a, b); }
   static __device__ __forceinline__ dd sub(dd a, dd b) { return dd_sub(a, b); }
   static __device__ __forceinline__ dd mul(dd a, dd b) { return dd_mul(a, b); }
-  static __device__ __forceinline__ dd div(dd a, dd b) { return dd_div(a, b); }
   static __device__ __forceinline__ dd sqrt(dd a) { return dd_sqrt(a); }
   static __device__ __forceinline__ dd fma(dd a, dd b, dd c) { return dd_add(dd_mul(a, b), c); }
   // 1/a for a > 0: y0 = RN(1/a.hi), whose residual 1 - a.hi y0 is exact in
@@ -68,33 +63,6 @@ struct Ar<MODE_DD> {
     double e = __fma_rn(-a.hi, y0, 1.0);
     e = __fma_rn(-a.lo, y0, e);
     return fast_two_sum(y0, y0 * __fma_rn(e, e, e));
-  }
-  // a x + b y: the two leading products exactly, their sum exactly, the
-  // cross terms by FMAs into the low part, one renormalization.  The error
-  // is about 2^-104 (|a x| + |b y|), not relative to the result: enough for
-  // a plane rotation, whose rounding errors count against the norm of what
-  // it rotates (and it costs about 22 FP64 operations, against 34 for two
-  // products and an accurate sum).
-  static __device__ __forceinline__ dd dot2(dd a, dd x, dd b, dd y) {
-    const dd p = two_prod(a.hi, x.hi), q = two_prod(b.hi, y.hi);
-    const dd h = two_sum(p.hi, q.hi);
-    double lo = __dadd_rn(p.lo, q.lo);
-    lo = __fma_rn(a.hi, x.lo, lo);
-    lo = __fma_rn(a.lo, x.hi, lo);
-    lo = __fma_rn(b.hi, y.lo, lo);
-    lo = __fma_rn(b.lo, y.hi, lo);
-    return two_sum(h.hi, __dadd_rn(h.lo, lo));
-  }
-  // 1/sqrt(a) for a > 0: y0 = RN(1/RN(sqrt(a.hi))); r = 1 - a y0^2 to about
-  // 2^-105 (y0^2 and a.hi y0^2 split exactly, 1 - hi exact as hi is near 1);
-  // 1/sqrt(a) = y0 (1 - r)^(-1/2) = y0 (1 + r/2 + 3 r^2/8 + ...), |r| < 2^-50.
-  static __device__ __forceinline__ dd rsqrt(dd a) {
-    const double y0 = __drcp_rn(__dsqrt_rn(a.hi));
-    const dd q = two_prod(y0, y0), p = two_prod(a.hi, q.hi);
-    double r = __dsub_rn(__dsub_rn(1.0, p.hi), p.lo);
-    r = __fma_rn(-a.hi, q.lo, r);
-    r = __fma_rn(-a.lo, q.hi, r);
-    return fast_two_sum(y0, y0 * __fma_rn(0.375 * r, r, 0.5 * r));
   }
 };
 

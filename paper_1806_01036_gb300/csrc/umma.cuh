@@ -92,11 +92,7 @@ static inline cudaError_t take_wait_record(unsigned* out) {
 __device__ __forceinline__ void mbar_arrive(unsigned bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
-// Barrier 1 among the NT threads of the converter warps only.
-template <int NT>
-__device__ __forceinline__ void bar_conv() {
-  asm volatile("bar.sync 1, %0;" ::"n"(NT) : "memory");
-}
+// Barrier 1 among the NT threads of the converter warps only, true if any of them passes true.
 template <int NT>
 __device__ __forceinline__ bool bar_conv_or(bool v) {
   unsigned r;

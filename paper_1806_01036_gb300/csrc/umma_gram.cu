@@ -8,7 +8,7 @@
 //  * each value x of a column is aligned to the column's alignment exponent
 //    A and held as X = floor(|x| 2^(1132 - A)) < 2^110, written with 14
 //    balanced base-256 digits, X = sum_s D_s 2^(104 - 8s), D_s in [-128, 127]
-//    (D_0 in [0, 65]; the fields of X + sum_s 128 2^(104 - 8s), less 128);
+//    (D_0 in [0, 64]; the fields of X + sum_s 128 2^(104 - 8s), less 128);
 //  * a digit is the FP16 integer sign(x) D_s, so a product of two digits is
 //    an integer of at most 2^14 and FP32 sums of up to 1024 such products are
 //    exact;
