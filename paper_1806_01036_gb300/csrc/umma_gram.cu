@@ -442,11 +442,9 @@ __global__ void __launch_bounds__(kThreads, 1)
   auto unit = [&](int p, int u) {
     return (unsigned)(p & 1) * G::stage_bytes + item + (((unsigned)(4 * (kc & 1) + u) ^ (unsigned)(lc & 7)) << 4);
   };
-  [[maybe_unused]] int fetched = 0;  // panels whose copies were issued (the thread that fetches)
   auto fetch = [&](int p) {
     if constexpr (TMA) {
       if (tid == kIssuer) {
-        fetched = p + 1;
         const unsigned bar = sb0 + 8u * (unsigned)(p & 1), dst = stage_s + (unsigned)(p & 1) * G::stage_bytes;
         const int xr = (int)(r0 + (int64_t)p * P);
         fence_proxy_async();
@@ -532,13 +530,15 @@ __global__ void __launch_bounds__(kThreads, 1)
     below = __any_sync(0xffffffffu, low);
     return up;
   };
-  // the values of a panel that `below` holds for, and the lane words of their
-  // digits 10..13; touched rarely, so they are kept out of registers
+  // the values of a panel that `below` holds for, the lane words of their digits
+  // 10..13, and the barriers passed in the panel loop; touched rarely, so they are
+  // kept out of registers
   struct {
     double v[8];
-    unsigned low[8];
+    unsigned low[8], syncs;
   } rare_, *rare = &rare_;
   asm volatile("" : "+l"(rare)::"memory");
+  rare->syncs = 0;
   if (npan > 0) {
     fetch(0);
     if (!TMA || npan > 1) fetch(1);
@@ -575,7 +575,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   asm volatile("" : "+l"(tot)::"memory");
   for (int y = 0; y < kParts * NY; ++y) tot[y] = 0;
   // bits of h that a total drops: 127 hold the sum of the chunk's rows (PACK: of all parts)
-  const int drop = fold_bits((unsigned)rows_per_chunk * (PACK ? 16u >> lg : 1u));
+  auto drop = [&]() { return fold_bits((unsigned)rows_per_chunk * (PACK ? 16u >> lg : 1u)); };
 
   // the running sums and, first, the accumulators at zero (this warp's share of the column blocks)
   auto zero_blocks = [&](unsigned t) {
@@ -633,12 +633,10 @@ __global__ void __launch_bounds__(kThreads, 1)
   // wait for the MMAs of step s (committed to its buffer's barrier)
   // Barrier of the panel loop over all warps, bounded like every wait in it, so
   // that warps which a wait that ran out has sent out of the loop hold up nobody.
-  int syncs = 0;
   auto sync_all = [&]() {
     __syncwarp();
     if (lane == 0) mbar_arrive(smem_u32(&cta_bar));
-    mbar_wait(smem_u32(&cta_bar), (unsigned)syncs & 1u, &bad);
-    ++syncs;
+    mbar_wait(smem_u32(&cta_bar), rare->syncs++ & 1u, &bad);
   };
   auto wait_step = [&](int s) { mbar_wait(fb0 + 8u * (unsigned)(s & 1), (unsigned)(s >> 1) & 1u, &bad); };
   // Empties the accumulators (after the MMAs of the steps before s) and, when
@@ -653,7 +651,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       tc_fence_before();
       sync_all();
       tc_fence_after();
-      fold<G, false>(tsum, jl, 8 * jl + drop, tot);
+      fold<G, false>(tsum, jl, 8 * jl + drop(), tot);
       tc_fence_before();
       sync_all();
       tc_fence_after();
@@ -730,8 +728,9 @@ __global__ void __launch_bounds__(kThreads, 1)
   }
   __syncthreads();
   if (TMA && npan > 2) fetch(2);  // (TMA: panel 0's values are in registers)
+  int p = 0;
 #pragma unroll 1
-  for (int p = 0; p < npan; ++p) {
+  for (; p < npan; ++p) {
     unsigned z[4][5];
     Sign2 sg[4];
     bool up = false, cut_all = below;
@@ -878,13 +877,14 @@ __global__ void __launch_bounds__(kThreads, 1)
   if (tid == kIssuer && *reinterpret_cast<volatile int*>(&bad)) {
     // after a wait that ran out: this thread's own MMAs and copies end before TMEM and shared memory are released
     if (step > 0) mbar_wait_final(fb0 + 8u * (unsigned)((step - 1) & 1), (unsigned)((step - 1) >> 1) & 1u, &bad);
-    for (int q = max(fetched - 2, 0); q < fetched; ++q) mbar_wait_final(sb0 + 8u * (unsigned)(q & 1), (unsigned)(q >> 1) & 1u, &bad);
+    // (at panel p the copies before panel p + 2 are issued, one phase of each buffer's barrier unwaited at most)
+    for (int f = min(p + 2, npan), q = max(f - 2, 0); TMA && q < f; ++q) mbar_wait_final(sb0 + 8u * (unsigned)(q & 1), (unsigned)(q >> 1) & 1u, &bad);
   }
   if (step > 0) {
     if (warp == 0) mbar_wait_final(fb0 + 8u * (unsigned)((step - 1) & 1), (unsigned)((step - 1) >> 1) & 1u, &bad);
     wait_step(step - 1);
     tc_fence_after();  // (the drains' running sums: before the barrier above)
-    fold<G, true>(tsum, jl, 8 * jl + drop, tot);
+    fold<G, true>(tsum, jl, 8 * jl + drop(), tot);
     tc_fence_before();
   }
   __syncthreads();
@@ -910,7 +910,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     FxPart o;
     o.wl = (long long)(unsigned long long)(u128)w;
     o.wh = (long long)(w >> 64);
-    o.s = max(Erun[i], 1) + max(Erun[(SHARED ? 0 : KXP) + yo], 1) - kOffsetDigits + drop;
+    o.s = max(Erun[i], 1) + max(Erun[(SHARED ? 0 : KXP) + yo], 1) - kOffsetDigits + drop();
     o.flag = flag | bad;
     o.pad = 0;
     return o;

@@ -11,7 +11,7 @@ SRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), 
 
 def test_panel_loop_has_bounded_waits_only():
     text = re.sub(r"//[^\n]*", "", open(SRC).read())
-    loop = text[text.index("for (int p = 0; p < npan; ++p) {"):]
+    loop = text[text.index("for (; p < npan; ++p) {"):]
     depth = 0
     for i, c in enumerate(loop):
         depth += (c == "{") - (c == "}")
