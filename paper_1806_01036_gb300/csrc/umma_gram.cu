@@ -88,7 +88,7 @@
 // f16x2 FMA on the other pipe each) where 7-bit digits took three, and ten
 // stored slabs instead of fifteen.  Measured, 4e6 rows against the 7-bit form
 // (15 slabs, items of two rows, 19 converter warps): V^T Y 64 x 16 1.41 -> 1.04
-// ms (2.5 TB/s), X^T X 16 columns 0.395 -> 0.283, 64 columns (strips) 4.6 ->
+// ms (2.5 TB/s), X^T X 16 columns 0.395 -> 0.264, 64 columns (strips) 4.6 ->
 // 3.06.  Tried and slower: loads straight into registers (each 128-bit load
 // costs 20 wavefronts of the shared data pipe: 1.30 ms), one bulk copy per
 // column (80 a panel: 2.41 ms), four warps that only drain (each drain takes

@@ -44,7 +44,7 @@
 // are NaN).  Each tile's loads precede its own stores, and no tile is written
 // by another CTA, so the update may run in place.
 //
-// Bound by the integer pipe (62% busy over a kernel, saturated inside the
+// Bound by the integer pipe (57% busy over a kernel, saturated inside the
 // conversion and the epilogue): 131 instructions an output and 40 to 60 a
 // value; memory needs a third of the time.  Y - V C of 4e6 rows, with 7-bit
 // digits and 128-bit roundings (280 instructions an output), then with 8-bit
