@@ -134,7 +134,8 @@ cudaError_t launch_fx_gram(int64_t n, int kx, const double* X, int64_t ldx, int 
 // kin <= 64, kout <= 16 (umma_rowprod_supported); Out may be A (in place).
 // ctas > 0 caps the CTAs of the launch (0 = one per SM).
 bool umma_rowprod_supported(int64_t n, int kin, int kout);
-// X = X Z in place for FP32 X, k <= 32: the exact sums rounded once to FP32.
+// X = X Z in place for FP32 X, k <= 32: the exact sums rounded once to FP32 (rows
+// that the digits do not hold: FP64 sums).
 cudaError_t launch_umma_update_f32(int64_t n, int k, float* X, int64_t ldx, const double* Zh, const double* Zl, int ldz,
                                    bool tri, const int* gate, cudaStream_t st);
 // Bounded device-side waits that ran out (tensor-core kernels): each unit's
